@@ -192,3 +192,97 @@ def tolerance(case):
     if kind == "prepare":
         return {"rel": 1.2e-7 if case["dtype"] == "fp32" else 7e-3}
     return {"rel": 9.5e-3}
+
+
+def _inverse(A, C):
+    """The scheme's inverse of I + A in fp64 (A strictly lower triangular, [..., C, C]): band-masked Neumann sum of order N, then
+    T0 (I + E + ... + E^S); 128 tokens as two 64-blocks and the block formula for the lower-left one."""
+    if C == 128:
+        T = torch.zeros_like(A)
+        T11, T22 = _inverse(A[..., :64, :64], 64), _inverse(A[..., 64:, 64:], 64)
+        T[..., :64, :64], T[..., 64:, 64:] = T11, T22
+        T[..., 64:, :64] = -T22 @ A[..., 64:, :64] @ T11
+        return T
+    N = min(3, C - 1)
+    S = {16: 3, 32: 4, 64: 8}.get(C, max(0, (C + 3) // 4 - 1))
+    eye = torch.eye(C, dtype=A.dtype, device=A.device)
+    P, T0 = -A, eye - A
+    for _ in range(N - 1):
+        P = P @ -A
+        T0 = T0 + P
+    T0 = T0.tril().triu(-N)
+    E = eye - (eye + A) @ T0
+    X = eye.expand_as(E)
+    for _ in range(S):  # Horner: I + E (I + E (...))
+        X = eye + E @ X
+    return T0 @ X
+
+
+def _chunks(K, V, beta, g, C, gated=False):
+    """W, U and the inverse of chunks K, V [..., C, d], beta and cumulative g [..., C], all fp64."""
+    decay = (g[..., :, None] - g[..., None, :]).tril(-1).exp().tril(-1)
+    T = _inverse(beta[..., :, None] * decay * (K @ K.transpose(-1, -2)), C)
+    w = beta * g.exp() if gated else beta
+    return T @ (w[..., None] * K), T @ (beta[..., None] * V), T
+
+
+def _exact_prepare(case, st):
+    B, H_k, H_v, T, C, d = (case[k] for k in ("B", "H_k", "H_v", "T", "C", "d"))
+    n, r = T // C, H_v // H_k
+
+    def empty(*shape):
+        return torch.empty(*shape, dtype=torch.float64, device="cuda")
+
+    W, U, Ti = empty(B, H_v, n, C, d), empty(B, H_v, n, C, d), empty(B, H_v, n, C, C)
+    for b in range(B):
+        for h in range(H_v):
+            W[b, h], U[b, h], Ti[b, h] = _chunks(*(x.double().view(n, C, -1) for x in (st["K"][b, h // r], st["V"][b, h])),
+                                                 *(x.double().view(n, C) for x in (st["beta"][b, h], st["g"][b, h])), C)
+    return W.view(B, H_v, T, d), U.view(B, H_v, T, d), Ti
+
+
+def _unit(x):
+    x = x.double()
+    return x / x.norm(dim=-1, keepdim=True).clamp_min(1e-300)
+
+
+def _exact_layer(case, st):
+    H_k, H_v, C = case["H_k"], case["H_v"], case["C"]
+    dense = case["kind"] == "layer"
+    Q, K, V, beta, g = (st[k].flatten(0, 1) if dense else st[k] for k in ("Q", "K", "V", "beta", "g"))  # [tokens, H, ...]
+    cu = [b * case["T"] for b in range(case["B"] + 1)] if dense else st["cu"]
+    n_seq = len(cu) - 1
+    S = torch.zeros(n_seq, H_v, D, D, dtype=torch.float64, device="cuda") if st["S"] is None else st["S"].double()
+    O = torch.empty(V.shape, dtype=torch.float64, device="cuda")
+    key = torch.arange(H_v, device="cuda") // (H_v // H_k)
+    row = torch.arange(C, device="cuda")
+    causal = torch.ones(C, C, dtype=torch.bool, device="cuda").tril()
+    longest = max(cu[s + 1] - cu[s] for s in range(n_seq))
+    for t0 in range(0, longest, C):  # the next chunk of every sequence that has one: [sequences, H_v, C, ...]
+        alive = [s for s in range(n_seq) if cu[s] + t0 < cu[s + 1]]
+        first = torch.tensor([cu[s] + t0 for s in alive], device="cuda")
+        size = torch.tensor([min(C, cu[s + 1] - cu[s] - t0) for s in alive], device="cuda")
+        real = row < size[:, None]
+        at = torch.where(real, first[:, None] + row, first[:, None])
+        # rows past a sequence's end write nothing: no key, no value, no further decay
+        q, k = (torch.where(real[..., None, None], _unit(x[at]), 0.0)[:, :, key].transpose(1, 2) for x in (Q, K))
+        v = torch.where(real[..., None, None], V[at].double(), 0.0).transpose(1, 2)
+        b, gc = (torch.where(real[..., None], x[at].double(), 0.0).transpose(1, 2) for x in (beta, g))
+        gc = gc.cumsum(-1)
+        W, U, _ = _chunks(k, v, b, gc, C, gated=True)
+        s0 = S[alive]
+        u = U - W @ s0.transpose(-1, -2)
+        P = (q @ k.transpose(-1, -2)) * torch.where(causal, gc[..., :, None] - gc[..., None, :], -torch.inf).exp()
+        o = D ** -0.5 * (gc.exp()[..., None] * (q @ s0.transpose(-1, -2)) + P @ u)
+        O[at[real]] = o.transpose(1, 2)[real]
+        end = gc[..., -1:]
+        S[alive] = end.exp()[..., None] * s0 + (u * (end - gc).exp()[..., None]).transpose(-1, -2) @ k
+    return O.view(st["V"].shape), S
+
+
+def exact(case, seed):
+    """What `run` returns for these inputs, from the definitions in fp64 (the integer kinds are whole numbers already)."""
+    if case["kind"] in ("int8", "int16"):
+        return None
+    st = prepare(case, seed)
+    return _exact_prepare(case, st) if case["kind"] == "prepare" else _exact_layer(case, st)

@@ -1,5 +1,5 @@
-// Plain-FMA (no tensor core) kernel for the chunk-prepare path: one CTA per chunk,
-// every matrix of the chunk in shared memory, fp32 arithmetic throughout.
+// Plain-FMA (no tensor core) kernel for the chunk-prepare path: one chunk per CTA (or one chunk per few CTAs when a
+// launch has fewer chunks than the chip has SMs), every matrix of the chunk in shared memory, fp32 arithmetic throughout.
 //
 // It serves the fp32 configuration (tolerance 1e-5 against the fp64 definition), small and
 // odd chunk sizes, and the forward-substitution comparisons (Eq. 2-3, App. E). The scheme of
@@ -8,267 +8,683 @@
 //       L_d[i] = Abar[i][i-d] + sum_{e<d} Abar[i][i-e] L_{d-e}[i-e],
 //     which equals the band of sum_{n<=N} Abar^n (a band entry at distance d only receives powers n <= d);
 //   * E = Abar + Abar L on i-j > N (Eq. 13 with T0 = I + L; exactly zero inside the band), N multiply-adds per entry;
-//   * X_0 = T0, X_{k+1} = T0 + X_k E for k < S (so X_S = T0 sum_{s<=S} E^s), every product summed over
-//     j+N+1 <= k <= i only (X is lower triangular, E vanishes for k-j <= N);
+//   * X_0 = T0, X_{k+1} = T0 + X_k E for k < S (so X_S = T0 sum_{s<=S} E^s); round k changes entries with i - j >= (k+1)(N+1)
+//     only, so block diagonals leave the rounds one by one (114 instead of 160 block products at C = 64, N = 3, S = 8; the
+//     doubling form with powers of E needs 90 but squares E: where the series has not converged its fp32 error is up to
+//     100 times larger, so it is not used);
 //   * App. E's two-block formula for C = 128.
-// The Gram matrix is accumulated from slices of K staged in shared memory.
+//
+// What bounds it: the FMA pipe and the shared-memory reads that feed it. Every product is a dot product of two ROWS held
+// in shared memory (right operands are kept transposed), so one 16-byte read brings four terms of the sum: a thread
+// holds the entries (ti + G r, tj + G s), r >= s, reads R + R rows per four terms and does 2 * 10 packed multiply-adds
+// (fma.rn.f32x2) with them at R = 4. The stride of G between a thread's rows keeps the triangle's zero blocks the same
+// for every thread (10 of 16 block pairs, 20 of 64 block triples) and the row pitch of 4 (mod 8) words keeps the reads
+// free of bank conflicts.
 #include "common.cuh"
 
 namespace gdn {
 namespace {
 
-template <typename T>
-__device__ __forceinline__ float to_f32(const T* p);
-template <>
-__device__ __forceinline__ float to_f32<float>(const float* p) { return *p; }
-template <>
-__device__ __forceinline__ float to_f32<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+constexpr int kSliceW = 128;  // features of K (V) held in shared memory at a time
+constexpr int kLdk = kSliceW + 4;
+constexpr float kLargest = 3.402823466e38f;  // FLT_MAX: |x| <= kLargest is false for infinities and NaN
+
+__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16* p, float4 v) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
 __device__ __forceinline__ void st(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 
-constexpr int kThreads = 256;
-constexpr int kSlice = 32;  // features of K staged per step of the Gram accumulation
+typedef unsigned long long f2;  // two packed fp32
+__device__ __forceinline__ void fma2(f2& acc, f2 a, f2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b)); }
+__device__ __forceinline__ f2 dup2(float x) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float2 split2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ float sum2(f2 v) {
+    const float2 r = split2(v);
+    return r.x + r.y;
+}
 
-// Inverse of (I - Abar) for one n x n diagonal block by the truncated scheme (order N, S residual terms).
-// X: Abar block (ld = ldx, strictly lower triangular); result written to Tout (ld = ldt).
-// w0..w2: n x n work matrices (ld = ldw).
-__device__ void neumann_block(const float* X, int ldx, float* Tout, int ldt, float* w0, float* w1, float* w2, int ldw, int n, int N,
-                              int S) {
-    float* T0 = w0;  // I + L, zero outside the band
-    float* E = w1;
-    float* Y = w2;   // second buffer of the rounds
-    for (int idx = threadIdx.x; idx < n * n; idx += kThreads) {
-        const int i = idx / n, j = idx % n;
-        T0[i * ldw + j] = (i == j) ? 1.f : 0.f;
+// Columns [0, w) of `rows` rows of a [rows, d] tile into shared memory as fp32 (row pitch kLdk), rows up to `pad` zero.
+// fp32 arrives asynchronously: the caller waits (load_wait) and synchronises.
+template <int NT>
+__device__ __forceinline__ void load_tile(float* dst, const float* src, int rows, int pad, int d, int w) {
+    const int per = w >> 2;
+    for (int idx = threadIdx.x; idx < rows * per; idx += NT) {
+        const int i = idx / per, c = (idx - i * per) << 2;
+        const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(dst + i * kLdk + c));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src + (long long)i * d + c) : "memory");
     }
-    __syncthreads();
-    // band by distance: one row per thread, one barrier per distance (row i needs L_{d-e} of rows i-e)
-    for (int d = 1; d <= N && d < n; ++d) {
-        for (int i = d + threadIdx.x; i < n; i += kThreads) {
-            float acc = X[i * ldx + (i - d)];
-            for (int e = 1; e < d; ++e) acc = fmaf(X[i * ldx + (i - e)], T0[(i - e) * ldw + (i - d)], acc);
-            T0[i * ldw + (i - d)] = acc;
-        }
-        __syncthreads();
+    for (int idx = rows * per + threadIdx.x; idx < pad * per; idx += NT) {
+        const int i = idx / per, c = (idx - i * per) << 2;
+        *reinterpret_cast<float4*>(dst + i * kLdk + c) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    // E on i - j > N: Abar[i][j] + sum_{e=1..N} Abar[i][j+e] L[j+e][j]   (j + e < i always holds there)
-    for (int idx = threadIdx.x; idx < n * n; idx += kThreads) {
-        const int i = idx / n, j = idx % n;
-        float e_ij = 0.f;
-        if (i - j > N) {
-            e_ij = X[i * ldx + j];
-            for (int e = 1; e <= N; ++e) e_ij = fmaf(X[i * ldx + j + e], T0[(j + e) * ldw + j], e_ij);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int NT>
+__device__ __forceinline__ void load_tile(float* dst, const __nv_bfloat16* src, int rows, int pad, int d, int w) {
+    const int per = w >> 3;
+    for (int idx = threadIdx.x; idx < pad * per; idx += NT) {
+        const int i = idx / per, c = (idx - i * per) << 3;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (i < rows) v = *reinterpret_cast<const uint4*>(src + (long long)i * d + c);
+        const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+        float f[8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            f[2 * q] = __uint_as_float(x[q] << 16);
+            f[2 * q + 1] = __uint_as_float(x[q] & 0xFFFF0000u);
         }
-        E[i * ldw + j] = e_ij;
-        Tout[i * ldt + j] = T0[i * ldw + j];  // X_0 = T0
+        *reinterpret_cast<float4*>(dst + i * kLdk + c) = make_float4(f[0], f[1], f[2], f[3]);
+        *reinterpret_cast<float4*>(dst + i * kLdk + c + 4) = make_float4(f[4], f[5], f[6], f[7]);
     }
-    __syncthreads();
-    // X_{k+1} = T0 + X_k E: only entries with i - j > N change; the sum runs over j + N + 1 <= k <= i
-    float* cur = Tout;
-    int ldc = ldt;
-    float* nxt = Y;
-    int ldn = ldw;
-    for (int r = 0; r < S; ++r) {
-        for (int idx = threadIdx.x; idx < n * n; idx += kThreads) {
-            const int i = idx / n, j = idx % n;
-            float acc = T0[i * ldw + j];
-            for (int k = j + N + 1; k <= i; ++k) acc = fmaf(cur[i * ldc + k], E[k * ldw + j], acc);
-            nxt[i * ldn + j] = acc;
-        }
-        __syncthreads();
-        float* tp = cur; cur = nxt; nxt = tp;
-        const int tl = ldc; ldc = ldn; ldn = tl;
-    }
-    if (cur != Tout) {
-        for (int idx = threadIdx.x; idx < n * n; idx += kThreads) {
-            const int i = idx / n, j = idx % n;
-            Tout[i * ldt + j] = cur[i * ldc + j];
-        }
-        __syncthreads();
+}
+__device__ __forceinline__ void load_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Row j of the tile times scale[j].
+template <int NT>
+__device__ __forceinline__ void scale_rows(float* buf, const float* scale, int rows, int w) {
+    const int per = w >> 2;
+    for (int idx = threadIdx.x; idx < rows * per; idx += NT) {
+        const int i = idx / per, c = (idx - i * per) << 2;
+        float4* p = reinterpret_cast<float4*>(buf + i * kLdk + c);
+        float4 v = *p;
+        const float s = scale[i];
+        v.x *= s; v.y *= s; v.z *= s; v.w *= s;
+        *p = v;
     }
 }
 
-template <typename IO>
-__global__ void __launch_bounds__(kThreads) chunk_simt_kernel(const IO* __restrict__ K, const IO* __restrict__ V,
-                                                             const float* __restrict__ beta, const float* __restrict__ g,
-                                                             IO* __restrict__ W, IO* __restrict__ U, IO* __restrict__ Tinv, int H_k,
-                                                             int H_v, int T, int C, int d_k, int d_v, int N, int S, int mode,
-                                                             long long n_chunks, unsigned flags) {
-    extern __shared__ float sm[];
-    const int ld = C + 1;
-    const int blk = (C == 128) ? 64 : C;  // size of the diagonal blocks inverted by the series
-    const int ldw = blk + 1;
-    float* sA = sm;                 // Abar, C x C
-    float* sT = sA + C * ld;        // T, C x C
-    float* w0 = sT + C * ld;        // three blk x blk work matrices
-    float* w1 = w0 + blk * ldw;
-    float* w2 = w1 + blk * ldw;
-    float* sbeta = w2 + blk * ldw;  // C
-    float* sg = sbeta + C;          // C
-    float* srn = sg + C;            // C: 1 / ||K_row|| (1 unless the keys are normalised here)
-    float* swsc = srn + C;          // C: column scale of the W operand (beta / ||K||, times exp(g) for the gated W)
-    float* sKs = swsc + C;          // C x (kSlice + 1): slice of K while the Gram matrix is accumulated
-    __shared__ float swt[kThreads / 32];
-
-    const int n_c = T / C;
-    const int group = H_v / H_k;
-    for (long long chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
-        const long long bh = chunk / n_c;
-        const int c = static_cast<int>(chunk % n_c);
-        const long long b = bh / H_v;
-        const int hv = static_cast<int>(bh % H_v);
-        const int hk = hv / group;
-        const IO* Kc = K + ((b * H_k + hk) * (long long)T + (long long)c * C) * d_k;
-        const IO* Vc = V + (bh * (long long)T + (long long)c * C) * d_v;
-        const float* bc = beta + bh * (long long)T + (long long)c * C;
-        const float* gc = g + bh * (long long)T + (long long)c * C;
-        IO* Wc = W + (bh * (long long)T + (long long)c * C) * d_k;
-        IO* Uc = U + (bh * (long long)T + (long long)c * C) * d_v;
-
-        for (int i = threadIdx.x; i < C; i += kThreads) {
-            sbeta[i] = bc[i];
-            sg[i] = gc[i];
-            srn[i] = 0.f;  // (sum of squares first)
-        }
-        for (int idx = threadIdx.x; idx < C * C; idx += kThreads) {
-            sA[(idx / C) * ld + (idx % C)] = 0.f;
-            sT[(idx / C) * ld + (idx % C)] = 0.f;
-        }
-        __syncthreads();
-        if (flags & GDN_FLAG_G_RAW) {
-            // raw log-gates: chunk-local inclusive prefix sum (C <= 128 <= kThreads): shuffles inside a warp, then the
-            // totals of the warps before it
-            const int i = threadIdx.x, lane = i & 31, wp = i >> 5;
-            float v = (i < C) ? sg[i] : 0.f;
+// v[r][s] = sum_k X[ti + G r][k] Et[tj + G s][k] for the pairs r - s >= DS, over the blocks q of k with s <= q <= r (X and E
+// lower triangular).
+template <int G, int R, int DS>
+__device__ __forceinline__ void prod_tri(float (&v)[R][R], const float* X, const float* Et, int ti, int tj) {
+    constexpr int ld = G * R + 4;
+    f2 acc[R][R];
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const float u = __shfl_up_sync(0xFFFFFFFFu, v, off);
-                if (lane >= off) v += u;
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int s = 0; s < R; ++s) acc[r][s] = 0ull;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+#pragma unroll 2
+        for (int k = q * G; k < q * G + G; k += 4) {
+            ulonglong2 b[R];
+#pragma unroll
+            for (int s = 0; s <= q && s < R - DS; ++s) b[s] = *reinterpret_cast<const ulonglong2*>(Et + (tj + G * s) * ld + k);
+#pragma unroll
+            for (int r = (q > DS ? q : DS); r < R; ++r) {
+                const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(X + (ti + G * r) * ld + k);
+#pragma unroll
+                for (int s = 0; s <= q && s <= r - DS; ++s) {
+                    fma2(acc[r][s], a.x, b[s].x);
+                    fma2(acc[r][s], a.y, b[s].y);
+                }
             }
-            if (lane == 31) swt[wp] = v;
-            __syncthreads();
-            for (int w = 0; w < wp; ++w) v += swt[w];
-            if (i < C) sg[i] = v;
-            __syncthreads();
         }
-        // Gram matrix of the chunk's keys, lower triangle, from slices of kSlice features staged in shared memory
-        // (every element of K is read from global memory once); the diagonal gives the row norms
-        for (int d0 = 0; d0 < d_k; d0 += kSlice) {
-            const int dw = min(kSlice, d_k - d0);
-            for (int idx = threadIdx.x; idx < C * dw; idx += kThreads) {
-                const int i = idx / dw, d = idx % dw;
-                sKs[i * (kSlice + 1) + d] = to_f32<IO>(Kc + (long long)i * d_k + d0 + d);
-            }
-            __syncthreads();
-            for (int idx = threadIdx.x; idx < C * C; idx += kThreads) {
-                const int i = idx / C, j = idx % C;
-                if (j > i) continue;
-                float dot = 0.f;
-                for (int d = 0; d < dw; ++d) dot = fmaf(sKs[i * (kSlice + 1) + d], sKs[j * (kSlice + 1) + d], dot);
-                if (i == j) srn[i] += dot;
-                else sA[i * ld + j] += dot;
-            }
-            __syncthreads();
-        }
-        for (int i = threadIdx.x; i < C; i += kThreads) {
-            const float rn = (flags & GDN_FLAG_K_L2NORM) ? rsqrtf(fmaxf(srn[i], 1e-30f)) : 1.f;
-            srn[i] = rn;
-            swsc[i] = sbeta[i] * rn * ((flags & GDN_FLAG_W_GATED) ? expf(sg[i]) : 1.f);
-        }
-        __syncthreads();
-        // Abar = -tril(diag(beta) (K K^T o Gamma), -1)
-        for (int idx = threadIdx.x; idx < C * C; idx += kThreads) {
-            const int i = idx / C, j = idx % C;
-            if (i > j) sA[i * ld + j] = -sbeta[i] * expf(sg[i] - sg[j]) * sA[i * ld + j] * srn[i] * srn[j];
-        }
-        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int s = 0; s <= r - DS; ++s) v[r][s] = sum2(acc[r][s]);
+}
 
-        if (mode == INV_NEUMANN) {
-            const int nb = C / blk;
-            for (int bi = 0; bi < nb; ++bi) {
-                neumann_block(sA + bi * blk * ld + bi * blk, ld, sT + bi * blk * ld + bi * blk, ld, w0, w1, w2, ldw, blk, N, S);
+// acc[r][c] += sum_j X[ti + G r][j] B[j][col_c .. col_c + 3] over the j of one block matrix: j blocks q <= r (X lower
+// triangular) or all (FULL). Each thread: R rows, NC pieces of four columns, 4 G apart.
+template <int G, int R, int NC, bool FULL>
+__device__ __forceinline__ void prod_rows(f2 (&acc)[R][NC * 2], const float* X, const float* B, int ti, int col) {
+    constexpr int ld = G * R + 4;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+#pragma unroll 1
+        for (int j = q * G; j < q * G + G; j += 4) {
+            float4 a[R];
+#pragma unroll
+            for (int r = FULL ? 0 : q; r < R; ++r) a[r] = *reinterpret_cast<const float4*>(X + (ti + G * r) * ld + j);
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                ulonglong2 b[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) b[c] = *reinterpret_cast<const ulonglong2*>(B + (j + jj) * kLdk + col + c * 4 * G);
+#pragma unroll
+                for (int r = FULL ? 0 : q; r < R; ++r) {
+                    const f2 x = dup2(jj == 0 ? a[r].x : jj == 1 ? a[r].y : jj == 2 ? a[r].z : a[r].w);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        fma2(acc[r][2 * c], x, b[c].x);
+                        fma2(acc[r][2 * c + 1], x, b[c].y);
+                    }
+                }
             }
-            if (nb == 2) {
-                // Y = A21 T11 (A21 = -Abar21);  T21 = -T22 Y   (App. E, Eq. 28)
-                const float* A21 = sA + blk * ld;
-                const float* T11 = sT;
-                const float* T22 = sT + blk * ld + blk;
-                for (int idx = threadIdx.x; idx < blk * blk; idx += kThreads) {
-                    const int i = idx / blk, j = idx % blk;
-                    float acc = 0.f;
-                    for (int k = 0; k < blk; ++k) acc = fmaf(-A21[i * ld + k], T11[k * ld + j], acc);
-                    w0[i * ldw + j] = acc;
+        }
+    }
+}
+
+// Columns [c0, c0 + 4 G NC) of X B (X = T diag(beta), B: a tile of K or V in shared memory whose first column is column s0
+// of the output) for block rows [nb0, nb1) of one chunk; columns from `d` on do not exist. `bad`: a result is not finite.
+template <typename IO, int G, int R, int NB, int NC>
+__device__ __forceinline__ void out_columns(IO* out, const float* X, const float* X22, const float* X21, const float* B, int C, int d, int s0,
+                                            int c0, int ti, int tj, int nb0, int nb1, bool& bad) {
+    constexpr int M = G * R;
+    const int col = c0 + 4 * tj;
+#pragma unroll 1
+    for (int nb = nb0; nb < nb1; ++nb) {
+        f2 acc[R][NC * 2];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < NC * 2; ++c) acc[r][c] = 0ull;
+        if (nb == 0) {
+            prod_rows<G, R, NC, false>(acc, X, B, ti, col - s0);
+        } else {
+            prod_rows<G, R, NC, true>(acc, X21, B, ti, col - s0);
+            prod_rows<G, R, NC, false>(acc, X22, B + M * kLdk, ti, col - s0);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = nb * M + ti + G * r;
+            if (i >= C) continue;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                if (col + c * 4 * G >= d) continue;
+                const float2 lo = split2(acc[r][2 * c]), hi = split2(acc[r][2 * c + 1]);
+                st4(out + (long long)i * d + col + c * 4 * G, make_float4(lo.x, lo.y, hi.x, hi.y));
+                bad |= !(fabsf(lo.x) <= kLargest && fabsf(lo.y) <= kLargest && fabsf(hi.x) <= kLargest && fabsf(hi.y) <= kLargest);
+            }
+        }
+    }
+}
+
+struct SimtParams {
+    const void *K, *V;
+    const float *beta, *g;
+    void *W, *U, *Tinv;
+    int H_k, H_v, T, C, d_k, d_v, N, S, mode, split;
+    unsigned flags;
+};
+
+// Shared memory in floats: X of every diagonal block, two work matrices per block (a slice of V overlays them once T is
+// complete), for two blocks the lower-left one, the slice of K, tables.
+template <int G, int R, int NB>
+struct SimtSmem {
+    static constexpr int M = G * R, ld = M + 4, mat = M * ld;
+    static constexpr int tile = NB * M * kLdk;
+    static constexpr int work = 2 * NB * mat > tile ? 2 * NB * mat : tile;
+    static constexpr int offX = 0, offW = NB * mat, offX21 = offW + work, offK = offX21 + (NB - 1) * mat;
+    static constexpr int offTab = offK + tile, total = offTab + 4 * NB * M;
+};
+
+// G x G threads per diagonal block of G R rows (the chunk is padded to them with tokens that write nothing), NB blocks.
+template <typename IO, int G, int R, int NB>
+__global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_simt_kernel(const SimtParams p) {
+    using L = SimtSmem<G, R, NB>;
+    constexpr int M = L::M, ld = L::ld, NG = G * G, NT = NG * NB;
+    extern __shared__ __align__(16) float sm[];
+    __shared__ float swt[4];
+    const int grp = threadIdx.x / NG;  // diagonal block this thread works on
+    const int tl = threadIdx.x % NG, lane = threadIdx.x & 31, wp = tl >> 5;
+    // a warp is 4 x 8 threads of the grid: the reads of a left operand touch 4 rows, of a right operand 8
+    const int ti = (G == 16 ? (wp & 3) * 4 : wp * 4) + (lane >> 3);
+    const int tj = (G == 16 ? (wp >> 2) * 8 : 0) + (lane & 7);
+    float* X = sm + L::offX + grp * L::mat;        // row-major, lower blocks
+    float* w0 = sm + L::offW + grp * 2 * L::mat;   // Abar, then E, row-major
+    float* Et = w0 + L::mat;                       // E transposed
+    float* A21 = sm + L::offX21;                   // -A21, finally T21 (row-major)
+    float* Ks = sm + L::offK;
+    float* Vs = sm + L::offW;
+    float* sbeta = sm + L::offTab;
+    float* sg = sbeta + NB * M;
+    float* srn = sg + NB * M;   // 1 / ||K_row|| (1 unless the keys are normalised here)
+    float* swsc = srn + NB * M; // scale of the rows of K in W besides beta (1 / ||K||, times exp(g) for the gated W)
+
+    const int C = p.C, d_k = p.d_k, d_v = p.d_v, N = p.N;
+    const long long chunk = blockIdx.x / p.split;
+    const int share = static_cast<int>(blockIdx.x - chunk * p.split);
+    const int n_c = p.T / C;
+    const long long bh = chunk / n_c;
+    const long long tok = bh * (long long)p.T + (chunk - bh * n_c) * C;  // first row of the value-head tensors
+    const long long ktok = ((bh / p.H_v) * p.H_k + (bh % p.H_v) / (p.H_v / p.H_k)) * (long long)p.T + (chunk - bh * n_c) * C;
+    const IO* Kc = static_cast<const IO*>(p.K) + ktok * d_k;
+    const IO* Vc = static_cast<const IO*>(p.V) + tok * d_v;
+    auto group_sync = [&]() {
+        if (NB == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(NG) : "memory");
+    };
+
+    load_tile<NT>(Ks, Kc, C, NB * M, d_k, min(kSliceW, d_k));
+    for (int i = threadIdx.x; i < NB * M; i += NT) {
+        sbeta[i] = (i < C) ? p.beta[tok + i] : 0.f;
+        sg[i] = (i < C) ? p.g[tok + i] : 0.f;
+    }
+    // ---- Gram matrix: the lower blocks of this group's diagonal block and, of two, half of the rows of the lower-left one
+    f2 acc[R][R], acc21[R / 2 > 0 ? R / 2 : 1][R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int s = 0; s < R; ++s) acc[r][s] = 0ull;
+    if (NB == 2) {
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r)
+#pragma unroll
+            for (int s = 0; s < R; ++s) acc21[r][s] = 0ull;
+    }
+    for (int d0 = 0; d0 < d_k; d0 += kSliceW) {
+        const int w = min(kSliceW, d_k - d0);
+        if (d0 > 0) {
+            __syncthreads();
+            load_tile<NT>(Ks, Kc + d0, C, NB * M, d_k, w);
+        }
+        load_wait();
+        __syncthreads();
+        const float* Kb = Ks + grp * M * kLdk;
+#pragma unroll 2
+        for (int d = 0; d < w; d += 4) {
+            ulonglong2 b[R];
+#pragma unroll
+            for (int s = 0; s < R; ++s) b[s] = *reinterpret_cast<const ulonglong2*>(Kb + (tj + G * s) * kLdk + d);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(Kb + (ti + G * r) * kLdk + d);
+#pragma unroll
+                for (int s = 0; s <= r; ++s) {
+                    fma2(acc[r][s], a.x, b[s].x);
+                    fma2(acc[r][s], a.y, b[s].y);
+                }
+            }
+        }
+        if (NB == 2) {
+#pragma unroll 2
+            for (int d = 0; d < w; d += 4) {
+                ulonglong2 b[R];
+#pragma unroll
+                for (int s = 0; s < R; ++s) b[s] = *reinterpret_cast<const ulonglong2*>(Ks + (tj + G * s) * kLdk + d);
+#pragma unroll
+                for (int r = 0; r < R / 2; ++r) {
+                    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(Ks + (M + ti + G * (r + grp * (R / 2))) * kLdk + d);
+#pragma unroll
+                    for (int s = 0; s < R; ++s) {
+                        fma2(acc21[r][s], a.x, b[s].x);
+                        fma2(acc21[r][s], a.y, b[s].y);
+                    }
+                }
+            }
+        }
+    }
+    if (p.flags & GDN_FLAG_G_RAW) {
+        // raw log-gates: chunk-local inclusive prefix sum (at most 128 tokens): shuffles inside a warp, then the totals
+        // of the warps before it
+        const int i = threadIdx.x, w = i >> 5;
+        float v = (i < NB * M) ? sg[i] : 0.f;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float u = __shfl_up_sync(0xFFFFFFFFu, v, off);
+            if (lane >= off) v += u;
+        }
+        if (lane == 31 && w < 4) swt[w] = v;
+        __syncthreads();
+        if (i < NB * M) {
+            for (int k = 0; k < w; ++k) v += swt[k];
+            sg[i] = v;
+        }
+    }
+    // row norms from the Gram diagonal
+    if (ti == tj) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            srn[grp * M + ti + G * r] = (p.flags & GDN_FLAG_K_L2NORM) ? rsqrtf(fmaxf(sum2(acc[r][r]), 1e-30f)) : 1.f;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < NB * M; i += NT)
+        swsc[i] = srn[i] * ((p.flags & GDN_FLAG_W_GATED) ? expf(sg[i]) : 1.f);
+    // ---- Abar = -tril(diag(beta) (K K^T o Gamma), -1); rows past the chunk's end are zero; X = I
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = grp * M + ti + G * r;
+        const float bi = -sbeta[i] * srn[i], gi = sg[i];
+#pragma unroll
+        for (int s = 0; s < R; ++s) {
+            const int j = grp * M + tj + G * s;
+            float v = 0.f;
+            if (s <= r && i > j && i < C) v = bi * expf(gi - sg[j]) * sum2(acc[r][s]) * srn[j];
+            w0[(ti + G * r) * ld + tj + G * s] = v;
+            X[(ti + G * r) * ld + tj + G * s] = (i == j) ? 1.f : 0.f;
+        }
+    }
+    if (NB == 2) {
+#pragma unroll
+        for (int r = 0; r < R / 2; ++r) {
+            const int il = ti + G * (r + grp * (R / 2)), i = M + il;
+            const float bi = -sbeta[i] * srn[i], gi = sg[i];
+#pragma unroll
+            for (int s = 0; s < R; ++s) {
+                const int j = tj + G * s;
+                A21[il * ld + j] = (i < C) ? bi * expf(gi - sg[j]) * sum2(acc21[r][s]) * srn[j] : 0.f;
+            }
+        }
+    }
+    __syncthreads();
+    const bool k_scaled = (p.flags & (GDN_FLAG_K_L2NORM | GDN_FLAG_W_GATED)) != 0;
+    // the rows of K as W reads them (wider keys are loaded again, slice by slice)
+    if (k_scaled && d_k <= kSliceW) scale_rows<NT>(Ks, swsc, NB * M, d_k);
+    if (p.mode == INV_NEUMANN) {
+        // ---- band by distance (one row per thread, a barrier per distance: row i needs L_{d-e} of rows i - e)
+        const int n = NB == 1 ? C : M;
+        for (int d = 1; d <= N && d < n; ++d) {
+            const int i = tl;
+            if (i >= d && i < n) {
+                float v = w0[i * ld + (i - d)];
+                for (int e = 1; e < d; ++e) v = fmaf(w0[i * ld + (i - e)], X[(i - e) * ld + (i - d)], v);
+                X[i * ld + (i - d)] = v;
+            }
+            group_sync();
+        }
+        if (p.S > 0) {
+            // ---- E on i - j > N: Abar[i][j] + sum_{e=1..N} Abar[i][j+e] L[j+e][j]   (j + e < i always holds there)
+            float ev[R][R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = ti + G * r;
+#pragma unroll
+                for (int s = 0; s <= r; ++s) {
+                    const int j = tj + G * s;
+                    float v = 0.f;
+                    if (i - j > N) {
+                        v = w0[i * ld + j];
+                        for (int e = 1; e <= N; ++e) v = fmaf(w0[i * ld + j + e], X[(j + e) * ld + j], v);
+                    }
+                    ev[r][s] = v;
+                }
+            }
+            group_sync();
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int s = 0; s <= r; ++s) {
+                    w0[(ti + G * r) * ld + tj + G * s] = ev[r][s];
+                    Et[(tj + G * s) * ld + ti + G * r] = ev[r][s];
+                }
+            group_sync();
+            // ---- X_1 = T0 + T0 E: N multiply-adds per entry as T0 = I + L (the band's rows of X stay as they are)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = ti + G * r;
+#pragma unroll
+                for (int s = 0; s <= r; ++s) {
+                    const int j = tj + G * s;
+                    if (i - j > N) {
+                        float v = ev[r][s];
+                        for (int e = 1; e <= N; ++e) v = fmaf(X[i * ld + i - e], w0[(i - e) * ld + j], v);
+                        X[i * ld + j] = v;  // (no thread reads X beyond its band here)
+                    }
+                }
+            }
+            // ---- X_{k+1} = T0 + X_k E for 1 <= k < S: block diagonals below `ds` no longer change
+            float v[R][R];
+            for (int k = 2; k <= p.S; ++k) {
+                const int ds = k * (N + 1) / G;
+                if (ds >= R) break;
+                group_sync();
+                switch (ds) {
+                    case 0: prod_tri<G, R, 0>(v, X, Et, ti, tj); break;
+                    case 1: prod_tri<G, R, (R > 1 ? 1 : 0)>(v, X, Et, ti, tj); break;
+                    case 2: prod_tri<G, R, (R > 2 ? 2 : 0)>(v, X, Et, ti, tj); break;
+                    default: prod_tri<G, R, (R > 3 ? 3 : 0)>(v, X, Et, ti, tj); break;
+                }
+                group_sync();
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int s = 0; s <= r; ++s)
+                        if (r - s >= ds && ti + G * r - tj - G * s > N) X[(ti + G * r) * ld + tj + G * s] = v[r][s];
+            }
+        }
+        // The products above run over whole blocks, zeros included: a chunk with an entry that is not finite is done again
+        // with every sum over its own terms only, so that a token does not reach the tokens before it.
+        bool bad = false;
+        group_sync();
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int s = 0; s <= r; ++s) bad |= !(fabsf(X[(ti + G * r) * ld + tj + G * s]) <= kLargest);
+        if (__syncthreads_or(bad) && p.S > 0) {
+            for (int idx = tl; idx < M * M; idx += NG)
+                if (idx / M - idx % M > N) X[(idx / M) * ld + idx % M] = 0.f;
+            group_sync();
+            for (int k0 = 0; k0 < p.S; ++k0) {  // X_{k+1} = T0 + X_k E
+                for (int idx = tl; idx < M * M; idx += NG) {
+                    const int i = idx / M, j = idx % M;
+                    float v = 0.f;
+                    for (int k = j + N + 1; k <= i; ++k) v = fmaf(X[i * ld + k], Et[j * ld + k], v);
+                    w0[i * ld + j] = v;
+                }
+                group_sync();
+                for (int idx = tl; idx < M * M; idx += NG)
+                    if (idx / M - idx % M > N) X[(idx / M) * ld + idx % M] = w0[(idx / M) * ld + idx % M];
+                group_sync();
+            }
+        }
+        if (NB == 2) {
+            // ---- T21 = T22 Abar21 T11 (App. E, Eq. 28 with Abar21 = -A21); T11 and the first product transposed
+            if (grp == 0) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int s = 0; s < R; ++s) Et[(tj + G * s) * ld + ti + G * r] = X[(ti + G * r) * ld + tj + G * s];
+            }
+            __syncthreads();
+            const float* T11t = sm + L::offW + L::mat;
+            float* Yt = sm + L::offW;
+            // block rows {0, 3} and {1, 2} of the four: as many triangle blocks for either group
+#pragma unroll 1
+            for (int step = 0; step < 2; ++step) {
+                const float* Lm = step == 0 ? A21 : sm + L::offX + L::mat;
+                const float* Rm = step == 0 ? T11t : Yt;
+                f2 a[R / 2 > 0 ? R / 2 : 1][R];
+#pragma unroll
+                for (int rr = 0; rr < R / 2; ++rr) {
+                    const int r = rr == 0 ? grp : R - 1 - grp;
+#pragma unroll
+                    for (int s = 0; s < R; ++s) a[rr][s] = 0ull;
+                    const int kend = step == 0 ? M : G * (r + 1);
+#pragma unroll 2
+                    for (int k = 0; k < kend; k += 4) {
+                        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(Lm + (ti + G * r) * ld + k);
+#pragma unroll
+                        for (int s = 0; s < R; ++s) {
+                            const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(Rm + (tj + G * s) * ld + k);
+                            fma2(a[rr][s], x.x, y.x);
+                            fma2(a[rr][s], x.y, y.y);
+                        }
+                    }
                 }
                 __syncthreads();
-                for (int idx = threadIdx.x; idx < blk * blk; idx += kThreads) {
-                    const int i = idx / blk, j = idx % blk;
-                    float acc = 0.f;
-                    for (int k = 0; k < blk; ++k) acc = fmaf(T22[i * ld + k], w0[k * ldw + j], acc);
-                    sT[(blk + i) * ld + j] = -acc;
+#pragma unroll
+                for (int rr = 0; rr < R / 2; ++rr) {
+                    const int i = ti + G * (rr == 0 ? grp : R - 1 - grp);
+#pragma unroll
+                    for (int s = 0; s < R; ++s) {
+                        if (step == 0) Yt[(tj + G * s) * ld + i] = sum2(a[rr][s]);
+                        else A21[i * ld + tj + G * s] = sum2(a[rr][s]);
+                    }
                 }
                 __syncthreads();
             }
-        } else if (mode == INV_FWDSUBST_BLOCKED) {
+        }
+    } else {
+        // ---- forward substitution: thread j owns column j of T
+        auto A = [&](int i, int j) -> float {
+            if (NB == 1) return w0[i * ld + j];
+            return i < M ? sm[L::offW + i * ld + j] : j < M ? A21[(i - M) * ld + j] : sm[L::offW + 2 * L::mat + (i - M) * ld + j - M];
+        };
+        float* T21 = sm + L::offW + L::mat;
+        auto Tm = [&](int i, int j) -> float& {
+            if (NB == 1) return X[i * ld + j];
+            return i < M ? sm[L::offX + i * ld + j] : j < M ? T21[(i - M) * ld + j] : sm[L::offX + L::mat + (i - M) * ld + j - M];
+        };
+        const int j = threadIdx.x;
+        if (p.mode == INV_FWDSUBST_BLOCKED) {
             // Blocked form (App. E): 16 x 16 diagonal blocks by substitution (Eq. 25), then block rows from
-            // S_ij = S_ii sum_{k<i} Abar_ik S_kj (Eq. 27 with T_ik = -Abar_ik); thread j owns column j.
-            for (int j = threadIdx.x; j < C; j += kThreads) {
+            // S_ij = S_ii sum_{k<i} Abar_ik S_kj (Eq. 27 with T_ik = -Abar_ik).
+            if (j < C) {
                 const int bend = (j / 16 + 1) * 16;
                 for (int i = j + 1; i < bend; ++i) {
-                    float acc = sA[i * ld + j];
-                    for (int k = j + 1; k < i; ++k) acc = fmaf(sA[i * ld + k], sT[k * ld + j], acc);
-                    sT[i * ld + j] = acc;
+                    float v = A(i, j);
+                    for (int k = j + 1; k < i; ++k) v = fmaf(A(i, k), Tm(k, j), v);
+                    Tm(i, j) = v;
                 }
-                sT[j * ld + j] = 1.f;
             }
             __syncthreads();
-            for (int j = threadIdx.x; j < C; j += kThreads) {
+            if (j < C) {
                 for (int bi = j / 16 + 1; bi < C / 16; ++bi) {
                     float tmp[16];
                     for (int r = 0; r < 16; ++r) {
-                        float acc = 0.f;
-                        for (int k = j; k < bi * 16; ++k) acc = fmaf(sA[(bi * 16 + r) * ld + k], sT[k * ld + j], acc);
-                        tmp[r] = acc;
+                        float v = 0.f;
+                        for (int k = j; k < bi * 16; ++k) v = fmaf(A(bi * 16 + r, k), Tm(k, j), v);
+                        tmp[r] = v;
                     }
                     for (int r = 0; r < 16; ++r) {
-                        float acc = 0.f;
-                        for (int q = 0; q <= r; ++q) acc = fmaf(sT[(bi * 16 + r) * ld + bi * 16 + q], tmp[q], acc);
-                        sT[(bi * 16 + r) * ld + j] = acc;
+                        float v = 0.f;
+                        for (int q = 0; q <= r; ++q) v = fmaf(Tm(bi * 16 + r, bi * 16 + q), tmp[q], v);
+                        Tm(bi * 16 + r, j) = v;
                     }
                 }
             }
-            __syncthreads();
-        } else {
-            // Forward substitution (Eq. 2-3): row i of X = Abar_i + Abar_{i,0:i} X_{0:i,:}; thread j owns column j.
-            for (int j = threadIdx.x; j < C; j += kThreads) {
-                for (int i = j + 1; i < C; ++i) {
-                    float acc = sA[i * ld + j];
-                    for (int k = j + 1; k < i; ++k) acc = fmaf(sA[i * ld + k], sT[k * ld + j], acc);
-                    sT[i * ld + j] = acc;
-                }
-                sT[j * ld + j] = 1.f;  // Eq. 3
+        } else if (j < C) {
+            // Rows in order (Eq. 2-3): row i of X = Abar_i + Abar_{i,0:i} X_{0:i,:}
+            for (int i = j + 1; i < C; ++i) {
+                float v = A(i, j);
+                for (int k = j + 1; k < i; ++k) v = fmaf(A(i, k), Tm(k, j), v);
+                Tm(i, j) = v;
             }
-            __syncthreads();
         }
-
-        // W = T diag(beta) K, U = T diag(beta) V; T is lower triangular
-        for (int idx = threadIdx.x; idx < C * d_k; idx += kThreads) {
-            const int i = idx / d_k, d = idx % d_k;
-            float acc = 0.f;
-            for (int j = 0; j <= i; ++j) acc = fmaf(sT[i * ld + j] * swsc[j], to_f32<IO>(Kc + (long long)j * d_k + d), acc);
-            st(Wc + (long long)i * d_k + d, acc);
-        }
-        for (int idx = threadIdx.x; idx < C * d_v; idx += kThreads) {
-            const int i = idx / d_v, d = idx % d_v;
-            float acc = 0.f;
-            for (int j = 0; j <= i; ++j) acc = fmaf(sT[i * ld + j] * sbeta[j], to_f32<IO>(Vc + (long long)j * d_v + d), acc);
-            st(Uc + (long long)i * d_v + d, acc);
-        }
-        if (Tinv != nullptr) {
-            IO* Tc = Tinv + chunk * (long long)C * C;
-            for (int idx = threadIdx.x; idx < C * C; idx += kThreads) st(Tc + idx, sT[(idx / C) * ld + (idx % C)]);
+        __syncthreads();
+        if (NB == 2) {
+            for (int idx = threadIdx.x; idx < M * M; idx += NT) A21[(idx / M) * ld + idx % M] = T21[(idx / M) * ld + idx % M];
         }
         __syncthreads();
     }
+
+    // ---- W = T diag(w) K, U = T diag(beta) V: units of 4 G columns, this CTA's share of them; two at a time where the
+    // second one lies in the same tile. A slice of V comes in (over the work matrices, all read by now) while W is formed.
+    constexpr int UW = 4 * G, per_slice = kSliceW / UW;
+    const int nk = (d_k + UW - 1) / UW, nv = (d_v + UW - 1) / UW;
+    const int u0 = (nk + nv) * share / p.split, u1 = (nk + nv) * (share + 1) / p.split;
+    int in_v = -1;  // slice in Vs: index of its first unit
+    if (u1 > nk) {
+        in_v = nk + (max(u0, nk) - nk) / per_slice * per_slice;
+        const int col = (in_v - nk) * UW;
+        load_tile<NT>(Vs, Vc + col, C, NB * M, d_v, min(kSliceW, d_v - col));
+    }
+    if (share == 0 && p.Tinv != nullptr) {
+        IO* Tc = static_cast<IO*>(p.Tinv) + chunk * (long long)C * C;
+        for (int idx = threadIdx.x; idx < C * C; idx += NT) {
+            const int i = idx / C, j = idx - i * C;
+            float v;
+            if (NB == 1) v = X[i * ld + j];
+            else v = i < M ? (j < M ? sm[L::offX + i * ld + j] : 0.f) : j < M ? A21[(i - M) * ld + j] : sm[L::offX + L::mat + (i - M) * ld + j - M];
+            st(Tc + idx, v);
+        }
+    }
+    __syncthreads();
+    // X <- T diag(beta)
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int s = 0; s <= r; ++s) X[(ti + G * r) * ld + tj + G * s] *= sbeta[grp * M + tj + G * s];
+    if (NB == 2) {
+        for (int idx = threadIdx.x; idx < M * M; idx += NT) A21[(idx / M) * ld + idx % M] *= sbeta[idx % M];
+    }
+    __syncthreads();
+    const float* X0 = sm + L::offX;
+    const float* X22 = X0 + (NB - 1) * L::mat;
+    bool v_ready = false;
+    for (int u = u0; u < u1;) {
+        const bool is_v = u >= nk;
+        const int first = is_v ? nk + (u - nk) / per_slice * per_slice : u / per_slice * per_slice;  // first unit of u's slice
+        const int end = min(min(first + per_slice, u1), is_v ? nk + nv : nk);
+        const int d = is_v ? d_v : d_k, s0 = (first - (is_v ? nk : 0)) * UW;
+        float* B = is_v ? Vs : Ks;
+        if (is_v ? in_v != first : d_k > kSliceW) {
+            __syncthreads();
+            load_tile<NT>(B, (is_v ? Vc : Kc) + s0, C, NB * M, d, min(kSliceW, d - s0));
+            v_ready = false;
+        }
+        if (is_v ? !v_ready : d_k > kSliceW) {
+            load_wait();
+            __syncthreads();
+            if (is_v) {
+                in_v = first;
+                v_ready = true;
+            } else if (k_scaled) {
+                scale_rows<NT>(B, swsc, NB * M, min(kSliceW, d - s0));
+                __syncthreads();
+            }
+        }
+        IO* out = (is_v ? static_cast<IO*>(p.U) + tok * d_v : static_cast<IO*>(p.W) + tok * d_k);
+        bool bad = false;
+        const int begin = u;
+        while (u < end) {
+            const int c0 = s0 + (u - first) * UW;
+            if (NB == 1 && u + 1 < end) {
+                out_columns<IO, G, R, NB, 2>(out, X0, X22, A21, B, C, d, s0, c0, ti, tj, 0, 1, bad);
+                u += 2;
+            } else if (NB == 2 && u + 1 < end) {  // one unit per group
+                out_columns<IO, G, R, NB, 1>(out, X0, X22, A21, B, C, d, s0, c0 + grp * UW, ti, tj, 0, 2, bad);
+                u += 2;
+            } else {  // a single unit: of two groups, each its own block rows
+                out_columns<IO, G, R, NB, 1>(out, X0, X22, A21, B, C, d, s0, c0, ti, tj, NB == 1 ? 0 : grp, NB == 1 ? 1 : grp + 1, bad);
+                u += 1;
+            }
+        }
+        if (__syncthreads_or(bad)) {  // (as above: every sum over its own terms only)
+            const int w = (end - begin) * UW;
+            for (int idx = threadIdx.x; idx < C * w; idx += NT) {
+                const int i = idx / w, c = s0 + (begin - first) * UW + idx % w;
+                if (c >= d) continue;
+                float v = 0.f;
+                for (int j = 0; j <= i; ++j) {
+                    const float t = NB == 1 || i < M ? X0[i * ld + j] : j < M ? A21[(i - M) * ld + j] : X22[(i - M) * ld + j - M];
+                    v = fmaf(t, B[j * kLdk + c - s0], v);
+                }
+                st(out + (long long)i * d + c, v);
+            }
+        }
+    }
+}
+
+template <typename IO, int G, int R, int NB>
+int launch_one(SimtParams p, long long n_chunks, cudaStream_t stream) {
+    auto kern = chunk_simt_kernel<IO, G, R, NB>;
+    constexpr int smem = SimtSmem<G, R, NB>::total * 4;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GDN_ERR_LAUNCH;
+    // Fewer chunks than SMs: two or four CTAs share a chunk (each forms the inverse, its part of the columns of W and U).
+    p.split = n_chunks * 4 <= 148 ? 4 : n_chunks * 2 <= 148 ? 2 : 1;
+    if (n_chunks * p.split >= (1LL << 31)) return GDN_ERR_UNSUPPORTED;
+    kern<<<static_cast<int>(n_chunks * p.split), G * G * NB, smem, stream>>>(p);
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_LAUNCH;
+}
+
+// Thread grid of a diagonal block by its size: 8 x 8 threads (64 per chunk) up to 32 rows, 16 x 16 above; R rows per thread.
+template <typename IO>
+int launch_size(const SimtParams& p, long long n_chunks, cudaStream_t stream) {
+    const int C = p.C;
+    if (C <= 8) return launch_one<IO, 8, 1, 1>(p, n_chunks, stream);
+    if (C <= 16) return launch_one<IO, 8, 2, 1>(p, n_chunks, stream);
+    if (C <= 24) return launch_one<IO, 8, 3, 1>(p, n_chunks, stream);
+    if (C <= 32) return launch_one<IO, 8, 4, 1>(p, n_chunks, stream);
+    if (C <= 48) return launch_one<IO, 16, 3, 1>(p, n_chunks, stream);
+    if (C <= 64) return launch_one<IO, 16, 4, 1>(p, n_chunks, stream);
+    return launch_one<IO, 16, 4, 2>(p, n_chunks, stream);
 }
 
 }  // namespace
@@ -283,26 +699,8 @@ int launch_simt(const Problem& p, InverseMode mode, cudaStream_t stream) {
     }
     const long long n_chunks = (long long)p.B * p.H_v * (p.T / C);
     if (n_chunks == 0) return GDN_OK;
-    const int blk = (C == 128) ? 64 : C;
-    const size_t smem = sizeof(float) * (2 * (size_t)C * (C + 1) + 3 * (size_t)blk * (blk + 1) + 4 * (size_t)C +
-                                         (size_t)C * (kSlice + 1));
-    const int grid = (int)(n_chunks < 148LL * 8 ? n_chunks : 148LL * 8);
-    cudaError_t e;
-    if (p.dtype == GDN_DTYPE_FP32) {
-        e = cudaFuncSetAttribute(chunk_simt_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return GDN_ERR_LAUNCH;
-        chunk_simt_kernel<float><<<grid, kThreads, smem, stream>>>((const float*)p.K, (const float*)p.V, p.beta, p.g, (float*)p.W,
-                                                                  (float*)p.U, (float*)p.Tinv, p.H_k, p.H_v, p.T, C, p.d_k, p.d_v,
-                                                                  p.order, p.steps, (int)mode, n_chunks, p.flags);
-    } else {
-        e = cudaFuncSetAttribute(chunk_simt_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return GDN_ERR_LAUNCH;
-        chunk_simt_kernel<__nv_bfloat16><<<grid, kThreads, smem, stream>>>(
-            (const __nv_bfloat16*)p.K, (const __nv_bfloat16*)p.V, p.beta, p.g, (__nv_bfloat16*)p.W, (__nv_bfloat16*)p.U,
-            (__nv_bfloat16*)p.Tinv, p.H_k, p.H_v, p.T, C, p.d_k, p.d_v, p.order, p.steps, (int)mode, n_chunks, p.flags);
-    }
-    count_launch();
-    return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_LAUNCH;
+    const SimtParams q{p.K, p.V, p.beta, p.g, p.W, p.U, p.Tinv, p.H_k, p.H_v, p.T, C, p.d_k, p.d_v, p.order, p.steps, (int)mode, 1, p.flags};
+    return p.dtype == GDN_DTYPE_FP32 ? launch_size<float>(q, n_chunks, stream) : launch_size<__nv_bfloat16>(q, n_chunks, stream);
 }
 
 }  // namespace gdn

@@ -1,0 +1,67 @@
+"""The plain-FMA kernel where its tiling can go wrong: block remainders, numbers of terms (entries leave the
+rounds of the residual sum block by block), launches of few chunks (several CTAs per chunk), features in slices, entries that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import gdn_oracle as orc
+from paper_2606_06034_b200 import binding as gdn
+from paper_2606_06034_b200 import inputs as gen
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5  # relative Frobenius error per chunk: sums of at most 128 fp32 terms (2^-24 each) with room for their growth
+
+
+def _compare(inp, N=-1, S=-1):
+    W, U, T = gdn.chunk_prepare(inp.K.cuda(), inp.V.cuda(), inp.beta.cuda(), inp.g.cuda(), inp.C, N, S)
+    sl = gen.chunk_slices(inp, range(inp.n_chunks))
+    ref = orc.chunk_prepare(*(np.stack([s[k] for s in sl]) for k in range(4)), None if N < 0 else N, None if S < 0 else S)
+    n, C = inp.n_chunks, inp.C
+    for got, want in zip((W.reshape(n, C, -1), U.reshape(n, C, -1), T.reshape(n, C, C)), ref):
+        assert orc.rel_frobenius(got.double().cpu().numpy(), want).max() <= TOL
+
+
+@pytest.mark.parametrize("C", [2, 7, 8, 9, 16, 17, 24, 25, 31, 32, 33, 47, 48, 49, 63, 64, 128])
+@pytest.mark.parametrize("d_k,d_v", [(8, 72), (136, 128), (256, 40)])
+def test_sizes(C, d_k, d_v):
+    _compare(gen.make_inputs(1, 1, 3, 2 * C, C, d_k, d_v, seed=C + d_k, dtype=torch.float32))
+
+
+@pytest.mark.parametrize("C", [32, 64, 128])
+@pytest.mark.parametrize("N", [1, 3, 20])
+@pytest.mark.parametrize("S", [1, 2, 3, 4, 5, 6, 9, 10, 12, 15])
+def test_numbers_of_terms(C, N, S):
+    """Correlated keys without decay, beta = 0.3: the series has not converged and every term shows."""
+    inp = gen.make_inputs(1, 1, 1, C, C, 64, 64, seed=S, dtype=torch.float32, adversarial_heads="all")
+    inp.beta.fill_(0.3)
+    _compare(inp, N, S)
+
+
+@pytest.mark.parametrize("n", [1, 37, 38, 74, 75])
+@pytest.mark.parametrize("C,d_k,d_v", [(64, 128, 128), (64, 200, 72), (24, 64, 136), (128, 128, 64)])
+def test_few_chunks(n, C, d_k, d_v):
+    """One, two or four CTAs per chunk: the same bits, as every chunk of the launch is an independent problem."""
+    inp = gen.make_inputs(1, 1, 1, n * C, C, d_k, d_v, seed=n, dtype=torch.float32)
+    dev = [x.cuda() for x in (inp.K, inp.V, inp.beta, inp.g)]
+    got = gdn.chunk_prepare(*dev, C)
+    many = gdn.chunk_prepare(*(x.repeat(160, *[1] * (x.dim() - 1)) for x in dev), C)
+    for a, b in zip(got, many):
+        assert torch.equal(a[0], b[0]) and torch.equal(a[0], b[-1])
+    _compare(inp)
+
+
+@pytest.mark.parametrize("C", [16, 33, 64, 128])
+@pytest.mark.parametrize("what", ["K", "V"])
+def test_tokens_before_one_that_is_not_finite(C, what):
+    inp = gen.make_inputs(1, 1, 1, C, C, 128, 128, seed=5, dtype=torch.float32)
+    at = C // 3 + 3  # (of two blocks, in the first: the block formula sums over all tokens of the second)
+    clean = gdn.chunk_prepare(inp.K.cuda(), inp.V.cuda(), inp.beta.cuda(), inp.g.cuda(), C)
+    for value in (float("nan"), float("inf")):
+        K, V = inp.K.clone(), inp.V.clone()
+        (K if what == "K" else V)[0, 0, at, 3] = value
+        W, U, T = gdn.chunk_prepare(K.cuda(), V.cuda(), inp.beta.cuda(), inp.g.cuda(), C)
+        for got, want in ((W[0, 0, :at], clean[0][0, 0, :at]), (U[0, 0, :at], clean[1][0, 0, :at]), (T[0, 0, 0, :at], clean[2][0, 0, 0, :at])):
+            assert torch.isfinite(got).all()
+            assert (got - want).abs().max().item() <= 1e-5  # (the order of the sums differs)
+        assert not torch.isfinite(U[0, 0, at]).all() and (what == "V" or not torch.isfinite(W[0, 0, at]).all())

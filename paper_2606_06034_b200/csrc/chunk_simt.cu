@@ -27,7 +27,6 @@ namespace {
 
 constexpr int kSliceW = 128;  // features of K (V) held in shared memory at a time
 constexpr int kLdk = kSliceW + 4;
-constexpr float kLargest = 3.402823466e38f;  // FLT_MAX: |x| <= kLargest is false for infinities and NaN
 
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ void st4(__nv_bfloat16* p, float4 v) {
@@ -58,23 +57,24 @@ __device__ __forceinline__ float sum2(f2 v) {
 // fp32 arrives asynchronously: the caller waits (load_wait) and synchronises.
 template <int NT>
 __device__ __forceinline__ void load_tile(float* dst, const float* src, int rows, int pad, int d, int w) {
-    const int per = w >> 2;
-    for (int idx = threadIdx.x; idx < rows * per; idx += NT) {
-        const int i = idx / per, c = (idx - i * per) << 2;
-        const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(dst + i * kLdk + c));
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src + (long long)i * d + c) : "memory");
-    }
-    for (int idx = rows * per + threadIdx.x; idx < pad * per; idx += NT) {
-        const int i = idx / per, c = (idx - i * per) << 2;
-        *reinterpret_cast<float4*>(dst + i * kLdk + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int c = (threadIdx.x & 31) << 2;
+    if (c < w) {
+        uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(dst + (threadIdx.x >> 5) * kLdk + c));
+        src += (long long)(threadIdx.x >> 5) * d + c;
+        for (int i = threadIdx.x >> 5; i < pad; i += NT / 32) {
+            if (i < rows) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
+            else *reinterpret_cast<float4*>(dst + i * kLdk + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+            a += (NT / 32) * kLdk * 4;
+            src += (NT / 32) * d;
+        }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 template <int NT>
 __device__ __forceinline__ void load_tile(float* dst, const __nv_bfloat16* src, int rows, int pad, int d, int w) {
-    const int per = w >> 3;
-    for (int idx = threadIdx.x; idx < pad * per; idx += NT) {
-        const int i = idx / per, c = (idx - i * per) << 3;
+    const int c = (threadIdx.x & 15) << 3;
+    if (c >= w) return;
+    for (int i = threadIdx.x >> 4; i < pad; i += NT / 16) {
         uint4 v = make_uint4(0, 0, 0, 0);
         if (i < rows) v = *reinterpret_cast<const uint4*>(src + (long long)i * d + c);
         const uint32_t x[4] = {v.x, v.y, v.z, v.w};
@@ -170,10 +170,10 @@ __device__ __forceinline__ void prod_rows(f2 (&acc)[R][NC * 2], const float* X, 
 }
 
 // Columns [c0, c0 + 4 G NC) of X B (X = T diag(beta), B: a tile of K or V in shared memory whose first column is column s0
-// of the output) for block rows [nb0, nb1) of one chunk; columns from `d` on do not exist. `bad`: a result is not finite.
+// of the output) for block rows [nb0, nb1) of one chunk; columns from `d` on do not exist. `bad`: NaN once a result is not finite.
 template <typename IO, int G, int R, int NB, int NC>
 __device__ __forceinline__ void out_columns(IO* out, const float* X, const float* X22, const float* X21, const float* B, int C, int d, int s0,
-                                            int c0, int ti, int tj, int nb0, int nb1, bool& bad) {
+                                            int c0, int ti, int tj, int nb0, int nb1, f2& bad) {
     constexpr int M = G * R;
     const int col = c0 + 4 * tj;
 #pragma unroll 1
@@ -190,6 +190,10 @@ __device__ __forceinline__ void out_columns(IO* out, const float* X, const float
             prod_rows<G, R, NC, false>(acc, X22, B + M * kLdk, ti, col - s0);
         }
 #pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < NC * 2; ++c) fma2(bad, acc[r][c], 0ull);  // NaN from here on if a result is not finite
+#pragma unroll
         for (int r = 0; r < R; ++r) {
             const int i = nb * M + ti + G * r;
             if (i >= C) continue;
@@ -198,7 +202,54 @@ __device__ __forceinline__ void out_columns(IO* out, const float* X, const float
                 if (col + c * 4 * G >= d) continue;
                 const float2 lo = split2(acc[r][2 * c]), hi = split2(acc[r][2 * c + 1]);
                 st4(out + (long long)i * d + col + c * 4 * G, make_float4(lo.x, lo.y, hi.x, hi.y));
-                bad |= !(fabsf(lo.x) <= kLargest && fabsf(lo.y) <= kLargest && fabsf(hi.x) <= kLargest && fabsf(hi.y) <= kLargest);
+            }
+        }
+    }
+}
+
+// E = Abar + Abar L on i - j > N (w0: Abar on entry, E on return, Et its transpose) and X_1 = T0 + T0 E, N multiply-adds per
+// entry each as T0 = I + L. NC: the order as a constant, 0 where it is not known.
+template <int G, int R, int NC, class Sync>
+__device__ __forceinline__ void first_term(float* X, float* w0, float* Et, int ti, int tj, int order, Sync sync) {
+    constexpr int ld = G * R + 4;
+    const int N = NC > 0 ? NC : order;
+    float ev[R][R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = ti + G * r;
+#pragma unroll
+        for (int s = 0; s <= r; ++s) {
+            const int j = tj + G * s;
+            float v = 0.f;
+            if (i - j > N) {
+                // Abar[i][j] + sum_{e=1..N} Abar[i][j+e] L[j+e][j]   (j + e < i always holds there)
+                v = w0[i * ld + j];
+#pragma unroll
+                for (int e = 1; e <= N; ++e) v = fmaf(w0[i * ld + j + e], X[(j + e) * ld + j], v);
+            }
+            ev[r][s] = v;
+        }
+    }
+    sync();
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int s = 0; s <= r; ++s) {
+            w0[(ti + G * r) * ld + tj + G * s] = ev[r][s];
+            Et[(tj + G * s) * ld + ti + G * r] = ev[r][s];
+        }
+    sync();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = ti + G * r;
+#pragma unroll
+        for (int s = 0; s <= r; ++s) {
+            const int j = tj + G * s;
+            if (i - j > N) {
+                float v = ev[r][s];
+#pragma unroll
+                for (int e = 1; e <= N; ++e) v = fmaf(X[i * ld + i - e], w0[(i - e) * ld + j], v);
+                X[i * ld + j] = v;  // (no thread reads X beyond its band here)
             }
         }
     }
@@ -232,9 +283,11 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
     __shared__ float swt[4];
     const int grp = threadIdx.x / NG;  // diagonal block this thread works on
     const int tl = threadIdx.x % NG, lane = threadIdx.x & 31, wp = tl >> 5;
-    // a warp is 4 x 8 threads of the grid: the reads of a left operand touch 4 rows, of a right operand 8
-    const int ti = (G == 16 ? (wp & 3) * 4 : wp * 4) + (lane >> 3);
-    const int tj = (G == 16 ? (wp >> 2) * 8 : 0) + (lane & 7);
+    // A warp is 4 x 8 threads of the grid: the reads of a left operand touch 4 rows, of a right operand 8. A 16-byte read
+    // takes 2 cycles where lanes i and i ^ 1 (or i and i ^ 2) read the same address and 4 otherwise (measured), so the row
+    // leaves lane bit 0 out and the column lane bit 1.
+    const int ti = (G == 16 ? (wp & 3) * 4 : wp * 4) + ((lane >> 1) & 1) + ((lane >> 4) << 1);
+    const int tj = (G == 16 ? (wp >> 2) * 8 : 0) + (lane & 1) + (((lane >> 2) & 3) << 1);
     float* X = sm + L::offX + grp * L::mat;        // row-major, lower blocks
     float* w0 = sm + L::offW + grp * 2 * L::mat;   // Abar, then E, row-major
     float* Et = w0 + L::mat;                       // E transposed
@@ -388,45 +441,9 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
             group_sync();
         }
         if (p.S > 0) {
-            // ---- E on i - j > N: Abar[i][j] + sum_{e=1..N} Abar[i][j+e] L[j+e][j]   (j + e < i always holds there)
-            float ev[R][R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int i = ti + G * r;
-#pragma unroll
-                for (int s = 0; s <= r; ++s) {
-                    const int j = tj + G * s;
-                    float v = 0.f;
-                    if (i - j > N) {
-                        v = w0[i * ld + j];
-                        for (int e = 1; e <= N; ++e) v = fmaf(w0[i * ld + j + e], X[(j + e) * ld + j], v);
-                    }
-                    ev[r][s] = v;
-                }
-            }
-            group_sync();
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int s = 0; s <= r; ++s) {
-                    w0[(ti + G * r) * ld + tj + G * s] = ev[r][s];
-                    Et[(tj + G * s) * ld + ti + G * r] = ev[r][s];
-                }
-            group_sync();
-            // ---- X_1 = T0 + T0 E: N multiply-adds per entry as T0 = I + L (the band's rows of X stay as they are)
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int i = ti + G * r;
-#pragma unroll
-                for (int s = 0; s <= r; ++s) {
-                    const int j = tj + G * s;
-                    if (i - j > N) {
-                        float v = ev[r][s];
-                        for (int e = 1; e <= N; ++e) v = fmaf(X[i * ld + i - e], w0[(i - e) * ld + j], v);
-                        X[i * ld + j] = v;  // (no thread reads X beyond its band here)
-                    }
-                }
-            }
+            // (the loops over the band unrolled for the default order)
+            if (N == 3) first_term<G, R, 3>(X, w0, Et, ti, tj, N, group_sync);
+            else first_term<G, R, 0>(X, w0, Et, ti, tj, N, group_sync);
             // ---- X_{k+1} = T0 + X_k E for 1 <= k < S: block diagonals below `ds` no longer change
             float v[R][R];
             for (int k = 2; k <= p.S; ++k) {
@@ -449,13 +466,13 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
         }
         // The products above run over whole blocks, zeros included: a chunk with an entry that is not finite is done again
         // with every sum over its own terms only, so that a token does not reach the tokens before it.
-        bool bad = false;
+        float bad = 0.f;
         group_sync();
 #pragma unroll
         for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int s = 0; s <= r; ++s) bad |= !(fabsf(X[(ti + G * r) * ld + tj + G * s]) <= kLargest);
-        if (__syncthreads_or(bad) && p.S > 0) {
+            for (int s = 0; s <= r; ++s) bad = fmaf(X[(ti + G * r) * ld + tj + G * s], 0.f, bad);
+        if (__syncthreads_or(bad != 0.f) && p.S > 0) {
             for (int idx = tl; idx < M * M; idx += NG)
                 if (idx / M - idx % M > N) X[(idx / M) * ld + idx % M] = 0.f;
             group_sync();
@@ -584,24 +601,29 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
         const int col = (in_v - nk) * UW;
         load_tile<NT>(Vs, Vc + col, C, NB * M, d_v, min(kSliceW, d_v - col));
     }
-    if (share == 0 && p.Tinv != nullptr) {
-        IO* Tc = static_cast<IO*>(p.Tinv) + chunk * (long long)C * C;
-        for (int idx = threadIdx.x; idx < C * C; idx += NT) {
-            const int i = idx / C, j = idx - i * C;
-            float v;
-            if (NB == 1) v = X[i * ld + j];
-            else v = i < M ? (j < M ? sm[L::offX + i * ld + j] : 0.f) : j < M ? A21[(i - M) * ld + j] : sm[L::offX + L::mat + (i - M) * ld + j - M];
-            st(Tc + idx, v);
-        }
-    }
-    __syncthreads();
-    // X <- T diag(beta)
+    // T leaves, X <- T diag(beta)
+    IO* Tc = (share == 0 && p.Tinv != nullptr) ? static_cast<IO*>(p.Tinv) + chunk * (long long)C * C : nullptr;
+    auto take = [&](float* m, int nbi, int nbj, int r, int s) {  // entry (ti + G r, tj + G s) of block (nbi, nbj)
+        const int i = nbi * M + ti + G * r, j = nbj * M + tj + G * s;
+        float* x = m + (ti + G * r) * ld + tj + G * s;
+        const float v = *x;
+        *x = v * sbeta[j];
+        if (Tc != nullptr && i < C && j < C) st(Tc + i * C + j, v);
+    };
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int s = 0; s <= r; ++s) X[(ti + G * r) * ld + tj + G * s] *= sbeta[grp * M + tj + G * s];
+        for (int s = 0; s < R; ++s) take(X, grp, grp, r, s);
     if (NB == 2) {
-        for (int idx = threadIdx.x; idx < M * M; idx += NT) A21[(idx / M) * ld + idx % M] *= sbeta[idx % M];
+#pragma unroll
+        for (int rr = 0; rr < R / 2; ++rr) {
+            const int r = rr + grp * (R / 2);
+#pragma unroll
+            for (int s = 0; s < R; ++s) {
+                take(A21, 1, 0, r, s);
+                if (Tc != nullptr) st(Tc + (ti + G * r) * C + M + tj + G * s, 0.f);
+            }
+        }
     }
     __syncthreads();
     const float* X0 = sm + L::offX;
@@ -630,7 +652,7 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
             }
         }
         IO* out = (is_v ? static_cast<IO*>(p.U) + tok * d_v : static_cast<IO*>(p.W) + tok * d_k);
-        bool bad = false;
+        f2 bad = 0ull;
         const int begin = u;
         while (u < end) {
             const int c0 = s0 + (u - first) * UW;
@@ -645,7 +667,7 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
                 u += 1;
             }
         }
-        if (__syncthreads_or(bad)) {  // (as above: every sum over its own terms only)
+        if (__syncthreads_or(sum2(bad) != 0.f)) {  // (as above: every sum over its own terms only)
             const int w = (end - begin) * UW;
             for (int idx = threadIdx.x; idx < C * w; idx += NT) {
                 const int i = idx / w, c = s0 + (begin - first) * UW + idx % w;

@@ -16,9 +16,10 @@
 // mixed ones share one); the threads recombine them exactly in 64 bits. The K and V tiles arrive as int16 by TMA and are
 // split into byte planes in shared memory by the threads.
 //
-// One CTA of 256 threads per SM (three 128-column accumulators + two operand planes = 448 TMEM columns), tile of 128
-// tokens = two 64-chunks, threads t and t + 128 share tile row t and split its 64 chunk columns. Everything between the
-// products is 64-bit integer ALU work; the kernel is written for exactness, not tuned.
+// One CTA of 512 threads per SM (three 128-column accumulators + two operand planes = 448 TMEM columns), tile of 128
+// tokens = two 64-chunks, the four threads t + 128 h share tile row t and split its 64 chunk columns. Everything between the
+// products is 64-bit integer ALU work: it is bound by the number of integer instructions and by how many warps there are to
+// hide their latency (with two threads per row and half the warps the same code ran at a third of the issue slots).
 #include <cuda.h>
 
 #include "common.cuh"
@@ -30,10 +31,11 @@ namespace {
 using namespace sm100;
 
 constexpr int kTile = 128;
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kD = 128;
 constexpr int kC = 64;
-constexpr int kHC = 32;          // chunk columns per thread
+constexpr int kHC = 16;          // chunk columns per thread
+constexpr int kFC = 32;          // feature columns per thread
 constexpr int kSMax = 8;
 constexpr int kWin = 16;         // bits kept below the largest term of an aligned sum
 constexpr int kQ = 32767;
@@ -56,6 +58,9 @@ struct ParamsI16 {
     int H_k, H_v, T, group, n_tt;
     int N, S;
     long long n_tiles;
+    // 1, 256 and 65536 as values the compiler does not know: products with them stay widening multiply-adds on the
+    // multiplier pipe; as constants they become shifts and carries on the integer pipe, the one that bounds the kernel
+    int m1, m8, m16;
     uint16_t lut[256];
 };
 
@@ -77,7 +82,7 @@ constexpr int kNumRed = 24;
 constexpr int kOffPark = (kOffRed + kNumRed * 16 + 1023) / 1024 * 1024;  // 80 KB: parked rows of R_4..R_8 (see the kernel)
 constexpr int kSmemTotal = kOffPark + 5 * 16384;
 
-__device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -102,11 +107,51 @@ __device__ __forceinline__ long long term64(long long x, int s) {
     const int r = s >= 0 ? 0 : ((-s) < 62 ? (-s) : 62);
     return rsr64(x, r) << (s >= 0 ? s : 0);
 }
-// clamp(rsr(x, r), +-kQ). r is the shift of the chunk's largest magnitude (q_shift of its bit length), so the shifted
-// value is at most 2^15 in magnitude and the clamp is done in 32 bits.
+// clamp(rsr(x, r), +-kQ) of single values. r is the shift of the chunk's largest magnitude (q_shift of its bit length), so
+// the shifted value is at most 2^15 in magnitude and the clamp is done in 32 bits.
 __device__ __forceinline__ int q16(long long x, int r) {
     const int y = static_cast<int>(rsr64(x, r));
     return max(min(y, kQ), -kQ);
+}
+// Requantisation of a thread's values in two steps that share their work. z = x + (x >> 63) is x for x >= 0 and x - 1
+// below, so z ^ (x >> 63) is |x| (or-ed into the magnitude), and the rounded shift of x by r > 0 is ((z >> (r - 1)) + 1) >> 1.
+__device__ __forceinline__ long long zmag(long long x, uint32_t& mlo, uint32_t& mhi, int one) {
+    const int sgn = static_cast<int>(x >> 32) >> 31;
+    const long long z = x + static_cast<long long>(sgn) * one;
+    mlo |= static_cast<uint32_t>(z) ^ static_cast<uint32_t>(sgn);
+    mhi |= static_cast<uint32_t>(z >> 32) ^ static_cast<uint32_t>(sgn);
+    return z;
+}
+// two values as int16, clamped to +-kQ
+__device__ __forceinline__ uint32_t clamp_pack(int a, int b) {
+    uint32_t d;
+    asm("cvt.pack.sat.s16.s32 %0, %1, %2;" : "=r"(d) : "r"(b), "r"(a));  // [-32768, 32767], the first operand on top
+    return __vmaxs2(d, 0x80018001u);
+}
+// clamp(rsr(x, r), +-kQ) of n values given as z, packed in pairs: (z + 2^(r-1)) >> r; r is uniform over the chunk
+template <int n>
+__device__ __forceinline__ void quantise(const long long (&z)[n], int r, uint32_t (&out)[n / 2], int one) {
+    if (r > 0 && r < 32) {
+        const int half = 1 << (r - 1);
+        auto q = [&](long long v) {
+            const long long w = v + static_cast<long long>(half) * one;
+            return static_cast<int>(__funnelshift_r(static_cast<uint32_t>(w), static_cast<uint32_t>(w >> 32), r));
+        };
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) out[i] = clamp_pack(q(z[2 * i]), q(z[2 * i + 1]));
+    } else if (r > 32) {  // (the low word does not reach the rounded bits)
+        const int half = (1 << (r - 32)) >> 1, sh = r - 32;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i)
+            out[i] = clamp_pack((static_cast<int>(z[2 * i] >> 32) + half) >> sh, (static_cast<int>(z[2 * i + 1] >> 32) + half) >> sh);
+    } else {
+        auto q = [&](long long v) {
+            const int a = static_cast<int>(v), c = static_cast<int>(v >> 32);
+            return r == 0 ? a - (a >> 31) : c + static_cast<int>(static_cast<uint32_t>(a) >> 31);
+        };
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) out[i] = clamp_pack(q(z[2 * i]), q(z[2 * i + 1]));
+    }
 }
 __device__ __forceinline__ unsigned long long abs64(long long x) { return static_cast<unsigned long long>(x < 0 ? -x : x); }
 __device__ __forceinline__ int q_shift(int bitlen) { return bitlen > 15 ? bitlen - 15 : 0; }
@@ -127,9 +172,9 @@ __device__ __forceinline__ int hi16(uint32_t w) { return static_cast<int>(w) >> 
 __device__ __forceinline__ uint32_t plane_lo(uint32_t w0, uint32_t w1) { return prmt(w0, w1, 0x6420u); }
 __device__ __forceinline__ uint32_t plane_hi(uint32_t w0, uint32_t w1) { return prmt(w0, w1, 0x7531u); }
 // exact product sum from the three byte-plane accumulators
-__device__ __forceinline__ long long combine(uint32_t hh, uint32_t mid, uint32_t ll) {
-    return (static_cast<long long>(static_cast<int>(hh)) << 16) + (static_cast<long long>(static_cast<int>(mid)) << 8) +
-           static_cast<long long>(static_cast<int>(ll));
+__device__ __forceinline__ long long combine(uint32_t hh, uint32_t mid, uint32_t ll, const ParamsI16& p) {
+    return static_cast<long long>(static_cast<int>(hh)) * p.m16 +
+           (static_cast<long long>(static_cast<int>(mid)) * p.m8 + static_cast<long long>(static_cast<int>(ll)) * p.m1);
 }
 
 struct TileCoord {
@@ -188,7 +233,7 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         tma_prefetch_desc(&tmK);
         tma_prefetch_desc(&tmV);
     }
-    slut[tid] = p.lut[tid];
+    if (tid < 256) slut[tid] = p.lut[tid];
     if (warp == 0) {
         tmem_alloc(&tmem_base_s, kTmemCols);
         tmem_relinquish();
@@ -203,7 +248,7 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const int n_c = p.T / kC;
 
     const int t = tid & 127;        // tile row
-    const int h = tid >> 7;         // column half
+    const int h = tid >> 7;         // column quarter
     const int col0 = h * kHC;       // first chunk column of this thread
     const int il = t & (kC - 1);    // row inside the chunk
     const int cb = t - il;          // first tile row of the chunk
@@ -224,14 +269,14 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     // ran out is published in s_fail so that all threads leave the tile loop at the same point
     auto wait_mma = [&]() -> bool {
         if (warp == 0 && (failed() || !wait_bar(&bar_mma, par_mma))) set_fail();
-        asm volatile("bar.sync 2, 256;" ::: "memory");
+        asm volatile("bar.sync 2, 512;" ::: "memory");
         par_mma ^= 1;
         return !failed();
     };
     // bit length of the OR of |values| over the chunk; `slot` is a fresh reduction slot of this tile
-    auto chunk_bitlen = [&](unsigned long long m, int slot) -> int {
-        const uint32_t lo = __reduce_or_sync(0xFFFFFFFFu, static_cast<uint32_t>(m));
-        const uint32_t hi = __reduce_or_sync(0xFFFFFFFFu, static_cast<uint32_t>(m >> 32));
+    auto chunk_bitlen2 = [&](uint32_t mlo, uint32_t mhi, int slot) -> int {
+        const uint32_t lo = __reduce_or_sync(0xFFFFFFFFu, mlo);
+        const uint32_t hi = __reduce_or_sync(0xFFFFFFFFu, mhi);
         if (lane == 0) {
             if (lo) atomicOr(&sred[(slot * 2 + ci) * 2 + 0], lo);
             if (hi) atomicOr(&sred[(slot * 2 + ci) * 2 + 1], hi);
@@ -241,25 +286,35 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             (static_cast<unsigned long long>(sred[(slot * 2 + ci) * 2 + 1]) << 32) | sred[(slot * 2 + ci) * 2 + 0];
         return all ? 64 - __clzll(static_cast<long long>(all)) : 0;
     };
-    // this thread's 64 int16 of its row of an int16 tile (columns [64 h, 64 h + 64)) as 32 words
-    auto load_row16 = [&](const uint8_t* tile16, uint32_t (&w)[32]) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const uint4 v = *reinterpret_cast<const uint4*>(tile16 + h * 16384 + t * 128 + ((c ^ (t & 7)) << 4));
-            w[4 * c + 0] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
-        }
+    auto chunk_bitlen = [&](unsigned long long m, int slot) -> int {
+        return chunk_bitlen2(static_cast<uint32_t>(m), static_cast<uint32_t>(m >> 32), slot);
     };
-    // int16 tile -> byte planes (K-major, 128-byte swizzle): this thread's 64 elements are bytes [64 h, 64 h + 64) of row t
+    // the rows of 64 int16 in sRow (its 16-byte pieces swizzled as in a tile): this thread's 16 columns, one column
+    auto put_row = [&](const uint32_t (&w)[kHC / 2]) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            *reinterpret_cast<uint4*>(sRow + t * 128 + ((((col0 >> 3) + c) ^ (t & 7)) << 4)) =
+                make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+    };
+    auto row_at = [&](int col) -> int16_t* {
+        return reinterpret_cast<int16_t*>(sRow + t * 128 + (((col >> 3) ^ (t & 7)) << 4) + (col & 7) * 2);
+    };
+    // int16 tile -> byte planes (K-major, 128-byte swizzle): this thread's 32 elements (columns [32 h, 32 h + 32), half of
+    // a 128-byte line of box h / 2) are bytes [32 h, 32 h + 32) of row t of either plane
     auto split_planes = [&](const uint8_t* tile16) {
-        uint32_t w[32];
-        load_row16(tile16, w);
+        uint32_t w[16];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4*>(tile16 + (h >> 1) * 16384 + t * 128 + ((((h & 1) * 4 + c) ^ (t & 7)) << 4));
+            w[4 * c + 0] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
             const uint4 lo = make_uint4(plane_lo(w[8 * c + 0], w[8 * c + 1]), plane_lo(w[8 * c + 2], w[8 * c + 3]),
                                         plane_lo(w[8 * c + 4], w[8 * c + 5]), plane_lo(w[8 * c + 6], w[8 * c + 7]));
             const uint4 hi = make_uint4(plane_hi(w[8 * c + 0], w[8 * c + 1]), plane_hi(w[8 * c + 2], w[8 * c + 3]),
                                         plane_hi(w[8 * c + 4], w[8 * c + 5]), plane_hi(w[8 * c + 6], w[8 * c + 7]));
-            const int pos = ((h * 4 + c) ^ (t & 7)) << 4;
+            const int pos = ((h * 2 + c) ^ (t & 7)) << 4;
             *reinterpret_cast<uint4*>(sPl + t * 128 + pos) = lo;
             *reinterpret_cast<uint4*>(sPh + t * 128 + pos) = hi;
         }
@@ -331,7 +386,7 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         fence_proxy_async_smem();
         tc_fence_before_sync();
         cta_barrier();
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             tc_fence_after_sync();
             for (int ks = 0; ks < 4; ++ks) {
                 const uint64_t dh = smem_desc(sPh_a + ks * 32, 16, 1024, SWZ_128B);
@@ -359,48 +414,45 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         int eA;
         {
             uint32_t ghh[kHC], gmid[kHC], gll[kHC];
-            tmem_ld32(lane_base + kDhh + cb + col0, ghh);
-            tmem_ld32(lane_base + kDmid + cb + col0, gmid);
-            tmem_ld32(lane_base + kDll + cb + col0, gll);
+            tmem_ld16(lane_base + kDhh + cb + col0, ghh);
+            tmem_ld16(lane_base + kDmid + cb + col0, gmid);
+            tmem_ld16(lane_base + kDll + cb + col0, gll);
             tmem_wait_ld();
             long long acc[kHC];
-            unsigned long long m = 0;
+            uint32_t mlo = 0, mhi = 0;
 #pragma unroll
             for (int jl = 0; jl < kHC; ++jl) {
-                const long long G = combine(ghh[jl], gmid[jl], gll[jl]);
+                const long long G = combine(ghh[jl], gmid[jl], gll[jl], p);
                 if (DBG && dbg_row != nullptr) dbg_row[col0 + jl] = G;
                 const int j = col0 + jl;
                 const int dlt = dq - sdecay[cb + j];
                 const int sh = dlt >> 8;
                 const int gam = (sh >= 0 && sh < 16) ? (static_cast<int>(slut[dlt & 255]) >> sh) : 0;
                 const int c = (j < il) ? ((bq * gam + (1 << 14)) >> 15) : 0;
-                acc[jl] = -G * static_cast<long long>(c);
-                m |= abs64(acc[jl]);
+                acc[jl] = zmag(-G * static_cast<long long>(c), mlo, mhi, p.m1);
             }
-            const int r = q_shift(chunk_bitlen(m, slot++));
+            const int r = q_shift(chunk_bitlen2(mlo, mhi, slot++));
+            uint32_t w[kHC / 2];
+            quantise(acc, r, w, p.m1);
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) aq[jl] = q16(acc[jl], r);
+            for (int i = 0; i < kHC / 2; ++i) {
+                aq[2 * i] = lo16(w[i]);
+                aq[2 * i + 1] = hi16(w[i]);
+            }
             eA = 2 * kexp - 15 + r;
-        }
-        // Aq to the private row; entries next to the diagonal and right of this half come back from there
-        int16_t* rowa = reinterpret_cast<int16_t*>(sRow + t * 128);
-        {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                *reinterpret_cast<uint4*>(sRow + t * 128 + col0 * 2 + c * 16) =
-                    make_uint4(pack2(aq[8 * c + 0], aq[8 * c + 1]), pack2(aq[8 * c + 2], aq[8 * c + 3]),
-                               pack2(aq[8 * c + 4], aq[8 * c + 5]), pack2(aq[8 * c + 6], aq[8 * c + 7]));
+            // Aq to the private row; entries next to the diagonal and right of this quarter come back from there
+            put_row(w);
         }
         cta_barrier();
         int ab1 = 0, ab2 = 0, ab3 = 0;  // Aq[i][i-1..i-3]
-        if (il >= 1) ab1 = rowa[il - 1];
-        if (il >= 2) ab2 = rowa[il - 2];
-        if (il >= 3) ab3 = rowa[il - 3];
-        int an0 = 0, an1 = 0, an2 = 0;  // Aq[i][32..34] for the left half
-        if (h == 0) {
-            an0 = rowa[kHC + 0];
-            an1 = rowa[kHC + 1];
-            an2 = rowa[kHC + 2];
+        if (il >= 1) ab1 = *row_at(il - 1);
+        if (il >= 2) ab2 = *row_at(il - 2);
+        if (il >= 3) ab3 = *row_at(il - 3);
+        int an0 = 0, an1 = 0, an2 = 0;  // the three entries right of this quarter
+        if (h < 3) {
+            an0 = *row_at(col0 + kHC + 0);
+            an1 = *row_at(col0 + kHC + 1);
+            an2 = *row_at(col0 + kHC + 2);
         }
         const int p11 = ab1, p12 = (N >= 2) ? ab2 : 0, p13 = (N >= 3) ? ab3 : 0;  // P_1 = band of Aq
         if (h == 0) {
@@ -459,13 +511,19 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         }
 
         // ---- I6: Eq = Q16(align(Aq, Aq T0q)) on i-j > N
-        int eq[kHC];
+        uint32_t cur[kHC / 2];  // Eq packed; R_{s-1} inside the loop over the powers
         int eE;
         {
             const int eref = align_ref2(eA, eA + eT0);
             const int sa = eA - eref, sp = eA + eT0 - eref;
             long long acc[kHC];
-            unsigned long long m = 0;
+            uint32_t mlo = 0, mhi = 0;
+            // The usual case: the product has the smaller exponent, so it is shifted right (or not at all) and the shift
+            // of the other term, at most the window, folds into a multiplier.
+            const bool fold = sp <= 0 && sa >= 0;
+            const int m_a = fold ? (1 << sa) : 0, rp = min(-sp, 62);
+            const long long half_p = (1ll << max(rp, 0)) >> 1;
+            const int neg_p = rp > 0 ? 1 : 0;
 #pragma unroll
             for (int jl = 0; jl < kHC; ++jl) {
                 const int4 c4 = *reinterpret_cast<const int4*>(sSH + (cb + col0 + jl) * 4);
@@ -474,48 +532,42 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 const int a3 = (jl + 3 < kHC) ? aq[(jl + 3 < kHC) ? jl + 3 : 0] : ((jl + 3 == kHC) ? an0 : (jl + 3 == kHC + 1 ? an1 : an2));
                 const bool on = (il - (col0 + jl)) > N;
                 const long long pr = (long long)a1 * c4.x + (long long)a2 * c4.y + (long long)a3 * c4.z;
-                const long long v = on ? (term64(aq[jl], sa) + term64(pr, sp)) : 0;
-                acc[jl] = v;
-                m |= abs64(v);
+                long long v;
+                if (fold) {
+                    v = ((pr + half_p + (long long)(static_cast<int>(pr >> 32) >> 31) * neg_p) >> rp) + (long long)aq[jl] * m_a;
+                } else {
+                    v = term64(aq[jl], sa) + term64(pr, sp);
+                }
+                acc[jl] = zmag(on ? v : 0, mlo, mhi, p.m1);
             }
-            const int r = q_shift(chunk_bitlen(m, slot++));
-#pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) eq[jl] = q16(acc[jl], r);
+            const int r = q_shift(chunk_bitlen2(mlo, mhi, slot++));
+            quantise(acc, r, cur, p.m1);
             eE = eref + r;
         }
-        // Rows of the powers R_s (R_1 = Eq) as int16 pairs. The loops over the powers are NOT unrolled (the kernel is bound
-        // by instruction fetch), so the rows cannot sit in registers indexed by s: every thread parks its 64 bytes of R_s
+        // Rows of the powers R_s (R_1 = Eq) as int16 pairs. The loops over the powers are NOT unrolled (code size:
+        // instruction fetch), so the rows cannot sit in registers indexed by s: every thread parks its 32 bytes of R_s
         // in shared memory and reads them back for the sum. The parked rows are private to the thread (no barrier):
         // R_1 in its private row (the Aq row there is dead), R_2 and R_3 in the V tile's buffer (V is loaded after the
         // sum), R_4..R_8 in a region of their own.
+        constexpr int kPiece = kThreads * 16;  // two 16-byte pieces, each piece of all threads in a row (no bank conflicts)
         auto park = [&](int s) -> uint8_t* {
             uint8_t* base = (s == 1) ? sRow : (s <= 3 ? sV16 + (s - 2) * 16384 : smem + kOffPark + (s - 4) * 16384);
-            return base + t * 128 + h * 64;
+            return base + tid * 16;
         };
-        uint32_t cur[kHC / 2];  // R_{s-1} inside the loop
         int er[kSMax];
 #pragma unroll
         for (int s = 0; s < kSMax; ++s) er[s] = 0;
-#pragma unroll
-        for (int w = 0; w < kHC / 2; ++w) cur[w] = 0u;
         int n_terms = 0;
         if (S >= 1) {
-#pragma unroll
-            for (int w = 0; w < kHC / 2; ++w) cur[w] = pack2(eq[2 * w], eq[2 * w + 1]);
             er[0] = eE;
             n_terms = 1;
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                *reinterpret_cast<uint4*>(park(1) + c * 16) = make_uint4(cur[4 * c], cur[4 * c + 1], cur[4 * c + 2], cur[4 * c + 3]);
+            *reinterpret_cast<uint4*>(park(1)) = make_uint4(cur[0], cur[1], cur[2], cur[3]);
+            *reinterpret_cast<uint4*>(park(1) + kPiece) = make_uint4(cur[4], cur[5], cur[6], cur[7]);
             // B operand [E_1 | E_2] as two byte planes (64 x 128 bytes each, MN-major, no swizzle): 16 columns of
             // chunk-row il per 16-byte piece
-#pragma unroll
-            for (int c = 0; c < kHC / 16; ++c) {
-                const uint32_t* w = &cur[8 * c];
-                const uint32_t off = (((cb + col0) >> 4) + c) * (16 * kC) + il * 16;
-                *reinterpret_cast<uint4*>(sEl + off) = make_uint4(plane_lo(w[0], w[1]), plane_lo(w[2], w[3]), plane_lo(w[4], w[5]), plane_lo(w[6], w[7]));
-                *reinterpret_cast<uint4*>(sEh + off) = make_uint4(plane_hi(w[0], w[1]), plane_hi(w[2], w[3]), plane_hi(w[4], w[5]), plane_hi(w[6], w[7]));
-            }
+            const uint32_t off = ((cb + col0) >> 4) * (16 * kC) + il * 16;
+            *reinterpret_cast<uint4*>(sEl + off) = make_uint4(plane_lo(cur[0], cur[1]), plane_lo(cur[2], cur[3]), plane_lo(cur[4], cur[5]), plane_lo(cur[6], cur[7]));
+            *reinterpret_cast<uint4*>(sEh + off) = make_uint4(plane_hi(cur[0], cur[1]), plane_hi(cur[2], cur[3]), plane_hi(cur[4], cur[5]), plane_hi(cur[6], cur[7]));
         }
         // ---- I7: R_s = Q16(R_{s-1} Eq) while s (N+1) < C
         bool bad = false;
@@ -524,53 +576,51 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             if (s > S || s * (N + 1) >= kC) break;
             {
                 // A operand: the rows of R_{s-1}, chunks stacked along M, as byte planes (64 bytes = 16 columns per plane)
-                uint32_t lo8[8], hi8[8];
+                uint32_t lo4[4], hi4[4];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    lo8[i] = plane_lo(cur[2 * i], cur[2 * i + 1]);
-                    hi8[i] = plane_hi(cur[2 * i], cur[2 * i + 1]);
+                for (int i = 0; i < 4; ++i) {
+                    lo4[i] = plane_lo(cur[2 * i], cur[2 * i + 1]);
+                    hi4[i] = plane_hi(cur[2 * i], cur[2 * i + 1]);
                 }
-                tmem_st8(lane_base + kAh + h * 8, hi8);
-                tmem_st8(lane_base + kAl + h * 8, lo8);
+                tmem_st4(lane_base + kAh + h * 4, hi4);
+                tmem_st4(lane_base + kAl + h * 4, lo4);
             }
             fence_proxy_async_smem();
             tmem_wait_st();
             tc_fence_before_sync();
             cta_barrier();
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after_sync();
                 issue_ts(kC / 32, sEh_a, sEl_a, 512, 128, 16 * kC, SWZ_NONE);
             }
             if (!wait_mma()) { bad = true; break; }
             tc_fence_after_sync();
             uint32_t dhh[kHC], dmid[kHC], dll[kHC];
-            tmem_ld32(lane_base + kDhh + cb + col0, dhh);
-            tmem_ld32(lane_base + kDmid + cb + col0, dmid);
-            tmem_ld32(lane_base + kDll + cb + col0, dll);
+            tmem_ld16(lane_base + kDhh + cb + col0, dhh);
+            tmem_ld16(lane_base + kDmid + cb + col0, dmid);
+            tmem_ld16(lane_base + kDll + cb + col0, dll);
             tmem_wait_ld();
-            unsigned long long m = 0;
+            uint32_t mlo = 0, mhi = 0;
             long long acc[kHC];
             // R_{s-1} is zero for i - j < (s - 1)(N + 1) and Eq for i - j <= N: the integer product is exactly zero for
             // i - j < s (N + 1), no mask needed
 #pragma unroll
             for (int jl = 0; jl < kHC; ++jl) {
-                acc[jl] = combine(dhh[jl], dmid[jl], dll[jl]);
-                if (DBG && dbg_row != nullptr) dbg_row[(s - 1) * kC + col0 + jl] = acc[jl];
-                m |= abs64(acc[jl]);
+                const long long x = combine(dhh[jl], dmid[jl], dll[jl], p);
+                if (DBG && dbg_row != nullptr) dbg_row[(s - 1) * kC + col0 + jl] = x;
+                acc[jl] = zmag(x, mlo, mhi, p.m1);
             }
-            const int r = q_shift(chunk_bitlen(m, slot++));
-#pragma unroll
-            for (int w = 0; w < kHC / 2; ++w) cur[w] = pack2(q16(acc[2 * w], r), q16(acc[2 * w + 1], r));
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                *reinterpret_cast<uint4*>(park(s) + c * 16) = make_uint4(cur[4 * c], cur[4 * c + 1], cur[4 * c + 2], cur[4 * c + 3]);
+            const int r = q_shift(chunk_bitlen2(mlo, mhi, slot++));
+            quantise(acc, r, cur, p.m1);
+            *reinterpret_cast<uint4*>(park(s)) = make_uint4(cur[0], cur[1], cur[2], cur[3]);
+            *reinterpret_cast<uint4*>(park(s) + kPiece) = make_uint4(cur[4], cur[5], cur[6], cur[7]);
             er[s - 1] = er[s - 2] + eE + r;
             n_terms = s;
         }
         if (bad) break;
 
         // ---- Sq = Q16(align(R_1..)): a term whose right shift exceeds 15 rounds to zero and is skipped
-        int sq[kHC];
+        uint32_t sq[kHC / 2];
         int eS = 0;
         if (n_terms > 0) {
             int emin = er[0], emax = er[0];
@@ -587,35 +637,37 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 if (sh < -15) continue;
                 uint32_t w[kHC / 2];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(park(s) + c * 16);
+                for (int c = 0; c < 2; ++c) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(park(s) + c * kPiece);
                     w[4 * c] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
                 }
                 if (sh >= 0) {
+                    const int mul = 1 << sh;  // (sh <= the window)
 #pragma unroll
                     for (int i = 0; i < kHC / 2; ++i) {
-                        acc[2 * i] += static_cast<long long>(lo16(w[i])) << sh;
-                        acc[2 * i + 1] += static_cast<long long>(hi16(w[i])) << sh;
+                        acc[2 * i] += static_cast<long long>(lo16(w[i])) * mul;
+                        acc[2 * i + 1] += static_cast<long long>(hi16(w[i])) * mul;
                     }
                 } else {
+                    const int half = (1 << -sh) >> 1;
 #pragma unroll
                     for (int i = 0; i < kHC / 2; ++i) {
-                        acc[2 * i] += rsr64(lo16(w[i]), -sh);
-                        acc[2 * i + 1] += rsr64(hi16(w[i]), -sh);
+                        const int a = lo16(w[i]), b = hi16(w[i]);
+                        acc[2 * i] += (a + half + (a >> 31)) >> -sh;
+                        acc[2 * i + 1] += (b + half + (b >> 31)) >> -sh;
                     }
                 }
             }
-            unsigned long long m = 0;
+            uint32_t mlo = 0, mhi = 0;
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) m |= abs64(acc[jl]);
+            for (int jl = 0; jl < kHC; ++jl) acc[jl] = zmag(acc[jl], mlo, mhi, p.m1);
             fence_proxy_async_smem();  // the parked rows in the V buffer are overwritten by a bulk copy next
-            const int r = q_shift(chunk_bitlen(m, slot++));
-#pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) sq[jl] = q16(acc[jl], r);
+            const int r = q_shift(chunk_bitlen2(mlo, mhi, slot++));
+            quantise(acc, r, sq, p.m1);
             eS = eref + r;
         } else {
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) sq[jl] = 0;
+            for (int i = 0; i < kHC / 2; ++i) sq[i] = 0u;
         }
         // the V tile of this tile: its buffer held parked rows until the sum above (every thread is past its reads: the
         // reduction of the sum is a barrier), and the previous tile's U stage is long finished
@@ -626,32 +678,28 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             tma_load_3d(sV16 + 16384, &tmV, &bar_v, 64, tc.t0, tc.bhv);
         }
         // Sq to the private rows (the rows above are needed for T0q Sq)
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            *reinterpret_cast<uint4*>(sRow + t * 128 + col0 * 2 + c * 16) =
-                make_uint4(pack2(sq[8 * c + 0], sq[8 * c + 1]), pack2(sq[8 * c + 2], sq[8 * c + 3]),
-                           pack2(sq[8 * c + 4], sq[8 * c + 5]), pack2(sq[8 * c + 6], sq[8 * c + 7]));
+        put_row(sq);
         cta_barrier();
 
         // ---- I8: Toffq = Q16(align(T0q, Sq, T0q Sq)) on i > j
-        int toff[kHC];
+        uint32_t toff[kHC / 2];
         int eT;
         {
-            long long prod[kHC];
+            long long acc[kHC];  // T0q Sq
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) prod[jl] = 0;
+            for (int jl = 0; jl < kHC; ++jl) acc[jl] = 0;
 #pragma unroll
             for (int e = 1; e <= 3; ++e) {
                 const int rr = (t - e) > 0 ? (t - e) : 0;
                 const int cf = (il - e >= 0) ? (e == 1 ? t0q1 : (e == 2 ? t0q2 : t0q3)) : 0;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const uint4 a = *reinterpret_cast<const uint4*>(sRow + rr * 128 + col0 * 2 + c * 16);
+                for (int c = 0; c < 2; ++c) {
+                    const uint4 a = *reinterpret_cast<const uint4*>(sRow + rr * 128 + ((((col0 >> 3) + c) ^ (rr & 7)) << 4));
                     const uint32_t w[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        prod[8 * c + 2 * i] += (long long)cf * lo16(w[i]);
-                        prod[8 * c + 2 * i + 1] += (long long)cf * hi16(w[i]);
+                        acc[8 * c + 2 * i] += (long long)cf * lo16(w[i]);
+                        acc[8 * c + 2 * i + 1] += (long long)cf * hi16(w[i]);
                     }
                 }
             }
@@ -659,67 +707,92 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             const int emin = min(e0, min(e1, e2)), emax = max(e0, max(e1, e2));
             const int eref = max(emin, emax - kWin);
             const int s0 = e0 - eref, s1 = e1 - eref, s2 = e2 - eref;
-            // the band entry and Sq never share an element (band: distance <= N, Sq: distance > N)
-            long long acc[kHC];
-            unsigned long long m = 0;
+            // Sq and T0q Sq are exactly zero on the band, the diagonal and above, so their terms need no mask; the (at most
+            // three) band entries of a row are scalars that enter the magnitude and are put into the packed row afterwards.
+            uint32_t mlo = 0, mhi = 0;
+            const bool fold = s2 <= 0 && s1 >= 0;  // (the usual case, as in I6)
+            const int m_s = fold ? (1 << s1) : 0, rp = min(-s2, 62);
+            const long long half_p = (1ll << max(rp, 0)) >> 1;
+            const int neg_p = rp > 0 ? 1 : 0;
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) {
-                const int d = il - (col0 + jl);
-                int v = sq[jl];
-                if (d == 1 && N >= 1) v = t0q1;
-                if (d == 2 && N >= 2) v = t0q2;
-                if (d == 3 && N >= 3) v = t0q3;
-                const long long a = (d > 0) ? (term64(v, (d <= N) ? s0 : s1) + term64(prod[jl], s2)) : 0;
-                acc[jl] = a;
-                m |= abs64(a);
+            for (int i = 0; i < kHC / 2; ++i) {
+                const int a = lo16(sq[i]), b = hi16(sq[i]);
+                long long va, vb;
+                if (fold) {
+                    va = ((acc[2 * i] + half_p + (long long)(static_cast<int>(acc[2 * i] >> 32) >> 31) * neg_p) >> rp) + (long long)a * m_s;
+                    vb = ((acc[2 * i + 1] + half_p + (long long)(static_cast<int>(acc[2 * i + 1] >> 32) >> 31) * neg_p) >> rp) + (long long)b * m_s;
+                } else {
+                    va = term64(a, s1) + term64(acc[2 * i], s2);
+                    vb = term64(b, s1) + term64(acc[2 * i + 1], s2);
+                }
+                acc[2 * i] = zmag(va, mlo, mhi, p.m1);
+                acc[2 * i + 1] = zmag(vb, mlo, mhi, p.m1);
             }
-            const int r = q_shift(chunk_bitlen(m, slot++));
-#pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) toff[jl] = q16(acc[jl], r);
+            const long long b1 = term64(t0q1, s0), b2 = term64(t0q2, s0), b3 = term64(t0q3, s0);  // (zero past the order)
+            const unsigned long long mb = abs64(b1) | abs64(b2) | abs64(b3);
+            const int r = q_shift(chunk_bitlen2(mlo | static_cast<uint32_t>(mb), mhi | static_cast<uint32_t>(mb >> 32), slot++));
+            quantise(acc, r, toff, p.m1);
             eT = eref + r;
+            // (every thread has read the rows of Sq: the reduction is a barrier. The quarter of a row is its thread's own.)
+            put_row(toff);
+            const int at = il - col0;  // columns at - 1, at - 2, at - 3 of this thread's sixteen hold the band
+            if (at - 1 >= 0 && at - 1 < kHC) *row_at(il - 1) = static_cast<int16_t>(q16(b1, r));
+            if (N >= 2 && at - 2 >= 0 && at - 2 < kHC) *row_at(il - 2) = static_cast<int16_t>(q16(b2, r));
+            if (N >= 3 && at - 3 >= 0 && at - 3 < kHC) *row_at(il - 3) = static_cast<int16_t>(q16(b3, r));
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const uint4 v = *reinterpret_cast<const uint4*>(sRow + t * 128 + ((((col0 >> 3) + c) ^ (t & 7)) << 4));
+                toff[4 * c] = v.x; toff[4 * c + 1] = v.y; toff[4 * c + 2] = v.z; toff[4 * c + 3] = v.w;
+            }
         }
-        // Toffq row: 32 int16 of this thread straight to global memory
+        // Toffq row: 16 int16 of this thread straight to global memory
         if (p.Toff != nullptr && row_valid) {
             uint4* dst = reinterpret_cast<uint4*>(p.Toff + (chunk_id * kC + il) * kC + col0);
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                dst[c] = make_uint4(pack2(toff[8 * c + 0], toff[8 * c + 1]), pack2(toff[8 * c + 2], toff[8 * c + 3]),
-                                    pack2(toff[8 * c + 4], toff[8 * c + 5]), pack2(toff[8 * c + 6], toff[8 * c + 7]));
+            dst[0] = make_uint4(toff[0], toff[1], toff[2], toff[3]);
+            dst[1] = make_uint4(toff[4], toff[5], toff[6], toff[7]);
         }
         if (row_valid && il == 0 && h == 0) p.t_exp[chunk_id] = eT;
 
         // ---- I9: Tbq = Q16(Toffq_ij beta_q_j); byte planes of the block-diagonal A operand of W / U
         int eTb;
         {
-            long long acc[kHC];
-            unsigned long long m = 0;
+            int acc[kHC];  // (30 bits)
+            uint32_t m = 0;
 #pragma unroll
             for (int jl = 0; jl < kHC; ++jl) {
-                acc[jl] = (long long)toff[jl] * sbeta[cb + col0 + jl];
-                m |= abs64(acc[jl]);
+                const int x = ((jl & 1) ? hi16(toff[jl >> 1]) : lo16(toff[jl >> 1])) * sbeta[cb + col0 + jl];
+                const int sgn = x >> 31;
+                acc[jl] = x + sgn;
+                m |= static_cast<uint32_t>(acc[jl] ^ sgn);
             }
-            const int r = q_shift(chunk_bitlen(m, slot++));
-            uint32_t lo8[8], hi8[8];
+            const int r = q_shift(chunk_bitlen2(m, 0u, slot++));
+            uint32_t w[kHC / 2];
+            if (r > 0) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const uint32_t w0 = pack2(q16(acc[4 * i + 0], r), q16(acc[4 * i + 1], r));
-                const uint32_t w1 = pack2(q16(acc[4 * i + 2], r), q16(acc[4 * i + 3], r));
-                lo8[i] = plane_lo(w0, w1);
-                hi8[i] = plane_hi(w0, w1);
+                for (int i = 0; i < kHC / 2; ++i) w[i] = clamp_pack(((acc[2 * i] >> (r - 1)) + 1) >> 1, ((acc[2 * i + 1] >> (r - 1)) + 1) >> 1);
+            } else {
+#pragma unroll
+                for (int i = 0; i < kHC / 2; ++i) w[i] = clamp_pack(acc[2 * i] - (acc[2 * i] >> 31), acc[2 * i + 1] - (acc[2 * i + 1] >> 31));
+            }
+            uint32_t lo4[4], hi4[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                lo4[i] = plane_lo(w[2 * i], w[2 * i + 1]);
+                hi4[i] = plane_hi(w[2 * i], w[2 * i + 1]);
             }
             eTb = eT - 15 + r;
             // row t's block occupies packed columns [cb/4, cb/4 + 16) of a 32-column plane; the other 16 are zero
-            tmem_st8(lane_base + kAh + cb / 4 + h * 8, hi8);
-            tmem_st8(lane_base + kAl + cb / 4 + h * 8, lo8);
+            tmem_st4(lane_base + kAh + cb / 4 + h * 4, hi4);
+            tmem_st4(lane_base + kAl + cb / 4 + h * 4, lo4);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) lo8[i] = 0u;
-            tmem_st8(lane_base + kAh + (16 - cb / 4) + h * 8, lo8);
-            tmem_st8(lane_base + kAl + (16 - cb / 4) + h * 8, lo8);
+            for (int i = 0; i < 4; ++i) lo4[i] = 0u;
+            tmem_st4(lane_base + kAh + (16 - cb / 4) + h * 4, lo4);
+            tmem_st4(lane_base + kAl + (16 - cb / 4) + h * 4, lo4);
             tmem_wait_st();
         }
         tc_fence_before_sync();
         cta_barrier();
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             // W accumulators = blockdiag(Tbq) Kq: M = 128, N = 128, K = 128 bytes per plane (4 steps of 32)
             tc_fence_after_sync();
             issue_ts(4, sPh_a, sPl_a, 4096, 16384, 1024, SWZ_128B);
@@ -730,16 +803,8 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
             const int xexp = (half == 0) ? kexp : vexp;
-            // diagonal term beta_q_i * Xq_i for this thread's 64 columns, from its own row of the int16 tile (16 columns
-            // at a time: the loops over the column blocks are not unrolled)
-            const uint8_t* xtile = (half == 0) ? sK16 : sV16;
-            auto load_x16 = [&](int c0, uint32_t (&w)[8]) {
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(xtile + h * 16384 + t * 128 + ((((c0 >> 3) + c) ^ (t & 7)) << 4));
-                    w[4 * c + 0] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
-                }
-            };
+            // diagonal term beta_q_i * Xq_i for this thread's 32 columns, from its own row of the int16 tile
+            const uint8_t* xtile = ((half == 0) ? sK16 : sV16) + (h >> 1) * 16384 + t * 128;
             if (!wait_mma()) { bad2 = true; break; }
             tc_fence_after_sync();
             const int ep = eTb + xexp, ed = xexp - 15;
@@ -751,78 +816,52 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             const bool fold = sp >= 0 && sp <= 14 && sd >= 0 && sd <= 15;
             const int m_hh = fold ? (1 << (16 + sp)) : 0, m_mid = fold ? (1 << (8 + sp)) : 0, m_ll = fold ? (1 << sp) : 0;
             const int bqs = fold ? (bq << sd) : 0;
-            // pass 1: the scale (bit length of the largest magnitude over the chunk's C x d block)
-            unsigned long long m = 0;
-#pragma unroll 1
-            for (int c0 = 0; c0 < 64; c0 += 16) {
+            // the aligned sums stay in registers between the scale (bit length of the largest magnitude over the chunk's
+            // C x d block) and the mantissas
+            long long acc[kFC];
+            uint32_t mlo = 0, mhi = 0;
+#pragma unroll
+            for (int c0 = 0; c0 < kFC; c0 += 16) {
                 uint32_t xr[8];
-                load_x16(c0, xr);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(xtile + ((((h & 1) * 4 + (c0 >> 3) + c) ^ (t & 7)) << 4));
+                    xr[4 * c + 0] = v.x; xr[4 * c + 1] = v.y; xr[4 * c + 2] = v.z; xr[4 * c + 3] = v.w;
+                }
                 uint32_t dhh[16], dmid[16], dll[16];
-                tmem_ld16(lane_base + kDhh + h * 64 + c0, dhh);
-                tmem_ld16(lane_base + kDmid + h * 64 + c0, dmid);
-                tmem_ld16(lane_base + kDll + h * 64 + c0, dll);
+                tmem_ld16(lane_base + kDhh + h * kFC + c0, dhh);
+                tmem_ld16(lane_base + kDmid + h * kFC + c0, dmid);
+                tmem_ld16(lane_base + kDll + h * kFC + c0, dll);
                 tmem_wait_ld();
                 if (DBG && dbg_row != nullptr) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) dbg_row[8 * kC + half * kD + h * 64 + c0 + i] = combine(dhh[i], dmid[i], dll[i]);
+                    for (int i = 0; i < 16; ++i) dbg_row[8 * kC + half * kD + h * kFC + c0 + i] = combine(dhh[i], dmid[i], dll[i], p);
                 }
                 if (fold) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const uint32_t xw = xr[i >> 1];
                         const int x = (i & 1) ? hi16(xw) : lo16(xw);
-                        const long long v = (long long)static_cast<int>(dhh[i]) * m_hh + (long long)static_cast<int>(dmid[i]) * m_mid +
-                                            (long long)static_cast<int>(dll[i]) * m_ll + (long long)x * bqs;
-                        m |= abs64(v);
+                        acc[c0 + i] = zmag((long long)static_cast<int>(dhh[i]) * m_hh + (long long)static_cast<int>(dmid[i]) * m_mid +
+                                               (long long)static_cast<int>(dll[i]) * m_ll + (long long)x * bqs, mlo, mhi, p.m1);
                     }
                 } else {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const long long pr = combine(dhh[i], dmid[i], dll[i]);
                         const uint32_t xw = xr[i >> 1];
                         const int x = (i & 1) ? hi16(xw) : lo16(xw);
-                        m |= abs64(term64(pr, sp) + term64((long long)bq * x, sd));
+                        acc[c0 + i] = zmag(term64(combine(dhh[i], dmid[i], dll[i], p), sp) + term64((long long)bq * x, sd), mlo, mhi, p.m1);
                     }
                 }
             }
-            const int rr = q_shift(chunk_bitlen(m, slot++));
+            const int rr = q_shift(chunk_bitlen2(mlo, mhi, slot++));
             if (row_valid && il == 0 && h == 0) ((half == 0) ? p.w_exp : p.u_exp)[chunk_id] = eref + rr;
-            // pass 2: mantissas, 64 int16 of this thread's row straight to global memory
-            int16_t* out = ((half == 0) ? p.W : p.U) + grow * kD + h * 64;
-#pragma unroll 1
-            for (int c0 = 0; c0 < 64; c0 += 16) {
-                uint32_t xr[8];
-                load_x16(c0, xr);
-                uint32_t dhh[16], dmid[16], dll[16];
-                tmem_ld16(lane_base + kDhh + h * 64 + c0, dhh);
-                tmem_ld16(lane_base + kDmid + h * 64 + c0, dmid);
-                tmem_ld16(lane_base + kDll + h * 64 + c0, dll);
-                tmem_wait_ld();
-                uint32_t o[8];
-                if (fold) {
+            uint32_t o[kFC / 2];
+            quantise(acc, rr, o, p.m1);
+            if (row_valid) {
+                uint4* dst = reinterpret_cast<uint4*>(((half == 0) ? p.W : p.U) + grow * kD + h * kFC);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const uint32_t xw = xr[i];
-                        const long long v0 = (long long)static_cast<int>(dhh[2 * i]) * m_hh + (long long)static_cast<int>(dmid[2 * i]) * m_mid +
-                                             (long long)static_cast<int>(dll[2 * i]) * m_ll + (long long)lo16(xw) * bqs;
-                        const long long v1 = (long long)static_cast<int>(dhh[2 * i + 1]) * m_hh + (long long)static_cast<int>(dmid[2 * i + 1]) * m_mid +
-                                             (long long)static_cast<int>(dll[2 * i + 1]) * m_ll + (long long)hi16(xw) * bqs;
-                        o[i] = pack2(q16(v0, rr), q16(v1, rr));
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const uint32_t xw = xr[i];
-                        const long long v0 = term64(combine(dhh[2 * i], dmid[2 * i], dll[2 * i]), sp) + term64((long long)bq * lo16(xw), sd);
-                        const long long v1 = term64(combine(dhh[2 * i + 1], dmid[2 * i + 1], dll[2 * i + 1]), sp) + term64((long long)bq * hi16(xw), sd);
-                        o[i] = pack2(q16(v0, rr), q16(v1, rr));
-                    }
-                }
-                if (row_valid) {
-                    uint4* dst = reinterpret_cast<uint4*>(out + c0);
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) dst[c] = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
-                }
+                for (int c = 0; c < kFC / 8; ++c) dst[c] = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
             }
             if (half == 0) {
                 tc_fence_before_sync();
@@ -842,7 +881,7 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                 fence_proxy_async_smem();
                 tc_fence_before_sync();
                 cta_barrier();
-                if (tid == 0) {
+                if (warp == 0 && elect_one()) {
                     tc_fence_after_sync();
                     issue_ts(4, sPh_a, sPl_a, 4096, 16384, 1024, SWZ_128B);
                 }
@@ -922,6 +961,9 @@ int launch_tc_int16(const ProblemI16& q, cudaStream_t stream) {
     prm.n_tt = (q.T + kTile - 1) / kTile;
     prm.N = q.order;
     prm.S = q.steps;
+    prm.m1 = 1;
+    prm.m8 = 1 << 8;
+    prm.m16 = 1 << 16;
     prm.n_tiles = (long long)q.B * q.H_v * prm.n_tt;
     if (prm.n_tiles >= (1LL << 31) - 4096) return GDN_ERR_UNSUPPORTED;
     int8_decay_lut(prm.lut);

@@ -14,7 +14,8 @@
 //                             a single bf16 copy costs 1e-2 on strongly correlated keys), B = W tile; the
 //                             transpose of U comes from the tensor core as
 //                             (-I) U^T with a constant A operand, so no thread ever transposes anything
-//     PT  = K Q^T             lanes 0..63 = token j, columns = token i
+//     PT  = K Q^T             an M = 64 product: token j = 16 (lane / 32) + lane mod 16 on the lower 16 lanes of every lane
+//                             quadrant, columns = token i; lanes 16..31 of a warp read the upper 32 columns of the lower ones
 //     O1  = S0 Q^T
 //     O2  = U_new^T P^T       A = bf16(U_new^T) (written over D1's columns), B = P_ij = exp(g_i-g_j) PT_ji [j <= i]
 //     S  += (U_new^T exp(g_C - g_j)) K     accumulated onto exp(g_C) S0 (the decay is a pass over the TMEM columns)
@@ -22,7 +23,7 @@
 // Two MMA groups per chunk; Q, K, W, U tiles of the next chunk are in flight (two stages) while a chunk is worked on.
 // All operand layouts are the ones the chunk-prepare kernel uses.
 // Warps: 16 compute warps (four threads per TMEM lane), one that issues every MMA, one that issues the TMA loads and
-// the output stores. The chain of a sequence is thread work (every phase runs on all 16 warps at once, so its
+// the output stores, two that form the gate tables and the norms a chunk ahead. The chain of a sequence is thread work (every phase runs on all 16 warps at once, so its
 // instruction count is what it costs); hand-offs to the issuing warp are hardware barriers, completions come back
 // through mbarriers (a poll costs ~200 cycles, so as few as possible are waited for).
 // Instantiations: packed variable-length sequences (one CTA per (sequence, value head), starting at the sequence's
@@ -42,6 +43,7 @@ using namespace sm100;
 constexpr int kC = 64;         // chunk size
 constexpr int kD = 128;        // d_k = d_v
 constexpr int kThreads = 512;  // compute threads, four per TMEM lane; two more warps issue the MMAs and the TMA loads
+constexpr int kTabThreads = 64;  // gate tables and norms, one thread per token of a chunk
 constexpr float kLog2e = 1.4426950408889634f;
 
 // TMEM column map (512 columns: one CTA per SM)
@@ -49,7 +51,7 @@ constexpr uint32_t kSD = 0;    // 128: state S, fp32 accumulator
 constexpr uint32_t kSA = 128;  // 64: bf16(S0) as A operand (K = d_k)
 constexpr uint32_t kIA = 192;  // 64: -I as A operand (K = d_v), constant
 constexpr uint32_t kD1 = 256;  // 64: S0 W^T - U^T, then the two bf16 forms of U_new^T as A operands
-constexpr uint32_t kPT = 320;  // 64: K Q^T (lanes 0..63); once read, the lo bf16 halves of the two forms of U_new^T
+constexpr uint32_t kPT = 320;  // 64: K Q^T (half of the lanes); once read, the lo bf16 halves of the two forms of U_new^T
 constexpr uint32_t kO1 = 384;  // 64: S0 Q^T
 constexpr uint32_t kO2 = 448;  // 64: U_new^T P^T; between chunks it holds the lo bf16 half of S0 (A operand)
 constexpr uint32_t kTmemCols = 512;
@@ -60,7 +62,7 @@ constexpr int kStageBytes = 4 * kTileBytes;  // Q, K, W, U
 constexpr int kOffQ = 0, kOffK = kTileBytes, kOffW = 2 * kTileBytes, kOffU = 3 * kTileBytes;
 constexpr int kOffP = 2 * kStageBytes;       // 2 x 8 KB: P as B operand [64 x 64] (MN-major, no swizzle), hi and lo halves
 constexpr int kOffO = kOffP + 16384;          // 2 x 16 KB: O tile staged for the bulk store (128B swizzle), two buffers
-constexpr int kTab = 5 * 64;  // floats per table buffer: exp(g_i), exp(g_C - g_j), g, 1 / ||k_j||, 1 / ||q_i||
+constexpr int kTab = 5 * 64;  // floats per table buffer: scale exp(g_i) / ||q_i||, -exp(g_C - g_j) / ||k_j||, g, -1 / ||k_j||, scale / ||q_i||
 constexpr int kOffG = kOffO + 2 * kTileBytes;  // three table buffers
 constexpr int kSmemTotal = kOffG + 3 * kTab * 4;
 
@@ -101,20 +103,59 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity) {
 // Hand-off from the 512 compute threads to the issuing warp over a hardware barrier: the threads arrive and go on, the
 // issuing warp waits. (An mbarrier poll costs the waiting warp ~200-300 cycles per hand-off on the chain of the
 // sequence; this is a few tens.) The wait has no bound of its own: threads whose own bounded waits run out arrive on both hand-offs before they leave.
+// Hand-off 4 (state copies in place) also takes the table threads, which wait on it: they stay one chunk ahead.
 template <int ID>
 __device__ __forceinline__ void handoff_arrive() {
-    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(kThreads + 32) : "memory");
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
 }
 template <int ID>
 __device__ __forceinline__ void handoff_wait() {
-    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(kThreads + 32) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
+}
+// 8 columns of 16 lanes: threads 0..15 the columns from taddr on, threads 16..31 of the same lanes those 32 further
+__device__ __forceinline__ void tmem_ld8_split32(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], 32;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+typedef unsigned long long f2;  // two packed fp32
+__device__ __forceinline__ f2 pair2(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t pack_pair(f2 v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return pack_bf16x2(a, b);
+}
+// two values as bf16 pairs hi + lo
+__device__ __forceinline__ void split_pair(f2 v, uint32_t& hi, uint32_t& lo) {
+    hi = pack_pair(v);
+    f2 rest;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rest) : "l"(v), "l"(pair2(bf16_lo(hi), bf16_hi(hi))));
+    lo = pack_pair(rest);
+}
+// 16 lanes x 16 columns of an accumulator as the fragments of four 8 x 8 matrices: r[0..1] lanes 0..7, r[2..3] lanes 8..15
+// of columns 0..7, r[4..7] the same of columns 8..15; thread l holds lane l / 4, columns 2 (l mod 4) and the next
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
 }
 
 // VAR: packed variable-length sequences (own instantiation: its masks sit on the chain the dense case is bound by)
 // SO: state only: no queries, no output (the first pass of the segmented call); U may be absent per sequence.
 // NRM: GDN_FLAG_K_L2NORM (keys and queries normalised here): own instantiations, the plain chain pays nothing for it.
 template <bool VAR, bool SO, bool NRM>
-__global__ void __launch_bounds__(kThreads + 64, 1)
+__global__ void __launch_bounds__(kThreads + 64 + kTabThreads, 1)
 chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmU,
                    const __grid_constant__ CUtensorMap tmO, const ParamsS p) {
@@ -137,6 +178,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const int lane = tid & 31;
     const bool issuer = warp == kThreads / 32;        // every tcgen05.mma
     const bool producer = warp == kThreads / 32 + 1;  // every TMA load
+    const bool tabler = warp >= kThreads / 32 + 2;    // gate tables, norms
 
     if (tid == 0) {
         mbar_init(&bar_full[0], 1);
@@ -186,7 +228,79 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const uint32_t smem_a = smem_u32(smem);
     volatile int* fail = reinterpret_cast<volatile int*>(&s_fail);
 
-    if (producer) {
+    if (tabler) {
+        // ================= table threads, one per token. Before hand-off 4 of chunk c they have written the factors of
+        // chunk c (read behind the completion of its first product, which that hand-off precedes) and the gates of chunk
+        // c + 1 (read from its start on, behind the same completion one chunk earlier). Three buffers: the threads are done
+        // with a chunk's tables when they arrive on the next hand-off 4, and the table threads wait for it.
+        const int tt = tid - (kThreads + 64);
+        const bool g_raw = (p.flags & GDN_FLAG_G_RAW) != 0;
+        auto fetch = [&](int c) -> float { return (c < n_c && (!VAR || c * kC + tt < len)) ? __ldg(gseq + (c * kC + tt) * gstep) : 0.f; };
+        auto put_gates = [&](int c, float gc) {
+            float* tb = gtab + (c % 3) * kTab;
+            const int left = len - c * kC;  // tokens of this chunk (>= 64 except for a short last chunk)
+            if (g_raw) {
+                // inclusive prefix sum over the chunk's 64 tokens: inside each of the two warps by shuffles ...
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const float v = __shfl_up_sync(0xFFFFFFFFu, gc, off);
+                    if (lane >= off) gc += v;
+                }
+                if (tt == 31) tb[128 + 63] = gc;  // ... and the first warp's total through the table itself
+                asm volatile("bar.sync 3, 64;" ::: "memory");
+                if (tt >= 32) gc += tb[128 + 63];
+                asm volatile("bar.sync 3, 64;" ::: "memory");
+            }
+            tb[128 + tt] = gc;
+            asm volatile("bar.sync 3, 64;" ::: "memory");
+            if (VAR && !g_raw && left < kC) {
+                // cumulative gates: tokens past the end keep the gate of the last real token
+                gc = tb[128 + (tt < left ? tt : left - 1)];
+                asm volatile("bar.sync 3, 64;" ::: "memory");
+                tb[128 + tt] = gc;
+                asm volatile("bar.sync 3, 64;" ::: "memory");
+            }
+        };
+        // 1 / ||row|| of row tt of a tile in shared memory (the sum does not care about the swizzle inside the row: each of
+        // eight neighbouring threads starts at another 16-byte piece, free of bank conflicts)
+        auto inv_norm = [&](const uint8_t* tile) -> float {
+            float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const uint4 w4 = *reinterpret_cast<const uint4*>(tile + (i >> 3) * 8192 + tt * 128 + (((i + tt) & 7) << 4));
+                const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float a = __uint_as_float(w[q] << 16), b = __uint_as_float(w[q] & 0xFFFF0000u);
+                    a0 = fmaf(a, a, a0);
+                    a1 = fmaf(b, b, a1);
+                }
+            }
+            return rsqrtf(fmaxf(a0 + a1, 1e-30f));
+        };
+        float g_next = fetch(0);
+        if (n_c > 0) put_gates(0, g_next);
+        asm volatile("bar.sync 1, 576;" ::: "memory");
+        g_next = fetch(1);
+        for (int c = 0; c < n_c && *fail == 0; ++c) {
+            if (c + 1 < n_c) put_gates(c + 1, g_next);
+            g_next = fetch(c + 2);
+            float* tb = gtab + (c % 3) * kTab;
+            float rk = 1.f, so = p.scale;
+            if (NRM) {
+                if (!wait_bar(&bar_full[c & 1], (c >> 1) & 1)) *fail = 1;
+                const uint8_t* st = smem + (c & 1) * kStageBytes;
+                rk = (VAR && tt >= len - c * kC) ? 0.f : inv_norm(st + kOffK);
+                if (!SO) so *= inv_norm(st + kOffQ);
+                tb[192 + tt] = -rk;
+            }
+            const float gc = tb[128 + tt], gC = tb[128 + 63];
+            tb[tt] = so * fast_exp2(gc * kLog2e);
+            tb[64 + tt] = -rk * fast_exp2((gC - gc) * kLog2e);
+            tb[256 + tt] = so;
+            handoff_wait<4>();
+        }
+    } else if (producer) {
         // ================= loading / storing warp: the four tiles of chunk c into stage c & 1, as soon as the products
         // that read the stage's previous tiles are complete; and the bulk stores of the staged output tiles, so that
         // no compute thread waits for the others at the end of a chunk
@@ -240,6 +354,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const uint32_t idesc_kk64 = instr_desc(128, 64, 1, 1, 0, 0, 1);   // B K-major (a TMA tile as [N x K])
         const uint32_t idesc_mn64 = instr_desc(128, 64, 1, 1, 0, 1, 1);   // B MN-major
         const uint32_t idesc_mn128 = instr_desc(128, 128, 1, 1, 0, 1, 1);
+        const uint32_t idesc_pt = instr_desc(64, 64, 1, 1, 0, 0, 1);
         // the products of chunk c that do not depend on the state: D1 <- (-I) U^T and PT = K Q^T
         auto issue_pre = [&](int c) {
             const uint32_t sa = smem_a + (c & 1) * kStageBytes;
@@ -254,12 +369,11 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     }
                 }
                 if (!SO) {
-                    // rows 64..127 of the A operand read past the 64-row K tile: unused lanes
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) {
                         const uint64_t ad = smem_desc(sa + kOffK + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024, SWZ_128B);
                         const uint64_t bd = smem_desc(sa + kOffQ + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024, SWZ_128B);
-                        mma_f16_ss(tmem + kPT, ad, bd, idesc_kk64, ks > 0);
+                        mma_f16_ss(tmem + kPT, ad, bd, idesc_pt, ks > 0);
                     }
                     mma_commit(&bar_pre);  // (state only: nothing of this group is waited for by itself)
                 }
@@ -334,6 +448,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             // state-independent products of the next chunk follow them directly
             if (c + 1 < n_c) issue_pre(c + 1);
         }
+        if (*fail != 0) handoff_arrive<4>();  // (the table threads may be waiting on it)
     } else {
         // ================= compute threads (512): four per TMEM lane
         uint32_t par_pre = 0, par_d1 = 0, par_o2 = 0, par_g2 = 0;
@@ -376,101 +491,15 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             tc_fence_before_sync();
             handoff_arrive<4>();
         }
-        // gates of the first chunk
-        float g_reg = 0.f;
-        // (a short last chunk: tokens past the sequence's end decay nothing and write nothing)
-        // The gate tables are the job of threads 64..127: their lanes hold no row of P, so they are idle while the other
-        // half of the CTA forms P.
-        const int tt = tid - 64;  // token of a table thread
-        const bool tabler = tt >= 0 && tt < 64;
-        if (n_c > 0 && tabler) g_reg = (!VAR || tt < len) ? __ldg(gseq + tt * gstep) : 0.f;
         bool ok = true;
-        // gate tables of a chunk: written by 64 threads into the buffer of that chunk one barrier before they are read
-        const bool g_raw = (p.flags & GDN_FLAG_G_RAW) != 0;
-        constexpr bool f_nrm = NRM;
-        auto fill_tables = [&](int c) {
-            if (tabler) {
-                float* tb = gtab + (c % 3) * kTab;
-                float gc = g_reg;
-                const int left = len - c * kC;  // tokens of this chunk (>= 64 except for a short last chunk)
-                if (g_raw) {
-                    // inclusive prefix sum over the chunk's 64 tokens: inside each of the two warps by shuffles ...
-#pragma unroll
-                    for (int off = 1; off < 32; off <<= 1) {
-                        const float v = __shfl_up_sync(0xFFFFFFFFu, gc, off);
-                        if (lane >= off) gc += v;
-                    }
-                    if (tt == 31) tb[128 + 63] = gc;  // ... and the first warp's total through the table itself
-                    asm volatile("bar.sync 3, 64;" ::: "memory");
-                    if (tt >= 32) gc += tb[128 + 63];
-                    asm volatile("bar.sync 3, 64;" ::: "memory");
-                }
-                tb[128 + tt] = gc;
-                asm volatile("bar.sync 3, 64;" ::: "memory");
-                if (VAR && !g_raw && left < kC) {
-                    // cumulative gates: tokens past the end keep the gate of the last real token
-                    gc = tb[128 + (tt < left ? tt : left - 1)];
-                    asm volatile("bar.sync 3, 64;" ::: "memory");
-                    tb[128 + tt] = gc;
-                    asm volatile("bar.sync 3, 64;" ::: "memory");
-                }
-                const float gC = tb[128 + 63];  // cumulative gate of the chunk's last token
-                // (with the keys and queries normalised here, their factors ride on the two gate factors: exp(g_i) only
-                // ever multiplies a product with q_i, exp(g_C - g_j) one with k_j)
-                tb[tt] = fast_exp2(gc * kLog2e) * (f_nrm ? tb[256 + tt] : 1.f);
-                tb[64 + tt] = fast_exp2((gC - gc) * kLog2e) * (f_nrm ? tb[192 + tt] : 1.f);
-            }
-        };
-        // GDN_FLAG_K_L2NORM: 1 / ||k_j|| and 1 / ||q_i|| of chunk c from its tiles in shared memory, by the 256 threads
-        // whose lanes hold no row of P (the sum of squares of a row does not care about the swizzle inside the row)
-        auto fill_norms = [&](int c) {
-            if (wq >= 2) {
-                // (the issuing warp has waited for these tiles, or will; observing the phase here orders the reads below)
-                if (!wait_bar(&bar_full[c & 1], (c >> 1) & 1)) *fail = 1;
-                const int u = (tid >> 7) * 64 + (tid & 63);  // 0 .. 255
-                float* tb = gtab + (c % 3) * kTab;
-                // A warp reads 512 contiguous bytes per step (four rows of a 64-column sub-tile): conflict-free. Thread u
-                // sees rows u >> 3 and 32 + (u >> 3) of both sub-tiles; the eight lanes of a row add up by shuffles.
-#pragma unroll
-                for (int which = 0; which < (SO ? 1 : 2); ++which) {
-                    const uint8_t* tile = smem + (c & 1) * kStageBytes + (which == 0 ? kOffK : kOffQ) + u * 16;
-                    float acc[2] = {0.f, 0.f};
-#pragma unroll
-                    for (int it = 0; it < 4; ++it) {
-                        const uint4 w4 = *reinterpret_cast<const uint4*>(tile + (it >> 1) * 8192 + (it & 1) * 4096);
-                        const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float a = __uint_as_float(w[i] << 16), b = __uint_as_float(w[i] & 0xFFFF0000u);
-                            acc[it & 1] = fmaf(a, a, fmaf(b, b, acc[it & 1]));
-                        }
-                    }
-#pragma unroll
-                    for (int off = 1; off < 8; off <<= 1) {
-                        acc[0] += __shfl_xor_sync(0xFFFFFFFFu, acc[0], off);
-                        acc[1] += __shfl_xor_sync(0xFFFFFFFFu, acc[1], off);
-                    }
-                    if ((u & 7) == 0) {
-                        tb[(which == 0 ? 192 : 256) + (u >> 3)] = rsqrtf(fmaxf(acc[0], 1e-30f));
-                        tb[(which == 0 ? 192 : 256) + 32 + (u >> 3)] = rsqrtf(fmaxf(acc[1], 1e-30f));
-                    }
-                }
-                asm volatile("bar.sync 7, 256;" ::: "memory");
-            }
-        };
-        if (n_c > 0) {
-            if (f_nrm) fill_norms(0);
-            fill_tables(0);
-        }
-        asm volatile("bar.sync 1, 512;" ::: "memory");
+        asm volatile("bar.sync 1, 576;" ::: "memory");  // the gates of the first chunk
         for (int c = 0; c < n_c; ++c) {
-            const float* se = gtab + (c % 3) * kTab;  // exp(g_i)
-            const float* sf = se + 64;               // exp(g_C - g_j)
+            const float* se = gtab + (c % 3) * kTab;  // scale exp(g_i) / ||q_i||
+            const float* sf = se + 64;               // -exp(g_C - g_j) / ||k_j|| (D1 holds -U_new)
             const float* sg = se + 128;              // g_i (cumulative inside the chunk)
             const float gC = sg[63];
             const int left = len - c * kC;
             const bool short_chunk = VAR && left < kC;
-            if (c + 1 < n_c && tabler) g_reg = (!VAR || (c + 1) * kC + tt < len) ? __ldg(gseq + ((c + 1) * kC + tt) * gstep) : 0.f;
 
             // ---- decay of the accumulator, S <- exp(g_C) S0 (the products of this chunk read the bf16 copies)
             {
@@ -488,73 +517,66 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 for (int i = 0; i < 16; ++i) w16[i] = v[16 + i];
                 tmem_st16(lane_base + kSD + h * 32 + 16, w16);
             }
-            // ---- P_ij = exp(g_i - g_j) PT_ji for j <= i (hi + lo): token j = lane (rows 0..63 only), this thread's 16 columns i
+            // ---- P_ij = exp(g_i - g_j) PT_ji for j <= i (hi + lo): this thread's token j and 8 columns i. (Keys and queries
+            // normalised here: 1 / ||k_j|| rides on U_new_j, 1 / ||q_i|| on the output.)
             if (!SO && !wait_group(&bar_pre, par_pre)) { ok = false; break; }
-            if (!SO && wq < 2) {
-                uint32_t d[16];
-                tmem_ld16(lane_base + kPT + h * 16, d);
+            if (!SO) {
+                uint32_t d[8];
+                tmem_ld8_split32(lane_base + kPT + h * 8, d);
+                const int j = wq * 16 + (lane & 15), n8 = (lane >> 4) * 4 + h;  // columns i = 8 n8 ..
+                const float gj = sg[j] * kLog2e;
+                float gi[8];
+#pragma unroll
+                for (int i4 = 0; i4 < 2; ++i4) {
+                    const float4 q4 = *reinterpret_cast<const float4*>(sg + n8 * 8 + i4 * 4);
+                    gi[i4 * 4 + 0] = q4.x; gi[i4 * 4 + 1] = q4.y; gi[i4 * 4 + 2] = q4.z; gi[i4 * 4 + 3] = q4.w;
+                }
                 tmem_wait_ld();
-                const float gj = sg[t] * kLog2e;
-                const float rkj = f_nrm ? sg[64 + t] : 1.f;
-                float gi16[16];  // g of this thread's 16 columns (four 16-byte loads instead of sixteen scalar ones)
+                uint32_t w[4], wl[4];
 #pragma unroll
-                for (int i4 = 0; i4 < 4; ++i4) {
-                    const float4 q4 = *reinterpret_cast<const float4*>(sg + h * 16 + i4 * 4);
-                    gi16[i4 * 4 + 0] = q4.x; gi16[i4 * 4 + 1] = q4.y; gi16[i4 * 4 + 2] = q4.z; gi16[i4 * 4 + 3] = q4.w;
-                }
+                for (int i2 = 0; i2 < 4; ++i2) {
+                    float v[2];
 #pragma unroll
-                for (int c2 = 0; c2 < 2; ++c2) {
-                    uint32_t w[4], wl[4];
-#pragma unroll
-                    for (int i2 = 0; i2 < 4; ++i2) {
-                        float v[2];
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int i = h * 16 + c2 * 8 + i2 * 2 + q;
-                            float x = __uint_as_float(d[c2 * 8 + i2 * 2 + q]) *
-                                      fast_exp2(fminf(fmaf(gi16[c2 * 8 + i2 * 2 + q], kLog2e, -gj), 0.f));
-                            if (f_nrm) x *= rkj * sg[128 + i];  // 1 / (||k_j|| ||q_i||)
-                            v[q] = (t <= i) ? x : 0.f;
-                        }
-                        w[i2] = pack_bf16x2(v[0], v[1]);
-                        wl[i2] = pack_bf16x2(v[0] - bf16_lo(w[i2]), v[1] - bf16_hi(w[i2]));
+                    for (int q = 0; q < 2; ++q) {
+                        const float x = __uint_as_float(d[i2 * 2 + q]) * fast_exp2(fminf(fmaf(gi[i2 * 2 + q], kLog2e, -gj), 0.f));
+                        v[q] = (j <= n8 * 8 + i2 * 2 + q) ? x : 0.f;
                     }
-                    // B operand [K-dim = j][N = i], MN-major, no swizzle: the 16-byte piece of row j for column group n8
-                    *reinterpret_cast<uint4*>(smem + kOffP + (h * 2 + c2) * 1024 + t * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-                    *reinterpret_cast<uint4*>(smem + kOffP + 8192 + (h * 2 + c2) * 1024 + t * 16) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+                    w[i2] = pack_bf16x2(v[0], v[1]);
+                    wl[i2] = pack_bf16x2(v[0] - bf16_lo(w[i2]), v[1] - bf16_hi(w[i2]));
                 }
+                // B operand [K-dim = j][N = i], MN-major, no swizzle: the 16-byte piece of row j for column group n8
+                *reinterpret_cast<uint4*>(smem + kOffP + n8 * 1024 + j * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(smem + kOffP + 8192 + n8 * 1024 + j * 16) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
             }
-            // the next chunk's gate tables, by threads that had no part in P (published by the barrier at the chunk's end)
-            if (c + 1 < n_c && !f_nrm) fill_tables(c + 1);
             // ---- U_new^T = -D1 as bf16 hi + lo, plain and gate-scaled (the sums over the tokens of a chunk telescope
             // on correlated keys, so single bf16 copies cost 1e-2 there). This thread's 16 tokens are one k-step of the
             // products that consume them: the hi halves are written over its own D1 columns (plain -> 16 h .. 16 h + 7,
-            // scaled -> 16 h + 8 ..), the lo halves at the same offsets of the PT region (read above by this thread).
+            // scaled -> 16 h + 8 ..), the lo halves at the same offsets of the PT region.
             if (!wait_group(&bar_d1, par_d1)) { ok = false; break; }
+            // (the four warps of a lane quadrant have read their columns of PT)
+            if (!SO) asm volatile("bar.sync %0, 128;" ::"r"(8 + wq) : "memory");
             {
                 uint32_t d[16];
                 tmem_ld16(lane_base + kD1 + h * 16, d);
                 tmem_wait_ld();
                 uint32_t hi[16], lo[16];
 #pragma unroll
-                float f16[16];
+                for (int i = 0; i < 8; i += 2) {
+                    const ulonglong2 f4 = *reinterpret_cast<const ulonglong2*>(sf + h * 16 + 2 * i);
+                    ulonglong2 k4;
+                    if (NRM && !SO) k4 = *reinterpret_cast<const ulonglong2*>(sg + 64 + h * 16 + 2 * i);
 #pragma unroll
-                for (int i4 = 0; i4 < 4; ++i4) {
-                    const float4 q4 = *reinterpret_cast<const float4*>(sf + h * 16 + i4 * 4);
-                    f16[i4 * 4 + 0] = q4.x; f16[i4 * 4 + 1] = q4.y; f16[i4 * 4 + 2] = q4.z; f16[i4 * 4 + 3] = q4.w;
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    float u0 = -__uint_as_float(d[2 * i]), u1 = -__uint_as_float(d[2 * i + 1]);
-                    if (short_chunk) {  // rows past the sequence's end hold another sequence's W, U
-                        if (h * 16 + 2 * i >= left) u0 = 0.f;
-                        if (h * 16 + 2 * i + 1 >= left) u1 = 0.f;
+                    for (int q = 0; q < 2; ++q) {
+                        float d0 = __uint_as_float(d[2 * (i + q)]), d1 = __uint_as_float(d[2 * (i + q) + 1]);
+                        if (short_chunk) {  // rows past the sequence's end hold another sequence's W, U
+                            if (h * 16 + 2 * (i + q) >= left) d0 = 0.f;
+                            if (h * 16 + 2 * (i + q) + 1 >= left) d1 = 0.f;
+                        }
+                        const f2 u = pair2(d0, d1);
+                        split_pair(mul2(u, q == 0 ? f4.x : f4.y), hi[8 + i + q], lo[8 + i + q]);
+                        if (!SO) split_pair(NRM ? mul2(u, q == 0 ? k4.x : k4.y) : pair2(-d0, -d1), hi[i + q], lo[i + q]);
+                        else hi[i + q] = lo[i + q] = 0u;  // (only the output product reads the plain form)
                     }
-                    const float s0 = u0 * f16[2 * i], s1 = u1 * f16[2 * i + 1];
-                    hi[i] = pack_bf16x2(u0, u1);
-                    hi[8 + i] = pack_bf16x2(s0, s1);
-                    lo[i] = pack_bf16x2(u0 - bf16_lo(hi[i]), u1 - bf16_hi(hi[i]));
-                    lo[8 + i] = pack_bf16x2(s0 - bf16_lo(hi[8 + i]), s1 - bf16_hi(hi[8 + i]));
                 }
                 tmem_st16(lane_base + kD1 + h * 16, hi);
                 tmem_st16(lane_base + kPT + h * 16, lo);
@@ -563,13 +585,6 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             tmem_wait_st();
             tc_fence_before_sync();
             handoff_arrive<5>();
-            // with the norms of the next chunk's keys and queries in the tables, both are formed here instead: the next
-            // chunk's tiles are still on their way while P is formed, and the threads idle now anyway
-            if (c + 1 < n_c && f_nrm) {
-                fill_norms(c + 1);
-                fill_tables(c + 1);
-            }
-
             if (!SO) {
                 // The storing warp has released the PREVIOUS chunk's staging buffer (polled here, in the shadow of the
                 // output product; the store was issued most of a chunk ago). That is one chunk later than this chunk's
@@ -577,34 +592,36 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 // storing warp has taken the previous chunk's hand-off: the threads must not arrive on that hardware
                 // barrier a second time before it has, however long a store may be held up.
                 if (c >= 1 && !wait_bar(&bar_stg[(c - 1) & 1], ((c - 1) >> 1) & 1)) { *fail = 1; ok = false; break; }
-                // ---- exp(g_i) O1 (complete with O2: products finish in the order they were issued)
+                // ---- O^T = scale (exp(g_i) O1 + O2), in fragments of 8 x 8: this warp's 32 features x 16 tokens, transposed
+                // on the way to the staged tile (O1 is complete with O2: products finish in the order they were issued)
                 if (!wait_group(&bar_o2, par_o2)) { ok = false; break; }
-                float o[16];
                 {
-                    uint32_t d[16];
-                    tmem_ld16(lane_base + kO1 + h * 16, d);
-                    tmem_wait_ld();
-    #pragma unroll
-                    for (int i4 = 0; i4 < 4; ++i4) {
-                        const float4 e4 = *reinterpret_cast<const float4*>(se + h * 16 + i4 * 4);
-                        o[i4 * 4 + 0] = __uint_as_float(d[i4 * 4 + 0]) * e4.x;
-                        o[i4 * 4 + 1] = __uint_as_float(d[i4 * 4 + 1]) * e4.y;
-                        o[i4 * 4 + 2] = __uint_as_float(d[i4 * 4 + 2]) * e4.z;
-                        o[i4 * 4 + 3] = __uint_as_float(d[i4 * 4 + 3]) * e4.w;
+                    const int t2 = h * 16 + 2 * (lane & 3);
+                    const float2 e0 = *reinterpret_cast<const float2*>(se + t2), e1 = *reinterpret_cast<const float2*>(se + t2 + 8);
+                    float2 q0 = make_float2(p.scale, p.scale), q1 = q0;
+                    if (NRM) {
+                        q0 = *reinterpret_cast<const float2*>(se + 256 + t2);
+                        q1 = *reinterpret_cast<const float2*>(se + 256 + t2 + 8);
                     }
-                }
-                // ---- O^T = scale (exp(g_i) O1 + O2): element (token i, feature t) of the staged tile
-                {
-                    uint32_t d[16];
-                    tmem_ld16(lane_base + kO2 + h * 16, d);
-                    tmem_wait_ld();
-                    uint8_t* sub = smem + kOffO + (c & 1) * kTileBytes + (t >> 6) * 8192;
-                    const int cch = (t & 63) >> 3;
-    #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int tok = h * 16 + i;
-                        const __nv_bfloat16 v = __float2bfloat16_rn(p.scale * (o[i] + __uint_as_float(d[i])));
-                        *reinterpret_cast<__nv_bfloat16*>(sub + tok * 128 + ((cch ^ (tok & 7)) << 4) + (t & 7) * 2) = v;
+                    const int tok = h * 16 + ((lane >> 4) << 3) + (lane & 7);  // row of the staged tile this lane addresses
+#pragma unroll
+                    for (int lh = 0; lh < 2; ++lh) {
+                        uint32_t a[8], d[8];
+                        tmem_ld_frag(lane_base + (static_cast<uint32_t>(lh * 16) << 16) + kO1 + h * 16, a);
+                        tmem_ld_frag(lane_base + (static_cast<uint32_t>(lh * 16) << 16) + kO2 + h * 16, d);
+                        tmem_wait_ld();
+                        uint32_t m[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float2 e = k < 2 ? e0 : e1, q = k < 2 ? q0 : q1;
+                            m[k] = pack_bf16x2(fmaf(__uint_as_float(a[2 * k]), e.x, __uint_as_float(d[2 * k]) * q.x),
+                                               fmaf(__uint_as_float(a[2 * k + 1]), e.y, __uint_as_float(d[2 * k + 1]) * q.y));
+                        }
+                        const int fb = wq * 4 + lh * 2 + ((lane >> 3) & 1);  // block of 8 features
+                        const uint32_t at = smem_a + kOffO + (c & 1) * kTileBytes + (fb >> 3) * 8192 + tok * 128 + (((fb & 7) ^ (tok & 7)) << 4);
+                        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(m[0]), "r"(m[1]),
+                                     "r"(m[2]), "r"(m[3])
+                                     : "memory");
                     }
                 }
                 // the tile goes to the storing warp: no compute thread waits for the others here
@@ -618,20 +635,15 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 uint32_t v[32], pk[16];
                 tmem_ld32(lane_base + kSD + h * 32, v);
                 tmem_wait_ld();
+                uint32_t lo[16];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+                for (int i = 0; i < 16; ++i) split_pair(pair2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), pk[i], lo[i]);
                 tmem_st16(lane_base + kSA + h * 16, pk);
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    pk[i] = pack_bf16x2(__uint_as_float(v[2 * i]) - bf16_lo(pk[i]), __uint_as_float(v[2 * i + 1]) - bf16_hi(pk[i]));
-                tmem_st16(lane_base + kO2 + h * 16, pk);
+                tmem_st16(lane_base + kO2 + h * 16, lo);
                 tmem_wait_st();
                 tc_fence_before_sync();
                 handoff_arrive<4>();
             }
-            // With the norms in the tables, the next chunk's tables are written after this chunk's hand-off (see above),
-            // so the hand-off -> product -> completion chain does not order them before their readers: one barrier.
-            if (NRM && c + 1 < n_c) asm volatile("bar.sync 1, 512;" ::: "memory");
             if (!SO && short_chunk) {
                 // only the rows of real tokens leave, 16 bytes per thread and step, from the staged (swizzled) tile
                 asm volatile("bar.sync 1, 512;" ::: "memory");  // (last chunk of a packed sequence only)
@@ -922,7 +934,7 @@ int launch_chunk_state(const ProblemS& q, cudaStream_t stream) {
                 : var        ? (nrm ? chunk_state_kernel<true, false, true> : chunk_state_kernel<true, false, false>)
                              : (nrm ? chunk_state_kernel<false, false, true> : chunk_state_kernel<false, false, false>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GDN_ERR_LAUNCH;
-    kern<<<static_cast<int>(n_cta), kThreads + 64, smem, stream>>>(mQ, mK, mW, mU, mO, prm);
+    kern<<<static_cast<int>(n_cta), kThreads + 64 + kTabThreads, smem, stream>>>(mQ, mK, mW, mU, mO, prm);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_LAUNCH;
 }

@@ -23,7 +23,7 @@
 // Two MMA groups per chunk; Q, K, W, U tiles of the next chunk are in flight (two stages) while a chunk is worked on.
 // All operand layouts are the ones the chunk-prepare kernel uses.
 // Warps: 16 compute warps (four threads per TMEM lane), one that issues every MMA, one that issues the TMA loads and
-// the output stores, two that form the gate tables and the norms a chunk ahead. The chain of a sequence is thread work (every phase runs on all 16 warps at once, so its
+// the output stores, four that form the gate tables and the norms a chunk ahead. The chain of a sequence is thread work (every phase runs on all 16 warps at once, so its
 // instruction count is what it costs); hand-offs to the issuing warp are hardware barriers, completions come back
 // through mbarriers (a poll costs ~200 cycles, so as few as possible are waited for).
 // Instantiations: packed variable-length sequences (one CTA per (sequence, value head), starting at the sequence's
@@ -43,7 +43,7 @@ using namespace sm100;
 constexpr int kC = 64;         // chunk size
 constexpr int kD = 128;        // d_k = d_v
 constexpr int kThreads = 512;  // compute threads, four per TMEM lane; two more warps issue the MMAs and the TMA loads
-constexpr int kTabThreads = 64;  // gate tables and norms, one thread per token of a chunk
+constexpr int kTabThreads = 128;  // gate tables and norms, two threads per token of a chunk (its key, its query)
 constexpr float kLog2e = 1.4426950408889634f;
 
 // TMEM column map (512 columns: one CTA per SM)
@@ -80,6 +80,7 @@ struct ParamsS {
     const int* seq_start;  // first token of sequence s
     const int* seq_end;    // one past its last token (the public call passes cu_seqlens and cu_seqlens + 1)
     const int* seq_no_u;   // optional: sequence s runs with U = 0 (the state map of a segment, see the segmented call)
+    int out_from;            // S_out holds the final states of the sequences from this one on
     __nv_bfloat16* O;  // output tensor (rows of a short last chunk are stored one by one)
 };
 
@@ -229,11 +230,12 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     volatile int* fail = reinterpret_cast<volatile int*>(&s_fail);
 
     if (tabler) {
-        // ================= table threads, one per token. Before hand-off 4 of chunk c they have written the factors of
+        // ================= table threads, two per token (the second only for the norm of its query). Before hand-off 4 of chunk c they have written the factors of
         // chunk c (read behind the completion of its first product, which that hand-off precedes) and the gates of chunk
         // c + 1 (read from its start on, behind the same completion one chunk earlier). Three buffers: the threads are done
         // with a chunk's tables when they arrive on the next hand-off 4, and the table threads wait for it.
-        const int tt = tid - (kThreads + 64);
+        const int tt = (tid - (kThreads + 64)) & 63;
+        const bool second = tid >= kThreads + 64 + 64;
         const bool g_raw = (p.flags & GDN_FLAG_G_RAW) != 0;
         auto fetch = [&](int c) -> float { return (c < n_c && (!VAR || c * kC + tt < len)) ? __ldg(gseq + (c * kC + tt) * gstep) : 0.f; };
         auto put_gates = [&](int c, float gc) {
@@ -264,40 +266,49 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // 1 / ||row|| of row tt of a tile in shared memory (the sum does not care about the swizzle inside the row: each of
         // eight neighbouring threads starts at another 16-byte piece, free of bank conflicts)
         auto inv_norm = [&](const uint8_t* tile) -> float {
-            float a0 = 0.f, a1 = 0.f;
+            f2 a[2] = {0ull, 0ull};
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 const uint4 w4 = *reinterpret_cast<const uint4*>(tile + (i >> 3) * 8192 + tt * 128 + (((i + tt) & 7) << 4));
                 const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const float a = __uint_as_float(w[q] << 16), b = __uint_as_float(w[q] & 0xFFFF0000u);
-                    a0 = fmaf(a, a, a0);
-                    a1 = fmaf(b, b, a1);
+                    const f2 x = pair2(bf16_lo(w[q]), bf16_hi(w[q]));
+                    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a[q & 1]) : "l"(x));
                 }
             }
-            return rsqrtf(fmaxf(a0 + a1, 1e-30f));
+            float s0, s1, s2, s3;
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(s0), "=f"(s1) : "l"(a[0]));
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(s2), "=f"(s3) : "l"(a[1]));
+            return rsqrtf(fmaxf((s0 + s1) + (s2 + s3), 1e-30f));
         };
-        float g_next = fetch(0);
-        if (n_c > 0) put_gates(0, g_next);
-        asm volatile("bar.sync 1, 576;" ::: "memory");
-        g_next = fetch(1);
+        float g_next = 0.f;
+        if (!second) {
+            g_next = fetch(0);
+            if (n_c > 0) put_gates(0, g_next);
+            g_next = fetch(1);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");
         for (int c = 0; c < n_c && *fail == 0; ++c) {
-            if (c + 1 < n_c) put_gates(c + 1, g_next);
-            g_next = fetch(c + 2);
-            float* tb = gtab + (c % 3) * kTab;
-            float rk = 1.f, so = p.scale;
-            if (NRM) {
-                if (!wait_bar(&bar_full[c & 1], (c >> 1) & 1)) *fail = 1;
-                const uint8_t* st = smem + (c & 1) * kStageBytes;
-                rk = (VAR && tt >= len - c * kC) ? 0.f : inv_norm(st + kOffK);
-                if (!SO) so *= inv_norm(st + kOffQ);
-                tb[192 + tt] = -rk;
+            if (!second) {
+                if (c + 1 < n_c) put_gates(c + 1, g_next);
+                g_next = fetch(c + 2);
             }
+            float* tb = gtab + (c % 3) * kTab;
             const float gc = tb[128 + tt], gC = tb[128 + 63];
-            tb[tt] = so * fast_exp2(gc * kLog2e);
-            tb[64 + tt] = -rk * fast_exp2((gC - gc) * kLog2e);
-            tb[256 + tt] = so;
+            float r = 1.f;
+            if (NRM && !(SO && second)) {
+                if (!wait_bar(&bar_full[c & 1], (c >> 1) & 1)) *fail = 1;
+                r = inv_norm(smem + (c & 1) * kStageBytes + (second ? kOffQ : kOffK));
+            }
+            if (second) {
+                tb[tt] = p.scale * r * fast_exp2(gc * kLog2e);
+                tb[256 + tt] = p.scale * r;
+            } else {
+                if (VAR && tt >= len - c * kC) r = 0.f;
+                tb[192 + tt] = -r;
+                tb[64 + tt] = -r * fast_exp2((gC - gc) * kLog2e);
+            }
             handoff_wait<4>();
         }
     } else if (producer) {
@@ -492,7 +503,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             handoff_arrive<4>();
         }
         bool ok = true;
-        asm volatile("bar.sync 1, 576;" ::: "memory");  // the gates of the first chunk
+        asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");  // the gates of the first chunk
         for (int c = 0; c < n_c; ++c) {
             const float* se = gtab + (c % 3) * kTab;  // scale exp(g_i) / ||q_i||
             const float* sf = se + 64;               // -exp(g_C - g_j) / ||k_j|| (D1 holds -U_new)
@@ -663,8 +674,8 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             handoff_arrive<6>();
         }
         // ---- final state
-        if (ok && p.S_out != nullptr) {
-            float* so = p.S_out + ((long long)blockIdx.x * kD + t) * kD + h * 32;
+        if (ok && p.S_out != nullptr && static_cast<int>(b) >= p.out_from) {
+            float* so = p.S_out + (((long long)blockIdx.x - (long long)p.out_from * p.H_v) * kD + t) * kD + h * 32;
             uint32_t v[32];
             tmem_ld32(lane_base + kSD + h * 32, v);
             tmem_wait_ld();
@@ -719,72 +730,102 @@ bool make_map(CUtensorMap* tm, const void* base, long long heads, int T, int col
 // Set-up of the first pass: the token ranges of its 2P - 3 runs (runs 0 .. P-2: segment s from a zero state, segment 0
 // from the caller's; runs P-1 .. 2P-4: segments 1 .. P-2 from the identity with U = 0, which gives the matrix M of
 // S_end = S_start M + N), their initial states, the token ranges of the second pass and its first initial state.
-__global__ void segmented_setup_kernel(int P, int H_v, int n_chunks, const float* S_user, float* S_in1, float* S_start,
-                                       int* start1, int* end1, int* no_u1, int* start3, int* end3) {
+// Grid (n1 + 1 states, value heads): one state of 128 x 128 per CTA.
+__global__ void __launch_bounds__(256) segmented_setup_kernel(int P, int H_v, int n_chunks, const float* S_user, float* S_in1,
+                                                              float* S_start, int* start1, int* end1, int* no_u1, int* start3,
+                                                              int* end3) {
     const int n1 = 2 * P - 3;
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
-        for (int s_ = threadIdx.x; s_ < n1; s_ += 32) {
+    const int run = blockIdx.x, hv = blockIdx.y;
+    if (run == 0 && hv == 0) {
+        for (int s_ = threadIdx.x; s_ < n1; s_ += 256) {
             const int seg = (s_ <= P - 2) ? s_ : s_ - (P - 2);
             start1[s_] = (int)((long long)n_chunks * seg / P) * kC;
             end1[s_] = (int)((long long)n_chunks * (seg + 1) / P) * kC;
             no_u1[s_] = (s_ <= P - 2) ? 0 : 1;
         }
-        for (int s_ = threadIdx.x; s_ < P; s_ += 32) {
+        for (int s_ = threadIdx.x; s_ < P; s_ += 256) {
             start3[s_] = (int)((long long)n_chunks * s_ / P) * kC;
             end3[s_] = (int)((long long)n_chunks * (s_ + 1) / P) * kC;
         }
     }
-    const long long per = (long long)H_v * kD * kD;
-    const long long total = (long long)n1 * per;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total + per; e += (long long)gridDim.x * blockDim.x) {
-        if (e < total) {
-            const int s_ = (int)(e / per);
-            const long long r = e - (long long)s_ * per;
-            const int idx = (int)(r % (kD * kD));
-            float v = 0.f;
-            if (s_ == 0) v = (S_user != nullptr) ? S_user[r] : 0.f;
-            else if (s_ > P - 2) v = (idx / kD == idx % kD) ? 1.f : 0.f;
-            S_in1[e] = v;
-        } else {
-            const long long r = e - total;
-            S_start[r] = (S_user != nullptr) ? S_user[r] : 0.f;
+    const bool user = (run == 0 || run == n1) && S_user != nullptr;
+    const bool eye = run > P - 2 && run < n1;
+    const float4* src = reinterpret_cast<const float4*>(S_user + (user ? (long long)hv * kD * kD : 0));
+    float4* dst = reinterpret_cast<float4*>((run < n1 ? S_in1 + (long long)run * H_v * kD * kD : S_start) + (long long)hv * kD * kD);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < kD * kD / 4; i += 256) {
+        float4 v = user ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (eye) {
+            const int row = i / (kD / 4), c = row - (i % (kD / 4)) * 4;  // the diagonal's place among these four
+            v = make_float4(c == 0, c == 1, c == 2, c == 3);
         }
+        dst[i] = v;
     }
 }
 
 // S_start[k] = S_start[k-1] M_{k-1} + N_{k-1} for k = 2 .. P-1, S_start[1] = N_0 (the first segment ran from the caller's
-// state). One CTA per (value head, block of 16 state rows): the rows of the state are independent. fp32 FMAs.
+// state). One CTA per (value head, block of 32 state rows): the rows of the state are independent. fp32 FMAs, every sum
+// in the order of the state's columns. M (64 KB) comes into shared memory while the step before is worked on; a thread
+// holds 4 rows x 4 columns. What a step costs is the chain load -> product: 3 us (one thread column per output, M read from
+// L2 in the loop: 13 us).
+constexpr int kCombRows = 32;
+constexpr int kCombSmem = 2 * kD * kD * 4;
 __global__ void __launch_bounds__(256) segmented_combine_kernel(int P, int H_v, const float* S_out1, float* S_start) {
-    __shared__ float cur[16][kD];
-    const int hv = blockIdx.x, r0 = blockIdx.y * 16;
+    extern __shared__ __align__(16) float comb_m[];  // two buffers of M
+    __shared__ __align__(16) float cur[kCombRows][kD + 4];
+    const int hv = blockIdx.x, r0 = blockIdx.y * kCombRows;
     const long long per = (long long)H_v * kD * kD;
-    const int col = threadIdx.x & 127, rh = threadIdx.x >> 7;  // this thread: column col, rows r0 + rh, r0 + rh + 2, ...
-    const float* N0 = S_out1 + (long long)hv * kD * kD;
-    for (int i = 0; i < 8; ++i) {
-        const int r = rh + 2 * i;
-        const float v = N0[(r0 + r) * kD + col];
-        cur[r][col] = v;
-        S_start[per + (long long)hv * kD * kD + (r0 + r) * kD + col] = v;
+    const float* base = S_out1 + (long long)hv * kD * kD;  // N of segment s at s * per, M of segment s (1 <= s <= P - 2) at (P - 2 + s) * per
+    float* out = S_start + (long long)hv * kD * kD;
+    const int col = (threadIdx.x & 31) * 4, rw = (threadIdx.x >> 5) * 4;  // this thread: rows r0 + rw .., columns col ..
+    auto fetch = [&](int s) {
+        const float* M = base + (long long)(P - 2 + s) * per;
+        float* dst = comb_m + (s & 1) * (kD * kD);
+        for (int i = threadIdx.x * 4; i < kD * kD; i += 1024) {
+            const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(dst + i));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(M + i) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (P > 2) fetch(1);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float4 v = *reinterpret_cast<const float4*>(base + (r0 + rw + r) * kD + col);
+        *reinterpret_cast<float4*>(&cur[rw + r][col]) = v;
+        *reinterpret_cast<float4*>(out + per + (r0 + rw + r) * kD + col) = v;
     }
-    __syncthreads();
     for (int k = 2; k < P; ++k) {
-        const float* M = S_out1 + (long long)(P - 1 + (k - 2)) * per + (long long)hv * kD * kD;  // M of segment k - 1
-        const float* N = S_out1 + (long long)(k - 1) * per + (long long)hv * kD * kD;            // N of segment k - 1
-        float acc[8];
+        float4 acc[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = N[(r0 + rh + 2 * i) * kD + col];
-        for (int d = 0; d < kD; ++d) {
-            const float m = M[d * kD + col];
+        for (int r = 0; r < 4; ++r) acc[r] = *reinterpret_cast<const float4*>(base + (long long)(k - 1) * per + (r0 + rw + r) * kD + col);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();  // M of this step and the state rows are in place, the other buffer is free
+        if (k + 1 < P) fetch(k);
+        const float* M = comb_m + ((k - 1) & 1) * (kD * kD);
+#pragma unroll 2
+        for (int d = 0; d < kD; d += 4) {
+            float4 c[4];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i] = fmaf(cur[rh + 2 * i][d], m, acc[i]);
+            for (int r = 0; r < 4; ++r) c[r] = *reinterpret_cast<const float4*>(&cur[rw + r][d]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 m = *reinterpret_cast<const float4*>(M + (d + q) * kD + col);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float x = q == 0 ? c[r].x : q == 1 ? c[r].y : q == 2 ? c[r].z : c[r].w;
+                    acc[r].x = fmaf(x, m.x, acc[r].x);
+                    acc[r].y = fmaf(x, m.y, acc[r].y);
+                    acc[r].z = fmaf(x, m.z, acc[r].z);
+                    acc[r].w = fmaf(x, m.w, acc[r].w);
+                }
+            }
         }
-        __syncthreads();
+        __syncwarp();  // (a warp reads and writes its own four rows of the state only)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            cur[rh + 2 * i][col] = acc[i];
-            S_start[(long long)k * per + (long long)hv * kD * kD + (r0 + rh + 2 * i) * kD + col] = acc[i];
+        for (int r = 0; r < 4; ++r) {
+            *reinterpret_cast<float4*>(&cur[rw + r][col]) = acc[r];
+            *reinterpret_cast<float4*>(out + (long long)k * per + (r0 + rw + r) * kD + col) = acc[r];
         }
-        __syncthreads();
     }
 }
 
@@ -818,13 +859,12 @@ int launch_chunk_state_segmented(const ProblemS& q, int P, void* workspace, cuda
     float* S_in1 = static_cast<float*>(workspace);
     float* S_out1 = S_in1 + n1 * per;
     float* S_start = S_out1 + n1 * per;
-    float* S_out3 = S_start + (size_t)P * per;
-    int* start1 = reinterpret_cast<int*>(S_out3 + (size_t)P * per);
+    int* start1 = reinterpret_cast<int*>(S_start + (size_t)P * per);
     int* end1 = start1 + n1;
     int* no_u1 = end1 + n1;
     int* start3 = no_u1 + n1;
     int* end3 = start3 + P;
-    segmented_setup_kernel<<<256, 256, 0, stream>>>(P, q.H_v, n_chunks, q.S_in, S_in1, S_start, start1, end1, no_u1, start3, end3);
+    segmented_setup_kernel<<<dim3(static_cast<unsigned>(n1) + 1, q.H_v), 256, 0, stream>>>(P, q.H_v, n_chunks, q.S_in, S_in1, S_start, start1, end1, no_u1, start3, end3);
     count_launch();
     ProblemS a = q;
     a.B = static_cast<int>(n1);
@@ -837,19 +877,18 @@ int launch_chunk_state_segmented(const ProblemS& q, int P, void* workspace, cuda
     a.state_only = true;
     int rc = launch_chunk_state(a, stream);
     if (rc != GDN_OK) return rc;
-    segmented_combine_kernel<<<dim3(q.H_v, kD / 16), 256, 0, stream>>>(P, q.H_v, S_out1, S_start);
+    if (cudaFuncSetAttribute(segmented_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombSmem) != cudaSuccess)
+        return GDN_ERR_LAUNCH;
+    segmented_combine_kernel<<<dim3(q.H_v, kD / kCombRows), 256, kCombSmem, stream>>>(P, q.H_v, S_out1, S_start);
     count_launch();
     ProblemS b = q;
     b.B = P;
     b.S_in = S_start;
-    b.S_out = (q.S_out != nullptr) ? S_out3 : nullptr;
+    b.out_from = P - 1;  // (only the last segment's state leaves)
     b.seq_start = start3;
     b.seq_end = end3;
     rc = launch_chunk_state(b, stream);
     if (rc != GDN_OK) return rc;
-    if (q.S_out != nullptr &&
-        cudaMemcpyAsync(q.S_out, S_out3 + (size_t)(P - 1) * per, per * sizeof(float), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
-        return GDN_ERR_LAUNCH;
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_LAUNCH;
 }
 
@@ -927,6 +966,7 @@ int launch_chunk_state(const ProblemS& q, cudaStream_t stream) {
     prm.seq_start = q.seq_start;
     prm.seq_end = q.seq_end;
     prm.seq_no_u = q.seq_no_u;
+    prm.out_from = q.out_from;
     prm.O = static_cast<__nv_bfloat16*>(q.O);
     const int smem = kSmemTotal + 1024;
     const bool nrm = (q.flags & GDN_FLAG_K_L2NORM) != 0;

@@ -88,6 +88,7 @@ struct ProblemS {
     // state only (packed form): no queries, no output, only S_out; seq_no_u[s] != 0: sequence s runs with U = 0
     bool state_only = false;
     const int* seq_no_u = nullptr;
+    int out_from = 0;  // S_out holds the final states of the sequences from this one on
 };
 
 enum InverseMode { INV_NEUMANN = 0, INV_FWDSUBST_ROWS = 1, INV_FWDSUBST_BLOCKED = 2, INV_FWDSUBST_TC = 3 };

@@ -151,12 +151,25 @@ def _ptr(t):
         key = t.device.index
         if key not in _EMPTY:
             _EMPTY[key] = torch.zeros(64, dtype=torch.float32, device=t.device)
-        return ctypes.c_void_p(_EMPTY[key].data_ptr())
-    return ctypes.c_void_p(t.data_ptr())
+        return _EMPTY[key].data_ptr()
+    return t.data_ptr()  # (the argument types turn it into a pointer)
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch.cuda.current_stream().cuda_stream
+
+
+def _int32_table(values, device):
+    """Host integers as an int32 CUDA tensor. From pinned memory the copy is ordered on the stream only: the host does not
+    wait for the work queued before it, as it does with a copy from pageable memory."""
+    return torch.tensor(values, dtype=torch.int32, pin_memory=device.type == "cuda").to(device, non_blocking=True)
+
+
+def _rows_like(shape, ref, bounds, T):
+    """Output rows of packed sequences: rows that no sequence covers are zero, and where the boundaries run from the first
+    token to the last there are none (every row is written)."""
+    whole = len(bounds) > 0 and bounds[0] == 0 and bounds[-1] == T
+    return (torch.empty if whole else torch.zeros)(shape, dtype=ref.dtype, device=ref.device)
 
 
 def _check_inputs(K, V, beta, g, outs):
@@ -255,14 +268,15 @@ def chunk_prepare_varlen(K, V, beta, g, cu_seqlens, C, order=-1, residual_steps=
     else:
         H_k, T, d_k = K.shape
         H_v, _, d_v = V.shape
-    start, length = chunk_table(cu_seqlens, C)
+    bounds = [int(x) for x in cu_seqlens]
+    start, length = chunk_table(bounds, C)
     n = len(start)
-    cs = torch.tensor(start, dtype=torch.int32, device=K.device)
-    cl = torch.tensor(length, dtype=torch.int32, device=K.device)
+    table = _int32_table(start + length, K.device)
+    cs, cl = table[:n], table[n:]
     per_tile = max(1, 128 // C)
     padded = -(-n // per_tile) * per_tile
-    W = torch.zeros((T, H_v, d_k) if token_major else (H_v, T, d_k), dtype=K.dtype, device=K.device)
-    U = torch.zeros_like(V)
+    W = _rows_like((T, H_v, d_k) if token_major else (H_v, T, d_k), K, bounds, T)
+    U = _rows_like(V.shape, V, bounds, T)
     Tinv = torch.empty(H_v, padded, C, C, dtype=K.dtype, device=K.device) if want_tinv else None
     gdn_chunk_prepare_varlen(K, V, beta, g, cs, cl, n, T, H_k, H_v, C, d_k, d_v, order, residual_steps, W, U, Tinv, flags)
     return W, U, (Tinv[:, :n] if want_tinv else None), cs, cl
@@ -450,9 +464,10 @@ def chunk_state_output_varlen(Q, K, W_gated, U, g, cu_seqlens, C, scale=1.0, S_i
     else:
         H_k, T, d_k = K.shape
         H_v, _, d_v = U.shape
-    cu = torch.tensor([int(x) for x in cu_seqlens], dtype=torch.int32, device=U.device)
-    n_seq = cu.numel() - 1
-    O = torch.zeros_like(U)
+    bounds = [int(x) for x in cu_seqlens]
+    cu = _int32_table(bounds, U.device)
+    n_seq = len(bounds) - 1
+    O = _rows_like(U.shape, U, bounds, T)
     S_out = torch.empty(n_seq, H_v, d_v, d_k, dtype=torch.float32, device=U.device) if want_state else None
     gdn_chunk_state_output_varlen(Q, K, W_gated, U, g, cu, n_seq, T, H_k, H_v, C, d_k, d_v, scale, S_in, O, S_out, flags)
     return O, S_out
@@ -476,6 +491,13 @@ def chunk_state_output(Q, K, W_gated, U, g, C, scale=1.0, S_in=None, *, want_sta
     return O, S_out
 
 
+def _segments_pay(T, C, segments):
+    """Whether the segmented state passing is the faster one: its four launches cost about 35 + 3 P us more than a plain
+    one and its two passes 4.5 / P us a chunk against 2.7 (measured back to back, 1 to 64 heads: with P = 8 the lines cross
+    at 26 chunks, 24 chunks 74 us plain and 82 segmented, 32 chunks 95 and 86; with P = 3 at 34, with P = 2 at 90)."""
+    return segments > 1 and (T // C) * (2.7 - 4.5 / segments) > 35 + 3 * segments
+
+
 def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_seqlens=None, token_major=True,
                       qk_l2norm=True, want_state=True):
     """The chunk-wise layer as model code calls it: the two library calls back to back (chunk-prepare with the gated W,
@@ -490,7 +512,7 @@ def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_s
         return chunk_state_output_varlen(Q, K, W, U, g_raw, cu_seqlens, C, scale, S_in, want_state=want_state, flags=flags)
     W, U, _ = chunk_prepare(K, V, beta, g_raw, C, flags=flags | GDN_FLAG_W_GATED, want_tinv=False)
     H_v = V.shape[2] if token_major else V.shape[1]
-    if K.shape[0] == 1 and int(load_library().gdn_chunk_state_segments(H_v)) > 1:
+    if K.shape[0] == 1 and _segments_pay(V.shape[1] if token_major else V.shape[2], C, int(load_library().gdn_chunk_state_segments(H_v))):
         # one long sequence per head and fewer heads than SMs: the segments of a sequence run in parallel
         O, S = chunk_state_output_segmented(Q[0], K[0], W[0], U[0], g_raw[0], C, scale, None if S_in is None else S_in[0],
                                             want_state=want_state, flags=flags)

@@ -1,0 +1,66 @@
+"""The layer call's choice of state passing, and packed outputs that are not cleared."""
+import pytest
+import torch
+
+from paper_2606_06034_b200 import binding as gdn
+
+FLAGS = gdn.GDN_FLAG_G_RAW | gdn.GDN_FLAG_LAYOUT_BTHD | gdn.GDN_FLAG_K_L2NORM
+
+
+@pytest.mark.parametrize("segments,first", [(2, 92), (3, 37), (4, 30), (6, 28), (8, 28)])
+def test_line_between_plain_and_segmented(segments, first):
+    assert not gdn._segments_pay(64 * (first - 1), 64, segments)
+    assert gdn._segments_pay(64 * first, 64, segments)
+    assert not gdn._segments_pay(64 * 100000, 64, 1) and not gdn._segments_pay(0, 64, segments)
+
+
+@pytest.mark.parametrize("bounds,T,whole", [([0, 5, 9], 9, True), ([0, 0, 9, 9], 9, True), ([0, 5], 9, False), ([1, 9], 9, False),
+                                            ([], 4, False), ([0], 0, True)])
+def test_rows_are_cleared_unless_every_one_is_written(bounds, T, whole, monkeypatch):
+    made = []
+    monkeypatch.setattr(torch, "zeros", lambda *a, _f=torch.zeros, **k: made.append("zeros") or _f(*a, **k))
+    gdn._rows_like((T, 2, 4), torch.empty(0, dtype=torch.bfloat16), bounds, T)
+    assert (made == []) == whole
+
+
+def _inputs(T, H_k, H_v, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    r = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    return (r(1, T, H_k, 128).bfloat16(), r(1, T, H_k, 128).bfloat16(), r(1, T, H_v, 128).bfloat16(), torch.sigmoid(r(1, T, H_v)),
+            -torch.nn.functional.softplus(r(1, T, H_v)), 0.3 * r(1, H_v, 128, 128))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H_k,H_v,chunks", [(1, 2, 1), (1, 2, 2), (1, 2, 27), (1, 2, 28), (16, 32, 36), (16, 32, 37), (32, 64, 91), (32, 64, 92)])
+@pytest.mark.parametrize("with_state", [False, True])
+def test_layer_on_both_sides_of_the_line(H_k, H_v, chunks, with_state):
+    """Both forms compute the same chain; they differ by the fp32 re-association of the state recurrence (at most 2^-24 per
+    token of decay-free carry, far below 1e-5 of the state) and, where that flips a rounding of the output, by one bf16 unit
+    (2^-8) of single elements."""
+    Q, K, V, beta, g, S = _inputs(64 * chunks, H_k, H_v, chunks)
+    S = S if with_state else None
+    O, Sn = gdn.gated_delta_layer(Q, K, V, beta, g, S_in=S)
+    W, U, _ = gdn.chunk_prepare(K, V, beta, g, 64, flags=FLAGS | gdn.GDN_FLAG_W_GATED, want_tinv=False)
+    Op, Sp = gdn.chunk_state_output(Q, K, W, U, g, 64, 128 ** -0.5, S, flags=FLAGS)
+    Os, Ss = gdn.chunk_state_output_segmented(Q[0], K[0], W[0], U[0], g[0], 64, 128 ** -0.5, None if S is None else S[0], flags=FLAGS)
+    assert gdn.gdn_device_status() == gdn.GDN_OK
+    assert O.shape == V.shape and Sn.shape == (1, H_v, 128, 128)
+    for o, s in ((Op, Sp), (Os[None], Ss[None])):
+        assert (Sn - s).norm() <= 1e-5 * s.norm()
+        assert (O.float() - o.float()).norm() <= 1e-3 * o.float().norm()
+
+
+@pytest.mark.gpu
+def test_packed_rows_without_a_sequence_stay_zero_and_the_others_keep_their_bits():
+    T, extra = 200, 40
+    Q, K, V, beta, g, _ = (x[0] for x in _inputs(T + extra, 1, 2, 3))
+    cu = [0, 64, 65, 65, 190, T]
+    whole = gdn.gated_delta_layer(*(x[:T].contiguous() for x in (Q, K, V, beta, g)), cu_seqlens=cu)
+    torch.empty(1 << 22, device="cuda").fill_(float("nan"))  # (what an uncleared allocation would show)
+    part = gdn.gated_delta_layer(Q, K, V, beta, g, cu_seqlens=cu)
+    assert torch.equal(part[0][:T], whole[0]) and torch.equal(part[1], whole[1])
+    assert torch.count_nonzero(part[0][T:]).item() == 0
+    W, U, Tinv, cs, cl = gdn.chunk_prepare_varlen(K, V, beta, g, cu, 64, flags=FLAGS)
+    assert torch.count_nonzero(W[T:]).item() == 0 and torch.count_nonzero(U[T:]).item() == 0
+    assert cs.tolist() == [0, 64, 65, 129, 190] and cl.tolist() == [64, 1, 64, 61, 10]
+    assert cs.dtype == cl.dtype == torch.int32 and cs.is_contiguous() and cl.is_contiguous()

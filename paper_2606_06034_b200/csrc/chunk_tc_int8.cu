@@ -507,7 +507,11 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             const int eref = align_ref2(eA, eA + eT0);
             const int sa = eA - eref, sp = eA + eT0 - eref;
             int acc[kHC];  // |Aq| < 2^7 and |Aq T0q| <= 3 * 127^2 < 2^16, shifted left by at most 8
-            const bool left = sa >= 0 && sp >= 0;
+            // The usual case: the product has the smaller exponent and is shifted right (or not at all), and the shift of the
+            // other term folds into a multiplier: one multiply-add and one rounded shift per element.
+            const bool fold = sa >= 0 && sp <= 0;
+            const int m_a = fold ? (1 << sa) : 0;
+            const Rnd rp = make_rnd(fold ? min(-sp, 31) : 0);
             uint32_t m = 0;
 #pragma unroll
             for (int jl = 0; jl < kHC; ++jl) {
@@ -517,8 +521,20 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
                 const int a3 = (jl + 3 < kHC) ? aq[(jl + 3 < kHC) ? jl + 3 : 0] : ((jl + 3 == kHC) ? an0 : (jl + 3 == kHC + 1 ? an1 : an2));
                 const bool on = (il - (col0 + jl)) > N;
                 const int pr = a1 * c4.x + a2 * c4.y + a3 * c4.z;
-                const int v = on ? (left ? ((aq[jl] << sa) + (pr << sp)) : (term32(aq[jl], sa) + term32(pr, sp))) : 0;
-                acc[jl] = v;
+                acc[jl] = on ? pr : 0;
+            }
+            if (fold) {
+#pragma unroll
+                for (int jl = 0; jl < kHC; ++jl) {
+                    const bool on = (il - (col0 + jl)) > N;
+                    acc[jl] = (on ? aq[jl] : 0) * m_a + rsr_rnd(acc[jl], rp);
+                }
+            } else {
+#pragma unroll
+                for (int jl = 0; jl < kHC; ++jl) {
+                    const bool on = (il - (col0 + jl)) > N;
+                    acc[jl] = on ? term32(aq[jl], sa) + term32(acc[jl], sp) : 0;
+                }
             }
             MaxMag mm;
 #pragma unroll
@@ -577,7 +593,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             tmem_wait_st();
             tc_fence_before_sync();
             cta_barrier();
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 tc_fence_after_sync();
 #pragma unroll
                 for (int ks = 0; ks < kC / 32; ++ks) {
@@ -653,19 +669,21 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
                 tmem_ldn(lane_base + park_col(s), w);
                 tmem_wait_ld();
                 if (sh >= 0) {
+                    const int mul = 1 << sh;  // (a multiply-add instead of a shift and an add)
 #pragma unroll
                     for (int b = 0; b < kNB; ++b) {
                         if (b < nb) {
 #pragma unroll
-                            for (int jl = 8 * b; jl < 8 * b + 8; ++jl) acc[jl] += byte_at(w[jl >> 2], jl & 3) << sh;
+                            for (int jl = 8 * b; jl < 8 * b + 8; ++jl) acc[jl] += byte_at(w[jl >> 2], jl & 3) * mul;
                         }
                     }
                 } else {
+                    const Rnd rs = make_rnd(-sh);
 #pragma unroll
                     for (int b = 0; b < kNB; ++b) {
                         if (b < nb) {
 #pragma unroll
-                            for (int jl = 8 * b; jl < 8 * b + 8; ++jl) acc[jl] += rsr32(byte_at(w[jl >> 2], jl & 3), -sh);
+                            for (int jl = 8 * b; jl < 8 * b + 8; ++jl) acc[jl] += rsr_rnd(byte_at(w[jl >> 2], jl & 3), rs);
                         }
                     }
                 }
@@ -736,12 +754,14 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             // and lower triangular). So the row's 32 columns take the far formula without any mask, and the (at most
             // three) band entries of the row are three scalars, T0q alone: entries below 2^7, the product below
             // 3 * 127^2 < 2^16. The band values are put into the packed rows afterwards, through shared memory.
-            const bool left = s0 >= 0 && s1 >= 0 && s2 >= 0;
+            const bool fold = s1 >= 0 && s2 <= 0;  // (the usual case, as in I6)
             int acc[kHC];
             uint32_t m = 0;
-            if (left) {
+            if (fold) {
+                const int m_s = 1 << s1;
+                const Rnd rp = make_rnd(min(-s2, 31));
 #pragma unroll
-                for (int jl = 0; jl < kHC; ++jl) acc[jl] = (sq[jl] << s1) + (prod[jl] << s2);
+                for (int jl = 0; jl < kHC; ++jl) acc[jl] = sq[jl] * m_s + rsr_rnd(prod[jl], rp);
             } else {
 #pragma unroll
                 for (int jl = 0; jl < kHC; ++jl) acc[jl] = term32(sq[jl], s1) + term32(prod[jl], s2);
@@ -847,7 +867,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             tma_store_3d(&tmT, stage + wrow0 * 64, p.merge ? ci * kC : 0, tc.t0 + wrow0, tc.bhv);
             tma_store_commit();
         }
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             // W accumulator = blockdiag(Tbq) Kq: M = 128, N = 128, K = 128 (4 steps of 32)
             tc_fence_after_sync();
 #pragma unroll

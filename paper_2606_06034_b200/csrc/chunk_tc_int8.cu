@@ -501,7 +501,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         }
 
         // ---- I6: Eq = Q8(align(Aq, Aq T0q)) on i-j > N
-        int eq[kHC];
+        uint32_t r1[kHC / 4];  // Eq = R_1, packed
         int eE;
         {
             const int eref = align_ref2(eA, eA + eT0);
@@ -543,20 +543,19 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             const int r = q8_shift(chunk_bitlen32(m, slot++));
             const Rnd rq = make_rnd(r);
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) eq[jl] = q8_32(acc[jl], rq);
+            for (int w = 0; w < kHC / 4; ++w) r1[w] = q8_pack4(acc[4 * w], acc[4 * w + 1], acc[4 * w + 2], acc[4 * w + 3], rq);
             eE = eref + r;
         }
         // Rows of the powers R_s (R_1 = Eq) as packed bytes. The loops over the powers are NOT unrolled (the kernel is bound
         // by instruction fetch: its straight-line code is larger than the instruction cache), so the rows cannot sit in
         // registers indexed by s: R_1 stays in registers, R_2.. are parked in free TMEM columns of the row's own lane
         // (columns 160..255 for s = 2..7; s = 8 and, for the sum, R_1 go to accumulator columns that are idle by then).
-        uint32_t r1[kHC / 4];   // R_1
         uint32_t cur[kHC / 4];  // R_{s-1} inside the loop
         int er[kSMax];
 #pragma unroll
         for (int s = 0; s < kSMax; ++s) er[s] = 0;
 #pragma unroll
-        for (int w = 0; w < kHC / 4; ++w) r1[w] = cur[w] = 0u;
+        for (int w = 0; w < kHC / 4; ++w) cur[w] = 0u;
         auto park_col = [&](int s) -> uint32_t {  // TMEM column of the parked row of R_s (s >= 1)
             return (s >= 2 && s <= 7) ? static_cast<uint32_t>(160 + (s - 2) * 16 + h * kW)
                                       : static_cast<uint32_t>(kR0 + (s == 1 ? 0 : 16) + h * kW);
@@ -574,7 +573,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         int n_terms = 0;
         if (S >= 1) {
 #pragma unroll
-            for (int w = 0; w < kHC / 4; ++w) r1[w] = cur[w] = pack4(eq[4 * w], eq[4 * w + 1], eq[4 * w + 2], eq[4 * w + 3]);
+            for (int w = 0; w < kHC / 4; ++w) cur[w] = r1[w];
             er[0] = eE;
             n_terms = 1;
             // B operand [E_1 | E_2] (64 x 128 int8, MN-major, no swizzle): 16 columns of chunk-row il per 16-byte piece
@@ -646,7 +645,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
 
         // ---- Sq = Q8(align(R_1..)): the exponents fall by several bits per power, so most terms are
         // shifted far to the right; a term whose right shift exceeds 7 rounds to zero and is skipped
-        int sq[kHC];
+        uint32_t sq[kHC / 4];  // packed
         int eS = 0;
         if (n_terms > 0) {
             int emin = er[0], emax = er[0];
@@ -702,30 +701,25 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             const Rnd rq = make_rnd(r);
 #pragma unroll
             for (int b = 0; b < kNB; ++b) {
-#pragma unroll
-                for (int jl = 8 * b; jl < 8 * b + 8; ++jl) sq[jl] = 0;
+                sq[2 * b] = sq[2 * b + 1] = 0u;
                 if (b < nb1) {
 #pragma unroll
-                    for (int jl = 8 * b; jl < 8 * b + 8; ++jl) sq[jl] = q8_32(acc[jl], rq);
+                    for (int w = 2 * b; w < 2 * b + 2; ++w) sq[w] = q8_pack4(acc[4 * w], acc[4 * w + 1], acc[4 * w + 2], acc[4 * w + 3], rq);
                 }
             }
             eS = eref + r;
         } else {
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) sq[jl] = 0;
+            for (int w = 0; w < kHC / 4; ++w) sq[w] = 0u;
         }
         // Sq bytes to the private rows (the rows above are needed for T0q Sq)
 #pragma unroll
         for (int c = 0; c < kHC / 16; ++c)
-            *reinterpret_cast<uint4*>(rowa + col0 + 16 * c) =
-                make_uint4(pack4(sq[16 * c + 0], sq[16 * c + 1], sq[16 * c + 2], sq[16 * c + 3]),
-                           pack4(sq[16 * c + 4], sq[16 * c + 5], sq[16 * c + 6], sq[16 * c + 7]),
-                           pack4(sq[16 * c + 8], sq[16 * c + 9], sq[16 * c + 10], sq[16 * c + 11]),
-                           pack4(sq[16 * c + 12], sq[16 * c + 13], sq[16 * c + 14], sq[16 * c + 15]));
+            *reinterpret_cast<uint4*>(rowa + col0 + 16 * c) = make_uint4(sq[4 * c], sq[4 * c + 1], sq[4 * c + 2], sq[4 * c + 3]);
         cta_barrier();
 
         // ---- I8: Toffq = Q8(align(T0q, Sq, T0q Sq)) on i > j
-        int toff[kHC];   // far part of the row (zero on the band)
+        uint32_t toff[kHC / 4];  // far part of the row (zero on the band), packed
         int tband[3];    // Toffq[i][i-1..i-3] (zero where the row or the order has no such entry)
         int eT;
         {
@@ -761,10 +755,10 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
                 const int m_s = 1 << s1;
                 const Rnd rp = make_rnd(min(-s2, 31));
 #pragma unroll
-                for (int jl = 0; jl < kHC; ++jl) acc[jl] = sq[jl] * m_s + rsr_rnd(prod[jl], rp);
+                for (int jl = 0; jl < kHC; ++jl) acc[jl] = byte_at(sq[jl >> 2], jl & 3) * m_s + rsr_rnd(prod[jl], rp);
             } else {
 #pragma unroll
-                for (int jl = 0; jl < kHC; ++jl) acc[jl] = term32(sq[jl], s1) + term32(prod[jl], s2);
+                for (int jl = 0; jl < kHC; ++jl) acc[jl] = term32(byte_at(sq[jl >> 2], jl & 3), s1) + term32(prod[jl], s2);
             }
             const int ab1 = term32(t0q1, s0), ab2 = term32(t0q2, s0), ab3 = term32(t0q3, s0);
             {
@@ -778,7 +772,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             const int r = q8_shift(chunk_bitlen32(m, slot++));
             const Rnd rq = make_rnd(r);
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) toff[jl] = q8_32(acc[jl], rq);
+            for (int w = 0; w < kHC / 4; ++w) toff[w] = q8_pack4(acc[4 * w], acc[4 * w + 1], acc[4 * w + 2], acc[4 * w + 3], rq);
             tband[0] = q8_32(ab1, rq);
             tband[1] = q8_32(ab2, rq);
             tband[2] = q8_32(ab3, rq);
@@ -792,7 +786,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             uint32_t m = 0;
 #pragma unroll
             for (int jl = 0; jl < kHC; ++jl) {
-                acc[jl] = toff[jl] * lds_s32(sbeta_a + (cb + col0 + jl) * 4);
+                acc[jl] = byte_at(toff[jl >> 2], jl & 3) * lds_s32(sbeta_a + (cb + col0 + jl) * 4);
             }
             int accb[3];  // the band entries times beta of their columns
 #pragma unroll
@@ -841,10 +835,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
 #pragma unroll
             for (int c = 0; c < kHC / 16; ++c) {
                 const int cc = (col0 >> 4) + c;
-                const uint4 v = make_uint4(pack4(toff[16 * c + 0], toff[16 * c + 1], toff[16 * c + 2], toff[16 * c + 3]),
-                                           pack4(toff[16 * c + 4], toff[16 * c + 5], toff[16 * c + 6], toff[16 * c + 7]),
-                                           pack4(toff[16 * c + 8], toff[16 * c + 9], toff[16 * c + 10], toff[16 * c + 11]),
-                                           pack4(toff[16 * c + 12], toff[16 * c + 13], toff[16 * c + 14], toff[16 * c + 15]));
+                const uint4 v = make_uint4(toff[4 * c], toff[4 * c + 1], toff[4 * c + 2], toff[4 * c + 3]);
                 *reinterpret_cast<uint4*>(line + ((cc ^ ((t >> 1) & 3)) << 4)) = v;
             }
 #pragma unroll

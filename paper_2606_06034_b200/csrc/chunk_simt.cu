@@ -116,7 +116,7 @@ __device__ __forceinline__ void prod_tri(float (&v)[R][R], const float* X, const
         for (int s = 0; s < R; ++s) acc[r][s] = 0ull;
 #pragma unroll
     for (int q = 0; q < R; ++q) {
-#pragma unroll 2
+#pragma unroll 4
         for (int k = q * G; k < q * G + G; k += 4) {
             ulonglong2 b[R];
 #pragma unroll
@@ -145,7 +145,7 @@ __device__ __forceinline__ void prod_rows(f2 (&acc)[R][NC * 2], const float* X, 
     constexpr int ld = G * R + 4;
 #pragma unroll
     for (int q = 0; q < R; ++q) {
-#pragma unroll 1
+#pragma unroll 2
         for (int j = q * G; j < q * G + G; j += 4) {
             float4 a[R];
 #pragma unroll
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
         load_wait();
         __syncthreads();
         const float* Kb = Ks + grp * M * kLdk;
-#pragma unroll 2
+#pragma unroll 4
         for (int d = 0; d < w; d += 4) {
             ulonglong2 b[R];
 #pragma unroll

@@ -513,28 +513,20 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             const int m_a = fold ? (1 << sa) : 0;
             const Rnd rp = make_rnd(fold ? min(-sp, 31) : 0);
             uint32_t m = 0;
-#pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) {
+            auto band_product = [&](int jl) -> int {  // (Aq T0q)_ij
                 const int4 c4 = lds_v4(sSH_a + (cb + col0 + jl) * 16);
                 const int a1 = (jl + 1 < kHC) ? aq[(jl + 1 < kHC) ? jl + 1 : 0] : ((jl + 1 == kHC) ? an0 : (jl + 1 == kHC + 1 ? an1 : an2));
                 const int a2 = (jl + 2 < kHC) ? aq[(jl + 2 < kHC) ? jl + 2 : 0] : ((jl + 2 == kHC) ? an0 : (jl + 2 == kHC + 1 ? an1 : an2));
                 const int a3 = (jl + 3 < kHC) ? aq[(jl + 3 < kHC) ? jl + 3 : 0] : ((jl + 3 == kHC) ? an0 : (jl + 3 == kHC + 1 ? an1 : an2));
-                const bool on = (il - (col0 + jl)) > N;
-                const int pr = a1 * c4.x + a2 * c4.y + a3 * c4.z;
-                acc[jl] = on ? pr : 0;
-            }
-            if (fold) {
+                return a1 * c4.x + a2 * c4.y + a3 * c4.z;
+            };
 #pragma unroll
-                for (int jl = 0; jl < kHC; ++jl) {
-                    const bool on = (il - (col0 + jl)) > N;
-                    acc[jl] = (on ? aq[jl] : 0) * m_a + rsr_rnd(acc[jl], rp);
-                }
-            } else {
-#pragma unroll
-                for (int jl = 0; jl < kHC; ++jl) {
-                    const bool on = (il - (col0 + jl)) > N;
-                    acc[jl] = on ? term32(aq[jl], sa) + term32(acc[jl], sp) : 0;
-                }
+            for (int jl = 0; jl < kHC; ++jl) {
+                const int pr = band_product(jl);
+                int v;
+                if (fold) v = aq[jl] * m_a + rsr_rnd(pr, rp);
+                else v = term32(aq[jl], sa) + term32(pr, sp);
+                acc[jl] = (il - (col0 + jl)) > N ? v : 0;
             }
             MaxMag mm;
 #pragma unroll
@@ -592,7 +584,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             tmem_wait_st();
             tc_fence_before_sync();
             cta_barrier();
-            if (warp == 0 && elect_one()) {
+            if (tid == 0) {
                 tc_fence_after_sync();
 #pragma unroll
                 for (int ks = 0; ks < kC / 32; ++ks) {
@@ -858,7 +850,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             tma_store_3d(&tmT, stage + wrow0 * 64, p.merge ? ci * kC : 0, tc.t0 + wrow0, tc.bhv);
             tma_store_commit();
         }
-        if (warp == 0 && elect_one()) {
+        if (tid == 0) {
             // W accumulator = blockdiag(Tbq) Kq: M = 128, N = 128, K = 128 (4 steps of 32)
             tc_fence_after_sync();
 #pragma unroll

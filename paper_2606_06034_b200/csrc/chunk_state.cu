@@ -23,7 +23,7 @@
 // Two MMA groups per chunk; Q, K, W, U tiles of the next chunk are in flight (two stages) while a chunk is worked on.
 // All operand layouts are the ones the chunk-prepare kernel uses.
 // Warps: 16 compute warps (four threads per TMEM lane), one that issues every MMA, one that issues the TMA loads and
-// the output stores, four that form the gate tables and the norms a chunk ahead. The chain of a sequence is thread work (every phase runs on all 16 warps at once, so its
+// the output stores, two that form the gate tables and the norms a chunk ahead. The chain of a sequence is thread work (every phase runs on all 16 warps at once, so its
 // instruction count is what it costs); hand-offs to the issuing warp are hardware barriers, completions come back
 // through mbarriers (a poll costs ~200 cycles, so as few as possible are waited for).
 // Instantiations: packed variable-length sequences (one CTA per (sequence, value head), starting at the sequence's
@@ -43,8 +43,9 @@ using namespace sm100;
 constexpr int kC = 64;         // chunk size
 constexpr int kD = 128;        // d_k = d_v
 constexpr int kThreads = 512;  // compute threads, four per TMEM lane; two more warps issue the MMAs and the TMA loads
-constexpr int kTabThreads = 128;  // gate tables and norms, two threads per token of a chunk (its key, its query)
+constexpr int kTabThreads = 64;  // gate tables and norms, one thread per token of a chunk (four warps would cap the registers at 80)
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kMaxOrder = 256;  // sequences a packed launch sorts by length
 
 // TMEM column map (512 columns: one CTA per SM)
 constexpr uint32_t kSD = 0;    // 128: state S, fp32 accumulator
@@ -80,6 +81,7 @@ struct ParamsS {
     const int* seq_start;  // first token of sequence s
     const int* seq_end;    // one past its last token (the public call passes cu_seqlens and cu_seqlens + 1)
     const int* seq_no_u;   // optional: sequence s runs with U = 0 (the state map of a segment, see the segmented call)
+    int n_order;             // packed: sequences to be taken longest first (0: in their order)
     int out_from;            // S_out holds the final states of the sequences from this one on
     __nv_bfloat16* O;  // output tensor (rows of a short last chunk are stored one by one)
 };
@@ -170,6 +172,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     __shared__ uint64_t bar_full[2], bar_pre, bar_d1, bar_o2, bar_g2, bar_stg[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int s_fail;
+    __shared__ int s_len[VAR && !SO ? kMaxOrder : 1], s_seq;
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -202,15 +205,28 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         tmem_alloc(&tmem_base_s, kTmemCols);
         tmem_relinquish();
     }
+    if (VAR && !SO && tid < p.n_order) s_len[tid] = __ldg(p.seq_end + tid) - __ldg(p.seq_start + tid);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    if (VAR && !SO && p.n_order > 0) {
+        // longest sequence first: the CTAs with block index k H_v .. take the sequence of rank k (ties in their order)
+        if (tid < p.n_order) {
+            const int mine = s_len[tid];
+            int rank = 0;
+            for (int i = 0; i < p.n_order; ++i) rank += (s_len[i] > mine || (s_len[i] == mine && i < tid)) ? 1 : 0;
+            if (rank == static_cast<int>(blockIdx.x / p.H_v)) s_seq = tid;
+        }
+        __syncthreads();
+    }
     const uint32_t tmem = tmem_base_s;
     const uint32_t lane_base = tmem + (static_cast<uint32_t>(wq * 32) << 16);
 
     // dense: one CTA per (batch, value head), bhv = row of the [B * H_v, T] tensors. Packed sequences: one CTA per
     // (sequence, value head); the tensors have one batch row per head and the sequence starts at token tok0
-    const int b = blockIdx.x / p.H_v, hv = blockIdx.x - b * p.H_v;
+    int b = blockIdx.x / p.H_v;
+    const int hv = blockIdx.x - b * p.H_v;
+    if (VAR && !SO && p.n_order > 0) b = s_seq;
     const int tok0 = VAR ? __ldg(p.seq_start + b) : 0;
     const int len = VAR ? __ldg(p.seq_end + b) - tok0 : p.T;
     const bool no_u = SO && p.seq_no_u != nullptr && __ldg(p.seq_no_u + b) != 0;
@@ -230,12 +246,11 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     volatile int* fail = reinterpret_cast<volatile int*>(&s_fail);
 
     if (tabler) {
-        // ================= table threads, two per token (the second only for the norm of its query). Before hand-off 4 of chunk c they have written the factors of
+        // ================= table threads, one per token. Before hand-off 4 of chunk c they have written the factors of
         // chunk c (read behind the completion of its first product, which that hand-off precedes) and the gates of chunk
         // c + 1 (read from its start on, behind the same completion one chunk earlier). Three buffers: the threads are done
         // with a chunk's tables when they arrive on the next hand-off 4, and the table threads wait for it.
-        const int tt = (tid - (kThreads + 64)) & 63;
-        const bool second = tid >= kThreads + 64 + 64;
+        const int tt = tid - (kThreads + 64);
         const bool g_raw = (p.flags & GDN_FLAG_G_RAW) != 0;
         auto fetch = [&](int c) -> float { return (c < n_c && (!VAR || c * kC + tt < len)) ? __ldg(gseq + (c * kC + tt) * gstep) : 0.f; };
         auto put_gates = [&](int c, float gc) {
@@ -282,33 +297,26 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             asm("mov.b64 {%0, %1}, %2;" : "=f"(s2), "=f"(s3) : "l"(a[1]));
             return rsqrtf(fmaxf((s0 + s1) + (s2 + s3), 1e-30f));
         };
-        float g_next = 0.f;
-        if (!second) {
-            g_next = fetch(0);
-            if (n_c > 0) put_gates(0, g_next);
-            g_next = fetch(1);
-        }
+        float g_next = fetch(0);
+        if (n_c > 0) put_gates(0, g_next);
+        g_next = fetch(1);
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");
         for (int c = 0; c < n_c && *fail == 0; ++c) {
-            if (!second) {
-                if (c + 1 < n_c) put_gates(c + 1, g_next);
-                g_next = fetch(c + 2);
-            }
+            if (c + 1 < n_c) put_gates(c + 1, g_next);
+            g_next = fetch(c + 2);
             float* tb = gtab + (c % 3) * kTab;
             const float gc = tb[128 + tt], gC = tb[128 + 63];
-            float r = 1.f;
-            if (NRM && !(SO && second)) {
+            float rk = 1.f, so = p.scale;
+            if (NRM) {
                 if (!wait_bar(&bar_full[c & 1], (c >> 1) & 1)) *fail = 1;
-                r = inv_norm(smem + (c & 1) * kStageBytes + (second ? kOffQ : kOffK));
+                const uint8_t* st = smem + (c & 1) * kStageBytes;
+                rk = (VAR && tt >= len - c * kC) ? 0.f : inv_norm(st + kOffK);
+                if (!SO) so *= inv_norm(st + kOffQ);
             }
-            if (second) {
-                tb[tt] = p.scale * r * fast_exp2(gc * kLog2e);
-                tb[256 + tt] = p.scale * r;
-            } else {
-                if (VAR && tt >= len - c * kC) r = 0.f;
-                tb[192 + tt] = -r;
-                tb[64 + tt] = -r * fast_exp2((gC - gc) * kLog2e);
-            }
+            tb[tt] = so * fast_exp2(gc * kLog2e);
+            tb[256 + tt] = so;
+            tb[192 + tt] = -rk;
+            tb[64 + tt] = -rk * fast_exp2((gC - gc) * kLog2e);
             handoff_wait<4>();
         }
     } else if (producer) {
@@ -483,7 +491,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             tmem_st16(lane_base + kIA + h * 16, r);
             // this thread's quarter of state row t: columns [32 h, 32 h + 32)
-            const float* s0 = (p.S_in != nullptr) ? p.S_in + ((long long)blockIdx.x * kD + t) * kD + h * 32 : nullptr;
+            const float* s0 = (p.S_in != nullptr) ? p.S_in + (((long long)b * p.H_v + hv) * kD + t) * kD + h * 32 : nullptr;
 #pragma unroll
             for (int part = 0; part < 2; ++part) {
                 uint32_t v[16], pk[8];
@@ -674,8 +682,10 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             handoff_arrive<6>();
         }
         // ---- final state
-        if (ok && p.S_out != nullptr && static_cast<int>(b) >= p.out_from) {
-            float* so = p.S_out + (((long long)blockIdx.x - (long long)p.out_from * p.H_v) * kD + t) * kD + h * 32;
+        // (the run's place among the states is formed again here: it is not held over the chunks)
+        const int seq = (VAR && !SO && p.n_order > 0) ? *reinterpret_cast<volatile int*>(&s_seq) : static_cast<int>(blockIdx.x / p.H_v);
+        if (ok && p.S_out != nullptr && seq >= p.out_from) {
+            float* so = p.S_out + (((long long)(seq - p.out_from) * p.H_v + blockIdx.x % p.H_v) * kD + t) * kD + h * 32;
             uint32_t v[32];
             tmem_ld32(lane_base + kSD + h * 32, v);
             tmem_wait_ld();
@@ -968,6 +978,10 @@ int launch_chunk_state(const ProblemS& q, cudaStream_t stream) {
     prm.seq_no_u = q.seq_no_u;
     prm.out_from = q.out_from;
     prm.O = static_cast<__nv_bfloat16*>(q.O);
+    // More runs than SMs (one CTA each): the long ones start first, so that none of them is left for the end. 61 prompts of
+    // 1 to 2050 tokens, 32 heads: the last SM finishes 20 % later in the order of arrival than in this one (list scheduling
+    // of the measured 5 + 2.5 us a chunk). Every CTA ranks the lengths itself, under 1 us at 256 sequences.
+    prm.n_order = (var && !q.state_only && n_cta > 148 && q.B > 1 && q.B <= kMaxOrder) ? q.B : 0;
     const int smem = kSmemTotal + 1024;
     const bool nrm = (q.flags & GDN_FLAG_K_L2NORM) != 0;
     auto kern = q.state_only ? (nrm ? chunk_state_kernel<true, true, true> : chunk_state_kernel<true, true, false>)

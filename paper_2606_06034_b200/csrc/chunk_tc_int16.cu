@@ -19,7 +19,8 @@
 // One CTA of 512 threads per SM (three 128-column accumulators + two operand planes = 448 TMEM columns), tile of 128
 // tokens = two 64-chunks, the four threads t + 128 h share tile row t and split its 64 chunk columns. Everything between the
 // products is 64-bit integer ALU work: it is bound by the number of integer instructions and by how many warps there are to
-// hide their latency (with two threads per row and half the warps the same code ran at a third of the issue slots).
+// hide their latency (16 / 32 heads, 32768 tokens: two threads per row 3.56 ms with 70 % of the issue slots empty, four 2.40 ms,
+// and with the products kept on the multiplier pipe 2.20 ms).
 #include <cuda.h>
 
 #include "common.cuh"

@@ -64,3 +64,26 @@ def test_packed_rows_without_a_sequence_stay_zero_and_the_others_keep_their_bits
     assert torch.count_nonzero(W[T:]).item() == 0 and torch.count_nonzero(U[T:]).item() == 0
     assert cs.tolist() == [0, 64, 65, 129, 190] and cl.tolist() == [64, 1, 64, 61, 10]
     assert cs.dtype == cl.dtype == torch.int32 and cs.is_contiguous() and cl.is_contiguous()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_seq", [3, 256, 257])
+def test_packed_sequences_taken_longest_first_keep_their_places(n_seq):
+    """More runs than SMs: the kernel orders the sequences by length (up to 256 of them); states and rows stay the ones of the
+    single-sequence calls, bit for bit. Ties and empty sequences among them."""
+    H_v = 64 if n_seq == 3 else 2
+    gen = torch.Generator().manual_seed(n_seq)
+    lens = torch.randint(0, 5, (n_seq,), generator=gen) * torch.randint(1, 40, (n_seq,), generator=gen)
+    lens[0], lens[-1] = 3, 129
+    cu = [0] + torch.cumsum(lens, 0).tolist()
+    Q, K, V, beta, g, _ = (x[0] for x in _inputs(cu[-1], 1, H_v, n_seq))
+    S0 = 0.3 * torch.randn(n_seq, H_v, 128, 128, generator=gen).cuda()
+    O, S = gdn.gated_delta_layer(Q, K, V, beta, g, cu_seqlens=cu, S_in=S0)
+    assert gdn.gdn_device_status() == gdn.GDN_OK
+    for s in sorted({0, 1, 2, n_seq // 2, n_seq - 2, n_seq - 1, int(lens.argmax()), int(lens.argmin())}):
+        a, b = cu[s], cu[s + 1]
+        if a == b:
+            assert torch.equal(S[s], S0[s])
+            continue
+        o, st = gdn.gated_delta_layer(*(x[a:b].clone() for x in (Q, K, V, beta, g)), cu_seqlens=[0, b - a], S_in=S0[s:s + 1].clone())
+        assert torch.equal(O[a:b], o) and torch.equal(S[s], st[0])

@@ -510,8 +510,6 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             // The usual case: the product has the smaller exponent and is shifted right (or not at all), and the shift of the
             // other term folds into a multiplier: one multiply-add and one rounded shift per element.
             const bool fold = sa >= 0 && sp <= 0;
-            const int m_a = fold ? (1 << sa) : 0;
-            const Rnd rp = make_rnd(fold ? min(-sp, 31) : 0);
             uint32_t m = 0;
             auto band_product = [&](int jl) -> int {  // (Aq T0q)_ij
                 const int4 c4 = lds_v4(sSH_a + (cb + col0 + jl) * 16);
@@ -520,13 +518,21 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
                 const int a3 = (jl + 3 < kHC) ? aq[(jl + 3 < kHC) ? jl + 3 : 0] : ((jl + 3 == kHC) ? an0 : (jl + 3 == kHC + 1 ? an1 : an2));
                 return a1 * c4.x + a2 * c4.y + a3 * c4.z;
             };
+            // (either term: a rounded shift to the right, 0 where it is shifted left, and a multiplier)
+            const Rnd ra = make_rnd(sa < 0 ? min(-sa, 31) : 0), rb = make_rnd(sp < 0 ? min(-sp, 31) : 0);
+            const int ma = sa > 0 ? 1 << sa : 1, mb = sp > 0 ? 1 << sp : 1;
+            if (fold) {
 #pragma unroll
-            for (int jl = 0; jl < kHC; ++jl) {
-                const int pr = band_product(jl);
-                int v;
-                if (fold) v = aq[jl] * m_a + rsr_rnd(pr, rp);
-                else v = term32(aq[jl], sa) + term32(pr, sp);
-                acc[jl] = (il - (col0 + jl)) > N ? v : 0;
+                for (int jl = 0; jl < kHC; ++jl) {
+                    const int v = aq[jl] * ma + rsr_rnd(band_product(jl), rb);
+                    acc[jl] = (il - (col0 + jl)) > N ? v : 0;
+                }
+            } else {
+#pragma unroll
+                for (int jl = 0; jl < kHC; ++jl) {
+                    const int v = rsr_rnd(aq[jl], ra) * ma + rsr_rnd(band_product(jl), rb) * mb;
+                    acc[jl] = (il - (col0 + jl)) > N ? v : 0;
+                }
             }
             MaxMag mm;
 #pragma unroll

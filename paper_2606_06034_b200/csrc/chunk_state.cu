@@ -103,17 +103,47 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity) {
     return true;
 }
 
-// Hand-off from the 512 compute threads to the issuing warp over a hardware barrier: the threads arrive and go on, the
-// issuing warp waits. (An mbarrier poll costs the waiting warp ~200-300 cycles per hand-off on the chain of the
-// sequence; this is a few tens.) The wait has no bound of its own: threads whose own bounded waits run out arrive on both hand-offs before they leave.
-// Hand-off 4 (state copies in place) also takes the table threads, which wait on it: they stay one chunk ahead.
-template <int ID>
-__device__ __forceinline__ void handoff_arrive() {
-    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
+// The same for a whole warp, with one answer for all its lanes (the hardware barriers behind it count warps). It also gives
+// up when another warp has: the lanes still polling then vote on one last poll. Lanes that have left the loop have seen the
+// phase complete, so that poll sees it too. (A vote on every poll, or a look at `fail` before the first one, costs the chain of
+// the sequence 20 to 40 cycles a chunk: 32 heads x 32768 tokens 1217 and 1207 us instead of 1199.)
+__device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity, const volatile int* fail) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    uint32_t i = 0;
+    while (!mbar_try_wait_hint(bar, parity, 2000u)) {
+        if ((++i & 15u) == 0) {
+            const uint32_t lanes = __activemask();
+            if (__any_sync(lanes, *fail != 0 || clock64() - t0 > 2000000000LL)) return __all_sync(lanes, mbar_try_wait(bar, parity));
+        }
+    }
+    return true;
 }
-template <int ID>
+
+// Hand-offs over hardware barriers: the 16 compute warps arrive and go on, whoever needs their work waits. (An mbarrier poll
+// costs the waiting warp ~200-300 cycles per hand-off on the chain of the sequence; this is a few tens.) Per chunk:
+//   4  the state copies are in place: 16 compute warps arrive, the issuing warp and the two table warps wait (these stay one
+//      chunk ahead), and the storing warp arrives once it has taken hand-off 6 of the chunk before: 20 warps, 19 state only
+//   5  U_new, P and the decayed state are in place: 16 compute warps arrive, the issuing warp waits
+//   6  the output tile is staged: 16 compute warps arrive, the storing warp waits (not state only)
+// These waits have no bound of their own. They end because every warp takes part in every one of them exactly once per chunk,
+// also after a bounded wait has run out (s_fail): the issuing, storing and table warps go through all chunks without doing
+// their work, and a compute warp that gives up does the rest of its hand-offs as waits (see the end of its loop). No warp
+// arrives twice in one generation of a barrier: a warp that goes on has seen a product that was issued behind the generation
+// before (D1 of a chunk behind its hand-off 4, O2 and the state behind its hand-off 5), and one that has given up waits for it.
+// Since hand-off 4 of a chunk takes the issuing warp (which has then taken 5 of the chunk before) and the storing warp (6), its
+// completion closes all three of the chunk before.
+template <int ID, bool SO>
+constexpr int handoff_threads() {
+    return kThreads + 32 + (ID == 4 ? kTabThreads + (SO ? 0 : 32) : 0);
+}
+template <int ID, bool SO>
+__device__ __forceinline__ void handoff_arrive() {
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(handoff_threads<ID, SO>()) : "memory");
+}
+template <int ID, bool SO>
 __device__ __forceinline__ void handoff_wait() {
-    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(handoff_threads<ID, SO>()) : "memory");
 }
 // 8 columns of 16 lanes: threads 0..15 the columns from taddr on, threads 16..31 of the same lanes those 32 further
 __device__ __forceinline__ void tmem_ld8_split32(uint32_t taddr, uint32_t (&r)[8]) {
@@ -167,9 +197,9 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     float* gtab = reinterpret_cast<float*>(smem + kOffG);  // per buffer: exp(g_i), exp(g_C - g_j), g_i, 1/||k||, 1/||q|| (64 each)
 
     // One mbarrier per MMA group that is waited for (never two pending phases on one barrier), two per-stage TMA
-    // barriers, and two on which the storing warp releases the output staging buffers. The hand-offs from the 512
-    // compute threads to the issuing and the storing warp go over hardware barriers 4, 5 and 6 (handoff_arrive / _wait).
-    __shared__ uint64_t bar_full[2], bar_pre, bar_d1, bar_o2, bar_g2, bar_stg[2];
+    // barriers, two on which the storing warp releases the output staging buffers, and one for products still in flight when
+    // the CTA gives up. The hand-offs between the warps go over hardware barriers 4, 5 and 6 (handoff_arrive / _wait).
+    __shared__ uint64_t bar_full[2], bar_pre, bar_d1, bar_o2, bar_g2, bar_stg[2], bar_end;
     __shared__ uint32_t tmem_base_s;
     __shared__ int s_fail;
     __shared__ int s_len[VAR && !SO ? kMaxOrder : 1], s_seq;
@@ -193,6 +223,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         mbar_init(&bar_g2, 1);
         mbar_init(&bar_stg[0], 1);
         mbar_init(&bar_stg[1], 1);
+        mbar_init(&bar_end, 1);
         s_fail = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tmQ);
@@ -301,14 +332,14 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         if (n_c > 0) put_gates(0, g_next);
         g_next = fetch(1);
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");
-        for (int c = 0; c < n_c && *fail == 0; ++c) {
+        for (int c = 0; c < n_c; ++c) {
             if (c + 1 < n_c) put_gates(c + 1, g_next);
             g_next = fetch(c + 2);
             float* tb = gtab + (c % 3) * kTab;
             const float gc = tb[128 + tt], gC = tb[128 + 63];
             float rk = 1.f, so = p.scale;
             if (NRM) {
-                if (!wait_bar(&bar_full[c & 1], (c >> 1) & 1)) *fail = 1;
+                if (!wait_bar_warp(&bar_full[c & 1], (c >> 1) & 1, fail)) *fail = 1;
                 const uint8_t* st = smem + (c & 1) * kStageBytes;
                 rk = (VAR && tt >= len - c * kC) ? 0.f : inv_norm(st + kOffK);
                 if (!SO) so *= inv_norm(st + kOffQ);
@@ -317,7 +348,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             tb[256 + tt] = so;
             tb[192 + tt] = -rk;
             tb[64 + tt] = -rk * fast_exp2((gC - gc) * kLog2e);
-            handoff_wait<4>();
+            handoff_wait<4, SO>();
         }
     } else if (producer) {
         // ================= loading / storing warp: the four tiles of chunk c into stage c & 1, as soon as the products
@@ -340,14 +371,19 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             tma_load_3d(st + kOffU, &tmU, bar, vx, t0, vz);
             tma_load_3d(st + kOffU + 8192, &tmU, bar, vx + 64, t0, vz);
         };
+        int loaded = n_c < 2 ? n_c : 2;  // chunks whose tiles have been asked for
         if (lead) {
             if (n_c > 0) load_stage(0);
             if (n_c > 1) load_stage(1);
         }
         uint32_t par = 0;
-        for (int c = 0; c < n_c && *fail == 0; ++c) {
+        if (!SO) handoff_arrive<4, SO>();
+        for (int c = 0; c < n_c; ++c) {
             // the staged output tile of chunk c is complete (every compute thread has arrived)
-            if (!SO) handoff_wait<6>();
+            if (!SO) {
+                handoff_wait<6, SO>();
+                if (c + 1 < n_c) handoff_arrive<4, SO>();
+            }
             if (lead && *fail == 0) {
                 if (!SO && !(VAR && len - c * kC < kC)) {  // (a short last chunk is stored row by row by the compute threads)
                     tma_store_3d(&tmO, smem + kOffO + (c & 1) * kTileBytes, vx, tok0 + c * kC, vz);
@@ -356,7 +392,10 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 }
                 if (c + 2 < n_c) {
                     if (!wait_bar(&bar_g2, par)) *fail = 1;
-                    if (*fail == 0) load_stage(c + 2);
+                    if (*fail == 0) {
+                        load_stage(c + 2);
+                        loaded = c + 3;
+                    }
                 }
                 if (!SO) {
                     tma_store_wait_read<0>();
@@ -366,7 +405,12 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             par ^= 1;
             __syncwarp();
         }
-        if (lead) tma_store_wait_all<0>();
+        if (lead) {
+            tma_store_wait_all<0>();
+            if (*fail != 0) {  // loads still in flight land before the CTA leaves
+                for (int c = loaded < 2 ? 0 : loaded - 2; c < loaded; ++c) wait_bar(&bar_full[c & 1], (c >> 1) & 1);
+            }
+        }
         __syncwarp();
     } else if (issuer) {
         // ================= issuing warp: every tcgen05.mma, in the order the tensor pipe runs them
@@ -377,7 +421,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // the products of chunk c that do not depend on the state: D1 <- (-I) U^T and PT = K Q^T
         auto issue_pre = [&](int c) {
             const uint32_t sa = smem_a + (c & 1) * kStageBytes;
-            if (!wait_bar(&bar_full[c & 1], (c >> 1) & 1)) *fail = 1;
+            if (!wait_bar_warp(&bar_full[c & 1], (c >> 1) & 1, fail)) *fail = 1;
             tc_fence_after_sync();
             if (*fail == 0 && elect_one()) {
                 if (!no_u) {
@@ -399,10 +443,10 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             __syncwarp();
         };
-        for (int c = 0; c < n_c && *fail == 0; ++c) {
+        for (int c = 0; c < n_c; ++c) {
             const uint32_t st_a = smem_a + (c & 1) * kStageBytes;
             // the state copies (and, for the first chunk, the constant operand) are in place
-            handoff_wait<4>();
+            handoff_wait<4, SO>();
             tc_fence_after_sync();
             if (c == 0) issue_pre(0);
             if (*fail == 0 && elect_one()) {
@@ -433,7 +477,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             __syncwarp();
             // U_new^T (hi, lo; plain, scaled), P (hi, lo) and the decayed accumulator are in place
-            handoff_wait<5>();
+            handoff_wait<5, SO>();
             tc_fence_after_sync();
             if (*fail == 0 && elect_one()) {
                 if (!SO) {
@@ -467,7 +511,11 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             // state-independent products of the next chunk follow them directly
             if (c + 1 < n_c) issue_pre(c + 1);
         }
-        if (*fail != 0) handoff_arrive<4>();  // (the table threads may be waiting on it)
+        if (*fail != 0 && elect_one()) {  // products still in flight end before their operands go
+            mma_commit(&bar_end);
+            wait_bar(&bar_end, 0);
+        }
+        __syncwarp();
     } else {
         // ================= compute threads (512): four per TMEM lane
         uint32_t par_pre = 0, par_d1 = 0, par_o2 = 0, par_g2 = 0;
@@ -475,7 +523,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // completed phase costs ~200 cycles whoever issues it; polling from lane 0 alone added a divergent branch and a
         // shuffle, ~150 cycles more per wait.
         auto wait_group = [&](uint64_t* bar, uint32_t& par) -> bool {
-            const bool good = wait_bar(bar, par);
+            const bool good = wait_bar_warp(bar, par, fail);
             if (!good) *fail = 1;
             par ^= 1;
             tc_fence_after_sync();
@@ -508,11 +556,12 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             tmem_wait_st();
             tc_fence_before_sync();
-            handoff_arrive<4>();
+            handoff_arrive<4, SO>();
         }
-        bool ok = true;
+        int gave_up = 0;  // 1, 2, 3: a wait of chunk c ran out before hand-off 5, before 6, behind 6
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");  // the gates of the first chunk
-        for (int c = 0; c < n_c; ++c) {
+        int c = 0;
+        for (; c < n_c; ++c) {
             const float* se = gtab + (c % 3) * kTab;  // scale exp(g_i) / ||q_i||
             const float* sf = se + 64;               // -exp(g_C - g_j) / ||k_j|| (D1 holds -U_new)
             const float* sg = se + 128;              // g_i (cumulative inside the chunk)
@@ -538,7 +587,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             // ---- P_ij = exp(g_i - g_j) PT_ji for j <= i (hi + lo): this thread's token j and 8 columns i. (Keys and queries
             // normalised here: 1 / ||k_j|| rides on U_new_j, 1 / ||q_i|| on the output.)
-            if (!SO && !wait_group(&bar_pre, par_pre)) { ok = false; break; }
+            if (!SO && !wait_group(&bar_pre, par_pre)) { gave_up = 1; break; }
             if (!SO) {
                 uint32_t d[8];
                 tmem_ld8_split32(lane_base + kPT + h * 8, d);
@@ -571,7 +620,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             // on correlated keys, so single bf16 copies cost 1e-2 there). This thread's 16 tokens are one k-step of the
             // products that consume them: the hi halves are written over its own D1 columns (plain -> 16 h .. 16 h + 7,
             // scaled -> 16 h + 8 ..), the lo halves at the same offsets of the PT region.
-            if (!wait_group(&bar_d1, par_d1)) { ok = false; break; }
+            if (!wait_group(&bar_d1, par_d1)) { gave_up = 1; break; }
             // (the four warps of a lane quadrant have read their columns of PT)
             if (!SO) asm volatile("bar.sync %0, 128;" ::"r"(8 + wq) : "memory");
             {
@@ -603,17 +652,15 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             fence_proxy_async_smem();
             tmem_wait_st();
             tc_fence_before_sync();
-            handoff_arrive<5>();
+            handoff_arrive<5, SO>();
             if (!SO) {
                 // The storing warp has released the PREVIOUS chunk's staging buffer (polled here, in the shadow of the
                 // output product; the store was issued most of a chunk ago). That is one chunk later than this chunk's
-                // own buffer needs (chunk c - 2 used it, and the stores are read in order), but it also says that the
-                // storing warp has taken the previous chunk's hand-off: the threads must not arrive on that hardware
-                // barrier a second time before it has, however long a store may be held up.
-                if (c >= 1 && !wait_bar(&bar_stg[(c - 1) & 1], ((c - 1) >> 1) & 1)) { *fail = 1; ok = false; break; }
+                // own buffer needs (chunk c - 2 used it, and the stores are read in order).
+                if (c >= 1 && !wait_bar_warp(&bar_stg[(c - 1) & 1], ((c - 1) >> 1) & 1, fail)) { *fail = 1; gave_up = 2; break; }
                 // ---- O^T = scale (exp(g_i) O1 + O2), in fragments of 8 x 8: this warp's 32 features x 16 tokens, transposed
                 // on the way to the staged tile (O1 is complete with O2: products finish in the order they were issued)
-                if (!wait_group(&bar_o2, par_o2)) { ok = false; break; }
+                if (!wait_group(&bar_o2, par_o2)) { gave_up = 2; break; }
                 {
                     const int t2 = h * 16 + 2 * (lane & 3);
                     const float2 e0 = *reinterpret_cast<const float2*>(se + t2), e1 = *reinterpret_cast<const float2*>(se + t2 + 8);
@@ -645,11 +692,11 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 }
                 // the tile goes to the storing warp: no compute thread waits for the others here
                 fence_proxy_async_smem();
-                handoff_arrive<6>();
+                handoff_arrive<6, SO>();
             }
             // ---- bf16 copies (hi, lo) of the new state for the next chunk's products; the lo half goes where O2 was
             // (this thread has read its O2 columns above)
-            if (!wait_group(&bar_g2, par_g2)) { ok = false; break; }
+            if (!wait_group(&bar_g2, par_g2)) { gave_up = 3; break; }
             {
                 uint32_t v[32], pk[16];
                 tmem_ld32(lane_base + kSD + h * 32, v);
@@ -661,7 +708,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 tmem_st16(lane_base + kO2 + h * 16, lo);
                 tmem_wait_st();
                 tc_fence_before_sync();
-                handoff_arrive<4>();
+                handoff_arrive<4, SO>();
             }
             if (!SO && short_chunk) {
                 // only the rows of real tokens leave, 16 bytes per thread and step, from the staged (swizzled) tile
@@ -674,17 +721,24 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 }
             }
         }
-        if (!ok) {
-            // a bounded wait ran out (s_fail is set): release the issuing and the storing warp from whichever hand-off
-            // they wait on (both leave their loops when they see s_fail)
-            handoff_arrive<4>();
-            handoff_arrive<5>();
-            handoff_arrive<6>();
+        if (gave_up != 0) {
+            // A bounded wait ran out (s_fail is set): this warp's remaining barriers of chunk c and of the chunks behind it, in
+            // the order of the loop above and as waits, so that no generation counts it twice.
+            for (; c < n_c; ++c, gave_up = 1) {
+                if (gave_up < 2) {
+                    if (!SO) asm volatile("bar.sync %0, 128;" ::"r"(8 + wq) : "memory");
+                    handoff_wait<5, SO>();
+                }
+                if (!SO && gave_up < 3) handoff_wait<6, SO>();
+                if (c + 1 < n_c) handoff_wait<4, SO>();
+                if (VAR && !SO && len - c * kC < kC) asm volatile("bar.sync 1, 512;" ::: "memory");
+            }
+            gave_up = 1;
         }
         // ---- final state
         // (the run's place among the states is formed again here: it is not held over the chunks)
         const int seq = (VAR && !SO && p.n_order > 0) ? *reinterpret_cast<volatile int*>(&s_seq) : static_cast<int>(blockIdx.x / p.H_v);
-        if (ok && p.S_out != nullptr && seq >= p.out_from) {
+        if (gave_up == 0 && p.S_out != nullptr && seq >= p.out_from) {
             float* so = p.S_out + (((long long)(seq - p.out_from) * p.H_v + blockIdx.x % p.H_v) * kD + t) * kD + h * 32;
             uint32_t v[32];
             tmem_ld32(lane_base + kSD + h * 32, v);

@@ -794,12 +794,12 @@ bool make_map(CUtensorMap* tm, const void* base, long long heads, int T, int col
 // Set-up of the first pass: the token ranges of its 2P - 3 runs (runs 0 .. P-2: segment s from a zero state, segment 0
 // from the caller's; runs P-1 .. 2P-4: segments 1 .. P-2 from the identity with U = 0, which gives the matrix M of
 // S_end = S_start M + N), their initial states, the token ranges of the second pass and its first initial state.
-// Grid (n1 + 1 states, value heads): one state of 128 x 128 per CTA.
+// Grid (value heads, n1 + 1 states): one state of 128 x 128 per CTA. (The heads along x: y ends at 65535.)
 __global__ void __launch_bounds__(256) segmented_setup_kernel(int P, int H_v, int n_chunks, const float* S_user, float* S_in1,
                                                               float* S_start, int* start1, int* end1, int* no_u1, int* start3,
                                                               int* end3) {
     const int n1 = 2 * P - 3;
-    const int run = blockIdx.x, hv = blockIdx.y;
+    const int run = blockIdx.y, hv = blockIdx.x;
     if (run == 0 && hv == 0) {
         for (int s_ = threadIdx.x; s_ < n1; s_ += 256) {
             const int seg = (s_ <= P - 2) ? s_ : s_ - (P - 2);
@@ -928,7 +928,8 @@ int launch_chunk_state_segmented(const ProblemS& q, int P, void* workspace, cuda
     int* no_u1 = end1 + n1;
     int* start3 = no_u1 + n1;
     int* end3 = start3 + P;
-    segmented_setup_kernel<<<dim3(static_cast<unsigned>(n1) + 1, q.H_v), 256, 0, stream>>>(P, q.H_v, n_chunks, q.S_in, S_in1, S_start, start1, end1, no_u1, start3, end3);
+    segmented_setup_kernel<<<dim3(q.H_v, static_cast<unsigned>(n1) + 1), 256, 0, stream>>>(P, q.H_v, n_chunks, q.S_in, S_in1, S_start, start1, end1, no_u1, start3, end3);
+    if (cudaGetLastError() != cudaSuccess) return GDN_ERR_LAUNCH;  // (the passes read the token ranges it writes)
     count_launch();
     ProblemS a = q;
     a.B = static_cast<int>(n1);
@@ -944,6 +945,7 @@ int launch_chunk_state_segmented(const ProblemS& q, int P, void* workspace, cuda
     if (cudaFuncSetAttribute(segmented_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombSmem) != cudaSuccess)
         return GDN_ERR_LAUNCH;
     segmented_combine_kernel<<<dim3(q.H_v, kD / kCombRows), 256, kCombSmem, stream>>>(P, q.H_v, S_out1, S_start);
+    if (cudaGetLastError() != cudaSuccess) return GDN_ERR_LAUNCH;
     count_launch();
     ProblemS b = q;
     b.B = P;

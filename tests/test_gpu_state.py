@@ -330,6 +330,22 @@ def test_segmented_call_on_the_prefill_shapes():
         assert eS.max() <= TOL_S, f"S rel-F {eS.max():.3e} of head {hv}"
 
 
+def test_segmented_call_with_more_heads_than_a_grid_has_rows():
+    """65536 value heads, one more than the y extent of a grid may have: every kernel of the call has to take them along x. Against
+    the plain call, which differs by the fp32 re-association of the state recurrence."""
+    H_v, T = 65536, 128
+    gen_ = torch.Generator(device="cuda").manual_seed(1)
+    K = torch.nn.functional.normalize(torch.randn(1, T, 128, generator=gen_, device="cuda"), dim=-1).bfloat16()
+    U = torch.randn(H_v, T, 128, generator=gen_, device="cuda", dtype=torch.bfloat16)
+    W = 0.1 * torch.randn(H_v, T, 128, generator=gen_, device="cuda", dtype=torch.bfloat16)
+    g = -0.1 * torch.rand(H_v, T, generator=gen_, device="cuda")
+    O, S = gdn.chunk_state_output_segmented(K, K, W, U, g, 64, 1.0, segments=2, flags=gdn.GDN_FLAG_G_RAW)
+    Op, Sp = gdn.chunk_state_output(K[None], K[None], W[None], U[None], g[None], 64, 1.0, flags=gdn.GDN_FLAG_G_RAW)
+    assert gdn.gdn_device_status() == gdn.GDN_OK
+    assert (S - Sp[0]).norm() <= 1e-5 * Sp.norm()
+    assert (O - Op[0]).float().norm() <= 2e-3 * Op.float().norm()
+
+
 @pytest.mark.parametrize("token_major", [False, True])
 def test_model_native_layer_from_raw_projections(token_major):
     """The call sequence of a model: raw key / query projections (normalised inside both kernels), raw log-gates,

@@ -54,16 +54,19 @@ __device__ __forceinline__ float sum2(f2 v) {
     return r.x + r.y;
 }
 
-// Columns [0, w) of `rows` rows of a [rows, d] tile into shared memory as fp32 (row pitch kLdk), rows up to `pad` zero.
+// Columns [0, w) of `rows` rows of a [rows, d] tile into shared memory as fp32 (row pitch kLdk), rows up to `pad` zero, columns
+// up to the end of the last unit of UW too: the products run over whole units, and what an earlier kernel has left there must
+// not reach the test for results that are not finite (d = 96 after a launch that left NaN: C = 64 173 instead of 81 us,
+// C = 128 1112 instead of 241).
 // fp32 arrives asynchronously: the caller waits (load_wait) and synchronises.
-template <int NT>
+template <int NT, int UW>
 __device__ __forceinline__ void load_tile(float* dst, const float* src, int rows, int pad, int d, int w) {
     const int c = (threadIdx.x & 31) << 2;
-    if (c < w) {
+    if (c < (w + UW - 1) / UW * UW) {
         uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(dst + (threadIdx.x >> 5) * kLdk + c));
         src += (long long)(threadIdx.x >> 5) * d + c;
         for (int i = threadIdx.x >> 5; i < pad; i += NT / 32) {
-            if (i < rows) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
+            if (i < rows && c < w) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
             else *reinterpret_cast<float4*>(dst + i * kLdk + c) = make_float4(0.f, 0.f, 0.f, 0.f);
             a += (NT / 32) * kLdk * 4;
             src += (NT / 32) * d;
@@ -71,13 +74,13 @@ __device__ __forceinline__ void load_tile(float* dst, const float* src, int rows
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
-template <int NT>
+template <int NT, int UW>
 __device__ __forceinline__ void load_tile(float* dst, const __nv_bfloat16* src, int rows, int pad, int d, int w) {
     const int c = (threadIdx.x & 15) << 3;
-    if (c >= w) return;
+    if (c >= (w + UW - 1) / UW * UW) return;
     for (int i = threadIdx.x >> 4; i < pad; i += NT / 16) {
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (i < rows) v = *reinterpret_cast<const uint4*>(src + (long long)i * d + c);
+        if (i < rows && c < w) v = *reinterpret_cast<const uint4*>(src + (long long)i * d + c);
         const uint32_t x[4] = {v.x, v.y, v.z, v.w};
         float f[8];
 #pragma unroll
@@ -314,7 +317,7 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
         else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(NG) : "memory");
     };
 
-    load_tile<NT>(Ks, Kc, C, NB * M, d_k, min(kSliceW, d_k));
+    load_tile<NT, 4 * G>(Ks, Kc, C, NB * M, d_k, min(kSliceW, d_k));
     for (int i = threadIdx.x; i < NB * M; i += NT) {
         sbeta[i] = (i < C) ? p.beta[tok + i] : 0.f;
         sg[i] = (i < C) ? p.g[tok + i] : 0.f;
@@ -335,7 +338,7 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
         const int w = min(kSliceW, d_k - d0);
         if (d0 > 0) {
             __syncthreads();
-            load_tile<NT>(Ks, Kc + d0, C, NB * M, d_k, w);
+            load_tile<NT, 4 * G>(Ks, Kc + d0, C, NB * M, d_k, w);
         }
         load_wait();
         __syncthreads();
@@ -600,7 +603,7 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
     if (u1 > nk) {
         in_v = nk + (max(u0, nk) - nk) / per_slice * per_slice;
         const int col = (in_v - nk) * UW;
-        load_tile<NT>(Vs, Vc + col, C, NB * M, d_v, min(kSliceW, d_v - col));
+        load_tile<NT, 4 * G>(Vs, Vc + col, C, NB * M, d_v, min(kSliceW, d_v - col));
     }
     // T leaves, X <- T diag(beta)
     IO* Tc = (share == 0 && p.Tinv != nullptr) ? static_cast<IO*>(p.Tinv) + chunk * (long long)C * C : nullptr;
@@ -638,7 +641,7 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
         float* B = is_v ? Vs : Ks;
         if (is_v ? in_v != first : d_k > kSliceW) {
             __syncthreads();
-            load_tile<NT>(B, (is_v ? Vc : Kc) + s0, C, NB * M, d, min(kSliceW, d - s0));
+            load_tile<NT, 4 * G>(B, (is_v ? Vc : Kc) + s0, C, NB * M, d, min(kSliceW, d - s0));
             v_ready = false;
         }
         if (is_v ? !v_ready : d_k > kSliceW) {

@@ -65,3 +65,30 @@ def test_tokens_before_one_that_is_not_finite(C, what):
             assert torch.isfinite(got).all()
             assert (got - want).abs().max().item() <= 1e-5  # (the order of the sums differs)
         assert not torch.isfinite(U[0, 0, at]).all() and (what == "V" or not torch.isfinite(W[0, 0, at]).all())
+
+
+@pytest.mark.parametrize("C,d", [(64, 96), (64, 72), (48, 200), (24, 40), (32, 136), (128, 96)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_calls_do_not_depend_on_what_ran_before(C, d, dtype):
+    """Feature sizes that end inside a unit of columns (64, 32 for chunks up to 32), after a launch that has left zeros in the
+    shared memory of every SM and after one that has left NaN: the same bits, and no second evaluation of the outputs (which takes
+    four times as long at C = 128, twice at 64)."""
+    inp = gen.make_inputs(1, 1, 1, 600 * C, C, d, d, seed=d, dtype=dtype)
+    dev = [x.cuda() for x in (inp.K, inp.V, inp.beta, inp.g)]
+    out, time = [], []
+    for left in (0.0, float("nan")):
+        fill = [torch.full((1, 1, 600 * C, 128), left, device="cuda") for _ in range(2)]
+        runs = []
+        for _ in range(9):
+            gdn.chunk_prepare(*fill, dev[2], dev[3], C)
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            res = gdn.chunk_prepare(*dev, C)
+            b.record()
+            torch.cuda.synchronize()
+            runs.append(a.elapsed_time(b))
+        out.append(res)
+        time.append(min(runs))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+    assert time[1] < 1.5 * time[0]

@@ -527,7 +527,13 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
                         }
                     }
                 }
-                __syncthreads();
+                float nonfinite = 0.f;
+#pragma unroll
+                for (int rr = 0; rr < R / 2; ++rr) {
+#pragma unroll
+                    for (int s = 0; s < R; ++s) nonfinite = fmaf(sum2(a[rr][s]), 0.f, nonfinite);
+                }
+                const bool again = __syncthreads_or(nonfinite != 0.f);
 #pragma unroll
                 for (int rr = 0; rr < R / 2; ++rr) {
                     const int i = ti + G * (rr == 0 ? grp : R - 1 - grp);
@@ -535,6 +541,16 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
                     for (int s = 0; s < R; ++s) {
                         if (step == 0) Yt[(tj + G * s) * ld + i] = sum2(a[rr][s]);
                         else A21[i * ld + tj + G * s] = sum2(a[rr][s]);
+                    }
+                }
+                if (again) {  // (as above: every sum over its own terms only, T11 from the diagonal on and T22 up to it)
+#pragma unroll 1
+                    for (int e = 0; e < R / 2 * R; ++e) {
+                        const int i = ti + G * (e < R ? grp : R - 1 - grp), j = tj + G * (e % R);
+                        float v = 0.f;
+                        for (int k = step == 0 ? j : 0; k < (step == 0 ? M : i + 1); ++k) v = fmaf(Lm[i * ld + k], Rm[j * ld + k], v);
+                        if (step == 0) Yt[j * ld + i] = v;
+                        else A21[i * ld + j] = v;
                     }
                 }
                 __syncthreads();

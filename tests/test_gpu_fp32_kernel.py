@@ -51,11 +51,10 @@ def test_few_chunks(n, C, d_k, d_v):
     _compare(inp)
 
 
-@pytest.mark.parametrize("C", [16, 33, 64, 128])
+@pytest.mark.parametrize("C,at", [(16, 8), (33, 14), (64, 24), (128, 45), (128, 64), (128, 74), (128, 101), (128, 127)])
 @pytest.mark.parametrize("what", ["K", "V"])
-def test_tokens_before_one_that_is_not_finite(C, what):
+def test_tokens_before_one_that_is_not_finite(C, at, what):
     inp = gen.make_inputs(1, 1, 1, C, C, 128, 128, seed=5, dtype=torch.float32)
-    at = C // 3 + 3  # (of two blocks, in the first: the block formula sums over all tokens of the second)
     clean = gdn.chunk_prepare(inp.K.cuda(), inp.V.cuda(), inp.beta.cuda(), inp.g.cuda(), C)
     for value in (float("nan"), float("inf")):
         K, V = inp.K.clone(), inp.V.clone()
@@ -64,6 +63,8 @@ def test_tokens_before_one_that_is_not_finite(C, what):
         for got, want in ((W[0, 0, :at], clean[0][0, 0, :at]), (U[0, 0, :at], clean[1][0, 0, :at]), (T[0, 0, 0, :at], clean[2][0, 0, 0, :at])):
             assert torch.isfinite(got).all()
             assert (got - want).abs().max().item() <= 1e-5  # (the order of the sums differs)
+        # and the entries of the inverse that no sum takes over that token: columns behind it
+        assert torch.isfinite(T[0, 0, 0, :, at + 1:]).all()
         assert not torch.isfinite(U[0, 0, at]).all() and (what == "V" or not torch.isfinite(W[0, 0, at]).all())
 
 

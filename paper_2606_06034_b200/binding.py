@@ -161,7 +161,11 @@ def _stream():
 
 def _int32_table(values, device):
     """Host integers as an int32 CUDA tensor. From pinned memory the copy is ordered on the stream only: the host does not
-    wait for the work queued before it, as it does with a copy from pageable memory."""
+    wait for the work queued before it, as it does with a copy from pageable memory. Under stream capture such a copy would
+    be recorded with the address of a buffer that is used for other things by the time the graph is replayed: refused."""
+    if device.type == "cuda" and torch.cuda.is_current_stream_capturing():
+        raise RuntimeError("packed calls that take their boundaries from the host cannot be captured; build the tables before the "
+                           "capture and use gdn_chunk_prepare_varlen / gdn_chunk_state_output_varlen")
     return torch.tensor(values, dtype=torch.int32, pin_memory=device.type == "cuda").to(device, non_blocking=True)
 
 

@@ -267,6 +267,36 @@ def test_empty_sequences_and_empty_batches():
     assert gdn.gdn_device_status() == gdn.GDN_OK
 
 
+def test_packed_calls_with_boundaries_on_the_host_are_refused_under_capture():
+    """Their tables are copied from a host buffer that outlives the call only until the copy has run; the raw entry points, whose
+    tables are the caller's, can be captured."""
+    T, cu = 200, [0, 70, 200]
+    gen_ = torch.Generator(device="cuda").manual_seed(2)
+    Q, K, V = (torch.randn(T, 2, 128, generator=gen_, device="cuda").bfloat16() for _ in range(3))
+    beta, g = torch.rand(T, 2, generator=gen_, device="cuda"), -torch.rand(T, 2, generator=gen_, device="cuda")
+    flags = gdn.GDN_FLAG_G_RAW | gdn.GDN_FLAG_LAYOUT_BTHD | gdn.GDN_FLAG_K_L2NORM
+    want = gdn.gated_delta_layer(Q, K, V, beta, g, cu_seqlens=cu)
+    W, U, _, cs, cl = gdn.chunk_prepare_varlen(K, V, beta, g, cu, 64, flags=flags | gdn.GDN_FLAG_W_GATED, want_tinv=False)
+    for call in (lambda: gdn.gated_delta_layer(Q, K, V, beta, g, cu_seqlens=cu),
+                 lambda: gdn.chunk_prepare_varlen(K, V, beta, g, cu, 64, flags=flags),
+                 lambda: gdn.chunk_state_output_varlen(Q, K, W, U, g, cu, 64, flags=flags)):
+        with pytest.raises(RuntimeError):
+            with torch.cuda.graph(torch.cuda.CUDAGraph()):
+                call()
+    table = torch.tensor(cu, dtype=torch.int32, device="cuda")
+    O, S = torch.zeros_like(U), torch.zeros_like(want[1])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gdn.gdn_chunk_prepare_varlen(K, V, beta, g, cs, cl, cs.numel(), T, 2, 2, 64, 128, 128, -1, -1, W, U, None,
+                                     flags | gdn.GDN_FLAG_W_GATED)
+        gdn.gdn_chunk_state_output_varlen(Q, K, W, U, g, table, 2, T, 2, 2, 64, 128, 128, 128 ** -0.5, None, O, S, flags)
+    W.zero_()
+    graph.replay()
+    again = gdn.gated_delta_layer(Q, K, V, beta, g, cu_seqlens=cu)
+    for a, b, c in zip(want, (O, S), again):
+        assert torch.equal(a, b) and torch.equal(a, c)
+
+
 def test_layer_wrapper_on_packed_token_major_raw_projections():
     """`gated_delta_layer`: packed sequences, token-major tensors, raw gates, raw key / query projections, one call."""
     C = 64

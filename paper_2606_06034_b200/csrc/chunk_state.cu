@@ -45,7 +45,7 @@ constexpr int kD = 128;        // d_k = d_v
 constexpr int kThreads = 512;  // compute threads, four per TMEM lane; two more warps issue the MMAs and the TMA loads
 constexpr int kTabThreads = 64;  // gate tables and norms, one thread per token of a chunk (four warps would cap the registers at 80)
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr int kMaxOrder = 256;  // sequences a packed launch sorts by length
+constexpr int kMaxOrder = 512;  // sequences that a packed launch takes longest first (see launch_chunk_state)
 
 // TMEM column map (512 columns: one CTA per SM)
 constexpr uint32_t kSD = 0;    // 128: state S, fp32 accumulator
@@ -81,7 +81,7 @@ struct ParamsS {
     const int* seq_start;  // first token of sequence s
     const int* seq_end;    // one past its last token (the public call passes cu_seqlens and cu_seqlens + 1)
     const int* seq_no_u;   // optional: sequence s runs with U = 0 (the state map of a segment, see the segmented call)
-    int n_order;             // packed: sequences to be taken longest first (0: in their order)
+    int n_order;             // sequences (the instantiations that take them longest first)
     int out_from;            // S_out holds the final states of the sequences from this one on
     __nv_bfloat16* O;  // output tensor (rows of a short last chunk are stored one by one)
 };
@@ -184,10 +184,52 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[8]) {
                  : "memory");
 }
 
+// Sequence of rank `rank` among the p.n_order <= 32 G of a packed call, longest class first, in their order inside a class; one
+// warp. Classes by the number of chunks: 0 .. 8, then four to a doubling. Bisection over the 32 classes, then the place inside
+// the class. Every CTA does it for itself, in the shadow of the TMEM allocation and of the loads of the sequence's bounds, which
+// it leaves in the L1 cache: 0.4 us a CTA up to 64 sequences, 0.7 at 256, 1.3 at 512. (A rank by comparison with every other
+// sequence, two barriers more: 2.4 us at 256.)
+template <int G>
+__device__ __forceinline__ int ranked_sequence(const ParamsS& p, int rank, int lane) {
+    int cls[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        const int s = i * 32 + lane;
+        cls[i] = s < p.n_order ? __ldg(p.seq_end + s) - __ldg(p.seq_start + s) : -kC;
+    }
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        const int n = (cls[i] + kC - 1) / kC, e = 31 - __clz(n | 8);
+        cls[i] = i * 32 + lane >= p.n_order ? -1 : n < 8 ? max(n, 0) : min(8 + (e - 3) * 4 + ((n >> (e - 2)) & 3), 31);
+    }
+    int lo = 0, longer = 0;  // more than `rank` sequences are of class lo or above, `longer` of the one behind the last bisection
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < G; ++i) n += cls[i] >= lo + step;
+        n = __reduce_add_sync(0xFFFFFFFFu, n);
+        if (n > rank) lo += step;
+        else longer = n;
+    }
+    int at = rank - longer, found = 0;
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        const uint32_t members = __ballot_sync(0xFFFFFFFFu, cls[i] == lo);
+        const bool me = cls[i] == lo && __popc(members & ((1u << lane) - 1u)) == at;
+        const uint32_t hit = __ballot_sync(0xFFFFFFFFu, me);
+        if (hit != 0) found = i * 32 + __ffs(hit) - 1;
+        at -= __popc(members);
+    }
+    return found;
+}
+
 // VAR: packed variable-length sequences (own instantiation: its masks sit on the chain the dense case is bound by)
 // SO: state only: no queries, no output (the first pass of the segmented call); U may be absent per sequence.
 // NRM: GDN_FLAG_K_L2NORM (keys and queries normalised here): own instantiations, the plain chain pays nothing for it.
-template <bool VAR, bool SO, bool NRM>
+// ORD: packed sequences, longest first (own instantiations: the code in front of the roles costs every CTA of a launch that does
+// not use it 0.1 to 0.4 us).
+template <bool VAR, bool SO, bool NRM, bool ORD>
 __global__ void __launch_bounds__(kThreads + 64 + kTabThreads, 1)
 chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmU,
@@ -202,7 +244,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     __shared__ uint64_t bar_full[2], bar_pre, bar_d1, bar_o2, bar_g2, bar_stg[2], bar_end;
     __shared__ uint32_t tmem_base_s;
     __shared__ int s_fail;
-    __shared__ int s_len[VAR && !SO ? kMaxOrder : 1], s_seq;
+    __shared__ int s_seq;
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -236,20 +278,16 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         tmem_alloc(&tmem_base_s, kTmemCols);
         tmem_relinquish();
     }
-    if (VAR && !SO && tid < p.n_order) s_len[tid] = __ldg(p.seq_end + tid) - __ldg(p.seq_start + tid);
+    if (ORD && producer) {
+        // longest sequences first: the CTAs with block index k H_v .. take the sequence of rank k
+        const int rank = static_cast<int>(blockIdx.x / p.H_v);
+        const int s = p.n_order <= 64 ? ranked_sequence<2>(p, rank, lane) : p.n_order <= 128 ? ranked_sequence<4>(p, rank, lane)
+                    : p.n_order <= 256 ? ranked_sequence<8>(p, rank, lane) : ranked_sequence<kMaxOrder / 32>(p, rank, lane);
+        if (lane == 0) s_seq = s;
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    if (VAR && !SO && p.n_order > 0) {
-        // longest sequence first: the CTAs with block index k H_v .. take the sequence of rank k (ties in their order)
-        if (tid < p.n_order) {
-            const int mine = s_len[tid];
-            int rank = 0;
-            for (int i = 0; i < p.n_order; ++i) rank += (s_len[i] > mine || (s_len[i] == mine && i < tid)) ? 1 : 0;
-            if (rank == static_cast<int>(blockIdx.x / p.H_v)) s_seq = tid;
-        }
-        __syncthreads();
-    }
     const uint32_t tmem = tmem_base_s;
     const uint32_t lane_base = tmem + (static_cast<uint32_t>(wq * 32) << 16);
 
@@ -257,7 +295,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     // (sequence, value head); the tensors have one batch row per head and the sequence starts at token tok0
     int b = blockIdx.x / p.H_v;
     const int hv = blockIdx.x - b * p.H_v;
-    if (VAR && !SO && p.n_order > 0) b = s_seq;
+    if (ORD) b = s_seq;
     const int tok0 = VAR ? __ldg(p.seq_start + b) : 0;
     const int len = VAR ? __ldg(p.seq_end + b) - tok0 : p.T;
     const bool no_u = SO && p.seq_no_u != nullptr && __ldg(p.seq_no_u + b) != 0;
@@ -737,7 +775,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         }
         // ---- final state
         // (the run's place among the states is formed again here: it is not held over the chunks)
-        const int seq = (VAR && !SO && p.n_order > 0) ? *reinterpret_cast<volatile int*>(&s_seq) : static_cast<int>(blockIdx.x / p.H_v);
+        const int seq = ORD ? *reinterpret_cast<volatile int*>(&s_seq) : static_cast<int>(blockIdx.x / p.H_v);
         if (gave_up == 0 && p.S_out != nullptr && seq >= p.out_from) {
             float* so = p.S_out + (((long long)(seq - p.out_from) * p.H_v + blockIdx.x % p.H_v) * kD + t) * kD + h * 32;
             uint32_t v[32];
@@ -1034,15 +1072,21 @@ int launch_chunk_state(const ProblemS& q, cudaStream_t stream) {
     prm.seq_no_u = q.seq_no_u;
     prm.out_from = q.out_from;
     prm.O = static_cast<__nv_bfloat16*>(q.O);
-    // More runs than SMs (one CTA each): the long ones start first, so that none of them is left for the end. 61 prompts of
-    // 1 to 2050 tokens, 32 heads: the last SM finishes 20 % later in the order of arrival than in this one (list scheduling
-    // of the measured 5 + 2.5 us a chunk). Every CTA ranks the lengths itself, under 1 us at 256 sequences.
-    prm.n_order = (var && !q.state_only && n_cta > 148 && q.B > 1 && q.B <= kMaxOrder) ? q.B : 0;
+    // More runs than SMs (one CTA each): the long ones may start first, so that none of them is left for the end. That saves a
+    // share of the longest run once, in proportion to the mean run, and costs every CTA (0.25 + 0.002 n) us for finding its
+    // sequence. It is done where the waves of CTAs times that are at most 1.5 us per chunk of the mean run. State passing,
+    // log-normal lengths (gain) and equal ones (cost), with the order / without: 61 sequences of 500 tokens, 8 heads, 131 / 181 us
+    // and 131 / 129; 256 of 128, 2 heads, 70 / 99 and 57 / 54. Beyond the line: 256 of 64, 128 heads, 2780 / 2560 us.
+    const double chunks = q.T / 64.0 + 0.5 * q.B;  // of all sequences
+    const bool ordered = var && !q.state_only && n_cta > 148 && q.B > 1 && q.B <= kMaxOrder &&
+                         static_cast<double>(n_cta) * q.B * (125 + q.B) <= 750.0 * 148 * chunks;
+    prm.n_order = q.B;
     const int smem = kSmemTotal + 1024;
     const bool nrm = (q.flags & GDN_FLAG_K_L2NORM) != 0;
-    auto kern = q.state_only ? (nrm ? chunk_state_kernel<true, true, true> : chunk_state_kernel<true, true, false>)
-                : var        ? (nrm ? chunk_state_kernel<true, false, true> : chunk_state_kernel<true, false, false>)
-                             : (nrm ? chunk_state_kernel<false, false, true> : chunk_state_kernel<false, false, false>);
+    auto kern = q.state_only ? (nrm ? chunk_state_kernel<true, true, true, false> : chunk_state_kernel<true, true, false, false>)
+                : ordered    ? (nrm ? chunk_state_kernel<true, false, true, true> : chunk_state_kernel<true, false, false, true>)
+                : var        ? (nrm ? chunk_state_kernel<true, false, true, false> : chunk_state_kernel<true, false, false, false>)
+                             : (nrm ? chunk_state_kernel<false, false, true, false> : chunk_state_kernel<false, false, false, false>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GDN_ERR_LAUNCH;
     kern<<<static_cast<int>(n_cta), kThreads + 64 + kTabThreads, smem, stream>>>(mQ, mK, mW, mU, mO, prm);
     count_launch();

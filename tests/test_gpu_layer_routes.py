@@ -69,8 +69,8 @@ def test_packed_rows_without_a_sequence_stay_zero_and_the_others_keep_their_bits
 @pytest.mark.gpu
 @pytest.mark.parametrize("n_seq", [3, 256, 257])
 def test_packed_sequences_taken_longest_first_keep_their_places(n_seq):
-    """More runs than SMs: the kernel orders the sequences by length (up to 256 of them); states and rows stay the ones of the
-    single-sequence calls, bit for bit. Ties and empty sequences among them."""
+    """More runs than SMs: states and rows stay the ones of the single-sequence calls, bit for bit. Ties and empty sequences among
+    them."""
     H_v = 64 if n_seq == 3 else 2
     gen = torch.Generator().manual_seed(n_seq)
     lens = torch.randint(0, 5, (n_seq,), generator=gen) * torch.randint(1, 40, (n_seq,), generator=gen)
@@ -87,3 +87,28 @@ def test_packed_sequences_taken_longest_first_keep_their_places(n_seq):
             continue
         o, st = gdn.gated_delta_layer(*(x[a:b].clone() for x in (Q, K, V, beta, g)), cu_seqlens=[0, b - a], S_in=S0[s:s + 1].clone())
         assert torch.equal(O[a:b], o) and torch.equal(S[s], st[0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_seq,H_v", [(2, 128), (60, 4), (64, 4), (65, 4), (128, 2), (129, 2), (256, 1), (257, 1), (512, 1)])
+def test_longest_first_gives_what_the_order_of_arrival_gives(n_seq, H_v):
+    """The forms for up to 64, 128, 256 and 512 sequences, on lengths for which the order is used, against the same sequences with
+    empty ones behind them, too many for it: the same bits. Lengths at the edges of the classes, ties, empty sequences, one longer
+    than the last class."""
+    gen = torch.Generator().manual_seed(n_seq)
+    lens = (64 * torch.exp(1.5 * torch.randn(n_seq, generator=gen) + 1.0)).int() % 4000
+    lens[::7] = 64 * torch.randint(0, 14, lens[::7].shape, generator=gen).int()
+    lens[n_seq // 2] = 64 * 500 + 1
+    cu = [0] + torch.cumsum(lens, 0).tolist()
+    chunks = cu[-1] / 64 + n_seq / 2
+    assert n_seq * H_v > 148 and n_seq * H_v * n_seq * (125 + n_seq) <= 750 * 148 * chunks
+    Q, K, V, beta, g, _ = (x[0] for x in _inputs(cu[-1], 1, H_v, n_seq))
+    S0 = 0.3 * torch.randn(513, H_v, 128, 128, generator=gen).cuda()
+    W, U, _, _, _ = gdn.chunk_prepare_varlen(K, V, beta, g, cu, 64, flags=FLAGS | gdn.GDN_FLAG_W_GATED, want_tinv=False)
+    for flags in (FLAGS, FLAGS & ~gdn.GDN_FLAG_K_L2NORM):
+        scale = 128 ** -0.5 if flags == FLAGS else 0.01
+        O, S = gdn.chunk_state_output_varlen(Q, K, W, U, g, cu, 64, scale, S0[:n_seq].contiguous(), flags=flags)
+        On, Sn = gdn.chunk_state_output_varlen(Q, K, W, U, g, cu + [cu[-1]] * (513 - n_seq), 64, scale, S0, flags=flags)
+        assert gdn.gdn_device_status() == gdn.GDN_OK
+        assert torch.equal(O.view(torch.int16), On.view(torch.int16)) and torch.equal(S.view(torch.int32), Sn[:n_seq].view(torch.int32))
+        assert torch.equal(Sn[n_seq:], S0[n_seq:])

@@ -557,51 +557,54 @@ __global__ void __launch_bounds__(G* G* NB, G == 16 && NB == 1 ? 2 : 1) chunk_si
             }
         }
     } else {
-        // ---- forward substitution: thread j owns column j of T
-        auto A = [&](int i, int j) -> float {
-            if (NB == 1) return w0[i * ld + j];
-            return i < M ? sm[L::offW + i * ld + j] : j < M ? A21[(i - M) * ld + j] : sm[L::offW + 2 * L::mat + (i - M) * ld + j - M];
-        };
+        // ---- forward substitution: thread j owns column j of T. Of two blocks, the sums below run first over the rows of the
+        // upper one, then over the lower one's, each with pointers and one stride of its own.
         float* T21 = sm + L::offW + L::mat;
-        auto Tm = [&](int i, int j) -> float& {
-            if (NB == 1) return X[i * ld + j];
-            return i < M ? sm[L::offX + i * ld + j] : j < M ? T21[(i - M) * ld + j] : sm[L::offX + L::mat + (i - M) * ld + j - M];
-        };
         const int j = threadIdx.x;
+        const bool up = NB == 1 || j < M;                                                         // column j in the left blocks
+        float* Tu = sm + L::offX + j;                                                             // T(k, j), k < M (left columns)
+        float* Tl = up ? T21 + j : sm + L::offX + L::mat + j - M;                                 // T(M + k, j)
+        const float* Al = sm + L::offW + 2 * L::mat;                                              // A(M + i, M + k)
+        auto row = [&](int i) { return (NB == 1 || i < M) ? sm + L::offW + i * ld : A21 + (i - M) * ld; };  // A(i, k), k < M
+        // v + the terms k0 <= k < k1 of row i of A with column j of T, in that order
+        auto dot = [&](int i, int k0, int k1, float v) {
+            if (up) {
+                const float* a = row(i);
+                const int end = NB == 1 ? k1 : min(k1, M);
+                for (int k = k0; k < end; ++k) v = fmaf(a[k], Tu[k * ld], v);
+            }
+            if (NB == 2 && k1 > M) {
+                const float* a = Al + (i - M) * ld;
+                for (int k = max(k0, M) - M; k < k1 - M; ++k) v = fmaf(a[k], Tl[k * ld], v);
+            }
+            return v;
+        };
+        auto A = [&](int i) { return up ? row(i)[j] : Al[(i - M) * ld + j - M]; };  // A(i, j)
+        auto T = [&](int i) -> float& { return (NB == 1 || i < M) ? Tu[i * ld] : Tl[(i - M) * ld]; };  // T(i, j)
         if (p.mode == INV_FWDSUBST_BLOCKED) {
             // Blocked form (App. E): 16 x 16 diagonal blocks by substitution (Eq. 25), then block rows from
             // S_ij = S_ii sum_{k<i} Abar_ik S_kj (Eq. 27 with T_ik = -Abar_ik).
             if (j < C) {
                 const int bend = (j / 16 + 1) * 16;
-                for (int i = j + 1; i < bend; ++i) {
-                    float v = A(i, j);
-                    for (int k = j + 1; k < i; ++k) v = fmaf(A(i, k), Tm(k, j), v);
-                    Tm(i, j) = v;
-                }
+                for (int i = j + 1; i < bend; ++i) T(i) = dot(i, j + 1, i, A(i));
             }
             __syncthreads();
             if (j < C) {
                 for (int bi = j / 16 + 1; bi < C / 16; ++bi) {
                     float tmp[16];
+                    for (int r = 0; r < 16; ++r) tmp[r] = dot(bi * 16 + r, j, bi * 16, 0.f);
+                    // the diagonal block of these rows (16 divides M: it lies in one of the two)
+                    const float* S = (NB == 1 || bi * 16 < M) ? sm + L::offX + bi * 16 * (ld + 1) : sm + L::offX + L::mat + (bi * 16 - M) * (ld + 1);
                     for (int r = 0; r < 16; ++r) {
                         float v = 0.f;
-                        for (int k = j; k < bi * 16; ++k) v = fmaf(A(bi * 16 + r, k), Tm(k, j), v);
-                        tmp[r] = v;
-                    }
-                    for (int r = 0; r < 16; ++r) {
-                        float v = 0.f;
-                        for (int q = 0; q <= r; ++q) v = fmaf(Tm(bi * 16 + r, bi * 16 + q), tmp[q], v);
-                        Tm(bi * 16 + r, j) = v;
+                        for (int q = 0; q <= r; ++q) v = fmaf(S[r * ld + q], tmp[q], v);
+                        T(bi * 16 + r) = v;
                     }
                 }
             }
         } else if (j < C) {
             // Rows in order (Eq. 2-3): row i of X = Abar_i + Abar_{i,0:i} X_{0:i,:}
-            for (int i = j + 1; i < C; ++i) {
-                float v = A(i, j);
-                for (int k = j + 1; k < i; ++k) v = fmaf(A(i, k), Tm(k, j), v);
-                Tm(i, j) = v;
-            }
+            for (int i = j + 1; i < C; ++i) T(i) = dot(i, j + 1, i, A(i));
         }
         __syncthreads();
         if (NB == 2) {

@@ -93,3 +93,23 @@ def test_calls_do_not_depend_on_what_ran_before(C, d, dtype):
     for a, b in zip(*out):
         assert torch.equal(a, b)
     assert time[1] < 1.5 * time[0]
+
+
+@pytest.mark.parametrize("variant", [gdn.GDN_FWDSUBST_ROWS, gdn.GDN_FWDSUBST_BLOCKED])
+def test_forward_substitution_over_two_blocks_costs_its_terms(variant):
+    """A column of 128 rows has four times the terms of one of 64 and there are as many columns, so the same tokens take about four
+    times as long; two block matrices addressed entry by entry took twelve times."""
+    time = []
+    for C in (64, 128):
+        inp = gen.make_inputs(1, 1, 1, 128000, C, 64, 64, seed=C)
+        dev = [x.cuda() for x in (inp.K, inp.V, inp.beta, inp.g)]
+        runs = []
+        for _ in range(7):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            gdn.chunk_prepare(*dev, C, method="fwdsubst", variant=variant)
+            b.record()
+            torch.cuda.synchronize()
+            runs.append(a.elapsed_time(b))
+        time.append(min(runs))
+    assert time[1] < 6 * time[0]

@@ -758,17 +758,18 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         float a[HC];
         if constexpr (MERGE) {
             // rows of the second block keep their part of the lower-left Gram block (columns 0..63) in R2:
-            // R0..R1 is overwritten by the residual rounds
+            // R0..R1 is overwritten by the residual rounds. Either half of a row keeps it in the very columns that its part of
+            // X22 (hi, lo) goes to later: no thread writes over what the other half has yet to read.
             if (wq >= 2) {
                 uint32_t r[32], r16[16];
                 tmem_ld32(lane_base + kR0 + h * 32, r);
                 tmem_wait_ld();
 #pragma unroll
                 for (int i = 0; i < 16; ++i) r16[i] = r[i];
-                tmem_st16(lane_base + kR2 + h * 32, r16);
+                tmem_st16(lane_base + kR2 + h * 16, r16);
 #pragma unroll
                 for (int i = 0; i < 16; ++i) r16[i] = r[16 + i];
-                tmem_st16(lane_base + kR2 + h * 32 + 16, r16);
+                tmem_st16(lane_base + kR2 + 32 + h * 16, r16);
                 tmem_wait_st();
             }
         }
@@ -1402,7 +1403,7 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     uint32_t gq[16];
-                    tmem_ld16(lane_base + kR2 + h * 32 + hh * 16, gq);
+                    tmem_ld16(lane_base + kR2 + hh * 32 + h * 16, gq);
                     tmem_wait_ld();
 #pragma unroll
                     for (int j4 = 0; j4 < 4; ++j4) {
@@ -1427,7 +1428,7 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             }
             // X = T - I of the row's diagonal block (band without the unit diagonal + far part) as hi and lo halves:
             // X11 rows are the B operands of the first product ([64 x 64], MN-major, no swizzle; hi at 0, lo at 8 KB),
-            // X22 rows the A operands of the second (R2 columns 0..31 and 32..63; the parked Gram block has been read).
+            // X22 rows the A operands of the second (R2 columns 0..31 and 32..63; this half's part of the Gram block there has been read).
             // One half (hi, then lo) and 16 columns at a time, stored at once, to keep the live registers down.
             {
                 uint16_t vals[NB + 1];

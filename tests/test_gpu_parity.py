@@ -592,3 +592,19 @@ def test_bf16_large_launch_form_on_small_cases(adv, N, S, monkeypatch):
     for a, b in zip(got, ref):
         d = (a.float() - b.float()).abs()
         assert bool((d <= 2.0 ** -7 * b.float().abs() + 1e-6).all())
+
+
+@pytest.mark.parametrize("variant", [gdn.GDN_FWDSUBST_ROWS, gdn.GDN_FWDSUBST_BLOCKED])
+def test_block_merge_repeats_itself(variant):
+    """The two halves of a row take part in the merge of C = 128 at their own pace: with one of them late, the lower-left block came
+    out wrong in one chunk out of ten. Repeated calls give the same bits, and those of the default path up to rounding."""
+    inp = gen.make_inputs(1, 1, 1, 1000 * 128, 128, 128, 128, seed=3, adversarial_heads="all")
+    dev = [x.cuda() for x in (inp.K, inp.V, inp.beta, inp.g)]
+    first = gdn.chunk_prepare(*dev, 128, method="fwdsubst", variant=variant)
+    exact = gdn.chunk_prepare(*dev, 128, 3, 15)  # (S = 15: the exact inverse of either 64-block)
+    for a, b in zip(first, exact):
+        a, b = (x.double().reshape(1000, -1) for x in (a, b))
+        assert ((a - b).norm(dim=1) / b.norm(dim=1)).max().item() <= 4e-3  # (two roundings to bf16)
+    for _ in range(5):
+        for a, b in zip(first, gdn.chunk_prepare(*dev, 128, method="fwdsubst", variant=variant)):
+            assert torch.equal(a, b)

@@ -818,29 +818,25 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             const int m_hh = fold ? (1 << (16 + sp)) : 0, m_mid = fold ? (1 << (8 + sp)) : 0, m_ll = fold ? (1 << sp) : 0;
             const int bqs = fold ? (bq << sd) : 0;
             // the aligned sums stay in registers between the scale (bit length of the largest magnitude over the chunk's
-            // C x d block) and the mantissas
+            // C x d block) and the mantissas; eight columns at a time (sixteen spill: 2198 instead of 2172 us on the prefill shape)
             long long acc[kFC];
             uint32_t mlo = 0, mhi = 0;
 #pragma unroll
-            for (int c0 = 0; c0 < kFC; c0 += 16) {
-                uint32_t xr[8];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(xtile + ((((h & 1) * 4 + (c0 >> 3) + c) ^ (t & 7)) << 4));
-                    xr[4 * c + 0] = v.x; xr[4 * c + 1] = v.y; xr[4 * c + 2] = v.z; xr[4 * c + 3] = v.w;
-                }
-                uint32_t dhh[16], dmid[16], dll[16];
-                tmem_ld16(lane_base + kDhh + h * kFC + c0, dhh);
-                tmem_ld16(lane_base + kDmid + h * kFC + c0, dmid);
-                tmem_ld16(lane_base + kDll + h * kFC + c0, dll);
+            for (int c0 = 0; c0 < kFC; c0 += 8) {
+                const uint4 xv = *reinterpret_cast<const uint4*>(xtile + ((((h & 1) * 4 + (c0 >> 3)) ^ (t & 7)) << 4));
+                const uint32_t xr[4] = {xv.x, xv.y, xv.z, xv.w};
+                uint32_t dhh[8], dmid[8], dll[8];
+                tmem_ld8(lane_base + kDhh + h * kFC + c0, dhh);
+                tmem_ld8(lane_base + kDmid + h * kFC + c0, dmid);
+                tmem_ld8(lane_base + kDll + h * kFC + c0, dll);
                 tmem_wait_ld();
                 if (DBG && dbg_row != nullptr) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) dbg_row[8 * kC + half * kD + h * kFC + c0 + i] = combine(dhh[i], dmid[i], dll[i], p);
+                    for (int i = 0; i < 8; ++i) dbg_row[8 * kC + half * kD + h * kFC + c0 + i] = combine(dhh[i], dmid[i], dll[i], p);
                 }
                 if (fold) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
+                    for (int i = 0; i < 8; ++i) {
                         const uint32_t xw = xr[i >> 1];
                         const int x = (i & 1) ? hi16(xw) : lo16(xw);
                         acc[c0 + i] = zmag((long long)static_cast<int>(dhh[i]) * m_hh + (long long)static_cast<int>(dmid[i]) * m_mid +
@@ -848,7 +844,7 @@ chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     }
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
+                    for (int i = 0; i < 8; ++i) {
                         const uint32_t xw = xr[i >> 1];
                         const int x = (i & 1) ? hi16(xw) : lo16(xw);
                         acc[c0 + i] = zmag(term64(combine(dhh[i], dmid[i], dll[i], p), sp) + term64((long long)bq * x, sd), mlo, mhi, p.m1);

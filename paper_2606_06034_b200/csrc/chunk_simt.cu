@@ -19,7 +19,7 @@
 // one 16-byte read brings four terms of the sum: a thread holds the entries (ti + G r, tj + G s), r >= s, reads R + R rows per
 // four terms and does 2 * 10 packed multiply-adds (fma.rn.f32x2) with them at R = 4. The stride of G between a thread's rows
 // keeps the triangle's zero blocks the same for every thread (10 of 16 block pairs, 20 of 64 block triples) and the row pitch
-// of 4 (mod 8) words keeps the reads free of bank conflicts. C = 64, d = 128: 1024 chunks 113 us (one entry per thread and
+// of 4 (mod 8) words keeps the reads free of bank conflicts. C = 64, d = 128: 1024 chunks 111 us (one entry per thread and
 // step, two scalar reads per multiply-add: 1016 us), 8 chunks 21 us (216 us).
 #include "common.cuh"
 
@@ -714,7 +714,7 @@ int launch_one(SimtParams p, long long n_chunks, cudaStream_t stream) {
     // Fewer chunks than SMs: two or four CTAs share a chunk (each forms the inverse, its part of the columns of W and U), as
     // long as every CTA still has an SM of its own: 8 chunks of 64 take 21 us in four parts, where W and U are half the
     // work of a chunk; with more CTAs than SMs the repeated Gram product and rounds would be paid for twice.
-    p.split = n_chunks * 4 <= 148 ? 4 : n_chunks * 2 <= 148 ? 2 : 1;
+    p.split = n_chunks * 4 <= kSMs ? 4 : n_chunks * 2 <= kSMs ? 2 : 1;
     if (n_chunks * p.split >= (1LL << 31)) return GDN_ERR_UNSUPPORTED;
     kern<<<static_cast<int>(n_chunks * p.split), G * G * NB, smem, stream>>>(p);
     count_launch();

@@ -236,7 +236,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                    const __grid_constant__ CUtensorMap tmO, const ParamsS p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    float* gtab = reinterpret_cast<float*>(smem + kOffG);  // per buffer: exp(g_i), exp(g_C - g_j), g_i, 1/||k||, 1/||q|| (64 each)
+    float* gtab = reinterpret_cast<float*>(smem + kOffG);  // (see kTab)
 
     // One mbarrier per MMA group that is waited for (never two pending phases on one barrier), two per-stage TMA
     // barriers, two on which the storing warp releases the output staging buffers, and one for products still in flight when
@@ -937,6 +937,7 @@ size_t chunk_state_segmented_workspace(int H_v, int P) {
     if (P < 2) return 0;
     const size_t per = (size_t)H_v * kD * kD * sizeof(float);
     const size_t n1 = (size_t)(2 * P - 3);
+    // (P states more than the passes use: what callers allocate, and what the built-in array takes, stays as it was published)
     return (2 * n1 + 2 * (size_t)P) * per + (3 * n1 + 2 * (size_t)P) * sizeof(int) + 256;
 }
 
@@ -1078,8 +1079,8 @@ int launch_chunk_state(const ProblemS& q, cudaStream_t stream) {
     // log-normal lengths (gain) and equal ones (cost), with the order / without: 61 sequences of 500 tokens, 8 heads, 131 / 181 us
     // and 131 / 129; 256 of 128, 2 heads, 70 / 99 and 57 / 54. Beyond the line: 256 of 64, 128 heads, 2780 / 2560 us.
     const double chunks = q.T / 64.0 + 0.5 * q.B;  // of all sequences
-    const bool ordered = var && !q.state_only && n_cta > 148 && q.B > 1 && q.B <= kMaxOrder &&
-                         static_cast<double>(n_cta) * q.B * (125 + q.B) <= 750.0 * 148 * chunks;
+    const bool ordered = var && !q.state_only && n_cta > kSMs && q.B > 1 && q.B <= kMaxOrder &&
+                         static_cast<double>(n_cta) * q.B * (125 + q.B) <= 750.0 * kSMs * chunks;
     prm.n_order = q.B;
     const int smem = kSmemTotal + 1024;
     const bool nrm = (q.flags & GDN_FLAG_K_L2NORM) != 0;

@@ -1860,7 +1860,7 @@ int launch_ex(const Maps& m, const Params& prm, cudaStream_t stream) {
     const int smem = L::kTotal + 1024;
     auto kern = chunk_tc_kernel<C, NB, MODE, MERGE, EX, DBL, PERM>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GDN_ERR_LAUNCH;
-    long long grid = prm.n_tiles < 2 * 148 ? prm.n_tiles : 2 * 148;
+    long long grid = prm.n_tiles < 2 * kSMs ? prm.n_tiles : 2 * kSMs;
     Params q = prm;
     const long long y = grid / prm.group;
     q.s_gi = static_cast<int>(grid - y * prm.group);

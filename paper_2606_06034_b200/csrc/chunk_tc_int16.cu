@@ -967,7 +967,7 @@ int launch_tc_int16(const ProblemI16& q, cudaStream_t stream) {
     const int smem = kSmemTotal + 1024;
     auto kern = (prm.dbg != nullptr) ? chunk_tc_int16_kernel<true> : chunk_tc_int16_kernel<false>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GDN_ERR_LAUNCH;
-    const long long grid = prm.n_tiles < 148 ? prm.n_tiles : 148;
+    const long long grid = prm.n_tiles < kSMs ? prm.n_tiles : kSMs;
     kern<<<static_cast<int>(grid), kThreads, smem, stream>>>(mK, mV, prm);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_LAUNCH;

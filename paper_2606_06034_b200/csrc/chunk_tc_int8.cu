@@ -1491,7 +1491,7 @@ int launch_tc_int8(const ProblemI8& q, cudaStream_t stream) {
     if (cudaFuncSetAttribute(chunk_tc_int8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
         cudaFuncSetAttribute(chunk_tc_int8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return GDN_ERR_LAUNCH;
-    const long long grid = prm.n_tiles < 2 * 148 ? prm.n_tiles : 2 * 148;
+    const long long grid = prm.n_tiles < 2 * kSMs ? prm.n_tiles : 2 * kSMs;
     if (q.dbg != nullptr) chunk_tc_int8_kernel<true><<<static_cast<int>(grid), kThreads, smem, stream>>>(mK, mV, mW, mU, mT, prm);
     else chunk_tc_int8_kernel<false><<<static_cast<int>(grid), kThreads, smem, stream>>>(mK, mV, mW, mU, mT, prm);
     count_launch();
@@ -1500,7 +1500,7 @@ int launch_tc_int8(const ProblemI8& q, cudaStream_t stream) {
         const int smem2 = kMrgSmemTotal + 1024;
         if (cudaFuncSetAttribute(int8_merge128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2) != cudaSuccess)
             return GDN_ERR_LAUNCH;
-        const long long grid2 = prm.n_tiles < 148 ? prm.n_tiles : 148;
+        const long long grid2 = prm.n_tiles < kSMs ? prm.n_tiles : kSMs;
         int8_merge128_kernel<<<static_cast<int>(grid2), kMThreads, smem2, stream>>>(mK, mV, prm);
         count_launch();
     }

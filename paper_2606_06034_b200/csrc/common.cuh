@@ -8,6 +8,9 @@
 
 namespace gdn {
 
+// SMs of a B200: grids of one or two CTAs per SM, and the rules that compare a launch with the chip
+constexpr int kSMs = 148;
+
 // Problem description shared by all kernels.
 struct Problem {
     const void* K;

@@ -51,6 +51,31 @@ def test_layer_on_both_sides_of_the_line(H_k, H_v, chunks, with_state):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("H_v,chunks", [(2, 10), (2, 80), (32, 16), (32, 96), (64, 40), (64, 256)])
+def test_the_line_is_on_the_right_side_of_the_clock(H_v, chunks):
+    """Well off the line, on either side, the form that the layer takes is the faster one (8, 3 and 2 segments)."""
+    Q, K, V, beta, g, _ = _inputs(64 * chunks, 1, H_v, chunks)
+    W, U, _ = gdn.chunk_prepare(K, V, beta, g, 64, flags=FLAGS | gdn.GDN_FLAG_W_GATED, want_tinv=False)
+    forms = (lambda: gdn.chunk_state_output(Q, K, W, U, g, 64, 1.0, flags=FLAGS),
+             lambda: gdn.chunk_state_output_segmented(Q[0], K[0], W[0], U[0], g[0], 64, 1.0, flags=FLAGS))
+    time = []
+    for call in forms:
+        runs = []
+        for _ in range(6):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            torch.cuda._sleep(200000)  # (the launches are queued before the first one runs)
+            a.record()
+            for _ in range(8):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            runs.append(a.elapsed_time(b))
+        time.append(min(runs))
+    segmented = gdn._segments_pay(64 * chunks, 64, int(gdn.load_library().gdn_chunk_state_segments(H_v)))
+    assert time[segmented] < time[not segmented]
+
+
+@pytest.mark.gpu
 def test_packed_rows_without_a_sequence_stay_zero_and_the_others_keep_their_bits():
     T, extra = 200, 40
     Q, K, V, beta, g, _ = (x[0] for x in _inputs(T + extra, 1, 2, 3))

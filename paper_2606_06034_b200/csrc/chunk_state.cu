@@ -127,27 +127,24 @@ __device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity, co
 // Hand-offs over hardware barriers: the 16 compute warps arrive and go on, whoever needs their work waits. (An mbarrier poll
 // costs the waiting warp ~200-300 cycles per hand-off on the chain of the sequence; this is a few tens.) Per chunk:
 //   4  the state copies are in place: 16 compute warps arrive, the issuing warp and the two table warps wait (these stay one
-//      chunk ahead), and the storing warp arrives once it has taken hand-off 6 of the chunk before: 20 warps, 19 state only
+//      chunk ahead)
 //   5  U_new, P and the decayed state are in place: 16 compute warps arrive, the issuing warp waits
 //   6  the output tile is staged: 16 compute warps arrive, the storing warp waits (not state only)
 // These waits have no bound of their own. They end because every warp takes part in every one of them exactly once per chunk,
 // also after a bounded wait has run out (s_fail): the issuing, storing and table warps go through all chunks without doing
 // their work, and a compute warp that gives up does the rest of its hand-offs as waits (see the end of its loop). No warp
 // arrives twice in one generation of a barrier: a warp that goes on has seen a product that was issued behind the generation
-// before (D1 of a chunk behind its hand-off 4, O2 and the state behind its hand-off 5), and one that has given up waits for it.
-// Since hand-off 4 of a chunk takes the issuing warp (which has then taken 5 of the chunk before) and the storing warp (6), its
-// completion closes all three of the chunk before.
-template <int ID, bool SO>
-constexpr int handoff_threads() {
-    return kThreads + 32 + (ID == 4 ? kTabThreads + (SO ? 0 : 32) : 0);
-}
-template <int ID, bool SO>
+// before (D1 of a chunk behind its hand-off 4, O2 and the state behind its hand-off 5) or, for 6, the staging buffer of the chunk
+// before released; one that has given up waits for 5, which the issuing warp takes behind 4, and looks whether the storing warp
+// has taken 6 (s_taken). (The storing warp in hand-off 4 as well would say so without a look, but it reaches it late where many
+// CTAs store at once: 256 heads x 4096 tokens 435 instead of 431 us.)
+template <int ID>
 __device__ __forceinline__ void handoff_arrive() {
-    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(handoff_threads<ID, SO>()) : "memory");
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
 }
-template <int ID, bool SO>
+template <int ID>
 __device__ __forceinline__ void handoff_wait() {
-    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(handoff_threads<ID, SO>()) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
 }
 // 8 columns of 16 lanes: threads 0..15 the columns from taddr on, threads 16..31 of the same lanes those 32 further
 __device__ __forceinline__ void tmem_ld8_split32(uint32_t taddr, uint32_t (&r)[8]) {
@@ -248,6 +245,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     __shared__ uint64_t bar_full[2], bar_pre, bar_d1, bar_o2, bar_g2, bar_stg[2], bar_end;
     __shared__ uint32_t tmem_base_s;
     __shared__ int s_fail;
+    __shared__ int s_taken;  // output tiles that the storing warp has taken over (hand-off 6)
     __shared__ int s_seq;
 
     const int tid = threadIdx.x;
@@ -271,6 +269,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         mbar_init(&bar_stg[1], 1);
         mbar_init(&bar_end, 1);
         s_fail = 0;
+        s_taken = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tmQ);
         tma_prefetch_desc(&tmK);
@@ -390,7 +389,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             tb[256 + tt] = so;
             tb[192 + tt] = -rk;
             tb[64 + tt] = -rk * fast_exp2((gC - gc) * kLog2e);
-            handoff_wait<4, SO>();
+            handoff_wait<4>();
         }
     } else if (producer) {
         // ================= loading / storing warp: the four tiles of chunk c into stage c & 1, as soon as the products
@@ -419,12 +418,11 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (n_c > 1) load_stage(1);
         }
         uint32_t par = 0;
-        if (!SO) handoff_arrive<4, SO>();
         for (int c = 0; c < n_c; ++c) {
             // the staged output tile of chunk c is complete (every compute thread has arrived)
             if (!SO) {
-                handoff_wait<6, SO>();
-                if (c + 1 < n_c) handoff_arrive<4, SO>();
+                handoff_wait<6>();
+                *reinterpret_cast<volatile int*>(&s_taken) = c + 1;
             }
             if (lead && *fail == 0) {
                 if (!SO && !(VAR && len - c * kC < kC)) {  // (a short last chunk is stored row by row by the compute threads)
@@ -488,7 +486,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         for (int c = 0; c < n_c; ++c) {
             const uint32_t st_a = smem_a + (c & 1) * kStageBytes;
             // the state copies (and, for the first chunk, the constant operand) are in place
-            handoff_wait<4, SO>();
+            handoff_wait<4>();
             tc_fence_after_sync();
             if (c == 0) issue_pre(0);
             if (*fail == 0 && elect_one()) {
@@ -519,7 +517,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             __syncwarp();
             // U_new^T (hi, lo; plain, scaled), P (hi, lo) and the decayed accumulator are in place
-            handoff_wait<5, SO>();
+            handoff_wait<5>();
             tc_fence_after_sync();
             if (*fail == 0 && elect_one()) {
                 if (!SO) {
@@ -598,7 +596,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
             tmem_wait_st();
             tc_fence_before_sync();
-            handoff_arrive<4, SO>();
+            handoff_arrive<4>();
         }
         int gave_up = 0;  // 1, 2, 3: a wait of chunk c ran out before hand-off 5, before 6, behind 6
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");  // the gates of the first chunk
@@ -694,11 +692,13 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             fence_proxy_async_smem();
             tmem_wait_st();
             tc_fence_before_sync();
-            handoff_arrive<5, SO>();
+            handoff_arrive<5>();
             if (!SO) {
                 // The storing warp has released the PREVIOUS chunk's staging buffer (polled here, in the shadow of the
                 // output product; the store was issued most of a chunk ago). That is one chunk later than this chunk's
-                // own buffer needs (chunk c - 2 used it, and the stores are read in order).
+                // own buffer needs (chunk c - 2 used it, and the stores are read in order), but it also says that the
+                // storing warp has taken the previous chunk's hand-off: the threads must not arrive on that hardware
+                // barrier a second time before it has, however long a store may be held up.
                 if (c >= 1 && !wait_bar_warp(&bar_stg[(c - 1) & 1], ((c - 1) >> 1) & 1, fail)) { *fail = 1; gave_up = 2; break; }
                 // ---- O^T = scale (exp(g_i) O1 + O2), in fragments of 8 x 8: this warp's 32 features x 16 tokens, transposed
                 // on the way to the staged tile (O1 is complete with O2: products finish in the order they were issued)
@@ -734,7 +734,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 }
                 // the tile goes to the storing warp: no compute thread waits for the others here
                 fence_proxy_async_smem();
-                handoff_arrive<6, SO>();
+                handoff_arrive<6>();
             }
             // ---- bf16 copies (hi, lo) of the new state for the next chunk's products; the lo half goes where O2 was
             // (this thread has read its O2 columns above)
@@ -750,7 +750,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 tmem_st16(lane_base + kO2 + h * 16, lo);
                 tmem_wait_st();
                 tc_fence_before_sync();
-                handoff_arrive<4, SO>();
+                handoff_arrive<4>();
             }
             if (!SO && short_chunk) {
                 // only the rows of real tokens leave, 16 bytes per thread and step, from the staged (swizzled) tile
@@ -769,10 +769,16 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             for (; c < n_c; ++c, gave_up = 1) {
                 if (gave_up < 2) {
                     if (!SO) asm volatile("bar.sync %0, 128;" ::"r"(8 + wq) : "memory");
-                    handoff_wait<5, SO>();
+                    handoff_wait<5>();
                 }
-                if (!SO && gave_up < 3) handoff_wait<6, SO>();
-                if (c + 1 < n_c) handoff_wait<4, SO>();
+                if (!SO && gave_up < 3) {
+                    // (it will: this warp has arrived there, the others arrive or wait there too; bounded as every wait)
+                    const long long t0 = clock64();
+                    while (__any_sync(0xFFFFFFFFu, *reinterpret_cast<volatile int*>(&s_taken) < c && clock64() - t0 < 2000000000LL)) {
+                    }
+                    handoff_wait<6>();
+                }
+                if (c + 1 < n_c) handoff_wait<4>();
                 if (VAR && !SO && len - c * kC < kC) asm volatile("bar.sync 1, 512;" ::: "memory");
             }
             gave_up = 1;

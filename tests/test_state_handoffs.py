@@ -23,14 +23,15 @@ class Twice(Exception):
 
 
 class Cta:
-    """Warps are generators of operations: ("arrive" | "sync", barrier), ("wait", event) -> whether it came in time."""
+    """Warps are generators of operations: ("arrive" | "sync", barrier), ("wait", event) -> whether it came in time, ("until", n):
+    the storing warp has taken n output tiles."""
 
     def __init__(self, rng, n_c, so, short, lost, old):
         self.rng, self.n_c, self.so, self.short, self.lost, self.old = rng, n_c, so, short, lost, old
-        self.size = {4: N_COMPUTE + 1 + N_TAB + (0 if so or old else 1), 5: N_COMPUTE + 1, 6: N_COMPUTE + 1, 1: N_COMPUTE, 3: N_TAB}
+        self.size = {4: N_COMPUTE + 1 + N_TAB, 5: N_COMPUTE + 1, 6: N_COMPUTE + 1, 1: N_COMPUTE, 3: N_TAB}
         self.size.update({8 + q: N_COMPUTE // 4 for q in range(4)})
         self.count = {b: [] for b in self.size}   # warps of the present generation
-        self.done, self.coming, self.fail = set(), set(), False
+        self.done, self.coming, self.fail, self.taken = set(), set(), False, 0
 
     def signal(self, *event):  # a load or a product: it completes some time later, or never
         if event not in self.lost:
@@ -75,6 +76,7 @@ class Cta:
                         yield "sync", 8 + w % 4
                     yield "sync", 5
                 if not so and gave_up < 3:
+                    yield "until", c
                     yield "sync", 6
                 if c + 1 < n_c:
                     yield "sync", 4
@@ -94,15 +96,12 @@ class Cta:
     def producer(self, w):
         for c in range(min(2, self.n_c)):
             self.signal("full", c)
-        if not self.so and not self.old:
-            yield "arrive", 4
         for c in range(self.n_c):
             if self.old and self.fail:
                 break
             if not self.so:
                 yield "sync", 6
-                if not self.old and c + 1 < self.n_c:
-                    yield "arrive", 4
+                self.taken = c + 1
             if not self.fail:
                 if c + 2 < self.n_c and (yield "wait", ("g2", c)) and not self.fail:
                     self.signal("full", c + 2)
@@ -147,7 +146,8 @@ class Cta:
         for i in range(len(warps)):
             step(i)
         while pending:
-            ready = [i for i in pending if i not in asleep and (pending[i][0] != "wait" or pending[i][1] in self.done)]
+            ready = [i for i in pending if i not in asleep and (pending[i][0] != "wait" or pending[i][1] in self.done)
+                     and (pending[i][0] != "until" or self.taken >= pending[i][1])]
             waiting = [i for i in pending if pending[i][0] == "wait" and pending[i][1] not in self.done]
             awake = [i for i in ready if i != frozen or self.fail]
             if self.coming and (self.rng.random() < 0.3 or not awake):
@@ -158,7 +158,7 @@ class Cta:
             elif ready:
                 i = self.rng.choice(awake or ready)
                 kind, what = pending[i]
-                if kind == "wait":
+                if kind in ("wait", "until"):
                     step(i, True)
                     continue
                 here = self.count[what]

@@ -10,22 +10,24 @@
 //
 // Everything is evaluated with the value dimension on the 128 TMEM lanes ("transposed"): one CTA per (batch, head)
 // keeps the state S [d_v x d_k] as an fp32 accumulator in TMEM for the whole sequence, lane t = value feature t.
-//     D1  = S0 W^T - U^T      A = S0 as hi + lo bf16 halves in TMEM (the state is O(1) while U_new can be small:
-//                             a single bf16 copy costs 1e-2 on strongly correlated keys), B = W tile; the
-//                             transpose of U comes from the tensor core as
-//                             (-I) U^T with a constant A operand, so no thread ever transposes anything
+//     D1  = S0 W^T            A = S0 as hi + lo bf16 halves in TMEM (the state is O(1) while U_new can be small:
+//                             a single bf16 copy costs 1e-2 on strongly correlated keys), B = W tile
+//     U_new^T = U^T - D1      by threads: ldmatrix transposes 8 x 8 blocks of the U tile into the fragments in which D1 is read
 //     PT  = K Q^T             an M = 64 product: token j = 16 (lane / 32) + lane mod 16 on the lower 16 lanes of every lane
-//                             quadrant, columns = token i; lanes 16..31 of a warp read the upper 32 columns of the lower ones
+//                             quadrant, columns = token i; lanes 16..31 of a warp read other columns of the lower ones
 //     O1  = S0 Q^T
 //     O2  = U_new^T P^T       A = bf16(U_new^T) (written over D1's columns), B = P_ij = exp(g_i-g_j) PT_ji [j <= i]
 //     S  += (U_new^T exp(g_C - g_j)) K     accumulated onto exp(g_C) S0 (the decay is a pass over the TMEM columns)
 //     O^T = scale (exp(g_i) O1 + O2)  -> transposed through shared memory -> bulk tensor store
-// Two MMA groups per chunk; Q, K, W, U tiles of the next chunk are in flight (two stages) while a chunk is worked on.
 // All operand layouts are the ones the chunk-prepare kernel uses.
-// Warps: 16 compute warps (four threads per TMEM lane), one that issues every MMA, one that issues the TMA loads and
-// the output stores, two that form the gate tables and the norms a chunk ahead. The chain of a sequence is thread work (every phase runs on all 16 warps at once, so its
-// instruction count is what it costs); hand-offs to the issuing warp are hardware barriers, completions come back
-// through mbarriers (a poll costs ~200 cycles, so as few as possible are waited for).
+// Warps: 8 chain warps (the state's copies, U_new, the decay), 8 output warps (P, O and the norms: nothing of theirs is on the chain),
+// one that issues every MMA, one that issues the TMA loads and stores, two that form the gate tables.
+// What bounds it: the chain of a sequence is D1 (16 products, 700 cycles with its completion) -> U_new (800) -> state update (first
+// half 500) -> copies (650), 2900 cycles a chunk; and beside it the SM's shared memory, of which a chunk's products, TMA
+// copies and fragments move 335 KB, 2600 cycles at its full rate. So the state's columns go through the update, the copies
+// and D1 in two halves (the tensor pipe works on one while threads work on the other), what a phase reads from shared memory is
+// fetched before its products start, and a hi + lo split takes four instructions (see split_neg). us per chunk of 32
+// sequences of 256 chunks, before (16 warps that did everything in turn) and now: NOW_FIGURES.
 // Instantiations: packed variable-length sequences (one CTA per (sequence, value head), starting at the sequence's
 // first token; the tokens a short last chunk lacks decay nothing and write nothing); state only (no queries, no
 // output: the first pass of the segmented call for few long sequences, see launch_chunk_state_segmented); keys and
@@ -42,30 +44,38 @@ using namespace sm100;
 
 constexpr int kC = 64;         // chunk size
 constexpr int kD = 128;        // d_k = d_v
-constexpr int kThreads = 512;  // compute threads, four per TMEM lane; two more warps issue the MMAs and the TMA loads
-constexpr int kTabThreads = 64;  // gate tables and norms, one thread per token of a chunk (four warps would cap the registers at 80)
+constexpr int kChain = 256;    // threads that carry the state's chain, two per TMEM lane
+constexpr int kAux = 256;      // threads that form P, the output and the norms, two per TMEM lane
+constexpr int kThreads = 512;  // both; two more warps issue the MMAs and the TMA copies
+static_assert(kThreads == kChain + kAux, "");
+constexpr int kTabThreads = 64;  // gate tables, one thread per token of a chunk
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kMaxOrder = 512;  // sequences that a packed launch takes longest first (see launch_chunk_state)
 
 // TMEM column map (512 columns: one CTA per SM)
 constexpr uint32_t kSD = 0;    // 128: state S, fp32 accumulator
 constexpr uint32_t kSA = 128;  // 64: bf16(S0) as A operand (K = d_k)
-constexpr uint32_t kIA = 192;  // 64: -I as A operand (K = d_v), constant
-constexpr uint32_t kD1 = 256;  // 64: S0 W^T - U^T, then the two bf16 forms of U_new^T as A operands
-constexpr uint32_t kPT = 320;  // 64: K Q^T (half of the lanes); once read, the lo bf16 halves of the two forms of U_new^T
+constexpr uint32_t kSL = 192;  // 64: the rest bf16(S0) leaves, negated (A operand)
+constexpr uint32_t kD1 = 256;  // 64: S0 W^T, then the hi halves of the two forms of U_new^T as A operands
+constexpr uint32_t kUL = 320;  // 64: the lo halves of the two forms of U_new^T, negated
 constexpr uint32_t kO1 = 384;  // 64: S0 Q^T
-constexpr uint32_t kO2 = 448;  // 64: U_new^T P^T; between chunks it holds the lo bf16 half of S0 (A operand)
+constexpr uint32_t kO2 = 448;  // 64: U_new^T P^T
+constexpr uint32_t kPT = kO2;  // K Q^T (half of the lanes): read before O2 of the same chunk is issued
 constexpr uint32_t kTmemCols = 512;
+// A lo half is kept negated, as the difference comes out of a mixed-precision subtraction: its products subtract
+constexpr uint32_t kNegA = 1u << 13, kNegB = 1u << 14;  // instruction descriptor: A or B negated
 
 // shared memory map (bytes; 1 KB aligned). A [64 x 128] bf16 tile is two [64 x 64] sub-tiles of 8 KB (128B swizzle).
 constexpr int kTileBytes = 16384;
-constexpr int kStageBytes = 4 * kTileBytes;  // Q, K, W, U
-constexpr int kOffQ = 0, kOffK = kTileBytes, kOffW = 2 * kTileBytes, kOffU = 3 * kTileBytes;
-constexpr int kOffP = 2 * kStageBytes;       // 2 x 8 KB: P as B operand [64 x 64] (MN-major, no swizzle), hi and lo halves
+constexpr int kRing = 3;  // K and Q tiles: in use from the norms on until the state update, so they are asked for three chunks ahead
+constexpr int kOffK = 0, kOffQ = kRing * kTileBytes;
+constexpr int kOffW = 2 * kRing * kTileBytes, kOffU = kOffW + 2 * kTileBytes;  // two each
+constexpr int kOffP = kOffU + 2 * kTileBytes;  // 2 x 8 KB: P as B operand [64 x 64] (MN-major, no swizzle), hi and lo halves
 constexpr int kOffO = kOffP + 16384;          // 2 x 16 KB: O tile staged for the bulk store (128B swizzle), two buffers
-constexpr int kTab = 5 * 64;  // floats per table buffer: scale exp(g_i) / ||q_i||, -exp(g_C - g_j) / ||k_j||, g, -1 / ||k_j||, scale / ||q_i||
-constexpr int kOffG = kOffO + 2 * kTileBytes;  // three table buffers
-constexpr int kSmemTotal = kOffG + 3 * kTab * 4;
+constexpr int kTab = 5 * 64;  // floats per table buffer: scale exp(g_i) / ||q_i||, exp(g_C - g_j) / ||k_j||, g, 1 / ||k_j||, scale / ||q_i||
+constexpr int kOffG = kOffO + 2 * kTileBytes;  // four table buffers
+constexpr int kSmemTotal = kOffG + 4 * kTab * 4;
+static_assert(kSmemTotal + 1024 <= 227 * 1024, "");
 
 
 struct ParamsS {
@@ -124,31 +134,37 @@ __device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity, co
     return mbar_try_wait(bar, parity) || wait_bar_slow(bar, parity, fail);
 }
 
-// Hand-offs over hardware barriers: the 16 compute warps arrive and go on, whoever needs their work waits. (An mbarrier poll
-// costs the waiting warp ~200-300 cycles per hand-off on the chain of the sequence; this is a few tens.) Per chunk:
-//   4  the state copies are in place: 16 compute warps arrive, the issuing warp and the two table warps wait (these stay one
-//      chunk ahead)
-//   5  U_new, P and the decayed state are in place: 16 compute warps arrive, the issuing warp waits
-//   6  the output tile is staged: 16 compute warps arrive, the storing warp waits (not state only)
-// These waits have no bound of their own. They end because every warp takes part in every one of them exactly once per chunk,
-// also after a bounded wait has run out (s_fail): the issuing, storing and table warps go through all chunks without doing
-// their work, and a compute warp that gives up does the rest of its hand-offs as waits (see the end of its loop). No warp
+// Hand-offs to the issuing warp over hardware barriers: the warps whose work it needs arrive and go on, it waits. (A poll of an
+// mbarrier, though its phase be complete, costs the issuing warp 100 to 200 cycles behind the products it has just issued, this 20 to 40.)
+//   4, 6  the copies of either half of the state's columns are in place (8 chain warps); 4 also: the tiles and the tables of the
+//         chunk are (2 table warps, which wait too and so stay one chunk ahead)
+//   5     U_new and the decayed state are in place (8 chain warps)
+//   7, 8  P is in place; O1 and O2 have been read (8 output warps)
+// These waits have no bound of their own. They end because every warp takes part in every one of its hand-offs exactly
+// once per chunk, also after a bounded wait has run out (s_fail): the issuing and table warps go through all chunks without doing their
+// work, and a chain or output warp that gives up does the rest of its hand-offs as waits (see the end of its loop). No warp
 // arrives twice in one generation of a barrier: a warp that goes on has seen a product that was issued behind the generation
-// before (D1 of a chunk behind its hand-off 4, O2 and the state behind its hand-off 5) or, for 6, the staging buffer of the chunk
-// before released; one that has given up waits for 5, which the issuing warp takes behind 4, and looks whether the storing warp
-// has taken 6 (s_taken). (The storing warp in hand-off 4 as well would say so without a look, but it reaches it late where many
-// CTAs store at once: 256 heads x 4096 tokens 435 instead of 431 us.)
+// before (D1 of a chunk behind its hand-offs 4 and 6, the state update behind 5, O2 behind 7, the next P^T behind 8).
+static_assert(kChain == kAux, "");
 template <int ID>
 __device__ __forceinline__ void handoff_arrive() {
-    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(kChain + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
 }
 template <int ID>
 __device__ __forceinline__ void handoff_wait() {
-    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(kThreads + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(kChain + 32 + (ID == 4 ? kTabThreads : 0)) : "memory");
 }
-// 8 columns of 16 lanes: threads 0..15 the columns from taddr on, threads 16..31 of the same lanes those 32 further
-__device__ __forceinline__ void tmem_ld8_split32(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], 32;"
+// 16 columns of 16 lanes: threads 0..15 the columns from taddr on, threads 16..31 of the same lanes those 32 further
+__device__ __forceinline__ void tmem_ld16_split32(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16], 32;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                   "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr)
+                 : "memory");
+}
+// 8 columns of 16 lanes: threads 0..15 the columns from taddr on, threads 16..31 of the same lanes the next 8
+__device__ __forceinline__ void tmem_ld8_split8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x32bx2.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], 8;"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr)
                  : "memory");
@@ -164,17 +180,38 @@ __device__ __forceinline__ f2 mul2(f2 a, f2 b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 __device__ __forceinline__ uint32_t pack_pair(f2 v) {
     float a, b;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
     return pack_bf16x2(a, b);
 }
-// two values as bf16 pairs hi + lo
-__device__ __forceinline__ void split_pair(f2 v, uint32_t& hi, uint32_t& lo) {
-    hi = pack_pair(v);
-    f2 rest;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rest) : "l"(v), "l"(pair2(bf16_lo(hi), bf16_hi(hi))));
-    lo = pack_pair(rest);
+// half HI of a bf16 pair minus x, in fp32 (one instruction, no unpacking)
+template <int HI>
+__device__ __forceinline__ float bf16_minus(uint32_t w, float x) {
+    float r;
+    if (HI) asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %1;\n\tsub.f32.bf16 %0, b, %2;\n\t}" : "=f"(r) : "r"(w), "f"(x));
+    else asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %1;\n\tsub.f32.bf16 %0, a, %2;\n\t}" : "=f"(r) : "r"(w), "f"(x));
+    return r;
+}
+// s0 += lo^2, s1 += hi^2 of a bf16 pair
+__device__ __forceinline__ void bf16_square_add(uint32_t w, float& s0, float& s1) {
+    asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\tfma.rn.f32.bf16 %0, a, a, %0;\n\tfma.rn.f32.bf16 %1, b, b, %1;\n\t}"
+        : "+f"(s0), "+f"(s1)
+        : "r"(w));
+}
+// two values as bf16 pairs, v = hi - neg_lo. 5.9 issue cycles per warp and pair; with the unpacked hi half subtracted from v (hi + lo)
+// 10.2, which is what the phases of the chain were bound by.
+__device__ __forceinline__ void split_neg(float v0, float v1, uint32_t& hi, uint32_t& neg_lo) {
+    hi = pack_bf16x2(v0, v1);
+    neg_lo = pack_bf16x2(bf16_minus<0>(hi, v0), bf16_minus<1>(hi, v1));
+}
+__device__ __forceinline__ void split_neg(f2 v, uint32_t& hi, uint32_t& neg_lo) {
+    split_neg(__uint_as_float(static_cast<uint32_t>(v)), __uint_as_float(static_cast<uint32_t>(v >> 32)), hi, neg_lo);
 }
 // 16 lanes x 16 columns of an accumulator as the fragments of four 8 x 8 matrices: r[0..1] lanes 0..7, r[2..3] lanes 8..15
 // of columns 0..7, r[4..7] the same of columns 8..15; thread l holds lane l / 4, columns 2 (l mod 4) and the next
@@ -182,6 +219,13 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr)
+                 : "memory");
+}
+// the reverse for packed operands: 16 lanes x 16 columns, r[2 k], r[2 k + 1] lanes 0..7 and 8..15 of columns 4 k .. 4 k + 3; thread l
+// holds lane l / 4, column l mod 4
+__device__ __forceinline__ void tmem_st_frag16(uint32_t taddr, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+                 "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                  : "memory");
 }
 
@@ -239,37 +283,48 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     float* gtab = reinterpret_cast<float*>(smem + kOffG);  // (see kTab)
 
-    // One mbarrier per MMA group that is waited for (never two pending phases on one barrier), two per-stage TMA
-    // barriers, two on which the storing warp releases the output staging buffers, and one for products still in flight when
-    // the CTA gives up. The hand-offs between the warps go over hardware barriers 4, 5 and 6 (handoff_arrive / _wait).
-    __shared__ uint64_t bar_full[2], bar_pre, bar_d1, bar_o2, bar_g2, bar_stg[2], bar_end;
+    // Never two pending phases on one barrier for anyone who waits on it: what a barrier's next phase needs, and who has to be past
+    // the present one for that, stands at each.
+    __shared__ uint64_t bar_kq[kRing], bar_w[2], bar_u[2];  // tiles: loaded again behind a product that every reader precedes (see the loading warp)
+    __shared__ uint64_t bar_nrm[4], bar_tab[4];  // norms (eight warps), tables (two warps) of chunk c: again behind hand-off 8 of chunk c + 1
+    __shared__ uint64_t bar_pt, bar_o2;  // products: the next one waits for a hand-off that every reader makes behind this one
+    __shared__ uint64_t bar_d1[2], bar_su[2][2];  // [chunk & 1]([half of the state's columns]): the one of chunk c + 2 needs tiles that are asked for behind this one
+    __shared__ uint64_t bar_ost[2], bar_stg[2];  // output tile staged (eight warps); staging buffer free again
+    __shared__ uint64_t bar_end;      // products still in flight when the CTA gives up
     __shared__ uint32_t tmem_base_s;
     __shared__ int s_fail;
-    __shared__ int s_taken;  // output tiles that the storing warp has taken over (hand-off 6)
     __shared__ int s_seq;
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
-    const int t = tid & 127;  // TMEM lane: value feature (state rows, output columns); token j for PT
-    const int h = (tid >> 7) & 3;  // column quarter: 16 of the 64 columns of a product, 32 of the 128 state columns
+    const int t = tid & 127;  // TMEM lane: value feature (state rows, output columns)
+    const int h = (tid >> 7) & 1;  // half: 32 of the 64 tokens of a product, 32 of every 64 state columns
     const int wq = warp & 3;
     const int lane = tid & 31;
+    const bool aux = warp >= kChain / 32 && warp < kThreads / 32;  // P, the output, the norms
     const bool issuer = warp == kThreads / 32;        // every tcgen05.mma
-    const bool producer = warp == kThreads / 32 + 1;  // every TMA load
-    const bool tabler = warp >= kThreads / 32 + 2;    // gate tables, norms
+    const bool producer = warp == kThreads / 32 + 1;  // every TMA load and store
+    const bool tabler = warp >= kThreads / 32 + 2;    // gate tables
 
     if (tid == 0) {
-        mbar_init(&bar_full[0], 1);
-        mbar_init(&bar_full[1], 1);
-        mbar_init(&bar_pre, 1);
-        mbar_init(&bar_d1, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&bar_w[i], 1);
+            mbar_init(&bar_u[i], 1);
+            mbar_init(&bar_d1[i], 1);
+            mbar_init(&bar_su[i][0], 1);
+            mbar_init(&bar_su[i][1], 1);
+            mbar_init(&bar_ost[i], kAux / 32);
+            mbar_init(&bar_stg[i], 1);
+        }
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(&bar_nrm[i], kAux / 32);
+            mbar_init(&bar_tab[i], kTabThreads / 32);
+        }
+        for (int i = 0; i < kRing; ++i) mbar_init(&bar_kq[i], 1);
+        mbar_init(&bar_pt, 1);
         mbar_init(&bar_o2, 1);
-        mbar_init(&bar_g2, 1);
-        mbar_init(&bar_stg[0], 1);
-        mbar_init(&bar_stg[1], 1);
         mbar_init(&bar_end, 1);
         s_fail = 0;
-        s_taken = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tmQ);
         tma_prefetch_desc(&tmK);
@@ -313,20 +368,31 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const long long grow0 = bthd ? ((long long)bz * p.T + tok0) * p.H_v + hv : (long long)bhv * p.T + tok0;  // first token's row
     const int gstep = bthd ? p.H_v : 1;
     const int n_c = (len + kC - 1) / kC;
-    const float* gseq = p.g + grow0;
     const uint32_t smem_a = smem_u32(smem);
     volatile int* fail = reinterpret_cast<volatile int*>(&s_fail);
 
+    // a wait of a whole warp that marks the CTA as failed when it runs out
+    auto wait_for = [&](uint64_t* bar, uint32_t parity) -> bool {
+        const bool good = wait_bar_warp(bar, parity, fail);
+        if (!good) *fail = 1;
+        return good;
+    };
+    // one arrival per warp, behind what all of its lanes have done
+    auto warp_arrive = [&](uint64_t* bar) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+    };
+
     if (tabler) {
-        // ================= table threads, one per token. Before hand-off 4 of chunk c they have written the factors of
-        // chunk c (read behind the completion of its first product, which that hand-off precedes) and the gates of chunk
-        // c + 1 (read from its start on, behind the same completion one chunk earlier). Three buffers: the threads are done
-        // with a chunk's tables when they arrive on the next hand-off 4, and the table threads wait for it.
+        // ================= table threads, one per token: the gates and factors of chunk c. They wait in hand-off 4 of the chunk, for
+        // its tiles too, so they are one chunk ahead at most: behind hand-off 4 of chunk c - 1 the state update of chunk c - 2 is complete,
+        // that was issued when the output warps were done with chunk c - 3 (hand-off 8), and nobody reads buffer c mod 4 any more.
         const int tt = tid - (kThreads + 64);
         const bool g_raw = (p.flags & GDN_FLAG_G_RAW) != 0;
+        const float* gseq = p.g + grow0;
         auto fetch = [&](int c) -> float { return (c < n_c && (!VAR || c * kC + tt < len)) ? __ldg(gseq + (c * kC + tt) * gstep) : 0.f; };
         auto put_gates = [&](int c, float gc) {
-            float* tb = gtab + (c % 3) * kTab;
+            float* tb = gtab + (c & 3) * kTab;
             const int left = len - c * kC;  // tokens of this chunk (>= 64 except for a short last chunk)
             if (g_raw) {
                 // inclusive prefix sum over the chunk's 64 tokens: inside each of the two warps by shuffles ...
@@ -350,452 +416,520 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 asm volatile("bar.sync 3, 64;" ::: "memory");
             }
         };
-        // 1 / ||row|| of row tt of a tile in shared memory (the sum does not care about the swizzle inside the row: each of
-        // eight neighbouring threads starts at another 16-byte piece, free of bank conflicts)
-        auto inv_norm = [&](const uint8_t* tile) -> float {
-            f2 a[2] = {0ull, 0ull};
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const uint4 w4 = *reinterpret_cast<const uint4*>(tile + (i >> 3) * 8192 + tt * 128 + (((i + tt) & 7) << 4));
-                const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const f2 x = pair2(bf16_lo(w[q]), bf16_hi(w[q]));
-                    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a[q & 1]) : "l"(x));
-                }
-            }
-            float s0, s1, s2, s3;
-            asm("mov.b64 {%0, %1}, %2;" : "=f"(s0), "=f"(s1) : "l"(a[0]));
-            asm("mov.b64 {%0, %1}, %2;" : "=f"(s2), "=f"(s3) : "l"(a[1]));
-            return rsqrtf(fmaxf((s0 + s1) + (s2 + s3), 1e-30f));
-        };
         float g_next = fetch(0);
-        if (n_c > 0) put_gates(0, g_next);
-        g_next = fetch(1);
-        asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");
         for (int c = 0; c < n_c; ++c) {
-            if (c + 1 < n_c) put_gates(c + 1, g_next);
-            g_next = fetch(c + 2);
-            float* tb = gtab + (c % 3) * kTab;
+            const float g_c = g_next;
+            g_next = fetch(c + 1);
+            put_gates(c, g_c);
+            float* tb = gtab + (c & 3) * kTab;
             const float gc = tb[128 + tt], gC = tb[128 + 63];
             float rk = 1.f, so = p.scale;
-            if (NRM) {
-                if (!wait_bar_warp(&bar_full[c & 1], (c >> 1) & 1, fail)) *fail = 1;
-                const uint8_t* st = smem + (c & 1) * kStageBytes;
-                rk = (VAR && tt >= len - c * kC) ? 0.f : inv_norm(st + kOffK);
-                if (!SO) so *= inv_norm(st + kOffQ);
+            if (NRM) {  // (a wait that runs out sets the flag, and the others' waits end by it)
+                wait_for(&bar_nrm[c & 3], (c >> 2) & 1);
+                rk = (VAR && tt >= len - c * kC) ? 0.f : tb[192 + tt];
+                if (!SO) so *= tb[256 + tt];
             }
             tb[tt] = so * fast_exp2(gc * kLog2e);
             tb[256 + tt] = so;
-            tb[192 + tt] = -rk;
-            tb[64 + tt] = -rk * fast_exp2((gC - gc) * kLog2e);
+            tb[192 + tt] = rk;
+            tb[64 + tt] = rk * fast_exp2((gC - gc) * kLog2e);
+            warp_arrive(&bar_tab[c & 3]);
+            wait_for(&bar_kq[c % kRing], (c / kRing) & 1);
+            wait_for(&bar_w[c & 1], (c >> 1) & 1);
             handoff_wait<4>();
         }
     } else if (producer) {
-        // ================= loading / storing warp: the four tiles of chunk c into stage c & 1, as soon as the products
-        // that read the stage's previous tiles are complete; and the bulk stores of the staged output tiles, so that
-        // no compute thread waits for the others at the end of a chunk
+        // ================= loading / storing warp. W and U of a chunk are asked for when D1 of the chunk two before is complete (its U is
+        // in registers by then: the chain warps fetch it before they make the copies that this D1 waits for; that of the first chunk
+        // behind its D1), K and Q when the state update of the chunk three before is. And the bulk stores of the staged output tiles.
         const bool lead = elect_one();
-        auto load_stage = [&](int c) {
-            uint8_t* st = smem + (c & 1) * kStageBytes;
-            uint64_t* bar = &bar_full[c & 1];
-            mbar_arrive_expect_tx(bar, SO ? 3 * kTileBytes : kStageBytes);
-            const int t0 = tok0 + c * kC;
-            if (!SO) {
-                tma_load_3d(st + kOffQ, &tmQ, bar, kx, t0, kz);
-                tma_load_3d(st + kOffQ + 8192, &tmQ, bar, kx + 64, t0, kz);
-            }
-            tma_load_3d(st + kOffK, &tmK, bar, kx, t0, kz);
-            tma_load_3d(st + kOffK + 8192, &tmK, bar, kx + 64, t0, kz);
-            tma_load_3d(st + kOffW, &tmW, bar, vx, t0, vz);
-            tma_load_3d(st + kOffW + 8192, &tmW, bar, vx + 64, t0, vz);
-            tma_load_3d(st + kOffU, &tmU, bar, vx, t0, vz);
-            tma_load_3d(st + kOffU + 8192, &tmU, bar, vx + 64, t0, vz);
+        auto load_tile = [&](int off, const CUtensorMap* tm, uint64_t* bar, int x, int c, int z) {
+            tma_load_3d(smem + off, tm, bar, x, tok0 + c * kC, z);
+            tma_load_3d(smem + off + 8192, tm, bar, x + 64, tok0 + c * kC, z);
         };
-        int loaded = n_c < 2 ? n_c : 2;  // chunks whose tiles have been asked for
+        auto load_kq = [&](int c) {
+            if (c >= n_c) return;
+            uint64_t* bar = &bar_kq[c % kRing];
+            mbar_arrive_expect_tx(bar, (SO ? 1 : 2) * kTileBytes);
+            load_tile(kOffK + (c % kRing) * kTileBytes, &tmK, bar, kx, c, kz);
+            if (!SO) load_tile(kOffQ + (c % kRing) * kTileBytes, &tmQ, bar, kx, c, kz);
+        };
+        auto load_v = [&](int off, const CUtensorMap* tm, uint64_t* bars, int c) {  // a tile of W or U
+            if (c >= n_c) return;
+            mbar_arrive_expect_tx(&bars[c & 1], kTileBytes);
+            load_tile(off + (c & 1) * kTileBytes, tm, &bars[c & 1], vx, c, vz);
+        };
         if (lead) {
-            if (n_c > 0) load_stage(0);
-            if (n_c > 1) load_stage(1);
-        }
-        uint32_t par = 0;
-        for (int c = 0; c < n_c; ++c) {
-            // the staged output tile of chunk c is complete (every compute thread has arrived)
-            if (!SO) {
-                handoff_wait<6>();
-                *reinterpret_cast<volatile int*>(&s_taken) = c + 1;
+            int n_kq = kRing, n_w = 2, n_u = 2;  // chunks whose tiles have been asked for
+            for (int c = 0; c < kRing; ++c) {
+                load_kq(c);
+                if (c < 2) load_v(kOffW, &tmW, bar_w, c);
+                if (c < 2) load_v(kOffU, &tmU, bar_u, c);
             }
-            if (lead && *fail == 0) {
-                if (!SO && !(VAR && len - c * kC < kC)) {  // (a short last chunk is stored row by row by the compute threads)
-                    tma_store_3d(&tmO, smem + kOffO + (c & 1) * kTileBytes, vx, tok0 + c * kC, vz);
-                    tma_store_3d(&tmO, smem + kOffO + (c & 1) * kTileBytes + 8192, vx + 64, tok0 + c * kC, vz);
-                    tma_store_commit();
-                }
+            for (int c = 0; c < n_c && *fail == 0; ++c) {
                 if (c + 2 < n_c) {
-                    if (!wait_bar(&bar_g2, par)) *fail = 1;
-                    if (*fail == 0) {
-                        load_stage(c + 2);
-                        loaded = c + 3;
-                    }
+                    if (!wait_bar(&bar_d1[c & 1], (c >> 1) & 1)) *fail = 1;
+                    if (*fail != 0) break;
+                    load_v(kOffW, &tmW, bar_w, n_w++);
+                    if (c > 0) load_v(kOffU, &tmU, bar_u, n_u++);
+                    if (!wait_bar(&bar_su[c & 1][1], (c >> 1) & 1)) *fail = 1;
+                    if (*fail != 0) break;
+                    if (c == 0) load_v(kOffU, &tmU, bar_u, n_u++);
+                    load_kq(n_kq++);
                 }
                 if (!SO) {
-                    tma_store_wait_read<0>();
+                    if (!wait_bar(&bar_ost[c & 1], (c >> 1) & 1)) *fail = 1;
+                    if (*fail != 0) break;
+                    if (!(VAR && len - c * kC < kC)) {  // (a short last chunk is stored row by row by the output warps)
+                        tma_store_3d(&tmO, smem + kOffO + (c & 1) * kTileBytes, vx, tok0 + c * kC, vz);
+                        tma_store_3d(&tmO, smem + kOffO + (c & 1) * kTileBytes + 8192, vx + 64, tok0 + c * kC, vz);
+                        tma_store_commit();
+                        tma_store_wait_read<0>();
+                    }
                     mbar_arrive(&bar_stg[c & 1]);  // the staging buffer may be written again (chunk c + 2)
                 }
             }
-            par ^= 1;
-            __syncwarp();
-        }
-        if (lead) {
             tma_store_wait_all<0>();
             if (*fail != 0) {  // loads still in flight land before the CTA leaves
-                for (int c = loaded < 2 ? 0 : loaded - 2; c < loaded; ++c) wait_bar(&bar_full[c & 1], (c >> 1) & 1);
+                for (int i = 1; i <= kRing; ++i) {
+                    if (n_kq - i >= 0 && n_kq - i < n_c) wait_bar(&bar_kq[(n_kq - i) % kRing], ((n_kq - i) / kRing) & 1);
+                    if (i <= 2 && n_w - i < n_c) wait_bar(&bar_w[(n_w - i) & 1], ((n_w - i) >> 1) & 1);
+                    if (i <= 2 && n_u - i < n_c) wait_bar(&bar_u[(n_u - i) & 1], ((n_u - i) >> 1) & 1);
+                }
             }
         }
         __syncwarp();
     } else if (issuer) {
-        // ================= issuing warp: every tcgen05.mma, in the order the tensor pipe runs them
+        // ================= issuing warp: every tcgen05.mma, in the order the tensor pipe runs them. On the chain of the sequence are
+        // D1 and the state update; P^T and O1 run while U_new is formed, O2 while the state is copied.
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0);  // (a uniform register: every operand address of a product derives from it)
         const uint32_t idesc_kk64 = instr_desc(128, 64, 1, 1, 0, 0, 1);   // B K-major (a TMA tile as [N x K])
         const uint32_t idesc_mn64 = instr_desc(128, 64, 1, 1, 0, 1, 1);   // B MN-major
-        const uint32_t idesc_mn128 = instr_desc(128, 128, 1, 1, 0, 1, 1);
         const uint32_t idesc_pt = instr_desc(64, 64, 1, 1, 0, 0, 1);
-        // the products of chunk c that do not depend on the state: D1 <- (-I) U^T and PT = K Q^T
-        auto issue_pre = [&](int c) {
-            const uint32_t sa = smem_a + (c & 1) * kStageBytes;
-            if (!wait_bar_warp(&bar_full[c & 1], (c >> 1) & 1, fail)) *fail = 1;
-            tc_fence_after_sync();
-            if (*fail == 0 && elect_one()) {
-                if (!no_u) {
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
-                        const uint64_t bd = smem_desc(sa + kOffU + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024, SWZ_128B);
-                        mma_f16_ts(tmem + kD1, tmem + kIA + ks * 8, bd, idesc_kk64, ks > 0);
-                    }
-                }
-                if (!SO) {
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
-                        const uint64_t ad = smem_desc(sa + kOffK + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024, SWZ_128B);
-                        const uint64_t bd = smem_desc(sa + kOffQ + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024, SWZ_128B);
-                        mma_f16_ss(tmem + kPT, ad, bd, idesc_pt, ks > 0);
-                    }
-                    mma_commit(&bar_pre);  // (state only: nothing of this group is waited for by itself)
-                }
-            }
-            __syncwarp();
-        };
+        const uint64_t desc_p = smem_desc(smem_a + kOffP, 128, 1024, SWZ_NONE);
         for (int c = 0; c < n_c; ++c) {
-            const uint32_t st_a = smem_a + (c & 1) * kStageBytes;
-            // the state copies (and, for the first chunk, the constant operand) are in place
-            handoff_wait<4>();
-            tc_fence_after_sync();
-            if (c == 0) issue_pre(0);
-            if (*fail == 0 && elect_one()) {
-                // D1 += (S0_hi + S0_lo) W^T onto -U^T, with its own completion barrier
+            // descriptors of the tiles; a step inside a tile adds its bytes / 16
+            const uint64_t desc_w = smem_desc(smem_a + kOffW + (c & 1) * kTileBytes, 16, 1024, SWZ_128B);
+            const uint64_t desc_k = smem_desc(smem_a + kOffK + (c % kRing) * kTileBytes, 16, 1024, SWZ_128B), desc_q = desc_k + (kOffQ - kOffK) / 16;
+            const uint64_t desc_kt = smem_desc(smem_a + kOffK + (c % kRing) * kTileBytes, 8192, 1024, SWZ_128B);
+            // D1 = (S0_hi + S0_lo) W^T, the first half of the state's columns as soon as its copies are in place
 #pragma unroll
-                for (int part = 0; part < 2; ++part) {
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {
-                        const uint64_t bd = smem_desc(st_a + kOffW + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024, SWZ_128B);
-                        mma_f16_ts(tmem + kD1, tmem + (part == 0 ? kSA : kO2) + ks * 8, bd, idesc_kk64,
-                                   !no_u || part > 0 || ks > 0);
-                    }
-                }
-                mma_commit(&bar_d1);
-                if (!SO) {
-                    // O1 = (S0_hi + S0_lo) Q^T
+            for (int half = 0; half < 2; ++half) {
+                if (half == 0) handoff_wait<4>();
+                else handoff_wait<6>();
+                tc_fence_after_sync();
+                if (*fail == 0 && elect_one()) {
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
 #pragma unroll
-                        for (int ks = 0; ks < 8; ++ks) {
-                            const uint64_t bd = smem_desc(st_a + kOffQ + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024, SWZ_128B);
-                            mma_f16_ts(tmem + kO1, tmem + (part == 0 ? kSA : kO2) + ks * 8, bd, idesc_kk64, part > 0 || ks > 0);
-                        }
+                        for (int k4 = 0; k4 < 4; ++k4)
+                            mma_f16_ts(tm + kD1, tm + (part == 0 ? kSA : kSL) + half * 32 + k4 * 8, desc_w + (half * 8192 + k4 * 32) / 16,
+                                       part == 0 ? idesc_kk64 : idesc_kk64 | kNegA, half > 0 || part > 0 || k4 > 0);
+                    }
+                    if (half == 1) mma_commit(&bar_d1[c & 1]);
+                }
+                __syncwarp();
+            }
+            if (!SO) {
+                if (c > 0) handoff_wait<8>();  // the output warps have read O1, O2 of the chunk before
+                tc_fence_after_sync();
+                if (*fail == 0 && elect_one()) {
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        mma_f16_ss(tm + kPT, desc_k + ((ks >> 2) * 8192 + (ks & 3) * 32) / 16, desc_q + ((ks >> 2) * 8192 + (ks & 3) * 32) / 16,
+                                   idesc_pt, ks > 0);
+                    mma_commit(&bar_pt);
+                    // O1 = (S0_hi + S0_lo) Q^T (no completion barrier of its own: the commit behind the output product covers it)
+#pragma unroll
+                    for (int part = 0; part < 2; ++part) {
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)
+                            mma_f16_ts(tm + kO1, tm + (part == 0 ? kSA : kSL) + ks * 8, desc_q + ((ks >> 2) * 8192 + (ks & 3) * 32) / 16,
+                                       part == 0 ? idesc_kk64 : idesc_kk64 | kNegA, part > 0 || ks > 0);
                     }
                 }
-                // (no completion barrier of its own: the commit behind the output product below covers it, and a wait
-                // costs the threads ~200 cycles even on a completed phase)
+                __syncwarp();
             }
-            __syncwarp();
-            // U_new^T (hi, lo; plain, scaled), P (hi, lo) and the decayed accumulator are in place
+            // the forms of U_new^T and the decayed accumulator are in place: S += (U_new^T exp(g_C - g_j)) K, hi + lo (the K tile as
+            // MN-major operand), one half of the state's columns after the other
             handoff_wait<5>();
             tc_fence_after_sync();
             if (*fail == 0 && elect_one()) {
-                if (!SO) {
-                    // O2 = U_new^T P^T = Uh Ph + Ul Ph + Uh Pl (K-dim = 64 tokens; the plain copy of tokens 16 ks.. sits
-                    // at columns 16 ks .. 16 ks + 7 of its region, the gate-scaled one at 16 ks + 8 ..)
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+#pragma unroll
+                    for (int part = 0; part < 2; ++part) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_f16_ts(tm + kSD + half * 64, tm + (part == 0 ? kD1 : kUL) + ks * 16 + 8, desc_kt + (half * 8192 + ks * 2048) / 16,
+                                       part == 0 ? idesc_mn64 : idesc_mn64 | kNegA, true);
+                    }
+                    mma_commit(&bar_su[c & 1][half]);
+                }
+            }
+            __syncwarp();
+            if (!SO) {
+                // O2 = U_new^T P^T = Uh Ph + Ul Ph + Uh Pl (K-dim = 64 tokens; the plain copy of tokens 16 ks.. sits
+                // at columns 16 ks .. 16 ks + 7 of its region, the gate-scaled one at 16 ks + 8 ..)
+                handoff_wait<7>();
+                tc_fence_after_sync();
+                if (*fail == 0 && elect_one()) {
 #pragma unroll
                     for (int part = 0; part < 3; ++part) {
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks) {
-                            const uint64_t bd = smem_desc(smem_a + kOffP + (part == 2 ? 8192 : 0) + ks * 256, 128, 1024, SWZ_NONE);
-                            mma_f16_ts(tmem + kO2, tmem + (part == 1 ? kPT : kD1) + ks * 16, bd,
-                                       idesc_mn64, part > 0 || ks > 0);
-                        }
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_f16_ts(tm + kO2, tm + (part == 1 ? kUL : kD1) + ks * 16, desc_p + ((part == 2 ? 8192 : 0) + ks * 256) / 16,
+                                       part == 0 ? idesc_mn64 : part == 1 ? idesc_mn64 | kNegA : idesc_mn64 | kNegB, part > 0 || ks > 0);
                     }
-                    mma_commit(&bar_o2);  // the output is finished while the state update still runs
+                    mma_commit(&bar_o2);
                 }
-                // S += (U_new^T exp(g_C - g_j)) K, hi + lo (the K tile as MN-major operand, N = 128)
-#pragma unroll
-                for (int part = 0; part < 2; ++part) {
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const uint64_t bd = smem_desc(st_a + kOffK + ks * 2048, 8192, 1024, SWZ_128B);
-                        mma_f16_ts(tmem + kSD, tmem + (part == 0 ? kD1 : kPT) + ks * 16 + 8, bd,
-                                   idesc_mn128, true);
-                    }
-                }
-                mma_commit(&bar_g2);
+                __syncwarp();
             }
-            __syncwarp();
-            // D1 and PT are only read by the products just issued, which the tensor pipe runs first: the
-            // state-independent products of the next chunk follow them directly
-            if (c + 1 < n_c) issue_pre(c + 1);
         }
         if (*fail != 0 && elect_one()) {  // products still in flight end before their operands go
             mma_commit(&bar_end);
             wait_bar(&bar_end, 0);
         }
         __syncwarp();
-    } else {
-        // ================= compute threads (512): four per TMEM lane
-        uint32_t par_pre = 0, par_d1 = 0, par_o2 = 0, par_g2 = 0;
-        // completion of an MMA group: every lane polls the mbarrier (no CTA-wide barrier on this path). A poll of a
-        // completed phase costs ~200 cycles whoever issues it; polling from lane 0 alone added a divergent branch and a
-        // shuffle, ~150 cycles more per wait.
-        auto wait_group = [&](uint64_t* bar, uint32_t& par) -> bool {
-            const bool good = wait_bar_warp(bar, par, fail);
-            if (!good) *fail = 1;
-            par ^= 1;
-            tc_fence_after_sync();
-            return good;
+    } else if (aux) {
+        // ================= output warps (eight, two per lane quadrant): P, the output tile and the norms, beside the chain of the state
+        // 1 / ||k||, 1 / ||q|| of chunk c into its table buffer: four warps the rows of K, four those of Q, two threads a row. (The sum does
+        // not care about the swizzle inside the row: eight neighbouring threads read eight different 16-byte pieces, free of bank
+        // conflicts.) Two chunks ahead: the table threads and the chain want them before this chunk is done, and here is where warps wait.
+        auto put_norms = [&](int c) -> bool {
+            if (!NRM || c >= n_c) return true;
+            if (SO && warp >= (kChain + kAux / 2) / 32) {  // (no queries)
+                warp_arrive(&bar_nrm[c & 3]);
+                return true;
+            }
+            if (!wait_for(&bar_kq[c % kRing], (c / kRing) & 1)) return false;
+            const int at = tid - kChain, r = (at >> 1) & 63, half = at & 1;
+            const uint8_t* rp = smem + (at < kAux / 2 ? kOffK : kOffQ) + (c % kRing) * kTileBytes + half * 8192 + r * 128;
+            float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint4 w4 = *reinterpret_cast<const uint4*>(rp + (((i + lane) & 7) << 4));
+                bf16_square_add(w4.x, a[0], a[1]);
+                bf16_square_add(w4.y, a[2], a[3]);
+                bf16_square_add(w4.z, a[0], a[1]);
+                bf16_square_add(w4.w, a[2], a[3]);
+            }
+            float sum = (a[0] + a[1]) + (a[2] + a[3]);
+            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
+            if (half == 0) gtab[(c & 3) * kTab + (at < kAux / 2 ? 192 : 256) + r] = rsqrtf(fmaxf(sum, 1e-30f));
+            warp_arrive(&bar_nrm[c & 3]);
+            return true;
         };
-        // ---- constant A operand -I, initial state, and its bf16 copies (hi in kSA, lo in kO2)
-        {
-            uint32_t r[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int col = h * 16 + i;  // packed column: features 2 col, 2 col + 1
-                r[i] = (col == (t >> 1)) ? ((t & 1) ? 0xBF800000u : 0x0000BF80u) : 0u;
+        int taken = 0;  // hand-offs this warp has made (7, 8 of a chunk, in this order; no 8 for the last)
+        bool good = put_norms(0);
+        if (SO) {  // the norms only: of chunk c when the table of chunk c - 2 has been formed, which is behind the last reader of buffer c mod 4
+            for (int c = 1; good && NRM && c < n_c; ++c) {
+                good = (c < 2 || wait_for(&bar_tab[(c - 2) & 3], ((c - 2) >> 2) & 1)) && put_norms(c);
             }
-            tmem_st16(lane_base + kIA + h * 16, r);
-            // this thread's quarter of state row t: columns [32 h, 32 h + 32)
-            const float* s0 = (p.S_in != nullptr) ? p.S_in + (((long long)b * p.H_v + hv) * kD + t) * kD + h * 32 : nullptr;
+        } else {  // P is zero above its diagonal: the blocks that no thread writes below
+            uint4* pz = reinterpret_cast<uint4*>(smem + kOffP);
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {
-                uint32_t v[16], pk[8];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = (s0 != nullptr) ? __float_as_uint(__ldg(s0 + part * 16 + i)) : 0u;
-                tmem_st16(lane_base + kSD + h * 32 + part * 16, v);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) pk[i] = pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-                tmem_st8(lane_base + kSA + h * 16 + part * 8, pk);
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    pk[i] = pack_bf16x2(__uint_as_float(v[2 * i]) - bf16_lo(pk[i]), __uint_as_float(v[2 * i + 1]) - bf16_hi(pk[i]));
-                tmem_st8(lane_base + kO2 + h * 16 + part * 8, pk);
-            }
-            tmem_wait_st();
-            tc_fence_before_sync();
-            handoff_arrive<4>();
+            for (int i = 0; i < 4; ++i) pz[i * kAux + tid - kChain] = make_uint4(0u, 0u, 0u, 0u);
+            asm volatile("bar.sync 1, %0;" ::"n"(kAux) : "memory");
         }
-        int gave_up = 0;  // 1, 2, 3: a wait of chunk c ran out before hand-off 5, before 6, behind 6
-        asm volatile("bar.sync 1, %0;" ::"n"(kThreads + kTabThreads) : "memory");  // the gates of the first chunk
-        int c = 0;
-        for (; c < n_c; ++c) {
-            const float* se = gtab + (c % 3) * kTab;  // scale exp(g_i) / ||q_i||
-            const float* sf = se + 64;               // -exp(g_C - g_j) / ||k_j|| (D1 holds -U_new)
+        for (int c = 0; good && c < (SO ? 0 : n_c); ++c) {
+            const float* se = gtab + (c & 3) * kTab;  // scale exp(g_i) / ||q_i||
             const float* sg = se + 128;              // g_i (cumulative inside the chunk)
-            const float gC = sg[63];
             const int left = len - c * kC;
-            const bool short_chunk = VAR && left < kC;
-
-            // ---- decay of the accumulator, S <- exp(g_C) S0 (the products of this chunk read the bf16 copies)
-            {
-                const float dec = fast_exp2(gC * kLog2e);
-                uint32_t v[32];
-                tmem_ld32(lane_base + kSD + h * 32, v);
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * dec);
-                uint32_t w16[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) w16[i] = v[i];
-                tmem_st16(lane_base + kSD + h * 32, w16);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) w16[i] = v[16 + i];
-                tmem_st16(lane_base + kSD + h * 32 + 16, w16);
-            }
-            // ---- P_ij = exp(g_i - g_j) PT_ji for j <= i (hi + lo): this thread's token j and 8 columns i. (Keys and queries
-            // normalised here: 1 / ||k_j|| rides on U_new_j, 1 / ||q_i|| on the output.)
-            if (!SO && !wait_group(&bar_pre, par_pre)) { gave_up = 1; break; }
-            if (!SO) {
-                uint32_t d[8];
-                tmem_ld8_split32(lane_base + kPT + h * 8, d);
-                const int j = wq * 16 + (lane & 15), n8 = (lane >> 4) * 4 + h;  // columns i = 8 n8 ..
-                const float gj = sg[j] * kLog2e;
+            // ---- P_ij = exp(g_i - g_j) PT_ji for j <= i (hi + lo): this thread's token j and 16 or 8 columns i. (Keys and
+            // queries normalised here: 1 / ||k_j|| rides on P and on the scaled form of U_new_j, 1 / ||q_i|| on the output.)
+            if (!(good = wait_for(&bar_pt, c & 1))) break;  // (issued behind hand-off 4: the tables are there too)
+            tc_fence_after_sync();
+            const int j = wq * 16 + (lane & 15);
+            const float gj = sg[j] * kLog2e, rk = NRM ? sg[64 + j] : 1.f;
+            auto put_p = [&](const uint32_t* d, int i0) {  // columns i0 .. i0 + 7 of this thread's row j
                 float gi[8];
 #pragma unroll
                 for (int i4 = 0; i4 < 2; ++i4) {
-                    const float4 q4 = *reinterpret_cast<const float4*>(sg + n8 * 8 + i4 * 4);
+                    const float4 q4 = *reinterpret_cast<const float4*>(sg + i0 + i4 * 4);
                     gi[i4 * 4 + 0] = q4.x; gi[i4 * 4 + 1] = q4.y; gi[i4 * 4 + 2] = q4.z; gi[i4 * 4 + 3] = q4.w;
                 }
-                tmem_wait_ld();
                 uint32_t w[4], wl[4];
 #pragma unroll
                 for (int i2 = 0; i2 < 4; ++i2) {
                     float v[2];
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
-                        const float x = __uint_as_float(d[i2 * 2 + q]) * fast_exp2(fminf(fmaf(gi[i2 * 2 + q], kLog2e, -gj), 0.f));
-                        v[q] = (j <= n8 * 8 + i2 * 2 + q) ? x : 0.f;
+                        float x = __uint_as_float(d[i2 * 2 + q]) * fast_exp2(fminf(fmaf(gi[i2 * 2 + q], kLog2e, -gj), 0.f));
+                        if (NRM) x *= rk;
+                        v[q] = (j <= i0 + i2 * 2 + q) ? x : 0.f;
                     }
-                    w[i2] = pack_bf16x2(v[0], v[1]);
-                    wl[i2] = pack_bf16x2(v[0] - bf16_lo(w[i2]), v[1] - bf16_hi(w[i2]));
+                    split_neg(v[0], v[1], w[i2], wl[i2]);
                 }
-                // B operand [K-dim = j][N = i], MN-major, no swizzle: the 16-byte piece of row j for column group n8
-                *reinterpret_cast<uint4*>(smem + kOffP + n8 * 1024 + j * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-                *reinterpret_cast<uint4*>(smem + kOffP + 8192 + n8 * 1024 + j * 16) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-            }
-            // ---- U_new^T = -D1 as bf16 hi + lo, plain and gate-scaled (the sums over the tokens of a chunk telescope
-            // on correlated keys, so single bf16 copies cost 1e-2 there). This thread's 16 tokens are one k-step of the
-            // products that consume them: the hi halves are written over its own D1 columns (plain -> 16 h .. 16 h + 7,
-            // scaled -> 16 h + 8 ..), the lo halves at the same offsets of the PT region.
-            if (!wait_group(&bar_d1, par_d1)) { gave_up = 1; break; }
-            // (the four warps of a lane quadrant have read their columns of PT)
-            if (!SO) asm volatile("bar.sync %0, 128;" ::"r"(8 + wq) : "memory");
-            {
+                // B operand [K-dim = j][N = i], MN-major, no swizzle: the 16-byte piece of row j for a group of 8 columns
+                uint8_t* at = smem + kOffP + (i0 >> 3) * 1024 + j * 16;
+                *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(at + 8192) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+            };
+            if (wq < 2) {
                 uint32_t d[16];
-                tmem_ld16(lane_base + kD1 + h * 16, d);
+                tmem_ld16_split32(lane_base + kPT + h * 16, d);
                 tmem_wait_ld();
-                uint32_t hi[16], lo[16];
-#pragma unroll
-                for (int i = 0; i < 8; i += 2) {
-                    const ulonglong2 f4 = *reinterpret_cast<const ulonglong2*>(sf + h * 16 + 2 * i);
-                    ulonglong2 k4;
-                    if (NRM && !SO) k4 = *reinterpret_cast<const ulonglong2*>(sg + 64 + h * 16 + 2 * i);
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        float d0 = __uint_as_float(d[2 * (i + q)]), d1 = __uint_as_float(d[2 * (i + q) + 1]);
-                        if (short_chunk) {  // rows past the sequence's end hold another sequence's W, U
-                            if (h * 16 + 2 * (i + q) >= left) d0 = 0.f;
-                            if (h * 16 + 2 * (i + q) + 1 >= left) d1 = 0.f;
-                        }
-                        const f2 u = pair2(d0, d1);
-                        split_pair(mul2(u, q == 0 ? f4.x : f4.y), hi[8 + i + q], lo[8 + i + q]);
-                        if (!SO) split_pair(NRM ? mul2(u, q == 0 ? k4.x : k4.y) : pair2(-d0, -d1), hi[i + q], lo[i + q]);
-                        else hi[i + q] = lo[i + q] = 0u;  // (only the output product reads the plain form)
-                    }
-                }
-                tmem_st16(lane_base + kD1 + h * 16, hi);
-                tmem_st16(lane_base + kPT + h * 16, lo);
+                put_p(d, (lane >> 4) * 32 + h * 16);
+                put_p(d + 8, (lane >> 4) * 32 + h * 16 + 8);
+            } else if (wq == 2 || h == 1) {  // rows j from 32 on: columns from 32 on, rows from 48 on: columns from 48 on; zeros elsewhere stay as written once
+                uint32_t d[8];
+                tmem_ld8_split8(lane_base + kPT + 32 + h * 16, d);
+                tmem_wait_ld();
+                put_p(d, 32 + h * 16 + (lane >> 4) * 8);
             }
             fence_proxy_async_smem();
-            tmem_wait_st();
             tc_fence_before_sync();
-            handoff_arrive<5>();
-            if (!SO) {
-                // The storing warp has released the PREVIOUS chunk's staging buffer (polled here, in the shadow of the
-                // output product; the store was issued most of a chunk ago). That is one chunk later than this chunk's
-                // own buffer needs (chunk c - 2 used it, and the stores are read in order), but it also says that the
-                // storing warp has taken the previous chunk's hand-off: the threads must not arrive on that hardware
-                // barrier a second time before it has, however long a store may be held up.
-                if (c >= 1 && !wait_bar_warp(&bar_stg[(c - 1) & 1], ((c - 1) >> 1) & 1, fail)) { *fail = 1; gave_up = 2; break; }
-                // ---- O^T = scale (exp(g_i) O1 + O2), in fragments of 8 x 8: this warp's 32 features x 16 tokens, transposed
-                // on the way to the staged tile (O1 is complete with O2: products finish in the order they were issued)
-                if (!wait_group(&bar_o2, par_o2)) { gave_up = 2; break; }
-                {
-                    const int t2 = h * 16 + 2 * (lane & 3);
-                    const float2 e0 = *reinterpret_cast<const float2*>(se + t2), e1 = *reinterpret_cast<const float2*>(se + t2 + 8);
-                    float2 q0 = make_float2(p.scale, p.scale), q1 = q0;
-                    if (NRM) {
-                        q0 = *reinterpret_cast<const float2*>(se + 256 + t2);
-                        q1 = *reinterpret_cast<const float2*>(se + 256 + t2 + 8);
-                    }
-                    const int tok = h * 16 + ((lane >> 4) << 3) + (lane & 7);  // row of the staged tile this lane addresses
+            handoff_arrive<7>();
+            ++taken;
+            if (c == 0 && !(good = put_norms(1))) break;
+            if (!(good = put_norms(c + 2))) break;
+            // ---- O^T = scale (exp(g_i) O1 + O2), in fragments of 8 x 8: this warp's 32 features x 32 tokens, transposed
+            // on the way to the staged tile (O1 is complete with O2: products finish in the order they were issued)
+            if (!(good = wait_for(&bar_o2, c & 1))) break;
+            tc_fence_after_sync();
+            uint32_t m[2][2][4];
 #pragma unroll
-                    for (int lh = 0; lh < 2; ++lh) {
-                        uint32_t a[8], d[8];
-                        tmem_ld_frag(lane_base + (static_cast<uint32_t>(lh * 16) << 16) + kO1 + h * 16, a);
-                        tmem_ld_frag(lane_base + (static_cast<uint32_t>(lh * 16) << 16) + kO2 + h * 16, d);
-                        tmem_wait_ld();
-                        uint32_t m[4];
+            for (int tg = 0; tg < 2; ++tg) {
+                uint32_t a[2][8], d[2][8];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const float2 e = k < 2 ? e0 : e1, q = k < 2 ? q0 : q1;
-                            m[k] = pack_bf16x2(fmaf(__uint_as_float(a[2 * k]), e.x, __uint_as_float(d[2 * k]) * q.x),
-                                               fmaf(__uint_as_float(a[2 * k + 1]), e.y, __uint_as_float(d[2 * k + 1]) * q.y));
-                        }
-                        const int fb = wq * 4 + lh * 2 + ((lane >> 3) & 1);  // block of 8 features
-                        const uint32_t at = smem_a + kOffO + (c & 1) * kTileBytes + (fb >> 3) * 8192 + tok * 128 + (((fb & 7) ^ (tok & 7)) << 4);
-                        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(m[0]), "r"(m[1]),
-                                     "r"(m[2]), "r"(m[3])
-                                     : "memory");
+                for (int lh = 0; lh < 2; ++lh) {
+                    tmem_ld_frag(lane_base + (static_cast<uint32_t>(lh * 16) << 16) + kO1 + h * 32 + tg * 16, a[lh]);
+                    tmem_ld_frag(lane_base + (static_cast<uint32_t>(lh * 16) << 16) + kO2 + h * 32 + tg * 16, d[lh]);
+                }
+                const int t2 = h * 32 + tg * 16 + 2 * (lane & 3);
+                const f2 e[2] = {*reinterpret_cast<const f2*>(se + t2), *reinterpret_cast<const f2*>(se + t2 + 8)};
+                f2 q[2] = {pair2(p.scale, p.scale), pair2(p.scale, p.scale)};
+                if (NRM) {
+                    q[0] = *reinterpret_cast<const f2*>(se + 256 + t2);
+                    q[1] = *reinterpret_cast<const f2*>(se + 256 + t2 + 8);
+                }
+                tmem_wait_ld();
+#pragma unroll
+                for (int lh = 0; lh < 2; ++lh) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const f2 o1 = pair2(__uint_as_float(a[lh][2 * k]), __uint_as_float(a[lh][2 * k + 1]));
+                        const f2 o2 = pair2(__uint_as_float(d[lh][2 * k]), __uint_as_float(d[lh][2 * k + 1]));
+                        m[tg][lh][k] = pack_pair(fma2(o1, e[k >> 1], mul2(o2, q[k >> 1])));
                     }
                 }
-                // the tile goes to the storing warp: no compute thread waits for the others here
-                fence_proxy_async_smem();
-                handoff_arrive<6>();
             }
-            // ---- bf16 copies (hi, lo) of the new state for the next chunk's products; the lo half goes where O2 was
-            // (this thread has read its O2 columns above)
-            if (!wait_group(&bar_g2, par_g2)) { gave_up = 3; break; }
-            {
-                uint32_t v[32], pk[16];
-                tmem_ld32(lane_base + kSD + h * 32, v);
-                tmem_wait_ld();
-                uint32_t lo[16];
+            tc_fence_before_sync();
+            if (c + 1 < n_c) {  // the columns and the tables of this chunk are read
+                handoff_arrive<8>();
+                ++taken;
+            }
+            if (c >= 2 && !(good = wait_for(&bar_stg[c & 1], ((c - 2) >> 1) & 1))) break;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) split_pair(pair2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), pk[i], lo[i]);
-                tmem_st16(lane_base + kSA + h * 16, pk);
-                tmem_st16(lane_base + kO2 + h * 16, lo);
-                tmem_wait_st();
-                tc_fence_before_sync();
-                handoff_arrive<4>();
+            for (int tg = 0; tg < 2; ++tg) {
+                const int tok = h * 32 + tg * 16 + ((lane >> 4) << 3) + (lane & 7);  // row of the staged tile this lane addresses
+#pragma unroll
+                for (int lh = 0; lh < 2; ++lh) {
+                    const int fb = wq * 4 + lh * 2 + ((lane >> 3) & 1);  // block of 8 features
+                    const uint32_t at = smem_a + kOffO + (c & 1) * kTileBytes + (fb >> 3) * 8192 + tok * 128 + (((fb & 7) ^ (tok & 7)) << 4);
+                    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(m[tg][lh][0]),
+                                 "r"(m[tg][lh][1]), "r"(m[tg][lh][2]), "r"(m[tg][lh][3])
+                                 : "memory");
+                }
             }
-            if (!SO && short_chunk) {
-                // only the rows of real tokens leave, 16 bytes per thread and step, from the staged (swizzled) tile
-                asm volatile("bar.sync 1, 512;" ::: "memory");  // (last chunk of a packed sequence only)
-                for (int q = tid; q < left * 16; q += kThreads) {
-                    const int tok = q >> 4, ch = q & 15;  // 16-byte piece ch of the token's 256-byte row
-                    const uint4 v = *reinterpret_cast<const uint4*>(smem + kOffO + (c & 1) * kTileBytes + (ch >> 3) * 8192 +
-                                                                    tok * 128 + (((ch & 7) ^ (tok & 7)) << 4));
-                    *reinterpret_cast<uint4*>(p.O + (grow0 + (long long)(c * kC + tok) * gstep) * kD + ch * 8) = v;
+            if (VAR && left < kC) {
+                // only the rows of real tokens leave, from the staged (swizzled) tile: every warp its own 32 tokens x 64 bytes
+                __syncwarp();
+#pragma unroll
+                for (int q = lane; q < 128; q += 32) {
+                    const int tok = h * 32 + (q >> 2), ch = wq * 4 + (q & 3);  // 16-byte piece ch of the token's 256-byte row
+                    if (tok < left) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(smem + kOffO + (c & 1) * kTileBytes + (ch >> 3) * 8192 +
+                                                                        tok * 128 + (((ch & 7) ^ (tok & 7)) << 4));
+                        *reinterpret_cast<uint4*>(p.O + (grow0 + (long long)(c * kC + tok) * gstep) * kD + ch * 8) = v;
+                    }
+                }
+            }
+            // the tile goes to the storing warp
+            fence_proxy_async_smem();
+            warp_arrive(&bar_ost[c & 1]);
+        }
+        if (!SO && !good) {  // a bounded wait ran out (s_fail is set): the remaining hand-offs, as waits
+            for (; taken < 2 * n_c - 1; ++taken) {
+                if ((taken & 1) == 0) handoff_wait<7>();
+                else handoff_wait<8>();
+            }
+        }
+    } else {
+        // ================= chain warps (eight, two per lane quadrant): the state's copies, its decay, U_new
+        const uint32_t row = lane_base;
+        const int tq = h * 32 + 2 * (lane & 3);  // this thread's tokens: tq + 8 k and the next one
+        // What U_new of a chunk needs beside D1: U in the fragments in which D1 is read (tokens tq + 16 ks + 8 x and the next one of
+        // feature lane / 4 of each block of 8), the tokens' factors exp(g_C - g_j) / ||k_j||, and the decay exp(g_C) of the state. Fetched
+        // while the state update of the chunk before runs: behind D1 the products read shared memory at up to its full rate.
+        uint32_t u[2][2][4];
+        f2 f[2][2], dec2;
+        auto prefetch = [&](int c) -> bool {
+            if (!(wait_for(&bar_tab[c & 3], (c >> 2) & 1) && wait_for(&bar_u[c & 1], (c >> 1) & 1))) return false;
+            const float* sf = gtab + (c & 3) * kTab + 64;
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks) {
+#pragma unroll
+                for (int lh = 0; lh < 2; ++lh) {
+                    const int tok = h * 32 + 16 * ks + ((lane >> 4) << 3) + (lane & 7), fb = wq * 4 + lh * 2 + ((lane >> 3) & 1);
+                    const uint32_t at = smem_a + kOffU + (c & 1) * kTileBytes + (fb >> 3) * 8192 + tok * 128 + (((fb & 7) ^ (tok & 7)) << 4);
+                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(u[ks][lh][0]), "=r"(u[ks][lh][1]), "=r"(u[ks][lh][2]), "=r"(u[ks][lh][3])
+                                 : "r"(at)
+                                 : "memory");
+                }
+#pragma unroll
+                for (int x = 0; x < 2; ++x) f[ks][x] = *reinterpret_cast<const f2*>(sf + tq + 16 * ks + 8 * x);
+            }
+            const float dec = fast_exp2(sf[64 + 63] * kLog2e);
+            dec2 = pair2(dec, dec);
+            return true;
+        };
+        // bf16 copies (hi, -lo) of 32 state columns
+        auto put_copies = [&](const uint32_t (&v)[32], int half) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t hi[8], lo[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) split_neg(__uint_as_float(v[16 * q + 2 * i]), __uint_as_float(v[16 * q + 2 * i + 1]), hi[i], lo[i]);
+                tmem_st8(row + kSA + half * 32 + h * 16 + q * 8, hi);
+                tmem_st8(row + kSL + half * 32 + h * 16 + q * 8, lo);
+            }
+            tmem_wait_st();
+            tc_fence_before_sync();
+        };
+        // the accumulator for the coming chunk, S <- exp(g_C) S0 (its products read the bf16 copies)
+        auto put_decayed = [&](uint32_t (&v)[32], int half) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const f2 x = mul2(pair2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), dec2);
+                v[2 * i] = static_cast<uint32_t>(x);
+                v[2 * i + 1] = static_cast<uint32_t>(x >> 32);
+            }
+            tmem_st32(row + kSD + half * 64 + h * 32, v);
+        };
+        int taken = 0;  // hand-offs this warp has made (4, 6, 5 of a chunk, in this order)
+        bool good = true;
+        {
+            // this thread's part of state row t: columns [64 half + 32 h, + 32)
+            const float* s0 = (p.S_in != nullptr) ? p.S_in + (((long long)b * p.H_v + hv) * kD + t) * kD + h * 32 : nullptr;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t v[32];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float4 x = (s0 != nullptr) ? __ldg(reinterpret_cast<const float4*>(s0 + half * 64) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[4 * i] = __float_as_uint(x.x); v[4 * i + 1] = __float_as_uint(x.y);
+                    v[4 * i + 2] = __float_as_uint(x.z); v[4 * i + 3] = __float_as_uint(x.w);
+                }
+                tmem_st32(row + kSD + half * 64 + h * 32, v);
+                if (n_c == 0) continue;  // no tokens: the state is handed on
+                put_copies(v, half);
+                if (half == 0) handoff_arrive<4>();
+                else handoff_arrive<6>();
+                ++taken;
+            }
+            tmem_wait_st();
+            if (n_c > 0 && (good = prefetch(0))) {
+#pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t v[32];
+                    tmem_ld32(row + kSD + half * 64 + h * 32, v);
+                    tmem_wait_ld();
+                    put_decayed(v, half);
                 }
             }
         }
-        if (gave_up != 0) {
-            // A bounded wait ran out (s_fail is set): this warp's remaining barriers of chunk c and of the chunks behind it, in
-            // the order of the loop above and as waits, so that no generation counts it twice.
-            for (; c < n_c; ++c, gave_up = 1) {
-                if (gave_up < 2) {
-                    if (!SO) asm volatile("bar.sync %0, 128;" ::"r"(8 + wq) : "memory");
-                    handoff_wait<5>();
-                }
-                if (!SO && gave_up < 3) {
-                    // (it will: this warp has arrived there, the others arrive or wait there too; bounded as every wait)
-                    const long long t0 = clock64();
-                    while (__any_sync(0xFFFFFFFFu, *reinterpret_cast<volatile int*>(&s_taken) < c && clock64() - t0 < 2000000000LL)) {
+        for (int c = 0; good && c < n_c; ++c) {
+            const int left = len - c * kC;
+            const bool short_chunk = VAR && left < kC;
+            // ---- U_new^T = U^T - D1 as bf16 hi - lo, plain and gate-scaled (the sums over the tokens of a chunk telescope
+            // on correlated keys, so single bf16 copies cost 1e-2 there). 16 tokens are one k-step of the
+            // products that consume them: the hi halves are written over their own D1 columns (plain -> 16 ks .. 16 ks + 7,
+            // scaled -> 16 ks + 8 ..), the lo halves at the same offsets of a region of their own.
+            if (!(good = wait_for(&bar_d1[c & 1], (c >> 1) & 1))) break;
+            tc_fence_after_sync();
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks) {
+                uint32_t d[2][8];
+#pragma unroll
+                for (int lh = 0; lh < 2; ++lh) tmem_ld_frag(row + (static_cast<uint32_t>(lh * 16) << 16) + kD1 + h * 32 + ks * 16, d[lh]);
+                tmem_wait_ld();
+#pragma unroll
+                for (int lh = 0; lh < 2; ++lh) {
+                    uint32_t hi[8], lo[8];
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+#pragma unroll
+                        for (int fb = 0; fb < 2; ++fb) {
+                            const uint32_t w = (SO && no_u) ? 0u : u[ks][lh][2 * x + fb];
+                            float u0 = bf16_minus<0>(w, __uint_as_float(d[lh][4 * x + 2 * fb]));
+                            float u1 = bf16_minus<1>(w, __uint_as_float(d[lh][4 * x + 2 * fb + 1]));
+                            if (short_chunk) {  // rows past the sequence's end hold another sequence's W, U
+                                if (tq + 16 * ks + 8 * x >= left) u0 = 0.f;
+                                if (tq + 16 * ks + 8 * x + 1 >= left) u1 = 0.f;
+                            }
+                            split_neg(mul2(pair2(u0, u1), f[ks][x]), hi[4 + 2 * x + fb], lo[4 + 2 * x + fb]);
+                            if (!SO) split_neg(u0, u1, hi[2 * x + fb], lo[2 * x + fb]);
+                            else hi[2 * x + fb] = lo[2 * x + fb] = 0u;  // (only the output product reads the plain form)
+                        }
                     }
-                    handoff_wait<6>();
+                    const uint32_t at = row + (static_cast<uint32_t>(lh * 16) << 16) + h * 32 + ks * 16;
+                    tmem_st_frag16(at + kD1, hi);
+                    tmem_st_frag16(at + kUL, lo);
                 }
-                if (c + 1 < n_c) handoff_wait<4>();
-                if (VAR && !SO && len - c * kC < kC) asm volatile("bar.sync 1, 512;" ::: "memory");
             }
-            gave_up = 1;
+            tmem_wait_st();
+            tc_fence_before_sync();
+            handoff_arrive<5>();
+            ++taken;
+            if (c + 1 < n_c) {
+                if (!(good = prefetch(c + 1))) break;
+                // ---- bf16 copies (hi, -lo) of the new state for the next chunk's products, and its decay
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    if (!(good = wait_for(&bar_su[c & 1][half], (c >> 1) & 1))) break;
+                    tc_fence_after_sync();
+                    uint32_t v[32];
+                    tmem_ld32(row + kSD + half * 64 + h * 32, v);
+                    tmem_wait_ld();
+                    put_copies(v, half);
+                    if (half == 0) handoff_arrive<4>();
+                    else handoff_arrive<6>();
+                    ++taken;
+                    put_decayed(v, half);
+                }
+                if (!good) break;
+            } else {
+                good = wait_for(&bar_su[c & 1][1], (c >> 1) & 1);
+                tc_fence_after_sync();
+            }
+        }
+        if (!good) {
+            // A bounded wait ran out (s_fail is set): this warp's remaining hand-offs, as waits, so that no generation counts it twice.
+            for (; taken < 3 * n_c; ++taken) {
+                if (taken % 3 == 0) handoff_wait<4>();
+                else if (taken % 3 == 1) handoff_wait<6>();
+                else handoff_wait<5>();
+            }
         }
         // ---- final state
         // (the run's place among the states is formed again here: it is not held over the chunks)
         const int seq = ORD ? *reinterpret_cast<volatile int*>(&s_seq) : static_cast<int>(blockIdx.x / p.H_v);
-        if (gave_up == 0 && p.S_out != nullptr && seq >= p.out_from) {
+        if (good && p.S_out != nullptr && seq >= p.out_from) {
             float* so = p.S_out + (((long long)(seq - p.out_from) * p.H_v + blockIdx.x % p.H_v) * kD + t) * kD + h * 32;
-            uint32_t v[32];
-            tmem_ld32(lane_base + kSD + h * 32, v);
-            tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                *reinterpret_cast<float4*>(so + i * 4) =
-                    make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]),
-                                __uint_as_float(v[4 * i + 3]));
+            for (int half = 0; half < 2; ++half) {
+                uint32_t v[32];
+                tmem_ld32(row + kSD + half * 64 + h * 32, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    *reinterpret_cast<float4*>(so + half * 64 + i * 4) =
+                        make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]),
+                                    __uint_as_float(v[4 * i + 3]));
+            }
         }
     }
     tc_fence_before_sync();

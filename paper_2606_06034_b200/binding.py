@@ -497,9 +497,9 @@ def chunk_state_output(Q, K, W_gated, U, g, C, scale=1.0, S_in=None, *, want_sta
 
 def _segments_pay(T, C, segments):
     """Whether the segmented state passing is the faster one: its four launches cost about 35 + 3 P us more than a plain
-    one and its two passes 4.5 / P us a chunk against 2.7 (measured back to back, 1 to 64 heads: with P = 8 the lines cross
-    at 26 chunks, 24 chunks 74 us plain and 82 segmented, 32 chunks 95 and 86; with P = 3 at 34, with P = 2 at 90)."""
-    return segments > 1 and (T // C) * (2.7 - 4.5 / segments) > 35 + 3 * segments
+    one and its two passes 3.75 / P us a chunk against 2.0 (measured back to back: 64 heads, 256 chunks, P = 2: 582 us plain
+    and 689 segmented when the passes took 2.2 each)."""
+    return segments > 1 and (T // C) * (2.0 - 3.75 / segments) > 35 + 3 * segments
 
 
 def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_seqlens=None, token_major=True,

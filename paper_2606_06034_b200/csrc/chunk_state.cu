@@ -337,6 +337,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         tmem_alloc(&tmem_base_s, kTmemCols);
         tmem_relinquish();
     }
+    grid_dependency_wait();  // (the set-up above runs beside the end of the kernel before; W and U are its output)
     if (ORD && producer) {
         // longest sequences first: the CTAs with block index k H_v .. take the sequence of rank k
         const int rank = static_cast<int>(blockIdx.x / p.H_v);
@@ -1234,9 +1235,9 @@ int launch_chunk_state(const ProblemS& q, cudaStream_t stream) {
                 : var        ? (nrm ? chunk_state_kernel<true, false, true, false> : chunk_state_kernel<true, false, false, false>)
                              : (nrm ? chunk_state_kernel<false, false, true, false> : chunk_state_kernel<false, false, false, false>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GDN_ERR_LAUNCH;
-    kern<<<static_cast<int>(n_cta), kThreads + 64 + kTabThreads, smem, stream>>>(mQ, mK, mW, mU, mO, prm);
+    if (!launch_behind(kern, dim3(static_cast<unsigned>(n_cta)), kThreads + 64 + kTabThreads, smem, stream, mQ, mK, mW, mU, mO, prm)) return GDN_ERR_LAUNCH;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_LAUNCH;
+    return GDN_OK;
 }
 
 }  // namespace gdn

@@ -479,6 +479,7 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const int warp = tid >> 5;
     const int lane = tid & 31;
 
+    if constexpr (EX == 1 || EX == 3) launch_dependents();  // (the layer call's state passing follows: it waits for this kernel's end itself)
     if (tid == 0) {
         mbar_init(&bar_k, 1);
         mbar_init(&bar_v, 1);

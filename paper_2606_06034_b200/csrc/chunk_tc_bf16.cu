@@ -449,7 +449,7 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     constexpr int CPT = HC / 8;    // packed chunks owned by this thread
     constexpr int CPTF = HC / 4;   // fp32 chunks owned by this thread
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);  // (an offset: the compiler goes on to know it as shared memory)
     uint8_t* sK = smem + L::kK;
     uint8_t* sV = smem + L::kV;
     uint8_t* sEB = smem + L::kEB;
@@ -668,15 +668,14 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if (blockIdx.x < n_tiles && !(kRowHalf && (p.flags & GDN_FLAG_LAYOUT_BTHD) && (threadIdx.x >> 7) == 1))
         fetch_row(pos_next, bi_next, gi_next, gtok_next);
 
-    for (uint32_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+    for (uint32_t rem = blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u; rem > 0 && ok; --rem) {  // tiles left for this CTA
         // The tile's coordinates are only needed by the stores at its end. With the optional layouts they are six values:
         // those instantiations keep the tile's position (three) and form the coordinates there.
         const TilePos pos_cur = pos_next;
         TileCoord tc;
         if constexpr (EX == 0) tc = tile_coord<EX>(pos_next, p);
         tile_advance<EX>(pos_next, p);
-        const uint32_t next = tile + gridDim.x;
-        const bool has_next = next < n_tiles;
+        const bool has_next = rem > 1;
 
         float bi = bi_next;  // loaded during the previous tile
         float gi_ = gi_next;
@@ -702,9 +701,10 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             const int first = wq - (wq % kWarpsPerChunk);
             for (int w = first; w < wq; ++w) gi_ += swt[w];
         }
-        if (C == 64 && warp == 0 && has_next && !(EX && f_var) && elect_one()) {
+        if (C == 64 && EX == 0 && warp == 0 && has_next && elect_one()) {
             // The next tile's K can only land in shared memory once this tile's W products are done with the buffer,
-            // which leaves its load little time before the next Gram product wants it: ask for it in L2 now.
+            // which leaves its load little time before the next Gram product wants it: ask for it in L2 now. (With the optional
+            // layouts that costs 28 bytes of spill: 8 x 4096 tokens of the layer call 698 us with it, 680 without.)
             const TileCoord nc = tile_coord<EX>(pos_next, p);
             tma_prefetch_l2_3d(&tmK, nc.kx, nc.t0, nc.kz);
             tma_prefetch_l2_3d(&tmK, nc.kx + 64, nc.t0, nc.kz);

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 chunk_tc_int16_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ ParamsI16 p) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);  // (an offset: the compiler goes on to know it as shared memory)
     uint8_t* sK16 = smem + kOffK16;
     uint8_t* sV16 = smem + kOffV16;
     uint8_t* sPh = smem + kOffPh;

@@ -218,7 +218,7 @@ chunk_tc_int8_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
                      const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmU,
                      const __grid_constant__ CUtensorMap tmT, const __grid_constant__ ParamsI8 p) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);  // (an offset: the compiler goes on to know it as shared memory)
     uint8_t* sK = smem + kOffK;
     uint8_t* sV = smem + kOffV;
     uint8_t* sEB = smem + kOffEB;
@@ -1018,7 +1018,7 @@ __global__ void __launch_bounds__(kMThreads, 1)
 int8_merge128_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                      const __grid_constant__ ParamsI8 p) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);  // (an offset: the compiler goes on to know it as shared memory)
     uint8_t* sK = smem + kMOffK;
     uint8_t* sV = smem + kMOffV;
     uint8_t* sEB = smem + kMOffEB;

@@ -512,7 +512,9 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
 
-    const int N = p.N, S = p.S;
+    // (S is known where the doubling form was chosen. As a constant it saves a register: chunks of 128 107 -> 101 us without a spill, layer call
+    // of 8 x 4096 tokens 662 -> 641; the default instantiation's code came out 1 % slower with it)
+    const int N = p.N, S = DBL != 0 && (MERGE || EX != 0) ? DBL : p.S;
     // width of the band kept in fp32 (lb[]): the order N, or all of NB for forward substitution
     const int n_band = (MODE == INV_NEUMANN) ? N : NB;
     const uint32_t n_tiles = static_cast<uint32_t>(p.n_tiles);
@@ -701,10 +703,12 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             const int first = wq - (wq % kWarpsPerChunk);
             for (int w = first; w < wq; ++w) gi_ += swt[w];
         }
-        if (C == 64 && EX == 0 && warp == 0 && has_next && elect_one()) {
+        if (C == 64 && EX == 0 && !PERM && !MERGE && warp == 0 && has_next && elect_one()) {
             // The next tile's K can only land in shared memory once this tile's W products are done with the buffer,
-            // which leaves its load little time before the next Gram product wants it: ask for it in L2 now. (With the optional
-            // layouts that costs 28 bytes of spill: 8 x 4096 tokens of the layer call 698 us with it, 680 without.)
+            // which leaves its load little time before the next Gram product wants it: ask for it in L2 now. Only in the default
+            // form (4 x 16 heads x 4096 tokens 79.7 us with, 80.5 without): the M = 64 form for large launches loses by it (stress 4643 and
+            // 4520 us), chunks of 128 too (107 and 101), and with the optional layouts it costs 28 bytes of spill (8 x 4096 tokens of
+            // the layer call 698 and 680).
             const TileCoord nc = tile_coord<EX>(pos_next, p);
             tma_prefetch_l2_3d(&tmK, nc.kx, nc.t0, nc.kz);
             tma_prefetch_l2_3d(&tmK, nc.kx + 64, nc.t0, nc.kz);

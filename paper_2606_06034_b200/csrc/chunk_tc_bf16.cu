@@ -100,6 +100,31 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
+// Two packed fp32: one instruction for two elements (the same roundings). In the A-build, the sums of the levels and the scaling of the W / U
+// operands: 4 x 16 heads x 4096 tokens 77.5 -> 76.8 us, chunks of 128 100.9 -> 99.9, layer call of 8 x 4096 tokens 636 -> 627.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pair2(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpair2(f2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 __device__ __forceinline__ void compute_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // bounded mbarrier wait: polls, and every 1024 polls compares the clock with a budget of about a second
@@ -313,7 +338,10 @@ __device__ __forceinline__ void build_wu_operands(uint32_t lane_base, uint32_t b
 #pragma unroll
     for (int i = 0; i < PCH / 2; ++i) {
         const float4 bb = lds128f(sb_a + i * 16);
-        const uint32_t w0 = pack_bf16x2(a[4 * i] * bb.x, a[4 * i + 1] * bb.y), w1 = pack_bf16x2(a[4 * i + 2] * bb.z, a[4 * i + 3] * bb.w);
+        float p0, p1, p2, p3;
+        unpair2(mul2(pair2(a[4 * i], a[4 * i + 1]), pair2(bb.x, bb.y)), p0, p1);
+        unpair2(mul2(pair2(a[4 * i + 2], a[4 * i + 3]), pair2(bb.z, bb.w)), p2, p3);
+        const uint32_t w0 = pack_bf16x2(p0, p1), w1 = pack_bf16x2(p2, p3);
         pk[2 * i] = (KEEP ? (w0 & keep[2 * i]) : w0) | bp[2 * i];
         pk[2 * i + 1] = (KEEP ? (w1 & keep[2 * i + 1]) : w1) | bp[2 * i + 1];
     }
@@ -811,6 +839,19 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     const float4 rq = sr4[j4];
                     rj[0] = rq.x; rj[1] = rq.y; rj[2] = rq.z; rj[3] = rq.w;
                 }
+                if constexpr (C == 64) {
+                    // (see below: entries on and above the diagonal only have to be finite)
+#pragma unroll
+                    for (int q = 0; q < 4; q += 2) {
+                        const int jl = j4 * 4 + q;
+                        float x0, x1;
+                        unpair2(fma2(pair2(gj[q], gj[q + 1]), pair2(-kLog2e, -kLog2e), pair2(gs, gs)), x0, x1);
+                        f2 v = mul2(mul2(pair2(nbi, nbi), pair2(fast_exp2(fminf(x0, 64.f)), fast_exp2(fminf(x1, 64.f)))), pair2(a[jl], a[jl + 1]));
+                        if (f_l2) v = mul2(v, pair2(rj[q], rj[q + 1]));
+                        unpair2(v, a[jl], a[jl + 1]);
+                    }
+                    continue;
+                }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int jl = j4 * 4 + q;
@@ -1292,7 +1333,9 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                                 for (int j = 0; j < 16; ++j) a[hh * 16 + j] = __uint_as_float(d[j]);
                             } else if (lv != 2 || kFull) {
 #pragma unroll
-                                for (int j = 0; j < 16; ++j) a[hh * 16 + j] += __uint_as_float(d[j]);
+                                for (int j = 0; j < 16; j += 2)
+                                    unpair2(add2(pair2(a[hh * 16 + j], a[hh * 16 + j + 1]), pair2(__uint_as_float(d[j]), __uint_as_float(d[j + 1]))),
+                                            a[hh * 16 + j], a[hh * 16 + j + 1]);
                             }
                             if (lv < 3) {
                                 uint32_t pk[8];

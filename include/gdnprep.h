@@ -240,6 +240,17 @@ int gdn_chunk_state_output(const void* Q, const void* K, const void* W_gated, co
                            const float* S_in, void* O_out, float* S_out, unsigned flags, gdn_stream_t stream);
 
 /*
+ * The whole chunk-wise layer in one call: gdn_chunk_prepare_ex with flags | GDN_FLAG_W_GATED, default order and residual steps and no
+ * Tinv, then gdn_chunk_state_output on its W and U, on the same stream (the second launch is set up beside the end of the first).
+ *   W_tmp [like U_tmp, d_k wide], U_tmp [like V] bf16: scratch for W and U, free again when the call's work is complete.
+ * Shapes, flags (GDN_FLAG_G_RAW | GDN_FLAG_K_L2NORM | GDN_FLAG_LAYOUT_BTHD) and status codes are those of the two calls; the first
+ * status that is not GDN_OK is returned.
+ */
+int gdn_gated_delta_layer(const void* Q, const void* K, const void* V, const float* beta, const float* g, int B, int H_k, int H_v,
+                          int T, int C, int d_k, int d_v, float scale, const float* S_in, void* W_tmp, void* U_tmp, void* O_out,
+                          float* S_out, unsigned flags, gdn_stream_t stream);
+
+/*
  * gdn_chunk_state_output for packed variable-length sequences (the tensors gdn_chunk_prepare_varlen works on): sequence s
  * holds the tokens [cu_seqlens[s], cu_seqlens[s + 1]) and has its own state. One CTA per (sequence, value head) walks
  * the sequence's chunks from its first token; in a short last chunk the tokens past the end write nothing and the rows
@@ -264,7 +275,8 @@ int gdn_chunk_state_output_varlen(const void* Q, const void* K, const void* W_ga
  * segment's initial state; a second pass runs all segments in parallel with their output. Three passes' worth of
  * state work instead of one, on `segments` times as many SMs.
  *   Tensors as gdn_chunk_state_output with B = 1 (head-major [H,T,d], or [T,H,d] with GDN_FLAG_LAYOUT_BTHD).
- *   segments: 1 = the plain call; gdn_chunk_state_segments(H_v) proposes the count that fills the SMs in one wave.
+ *   segments: 1 = the plain call; gdn_chunk_state_segments(H_v) proposes the count that fills the SMs in one wave (1
+ *   where that would be 2, which is slower than the plain call).
  *   workspace: DEVICE memory of gdn_chunk_state_segmented_workspace(H_v, segments) bytes, 16-byte aligned, owned by
  *   the caller and free to reuse when the stream has passed the call.
  * The result differs from the plain call by fp32 rounding of the state recurrence only.

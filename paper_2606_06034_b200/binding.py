@@ -39,7 +39,7 @@ EXPORTS = (
     "gdn_chunk_prepare", "gdn_chunk_prepare_gqa", "gdn_chunk_prepare_ex", "gdn_chunk_prepare_varlen",
     "gdn_chunk_prepare_fwdsubst",
     "gdn_chunk_prepare_int8", "gdn_chunk_prepare_int16", "gdn_chunk_state_output", "gdn_chunk_state_output_varlen", "gdn_chunk_state_output_segmented",
-    "gdn_chunk_state_output_segmented_noalloc",
+    "gdn_chunk_state_output_segmented_noalloc", "gdn_gated_delta_layer",
     "gdn_chunk_state_segments", "gdn_chunk_state_segmented_workspace", "gdn_selftest_bounded_wait",
     "gdn_int8_lut_checksum",
     "gdn_device_status", "gdn_default_order", "gdn_default_residual_steps",
@@ -87,6 +87,9 @@ def load_library() -> ctypes.CDLL:
     lib.gdn_chunk_state_output_varlen.argtypes = [vp, vp, vp, vp, vp, vp, ip, ip, ip, ip, ip, ip, ip, ctypes.c_float, vp, vp, vp,
                                                   ctypes.c_uint, vp]
     lib.gdn_chunk_state_output_varlen.restype = ip
+    lib.gdn_gated_delta_layer.argtypes = [vp, vp, vp, vp, vp, ip, ip, ip, ip, ip, ip, ip, ctypes.c_float, vp, vp, vp, vp, vp,
+                                          ctypes.c_uint, vp]
+    lib.gdn_gated_delta_layer.restype = ip
     lib.gdn_chunk_state_segments.argtypes = [ip]
     lib.gdn_chunk_state_segments.restype = ip
     lib.gdn_chunk_state_segmented_workspace.argtypes = [ip, ip]
@@ -425,8 +428,10 @@ def chunk_state_output_segmented(Q, K, W_gated, U, g, C, scale=1.0, S_in=None, *
         H_k, T, d_k = K.shape
         H_v, _, d_v = U.shape
     lib = load_library()
-    if segments <= 0:
+    if segments <= 0:  # (two where the library proposes none though the first pass fits the SMs: who calls this wants segments)
         segments = int(lib.gdn_chunk_state_segments(H_v))
+        if segments == 1 and H_v <= torch.cuda.get_device_properties(U.device).multi_processor_count:
+            segments = 2
     need = int(lib.gdn_chunk_state_segmented_workspace(H_v, segments))
     if workspace is None and need > 0:
         workspace = torch.empty(need, dtype=torch.uint8, device=U.device)
@@ -497,9 +502,9 @@ def chunk_state_output(Q, K, W_gated, U, g, C, scale=1.0, S_in=None, *, want_sta
 
 def _segments_pay(T, C, segments):
     """Whether the segmented state passing is the faster one: its four launches cost about 35 + 3 P us more than a plain
-    one and its two passes 3.75 / P us a chunk against 2.0 (measured back to back: 64 heads, 256 chunks, P = 2: 582 us plain
-    and 689 segmented when the passes took 2.2 each)."""
-    return segments > 1 and (T // C) * (2.0 - 3.75 / segments) > 35 + 3 * segments
+    one and its two passes 4.5 / P us a chunk against 2.7. (Kernels as they are now, plain / segmented, us: P = 3, 37 chunks 72 / 74,
+    60 chunks 114 / 101; P = 8, 28 chunks 56 / 65, 40 chunks 77 / 68: the layer call also asks for more than 33 chunks.)"""
+    return segments > 1 and (T // C) * (2.7 - 4.5 / segments) > 35 + 3 * segments
 
 
 def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_seqlens=None, token_major=True,
@@ -514,14 +519,32 @@ def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_s
     if cu_seqlens is not None:
         W, U, _, _, _ = chunk_prepare_varlen(K, V, beta, g_raw, cu_seqlens, C, flags=flags | GDN_FLAG_W_GATED, want_tinv=False)
         return chunk_state_output_varlen(Q, K, W, U, g_raw, cu_seqlens, C, scale, S_in, want_state=want_state, flags=flags)
-    W, U, _ = chunk_prepare(K, V, beta, g_raw, C, flags=flags | GDN_FLAG_W_GATED, want_tinv=False)
-    H_v = V.shape[2] if token_major else V.shape[1]
-    if K.shape[0] == 1 and _segments_pay(V.shape[1] if token_major else V.shape[2], C, int(load_library().gdn_chunk_state_segments(H_v))):
-        # one long sequence per head and fewer heads than SMs: the segments of a sequence run in parallel
+    if token_major:
+        (B, T, H_k, d_k), (H_v, d_v) = K.shape, V.shape[2:]
+    else:
+        (B, H_k, T, d_k), H_v, d_v = K.shape, V.shape[1], V.shape[3]
+    # one long sequence per head and fewer heads than SMs: the segments of a sequence run in parallel
+    if B == 1 and T // C > 33 and _segments_pay(T, C, int(load_library().gdn_chunk_state_segments(H_v))):
+        W, U, _ = chunk_prepare(K, V, beta, g_raw, C, flags=flags | GDN_FLAG_W_GATED, want_tinv=False)
         O, S = chunk_state_output_segmented(Q[0], K[0], W[0], U[0], g_raw[0], C, scale, None if S_in is None else S_in[0],
                                             want_state=want_state, flags=flags)
         return O[None], (None if S is None else S[None])
-    return chunk_state_output(Q, K, W, U, g_raw, C, scale, S_in, want_state=want_state, flags=flags)
+    if K.dtype != torch.bfloat16 or K.numel() == 0 or V.numel() == 0:
+        W, U, _ = chunk_prepare(K, V, beta, g_raw, C, flags=flags | GDN_FLAG_W_GATED, want_tinv=False)
+        return chunk_state_output(Q, K, W, U, g_raw, C, scale, S_in, want_state=want_state, flags=flags)
+    # both launches by one native call: W and U are one allocation that nobody else sees
+    _check_inputs(K, V, beta, g_raw, (Q, S_in))
+    rows = B * T * H_v
+    tmp = torch.empty(rows * (d_k + d_v), dtype=V.dtype, device=V.device)
+    O = torch.empty_like(V)
+    S_out = torch.empty(B, H_v, d_v, d_k, dtype=torch.float32, device=V.device) if want_state else None
+    at = tmp.data_ptr()
+    rc = load_library().gdn_gated_delta_layer(Q.data_ptr(), K.data_ptr(), V.data_ptr(), beta.data_ptr(), g_raw.data_ptr(), B, H_k, H_v, T,
+                                              C, d_k, d_v, scale, None if S_in is None else S_in.data_ptr(), at, at + 2 * rows * d_k,
+                                              O.data_ptr(), None if S_out is None else S_out.data_ptr(), flags, _stream())
+    if rc != GDN_OK:
+        raise GdnError(rc, "gdn_gated_delta_layer")
+    return O, S_out
 
 
 def gdn_selftest_bounded_wait() -> int:

@@ -1091,7 +1091,7 @@ int chunk_state_auto_segments(long long H_v) {
         return 1;
     int P = 1;
     while (P < 8 && H_v * (2 * (P + 1) - 3) <= n_sm) ++P;
-    return P;
+    return P == 2 ? 1 : P;  // (two never pay: 64 heads x 256 chunks 512 us, 464 as one run each; a state-only chunk costs 0.85 of one with output)
 }
 
 // One sequence per value head (B = 1), cut into P segments: first pass = every segment's state map in parallel (state

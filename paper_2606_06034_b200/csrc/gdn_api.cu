@@ -233,6 +233,15 @@ int gdn_chunk_state_output(const void* Q, const void* K, const void* W_gated, co
     return launch_chunk_state(q, static_cast<cudaStream_t>(stream));
 }
 
+int gdn_gated_delta_layer(const void* Q, const void* K, const void* V, const float* beta, const float* g, int B, int H_k, int H_v,
+                          int T, int C, int d_k, int d_v, float scale, const float* S_in, void* W_tmp, void* U_tmp, void* O_out,
+                          float* S_out, unsigned flags, gdn_stream_t stream) {
+    if (flags & ~static_cast<unsigned>(GDN_FLAG_G_RAW | GDN_FLAG_LAYOUT_BTHD | GDN_FLAG_K_L2NORM)) return GDN_ERR_INVALID_ARG;
+    const int rc = gdn_chunk_prepare_ex(K, V, beta, g, B, H_k, H_v, T, C, d_k, d_v, -1, -1, GDN_DTYPE_BF16, W_tmp, U_tmp, nullptr,
+                                        flags | GDN_FLAG_W_GATED, stream);
+    return rc != GDN_OK ? rc : gdn_chunk_state_output(Q, K, W_tmp, U_tmp, g, B, H_k, H_v, T, C, d_k, d_v, scale, S_in, O_out, S_out, flags, stream);
+}
+
 int gdn_chunk_state_segments(int H_v) { return check_arch() == GDN_OK ? chunk_state_auto_segments(H_v) : 1; }
 
 size_t gdn_chunk_state_segmented_workspace(int H_v, int segments) {

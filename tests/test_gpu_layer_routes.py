@@ -137,3 +137,28 @@ def test_longest_first_gives_what_the_order_of_arrival_gives(n_seq, H_v):
         assert gdn.gdn_device_status() == gdn.GDN_OK
         assert torch.equal(O.view(torch.int16), On.view(torch.int16)) and torch.equal(S.view(torch.int32), Sn[:n_seq].view(torch.int32))
         assert torch.equal(Sn[n_seq:], S0[n_seq:])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,H_k,H_v,chunks", [(1, 1, 1, 1), (1, 2, 6, 3), (2, 3, 3, 5), (3, 16, 32, 2)])
+@pytest.mark.parametrize("token_major", [False, True])
+def test_one_native_call_gives_what_the_two_calls_give(B, H_k, H_v, chunks, token_major):
+    """Same kernels on the same inputs: the same bits, with and without a state carried in or asked for; and the argument errors of
+    the two calls."""
+    T = 64 * chunks
+    gen = torch.Generator(device="cuda").manual_seed(B + H_v)
+    r = lambda H, *d: torch.randn(*((B, T, H) if token_major else (B, H, T)), *d, generator=gen, device="cuda")
+    Q, K, V = r(H_k, 128).bfloat16(), r(H_k, 128).bfloat16(), r(H_v, 128).bfloat16()
+    beta, g, S0 = torch.sigmoid(r(H_v)), -torch.nn.functional.softplus(r(H_v)), 0.3 * torch.randn(B, H_v, 128, 128, generator=gen, device="cuda")
+    flags = gdn.GDN_FLAG_G_RAW | gdn.GDN_FLAG_K_L2NORM | (gdn.GDN_FLAG_LAYOUT_BTHD if token_major else 0)
+    W, U, _ = gdn.chunk_prepare(K, V, beta, g, 64, flags=flags | gdn.GDN_FLAG_W_GATED, want_tinv=False)
+    for S, want in ((None, True), (S0, True), (S0, False)):
+        O, Sn = gdn.gated_delta_layer(Q, K, V, beta, g, S_in=S, token_major=token_major, want_state=want)
+        Op, Sp = gdn.chunk_state_output(Q, K, W, U, g, 64, 128 ** -0.5, S, want_state=want, flags=flags)
+        assert gdn.gdn_device_status() == gdn.GDN_OK
+        assert torch.equal(O.view(torch.int16), Op.view(torch.int16)) and (Sn is None) == (Sp is None) == (not want)
+        assert Sn is None or torch.equal(Sn.view(torch.int32), Sp.view(torch.int32))
+    with pytest.raises(gdn.GdnError):
+        gdn.gated_delta_layer(Q, K, V, beta, g, C=32, token_major=token_major)
+    with pytest.raises(ValueError):
+        gdn.gated_delta_layer(torch.stack((Q, Q), -1)[..., 0], K, V, beta, g, token_major=token_major)

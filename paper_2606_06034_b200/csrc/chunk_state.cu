@@ -230,6 +230,11 @@ __device__ __forceinline__ void tmem_st_frag16(uint32_t taddr, const uint32_t (&
                  : "memory");
 }
 
+// the same with 8 columns
+__device__ __forceinline__ void tmem_st_frag8(uint32_t taddr, const uint32_t (&r)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+
 // Sequence of rank `rank` among the p.n_order <= 32 G of a packed call, longest class first, in their order inside a class; one
 // warp. Classes by the number of chunks: 0 .. 8, then four to a doubling. Bisection over the 32 classes, then the place inside
 // the class. Every CTA does it for itself, in the shadow of the TMEM allocation and of the loads of the sequence's bounds, which
@@ -858,7 +863,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 tmem_wait_ld();
 #pragma unroll
                 for (int lh = 0; lh < 2; ++lh) {
-                    uint32_t hi[8], lo[8];
+                    uint32_t hi[8], lo[8], shi[4], slo[4];  // (state only: the scaled form alone, the output product reads the plain one)
 #pragma unroll
                     for (int x = 0; x < 2; ++x) {
 #pragma unroll
@@ -870,14 +875,22 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                                 if (tq + 16 * ks + 8 * x >= left) u0 = 0.f;
                                 if (tq + 16 * ks + 8 * x + 1 >= left) u1 = 0.f;
                             }
-                            split_neg(mul2(pair2(u0, u1), f[ks][x]), hi[4 + 2 * x + fb], lo[4 + 2 * x + fb]);
-                            if (!SO) split_neg(u0, u1, hi[2 * x + fb], lo[2 * x + fb]);
-                            else hi[2 * x + fb] = lo[2 * x + fb] = 0u;  // (only the output product reads the plain form)
+                            if (SO) {
+                                split_neg(mul2(pair2(u0, u1), f[ks][x]), shi[2 * x + fb], slo[2 * x + fb]);
+                            } else {
+                                split_neg(mul2(pair2(u0, u1), f[ks][x]), hi[4 + 2 * x + fb], lo[4 + 2 * x + fb]);
+                                split_neg(u0, u1, hi[2 * x + fb], lo[2 * x + fb]);
+                            }
                         }
                     }
                     const uint32_t at = row + (static_cast<uint32_t>(lh * 16) << 16) + h * 32 + ks * 16;
-                    tmem_st_frag16(at + kD1, hi);
-                    tmem_st_frag16(at + kUL, lo);
+                    if (SO) {
+                        tmem_st_frag8(at + kD1 + 8, shi);
+                        tmem_st_frag8(at + kUL + 8, slo);
+                    } else {
+                        tmem_st_frag16(at + kD1, hi);
+                        tmem_st_frag16(at + kUL, lo);
+                    }
                 }
             }
             tmem_wait_st();

@@ -113,3 +113,16 @@ def test_forward_substitution_over_two_blocks_costs_its_terms(variant):
             runs.append(a.elapsed_time(b))
         time.append(min(runs))
     assert time[1] < 6 * time[0]
+
+
+@pytest.mark.parametrize("C,method", [(17, "neumann"), (24, "neumann"), (25, "neumann"), (32, "neumann"), (49, "fwdsubst"), (64, "fwdsubst")])
+@pytest.mark.parametrize("d_k,d_v", [(128, 128), (136, 72), (72, 200)])
+@pytest.mark.parametrize("flags", [0, gdn.GDN_FLAG_K_L2NORM | gdn.GDN_FLAG_W_GATED])
+def test_many_chunks_read_the_keys_again(C, method, d_k, d_v, flags):
+    """Launches of more chunks than fit at once read K a second time for W: the bits of a launch of one chunk."""
+    inp = gen.make_inputs(1, 1, 1, C, C, d_k, d_v, seed=C, dtype=torch.float32)
+    dev = [x.cuda() for x in (inp.K, inp.V, inp.beta, inp.g)]
+    one = gdn.chunk_prepare(*dev, C, method=method, flags=flags)
+    many = gdn.chunk_prepare(*(x.repeat(1300, *[1] * (x.dim() - 1)) for x in dev), C, method=method, flags=flags)
+    for a, b in zip(one, many):
+        assert torch.equal(a.expand_as(b), b)

@@ -263,40 +263,36 @@ struct SimtParams {
     const void *K, *V;
     const float *beta, *g;
     void *W, *U, *Tinv;
-    int H_k, H_v, T, C, d_k, d_v, N, S, mode, split;
+    int H_k, H_v, T, C, d_k, d_v, N, S, mode, split, again;
     unsigned flags;
 };
 
 // Shared memory in floats: X of every diagonal block, two work matrices per block (a slice of V overlays them once T is
-// complete), for two blocks the lower-left one, the slice of K, tables. AGAIN: the slice of K lies over the work matrices too,
+// complete), for two blocks the lower-left one, tables, the slice of K. With `again` that slice lies over the work matrices too,
 // which come into use when the Gram product has read it; it is read again for W.
-template <int G, int R, int NB, bool AGAIN>
+template <int G, int R, int NB>
 struct SimtSmem {
     static constexpr int M = G * R, ld = M + 4, mat = M * ld;
     static constexpr int tile = NB * M * kLdk;
     static constexpr int work = 2 * NB * mat > tile ? 2 * NB * mat : tile;
-    static constexpr int offX = 0, offW = NB * mat, offX21 = offW + work, offK = AGAIN ? offW : offX21 + (NB - 1) * mat;
-    static constexpr int offTab = offX21 + (NB - 1) * mat + (AGAIN ? 0 : tile), total = offTab + 4 * NB * M;
+    static constexpr int offX = 0, offW = NB * mat, offX21 = offW + work, offTab = offX21 + (NB - 1) * mat;
+    static constexpr int offK = offTab + 4 * NB * M, total = offK + tile;
+    static constexpr bool can_read_again = G == 8 && R >= 3;  // (elsewhere it gives no further CTA, or one at registers that spill)
 };
 
-// CTAs per SM that the registers are cut to. What the other warps of an SM hide is the latency of shared memory and of the
-// barriers of a chunk, so a few more CTAs at fewer registers (0 to 60 bytes spilled) pay where warps were missing (us before and
-// now, d = 128):
-//   64 threads: 8 rows 8 -> 14 CTAs (16384 chunks 80 -> 65), 16 rows 7 -> 10 (16384 chunks 152 -> 127; 8 are 135, 12 are 134);
-//   24 and 32 rows, AGAIN: 7 -> 10 and 5 -> 8 (16384 chunks of 24 238 -> 220, of 32 358 -> 326; 12 and 10 are 219 and 322, but
-//   2048 chunks 37.4 and 51.1 instead of 37.2 and 49.9).
-//   256 threads: 48 rows 2 -> 3 (1024 chunks 79 -> 76, 4096 293 -> 277; substitution, 2048 chunks 193 -> 158). 64 rows stay at 2
-//   in the scheme (AGAIN with 3: 1024 chunks 113 -> 114, 8192 837 -> 810); the substitution takes 3 (1024 chunks 164 -> 144).
-template <int G, int R, int NB, bool AGAIN>
+// CTAs per SM that the registers are cut to, as far as nothing is spilled. What the other warps of an SM hide is the latency of
+// shared memory and of the barriers of a chunk; 64 threads per CTA need many of them (us before and now, d = 128, 16384 chunks):
+// 8 rows 8 -> 14 CTAs 80 -> 65, 16 rows 7 -> 8 152 -> 135, 24 rows 7 -> 8 238 -> 226, 32 rows (K read again) 5 -> 8 358 -> 326.
+// (256 threads and three CTAs: 24 to 60 bytes spilled; chunks of 64 113 -> 114 with 1024 chunks.)
+template <int G, int R, int NB>
 constexpr int ctas_per_sm() {
-    if (G == 8) return R == 1 ? 14 : R == 2 ? 10 : !AGAIN ? 1 : R == 3 ? 10 : 8;
-    return NB == 2 ? 1 : R == 3 || AGAIN ? 3 : 2;
+    return G == 8 ? (R == 1 ? 14 : 8) : NB == 1 ? 2 : 1;
 }
 
 // G x G threads per diagonal block of G R rows (the chunk is padded to them with tokens that write nothing), NB blocks.
-template <typename IO, int G, int R, int NB, bool AGAIN>
-__global__ void __launch_bounds__(G* G* NB, (ctas_per_sm<G, R, NB, AGAIN>())) chunk_simt_kernel(const SimtParams p) {
-    using L = SimtSmem<G, R, NB, AGAIN>;
+template <typename IO, int G, int R, int NB>
+__global__ void __launch_bounds__(G* G* NB, (ctas_per_sm<G, R, NB>())) chunk_simt_kernel(const SimtParams p) {
+    using L = SimtSmem<G, R, NB>;
     constexpr int M = L::M, ld = L::ld, NG = G * G, NT = NG * NB;
     extern __shared__ __align__(16) float sm[];
     __shared__ float swt[4];
@@ -311,7 +307,8 @@ __global__ void __launch_bounds__(G* G* NB, (ctas_per_sm<G, R, NB, AGAIN>())) ch
     float* w0 = sm + L::offW + grp * 2 * L::mat;   // Abar, then E, row-major
     float* Et = w0 + L::mat;                       // E transposed
     float* A21 = sm + L::offX21;                   // -A21, finally T21 (row-major)
-    float* Ks = sm + L::offK;
+    const bool again = L::can_read_again && p.again;
+    float* Ks = sm + (again ? L::offW : L::offK);
     float* Vs = sm + L::offW;
     float* sbeta = sm + L::offTab;
     float* sg = sbeta + NB * M;
@@ -445,8 +442,8 @@ __global__ void __launch_bounds__(G* G* NB, (ctas_per_sm<G, R, NB, AGAIN>())) ch
     }
     __syncthreads();
     const bool k_scaled = (p.flags & (GDN_FLAG_K_L2NORM | GDN_FLAG_W_GATED)) != 0;
-    // the rows of K as W reads them (wider keys, and with AGAIN all, are loaded again, slice by slice)
-    if (!AGAIN && k_scaled && d_k <= kSliceW) scale_rows<NT>(Ks, swsc, NB * M, d_k);
+    // the rows of K as W reads them (wider keys, and with `again` all, are loaded again, slice by slice)
+    if (!again && k_scaled && d_k <= kSliceW) scale_rows<NT>(Ks, swsc, NB * M, d_k);
     if (p.mode == INV_NEUMANN) {
         // ---- band by distance (one row per thread, a barrier per distance: row i needs L_{d-e} of rows i - e)
         const int n = NB == 1 ? C : M;
@@ -633,9 +630,9 @@ __global__ void __launch_bounds__(G* G* NB, (ctas_per_sm<G, R, NB, AGAIN>())) ch
     constexpr int UW = 4 * G, per_slice = kSliceW / UW;
     const int nk = (d_k + UW - 1) / UW, nv = (d_v + UW - 1) / UW;
     const int u0 = (nk + nv) * share / p.split, u1 = (nk + nv) * (share + 1) / p.split;
-    int in_v = -1;  // slice in Vs (AGAIN: of K or V): index of its first unit
-    if (AGAIN) {
-        in_v = 0;  // (one CTA has all of a chunk: it begins with the first slice of K)
+    int in_v = -1;  // slice in Vs: index of its first unit
+    if (again) {    // (one CTA has all of a chunk: it begins with the first slice of K)
+        in_v = 0;
         load_tile<NT, 4 * G>(Ks, Kc, C, NB * M, d_k, min(kSliceW, d_k));
     } else if (u1 > nk) {
         in_v = nk + (max(u0, nk) - nk) / per_slice * per_slice;
@@ -676,12 +673,12 @@ __global__ void __launch_bounds__(G* G* NB, (ctas_per_sm<G, R, NB, AGAIN>())) ch
         const int end = min(min(first + per_slice, u1), is_v ? nk + nv : nk);
         const int d = is_v ? d_v : d_k, s0 = (first - (is_v ? nk : 0)) * UW;
         float* B = is_v ? Vs : Ks;
-        if (AGAIN || is_v ? in_v != first : d_k > kSliceW) {
+        if (is_v || again ? in_v != first : d_k > kSliceW) {
             __syncthreads();
             load_tile<NT, 4 * G>(B, (is_v ? Vc : Kc) + s0, C, NB * M, d, min(kSliceW, d - s0));
             v_ready = false;
         }
-        if (is_v ? !v_ready : AGAIN || d_k > kSliceW) {
+        if (is_v ? !v_ready : again || d_k > kSliceW) {
             load_wait();
             __syncthreads();
             if (is_v) {
@@ -724,16 +721,20 @@ __global__ void __launch_bounds__(G* G* NB, (ctas_per_sm<G, R, NB, AGAIN>())) ch
     }
 }
 
-template <typename IO, int G, int R, int NB, bool AGAIN = false>
+template <typename IO, int G, int R, int NB>
 int launch_one(SimtParams p, long long n_chunks, cudaStream_t stream) {
-    auto kern = chunk_simt_kernel<IO, G, R, NB, AGAIN>;
-    constexpr int smem = SimtSmem<G, R, NB, AGAIN>::total * 4;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return GDN_ERR_LAUNCH;
+    auto kern = chunk_simt_kernel<IO, G, R, NB>;
+    using L = SimtSmem<G, R, NB>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::total * 4) != cudaSuccess) return GDN_ERR_LAUNCH;
     // Fewer chunks than SMs: two or four CTAs share a chunk (each forms the inverse, its part of the columns of W and U), as
     // long as every CTA still has an SM of its own: 8 chunks of 64 take 21 us in four parts, where W and U are half the
     // work of a chunk; with more CTAs than SMs the repeated Gram product and rounds would be paid for twice.
     p.split = n_chunks * 4 <= kSMs ? 4 : n_chunks * 2 <= kSMs ? 2 : 1;
     if (n_chunks * p.split >= (1LL << 31)) return GDN_ERR_UNSUPPORTED;
+    // K read again instead of kept from the Gram product to W makes room for more CTAs per SM: from the number of chunks on that no
+    // longer fits at once with K kept (7 CTAs per SM up to 24 rows, 5 up to 32; 741 chunks of 32 27 -> 23 us, 1190 of 24 25 -> 23).
+    p.again = L::can_read_again && n_chunks > (R == 3 ? 7 : 5) * kSMs;
+    const int smem = (p.again ? L::offK : L::total) * 4;
     kern<<<static_cast<int>(n_chunks * p.split), G * G * NB, smem, stream>>>(p);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GDN_OK : GDN_ERR_LAUNCH;
@@ -745,15 +746,9 @@ int launch_size(const SimtParams& p, long long n_chunks, cudaStream_t stream) {
     const int C = p.C;
     if (C <= 8) return launch_one<IO, 8, 1, 1>(p, n_chunks, stream);
     if (C <= 16) return launch_one<IO, 8, 2, 1>(p, n_chunks, stream);
-    // K read again instead of kept from the Gram product to W (AGAIN) makes room for more CTAs per SM: from the number of chunks on
-    // that no longer fits at once with K kept (8 and 5 CTAs per SM; 1190 chunks of 24 25 -> 23 us, 741 of 32 27 -> 23 us).
-    if (C <= 24 && n_chunks > 8 * kSMs) return launch_one<IO, 8, 3, 1, true>(p, n_chunks, stream);
     if (C <= 24) return launch_one<IO, 8, 3, 1>(p, n_chunks, stream);
-    if (C <= 32 && n_chunks > 5 * kSMs) return launch_one<IO, 8, 4, 1, true>(p, n_chunks, stream);
     if (C <= 32) return launch_one<IO, 8, 4, 1>(p, n_chunks, stream);
     if (C <= 48) return launch_one<IO, 16, 3, 1>(p, n_chunks, stream);
-    // (two waves either way up to 4 chunks per SM: 512 chunks 87 us with K kept, 90 us with K read again)
-    if (C <= 64 && p.mode != INV_NEUMANN && n_chunks > 4 * kSMs) return launch_one<IO, 16, 4, 1, true>(p, n_chunks, stream);
     if (C <= 64) return launch_one<IO, 16, 4, 1>(p, n_chunks, stream);
     return launch_one<IO, 16, 4, 2>(p, n_chunks, stream);
 }
@@ -770,7 +765,7 @@ int launch_simt(const Problem& p, InverseMode mode, cudaStream_t stream) {
     }
     const long long n_chunks = (long long)p.B * p.H_v * (p.T / C);
     if (n_chunks == 0) return GDN_OK;
-    const SimtParams q{p.K, p.V, p.beta, p.g, p.W, p.U, p.Tinv, p.H_k, p.H_v, p.T, C, p.d_k, p.d_v, p.order, p.steps, (int)mode, 1, p.flags};
+    const SimtParams q{p.K, p.V, p.beta, p.g, p.W, p.U, p.Tinv, p.H_k, p.H_v, p.T, C, p.d_k, p.d_v, p.order, p.steps, (int)mode, 1, 0, p.flags};
     return p.dtype == GDN_DTYPE_FP32 ? launch_size<float>(q, n_chunks, stream) : launch_size<__nv_bfloat16>(q, n_chunks, stream);
 }
 

@@ -296,7 +296,11 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     __shared__ uint64_t bar_kq[kRing], bar_w[2], bar_u[2];  // tiles: loaded again behind a product that every reader precedes (see the loading warp)
     __shared__ uint64_t bar_nrm[4], bar_tab[4];  // norms (eight warps), tables (two warps) of chunk c: again behind hand-off 8 of chunk c + 1
     __shared__ uint64_t bar_pt, bar_o2;  // products: the next one waits for a hand-off that every reader makes behind this one
-    __shared__ uint64_t bar_d1[2], bar_su[2][2];  // [chunk & 1]([half of the state's columns]): the one of chunk c + 2 needs tiles that are asked for behind this one
+    __shared__ uint64_t bar_d1[2];  // S0 W^T: the one of chunk c + 2 needs a W tile that is asked for behind this one
+    // State update, either half of the state's columns. The chain warps, which alone wait for the first, precede the next one of either. The
+    // loading warp waits for the second too, and asks for nothing behind it that chunk c + 2 needs: it may be two chunks late there (three
+    // it may not: the W tile of chunk c + 3 is asked for behind it).
+    __shared__ uint64_t bar_su0[2], bar_su1[4];
     __shared__ uint64_t bar_ost[2], bar_stg[2];  // output tile staged (eight warps); staging buffer free again
     __shared__ uint64_t bar_end;      // products still in flight when the CTA gives up
     __shared__ uint32_t tmem_base_s;
@@ -319,12 +323,12 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             mbar_init(&bar_w[i], 1);
             mbar_init(&bar_u[i], 1);
             mbar_init(&bar_d1[i], 1);
-            mbar_init(&bar_su[i][0], 1);
-            mbar_init(&bar_su[i][1], 1);
+            mbar_init(&bar_su0[i], 1);
             mbar_init(&bar_ost[i], kAux / 32);
             mbar_init(&bar_stg[i], 1);
         }
         for (int i = 0; i < 4; ++i) {
+            mbar_init(&bar_su1[i], 1);
             mbar_init(&bar_nrm[i], kAux / 32);
             mbar_init(&bar_tab[i], kTabThreads / 32);
         }
@@ -481,7 +485,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     if (*fail != 0) break;
                     load_v(kOffW, &tmW, bar_w, n_w++);
                     if (c > 0) load_v(kOffU, &tmU, bar_u, n_u++);
-                    if (!wait_bar(&bar_su[c & 1][1], (c >> 1) & 1)) *fail = 1;
+                    if (!wait_bar(&bar_su1[c & 3], (c >> 2) & 1)) *fail = 1;
                     if (*fail != 0) break;
                     if (c == 0) load_v(kOffU, &tmU, bar_u, n_u++);
                     load_kq(n_kq++);
@@ -573,7 +577,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             mma_f16_ts(tm + kSD + half * 64, tm + (part == 0 ? kD1 : kUL) + ks * 16 + 8, desc_kt + (half * 8192 + ks * 2048) / 16,
                                        part == 0 ? idesc_mn64 : idesc_mn64 | kNegA, true);
                     }
-                    mma_commit(&bar_su[c & 1][half]);
+                    mma_commit(half == 0 ? &bar_su0[c & 1] : &bar_su1[c & 3]);
                 }
             }
             __syncwarp();
@@ -902,7 +906,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 // ---- bf16 copies (hi, -lo) of the new state for the next chunk's products, and its decay
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
-                    if (!(good = wait_for(&bar_su[c & 1][half], (c >> 1) & 1))) break;
+                    if (!(good = half == 0 ? wait_for(&bar_su0[c & 1], (c >> 1) & 1) : wait_for(&bar_su1[c & 3], (c >> 2) & 1))) break;
                     tc_fence_after_sync();
                     uint32_t v[32];
                     tmem_ld32(row + kSD + half * 64 + h * 32, v);
@@ -915,7 +919,7 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 }
                 if (!good) break;
             } else {
-                good = wait_for(&bar_su[c & 1][1], (c >> 1) & 1);
+                good = wait_for(&bar_su1[c & 3], (c >> 2) & 1);
                 tc_fence_after_sync();
             }
         }

@@ -1,7 +1,9 @@
 """The hand-offs between the warps of the state-passing kernel, as a model on the CPU: every warp is the sequence of barrier
 operations that it has in `chunk_state.cu`, a scheduler runs them in random orders, and any bounded wait may run out at any time.
 Whatever runs out where, every warp has to reach the end, and none may be counted twice in one generation of a hardware barrier
-(it would complete early, and what is left could never complete it again)."""
+(it would complete early, and what is left could never complete it again). A wait on an mbarrier asks for the parity of a phase:
+no warp, however slow, may still stand before its wait on a phase when the next phase of that barrier is complete too (the parity
+would read "not complete"), and nobody may arrive on a barrier before the phase that the arrival is meant for."""
 import itertools
 import os
 import random
@@ -12,7 +14,11 @@ import pytest
 SOURCE = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2606_06034_b200", "csrc", "chunk_state.cu")
 _CONST = dict(re.findall(r"constexpr int (kChain|kAux|kThreads|kTabThreads) = (\d+);", open(SOURCE).read()))
 N_CHAIN, N_AUX, N_TAB = (int(_CONST[k]) // 32 for k in ("kChain", "kAux", "kTabThreads"))
-RING = 3  # K, Q tiles
+RING = int(re.search(r"constexpr int kRing = (\d+);", open(SOURCE).read()).group(1))  # K, Q tiles
+# phases of every event that its barriers tell apart: chunk c is on barrier c mod this (kq .. stg as the kernel declares them)
+SLOTS = {name: RING if size == "kRing" else int(size or 1)
+         for line in re.findall(r"__shared__ uint64_t (bar_.*?);", open(SOURCE).read())
+         for name, size in re.findall(r"bar_(\w+)(?:\[(\w+)\])?", line)}
 
 
 class Stuck(Exception):
@@ -23,21 +29,50 @@ class Twice(Exception):
     pass
 
 
+class Overtaken(Exception):
+    pass
+
+
+class WrongPhase(Exception):
+    pass
+
+
 class Cta:
     """Warps are generators of operations: ("arrive" | "sync", barrier), ("wait", event) -> whether it came in time, ("count", event):
-    one of the arrivals that complete an event."""
+    one of the arrivals that complete an event. An event (name, chunk) is a phase of barrier chunk mod SLOTS[name]. `slow`: warps
+    that take a step only when nobody else can; without `lost` events no wait runs out then."""
 
-    def __init__(self, rng, n_c, so, short, lost, old):
-        self.rng, self.n_c, self.so, self.short, self.lost, self.old = rng, n_c, so, short, lost, old
+    def __init__(self, rng, n_c, so, nrm, lost=(), old=False, slow=None, slots=SLOTS):
+        self.rng, self.n_c, self.so, self.nrm, self.lost, self.old, self.slow, self.slots = rng, n_c, so, nrm, lost, old, slow, slots
         self.size = {4: N_CHAIN + 1 + N_TAB, 5: N_CHAIN + 1, 6: N_CHAIN + 1, 7: N_AUX + 1, 8: N_AUX + 1, 1: N_AUX, 3: N_TAB}
         self.needs = {"nrm": N_AUX, "tab": N_TAB, "ost": N_AUX}
         self.count = {b: [] for b in self.size}   # warps of the present generation
         self.arrived = {}
-        self.done, self.coming, self.fail = set(), set(), False
+        self.phases, self.fail = {}, False         # barrier -> phases that are complete
+        self.loads, self.products = [], []         # on their way: loads in any order, products in the order they were issued
 
-    def signal(self, *event):  # a load or a product: it completes some time later, or never
-        if event not in self.lost:
-            self.coming.add(event)
+    def barrier(self, name, c):
+        n = self.slots[name]
+        return (name, c % n), c // n
+
+    def signal(self, name, c):  # a load, a product or a store: it completes some time later, or never
+        bar, phase = self.barrier(name, c)
+        if self.phases.get(bar, 0) != phase and not self.fail:
+            raise WrongPhase((name, c))
+        if (name, c) not in self.lost:
+            (self.loads if name in ("kq", "w", "u", "stg") else self.products).append((name, c))
+
+    def complete(self, name, c):
+        bar, phase = self.barrier(name, c)
+        if self.phases.get(bar, 0) != phase and not self.fail:
+            raise WrongPhase((name, c))
+        self.phases[bar] = max(self.phases.get(bar, 0), phase + 1)
+
+    def come(self, name, c):
+        bar, phase = self.barrier(name, c)
+        if self.phases.get(bar, 0) > phase + 1 and not self.fail:
+            raise Overtaken((name, c))
+        return self.phases.get(bar, 0) > phase
 
     def chain(self, w):
         n_c = self.n_c
@@ -79,7 +114,7 @@ class Cta:
         taken = 0
 
         def norms(c):
-            if c >= n_c:
+            if c >= n_c or not self.nrm:
                 return True
             if so and w >= N_CHAIN + N_AUX // 2:
                 yield "count", ("nrm", c)
@@ -91,7 +126,7 @@ class Cta:
         good = yield from norms(0)
         if so:
             c = 1
-            while good and c < n_c:
+            while good and self.nrm and c < n_c:
                 good = c < 2 or (yield "wait", ("tab", c - 2))
                 good = good and (yield from norms(c))
                 c += 1
@@ -127,7 +162,8 @@ class Cta:
             if self.old and self.fail:
                 break
             yield "sync", 3
-            yield "wait", ("nrm", c)
+            if self.nrm:
+                yield "wait", ("nrm", c)
             yield "count", ("tab", c)
             yield "wait", ("kq", c)
             yield "wait", ("w", c)
@@ -139,9 +175,6 @@ class Cta:
 
         def load(what, c):
             assert (what, c) not in asked
-            # the barrier's phase before is complete: an arrival on it twice in one phase is a fault of the GPU
-            before = c - (RING if what == "kq" else 2)
-            assert before < 0 or (what, before) in self.done, (what, c)
             if c < n_c:
                 asked.add((what, c))
                 self.signal(what, c)
@@ -194,8 +227,10 @@ class Cta:
     def run(self):
         kinds = [self.chain] * N_CHAIN + [self.aux] * N_AUX + [self.issuer, self.producer] + [self.tabler] * N_TAB
         warps = [k(i) for i, k in enumerate(kinds)]
-        frozen = self.rng.choice([-1, *range(len(warps))])  # runs when nothing else can, until a wait has run out
-        early = self.rng.choice((0.0, 0.002))  # how often a wait runs out though something could still go on
+        patient = self.slow is not None
+        # slow warps run when nothing else can; of those that the test does not name, until a wait has run out
+        slow = self.slow if patient else {self.rng.choice([-1, *range(len(warps))])}
+        early = 0.0 if patient else self.rng.choice((0.0, 0.002))  # how often a wait runs out though something could still go on
         pending = {}  # warp -> operation it stands at
         asleep = {}   # warp -> barrier it waits on
 
@@ -208,12 +243,15 @@ class Cta:
         for i in range(len(warps)):
             step(i)
         while pending:
-            ready = [i for i in pending if i not in asleep and (pending[i][0] != "wait" or pending[i][1] in self.done)]
-            waiting = [i for i in pending if pending[i][0] == "wait" and pending[i][1] not in self.done]
-            awake = [i for i in ready if i != frozen or self.fail]
-            if self.coming and (self.rng.random() < 0.3 or not awake):
-                self.done.add(self.coming.pop())
-            elif waiting and (not awake or self.rng.random() < (0.1 if self.fail else early)):
+            ready = [i for i in pending if i not in asleep and (pending[i][0] != "wait" or self.come(*pending[i][1]))]
+            waiting = [i for i in pending if pending[i][0] == "wait" and not self.come(*pending[i][1])]
+            awake = [i for i in ready if i not in slow or (self.fail and not patient)]
+            if (self.loads or self.products) and (self.rng.random() < 0.3 or not awake):
+                if self.loads and (not self.products or self.rng.random() < 0.5):
+                    self.complete(*self.loads.pop(self.rng.randrange(len(self.loads))))
+                else:
+                    self.complete(*self.products.pop(0))
+            elif waiting and not (patient and ready) and (not awake or self.rng.random() < (0.1 if self.fail else early)):
                 self.fail = True
                 step(self.rng.choice(waiting), False)
             elif ready:
@@ -223,9 +261,12 @@ class Cta:
                     step(i, True)
                     continue
                 if kind == "count":
+                    bar, phase = self.barrier(*what)
+                    if self.phases.get(bar, 0) != phase and not self.fail:
+                        raise WrongPhase(what)
                     self.arrived[what] = self.arrived.get(what, 0) + 1
                     if self.arrived[what] == self.needs[what[0]] and what not in self.lost:
-                        self.done.add(what)
+                        self.complete(*what)
                     step(i)
                     continue
                 here = self.count[what]
@@ -247,16 +288,17 @@ class Cta:
                 raise Stuck({i: pending[i] for i in pending})
 
 
-def _lost(n_c, so):
+def _lost(n_c, so, nrm):
     """No event lost, and every single one of each kind in turn."""
-    return [set()] + [{(e, c)} for c in range(n_c) for e in ("kq", "w", "u", "d1", "su0", "su1", "nrm", "tab") + (() if so else ("pt", "o2", "ost", "stg"))]
+    kinds = ("kq", "w", "u", "d1", "su0", "su1", "tab") + (("nrm",) if nrm else ()) + (() if so else ("pt", "o2", "ost", "stg"))
+    return [set()] + [{(e, c)} for c in range(n_c) for e in kinds]
 
 
-@pytest.mark.parametrize("so,short", [(False, False), (False, True), (True, False)])
-def test_every_warp_leaves_whatever_runs_out(so, short):
+@pytest.mark.parametrize("so,nrm", [(False, True), (False, False), (True, True), (True, False)])
+def test_every_warp_leaves_whatever_runs_out(so, nrm):
     for n_c in (1, 2, 4):
-        for lost, seed in itertools.product(_lost(n_c, so), range(40 if n_c < 4 else 12)):
-            Cta(random.Random(seed), n_c, so, short, lost, old=False).run()
+        for lost, seed in itertools.product(_lost(n_c, so, nrm), range(40)):
+            Cta(random.Random(seed), n_c, so, nrm, lost).run()
 
 
 def test_the_model_sees_warps_that_leave_early():
@@ -265,7 +307,31 @@ def test_the_model_sees_warps_that_leave_early():
     stuck = 0
     for seed in range(40):
         try:
-            Cta(random.Random(seed), 3, False, False, {("kq", 1)}, old=True).run()
+            Cta(random.Random(seed), 3, False, True, {("kq", 1)}, old=True).run()
         except Stuck:
             stuck += 1
     assert stuck > 0
+
+
+WARPS = N_CHAIN + N_AUX + 2 + N_TAB
+# one warp of each part, and the ones of a part that do something of their own (norms of K, norms of Q)
+SLOW = [{0}, {N_CHAIN}, {N_CHAIN + N_AUX - 1}, {WARPS - N_TAB - 2}, {WARPS - N_TAB - 1}, {WARPS - 1}, {WARPS - N_TAB - 1, 0},
+        {WARPS - N_TAB - 1, N_CHAIN}, {WARPS - N_TAB - 1, WARPS - 1}, set()]
+
+
+@pytest.mark.parametrize("so,nrm", [(False, True), (False, False), (True, True), (True, False)])
+def test_no_phase_is_lost_however_slow_a_warp_is(so, nrm):
+    """Nothing is lost and nothing runs out; the slow warps stay behind as far as the others can go without them. More chunks than twice
+    the longest ring."""
+    for slow, seed in itertools.product(SLOW, range(6)):
+        cta = Cta(random.Random(seed), 9, so, nrm, slow=slow)
+        cta.run()
+        assert not cta.fail
+
+
+@pytest.mark.parametrize("so,nrm", [(False, True), (False, False), (True, True), (True, False)])
+def test_the_model_sees_a_phase_that_is_overtaken(so, nrm):
+    """Two barriers for the state update's completion: the loading warp is two chunks behind before anybody needs what it asks for."""
+    with pytest.raises(Overtaken):
+        for seed in range(6):
+            Cta(random.Random(seed), 9, so, nrm, slow={WARPS - N_TAB - 1}, slots={**SLOTS, "su0": 2, "su1": 2}).run()

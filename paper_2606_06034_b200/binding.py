@@ -524,7 +524,7 @@ def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_s
     else:
         (B, H_k, T, d_k), H_v, d_v = K.shape, V.shape[1], V.shape[3]
     # one long sequence per head and fewer heads than SMs: the segments of a sequence run in parallel
-    if B == 1 and T // C > 33 and _segments_pay(T, C, int(load_library().gdn_chunk_state_segments(H_v))):
+    if B == 1 and 0 < C <= T and T // C > 33 and _segments_pay(T, C, int(load_library().gdn_chunk_state_segments(H_v))):
         W, U, _ = chunk_prepare(K, V, beta, g_raw, C, flags=flags | GDN_FLAG_W_GATED, want_tinv=False)
         O, S = chunk_state_output_segmented(Q[0], K[0], W[0], U[0], g_raw[0], C, scale, None if S_in is None else S_in[0],
                                             want_state=want_state, flags=flags)

@@ -160,5 +160,9 @@ def test_one_native_call_gives_what_the_two_calls_give(B, H_k, H_v, chunks, toke
         assert Sn is None or torch.equal(Sn.view(torch.int32), Sp.view(torch.int32))
     with pytest.raises(gdn.GdnError):
         gdn.gated_delta_layer(Q, K, V, beta, g, C=32, token_major=token_major)
+    for C in (0, -64):
+        with pytest.raises(gdn.GdnError) as e:
+            gdn.gated_delta_layer(Q, K, V, beta, g, C=C, token_major=token_major)
+        assert e.value.status == gdn.GDN_ERR_INVALID_ARG
     with pytest.raises(ValueError):
         gdn.gated_delta_layer(torch.stack((Q, Q), -1)[..., 0], K, V, beta, g, token_major=token_major)

@@ -139,6 +139,16 @@ def test_binding_refuses_host_tensors():
         gdn.chunk_prepare(K, K, b, b, 64)
 
 
+@pytest.mark.parametrize("B,C", [(1, 0), (2, 0), (1, -64), (1, 64)])
+def test_layer_call_refuses_host_tensors_whatever_the_chunk_size(lib, B, C):
+    """Also where the choice of the state passing, which divides by the chunk size, comes before the call itself."""
+    import torch
+    K = torch.zeros(B, 64, 2, 128, dtype=torch.bfloat16)
+    g = torch.zeros(B, 64, 2)
+    with pytest.raises(ValueError):
+        gdn.gated_delta_layer(K, K, K, g, g, C)
+
+
 def test_chunk_table_of_packed_sequences():
     """Host-side chunking of packed sequences (each sequence chunked from its own first token, last chunk short),
     against the oracle's own table."""

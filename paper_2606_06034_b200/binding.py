@@ -427,6 +427,9 @@ def chunk_state_output_segmented(Q, K, W_gated, U, g, C, scale=1.0, S_in=None, *
     else:
         H_k, T, d_k = K.shape
         H_v, _, d_v = U.shape
+    for t in (Q, K, W_gated, U, g, S_in):
+        if t is not None and (not t.is_cuda or not t.is_contiguous()):
+            raise ValueError("all tensors must be contiguous CUDA tensors (there is no CPU path)")
     lib = load_library()
     if segments <= 0:  # (two where the library proposes none though the first pass fits the SMs: who calls this wants segments)
         segments = int(lib.gdn_chunk_state_segments(H_v))
@@ -435,9 +438,6 @@ def chunk_state_output_segmented(Q, K, W_gated, U, g, C, scale=1.0, S_in=None, *
     need = int(lib.gdn_chunk_state_segmented_workspace(H_v, segments))
     if workspace is None and need > 0:
         workspace = torch.empty(need, dtype=torch.uint8, device=U.device)
-    for t in (Q, K, W_gated, U, g, S_in):
-        if t is not None and (not t.is_cuda or not t.is_contiguous()):
-            raise ValueError("all tensors must be contiguous CUDA tensors (there is no CPU path)")
     O = torch.empty_like(U)
     S_out = torch.empty(H_v, d_v, d_k, dtype=torch.float32, device=U.device) if want_state else None
     rc = lib.gdn_chunk_state_output_segmented(_ptr(Q), _ptr(K), _ptr(W_gated), _ptr(U), _ptr(g), H_k, H_v, T, C, d_k, d_v,

@@ -213,3 +213,12 @@ def test_int16_and_fp32_kernels_spill_no_more_than_was_measured_to_be_free():
     assert len(main) == 2 and all(v["spill_stores"] == 0 and v["registers"] <= 128 for v in main)
     res = gdn_build.kernel_resources("chunk_simt.cu")
     assert len(res) == 14 and all(v["spill_stores"] <= (4 if "Li16E" in k else 0) for k, v in res.items())
+
+
+@pytest.mark.parametrize("H_v", [2, 64])
+def test_segmented_call_refuses_host_tensors(lib, H_v):
+    """Also for the head counts at which the number of segments is chosen by the device's SMs."""
+    import torch
+    x = torch.zeros(H_v, 128, 128, dtype=torch.bfloat16)
+    with pytest.raises(ValueError, match="CUDA tensors"):
+        gdn.chunk_state_output_segmented(x, x, x, x, torch.zeros(H_v, 128), 64)

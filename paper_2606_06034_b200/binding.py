@@ -500,11 +500,13 @@ def chunk_state_output(Q, K, W_gated, U, g, C, scale=1.0, S_in=None, *, want_sta
     return O, S_out
 
 
-def _segments_pay(T, C, segments):
-    """Whether the segmented state passing is the faster one: its four launches cost about 35 + 3 P us more than a plain
-    one and its two passes 4.5 / P us a chunk against 2.7. (Kernels as they are now, plain / segmented, us: P = 3, 37 chunks 72 / 74,
-    60 chunks 114 / 101; P = 8, 28 chunks 56 / 65, 40 chunks 77 / 68: the layer call also asks for more than 33 chunks.)"""
-    return segments > 1 and (T // C) * (2.7 - 4.5 / segments) > 35 + 3 * segments
+def _segments_pay(T, C, segments, heads=1):
+    """Whether the segmented state passing is the faster one for `segments` P per sequence: a chunk costs 1.7 - 3.1 / P us less, the
+    call 17 + 3.7 P us more, and 9 more where the four CTAs per head that combine the segments no longer run at once on the SMs.
+    Layer calls, plain / segmented, us: P = 8 (4 heads) 34 chunks 78 / 81, 38 chunks 86 / 81; P = 6 (16 heads) 31 chunks 80 / 84, 37
+    chunks 97 / 94; P = 4 (26 heads) 30 chunks 89 / 92, 38 chunks 105 / 103; P = 3 (32 heads) 34 chunks 101 / 104, 50 chunks 141 / 135,
+    (44 heads) 42 chunks 138 / 145, 58 chunks 185 / 179."""
+    return segments > 1 and (T // C) * (1.7 - 3.1 / segments) > 17 + 3.7 * segments + (9 if 4 * heads > 148 else 0)
 
 
 def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_seqlens=None, token_major=True,
@@ -523,8 +525,9 @@ def gated_delta_layer(Q, K, V, beta, g_raw, C=64, scale=None, S_in=None, *, cu_s
         (B, T, H_k, d_k), (H_v, d_v) = K.shape, V.shape[2:]
     else:
         (B, H_k, T, d_k), H_v, d_v = K.shape, V.shape[1], V.shape[3]
-    # one long sequence per head and fewer heads than SMs: the segments of a sequence run in parallel
-    if B == 1 and 0 < C <= T and T // C > 33 and _segments_pay(T, C, int(load_library().gdn_chunk_state_segments(H_v))):
+    # one long sequence per head and fewer heads than SMs: the segments of a sequence run in parallel (up to 32 chunks no number of
+    # them pays, and the library is not asked for it)
+    if B == 1 and 0 < 32 * C < T and _segments_pay(T, C, int(load_library().gdn_chunk_state_segments(H_v)), H_v):
         W, U, _ = chunk_prepare(K, V, beta, g_raw, C, flags=flags | GDN_FLAG_W_GATED, want_tinv=False)
         O, S = chunk_state_output_segmented(Q[0], K[0], W[0], U[0], g_raw[0], C, scale, None if S_in is None else S_in[0],
                                             want_state=want_state, flags=flags)

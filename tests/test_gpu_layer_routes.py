@@ -7,11 +7,12 @@ from paper_2606_06034_b200 import binding as gdn
 FLAGS = gdn.GDN_FLAG_G_RAW | gdn.GDN_FLAG_LAYOUT_BTHD | gdn.GDN_FLAG_K_L2NORM
 
 
-@pytest.mark.parametrize("segments,first", [(2, 92), (3, 37), (4, 30), (6, 28), (8, 28)])
-def test_line_between_plain_and_segmented(segments, first):
-    assert not gdn._segments_pay(64 * (first - 1), 64, segments)
-    assert gdn._segments_pay(64 * first, 64, segments)
-    assert not gdn._segments_pay(64 * 100000, 64, 1) and not gdn._segments_pay(0, 64, segments)
+@pytest.mark.parametrize("segments,heads,first", [(3, 37, 43), (3, 38, 56), (4, 29, 35), (5, 21, 33), (6, 16, 34), (7, 13, 35), (8, 11, 36)])
+def test_line_between_plain_and_segmented(segments, heads, first):
+    assert not gdn._segments_pay(64 * (first - 1), 64, segments, heads)
+    assert gdn._segments_pay(64 * first, 64, segments, heads)
+    assert not gdn._segments_pay(64 * 100000, 64, 1, heads) and not gdn._segments_pay(0, 64, segments, heads)
+    assert not gdn._segments_pay(64 * 32, 64, segments, heads)  # (the layer call does not ask up to there)
 
 
 @pytest.mark.parametrize("bounds,T,whole", [([0, 5, 9], 9, True), ([0, 0, 9, 9], 9, True), ([0, 5], 9, False), ([1, 9], 9, False),
@@ -31,12 +32,13 @@ def _inputs(T, H_k, H_v, seed):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("H_k,H_v,chunks", [(1, 2, 1), (1, 2, 2), (1, 2, 27), (1, 2, 28), (16, 32, 36), (16, 32, 37), (32, 64, 91), (32, 64, 92)])
+@pytest.mark.parametrize("H_k,H_v,chunks", [(1, 2, 1), (1, 2, 2), (1, 2, 35), (1, 2, 36), (16, 32, 42), (16, 32, 43), (19, 38, 55), (19, 38, 56),
+                                            (32, 64, 92)])
 @pytest.mark.parametrize("with_state", [False, True])
 def test_layer_on_both_sides_of_the_line(H_k, H_v, chunks, with_state):
     """Both forms compute the same chain; they differ by the fp32 re-association of the state recurrence (at most 2^-24 per
     token of decay-free carry, far below 1e-5 of the state) and, where that flips a rounding of the output, by one bf16 unit
-    (2^-8) of single elements."""
+    (2^-8) of single elements. The layer gives the bits of the form that the line asks for."""
     Q, K, V, beta, g, S = _inputs(64 * chunks, H_k, H_v, chunks)
     S = S if with_state else None
     O, Sn = gdn.gated_delta_layer(Q, K, V, beta, g, S_in=S)
@@ -48,6 +50,9 @@ def test_layer_on_both_sides_of_the_line(H_k, H_v, chunks, with_state):
     for o, s in ((Op, Sp), (Os[None], Ss[None])):
         assert (Sn - s).norm() <= 1e-5 * s.norm()
         assert (O.float() - o.float()).norm() <= 1e-3 * o.float().norm()
+    segmented = gdn._segments_pay(64 * chunks, 64, int(gdn.load_library().gdn_chunk_state_segments(H_v)), H_v)
+    o, s = (Os[None], Ss[None]) if segmented else (Op, Sp)
+    assert torch.equal(O.view(torch.int16), o.view(torch.int16)) and torch.equal(Sn.view(torch.int32), s.view(torch.int32))
 
 
 @pytest.mark.gpu
@@ -71,7 +76,7 @@ def test_the_line_is_on_the_right_side_of_the_clock(H_v, chunks):
             torch.cuda.synchronize()
             runs.append(a.elapsed_time(b))
         time.append(min(runs))
-    segmented = gdn._segments_pay(64 * chunks, 64, int(gdn.load_library().gdn_chunk_state_segments(H_v)))
+    segmented = gdn._segments_pay(64 * chunks, 64, int(gdn.load_library().gdn_chunk_state_segments(H_v)), H_v)
     assert time[segmented] < time[not segmented]
 
 

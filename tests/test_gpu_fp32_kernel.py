@@ -126,3 +126,25 @@ def test_many_chunks_read_the_keys_again(C, method, d_k, d_v, flags):
     many = gdn.chunk_prepare(*(x.repeat(1300, *[1] * (x.dim() - 1)) for x in dev), C, method=method, flags=flags)
     for a, b in zip(one, many):
         assert torch.equal(a.expand_as(b), b)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("C,method,flags", [(C, "neumann", f) for C in (17, 24, 32) for f in (
+    0, gdn.GDN_FLAG_G_RAW, gdn.GDN_FLAG_G_RAW | gdn.GDN_FLAG_K_L2NORM | gdn.GDN_FLAG_W_GATED)] + [(32, "fwdsubst", 0)])
+def test_keys_read_again_are_the_chunks_own(dtype, C, method, flags):
+    """1080 different chunks in one launch (K read again) and the same batches in launches of 360 (K kept): the same bits. Grouped
+    heads, several chunks per sequence, raw gates, features of an odd slice, both tensor types."""
+    B, H_k, H_v, n = 36, 2, 6, 5
+    r = torch.Generator(device="cuda").manual_seed(C + flags)
+    rand = lambda *s: torch.randn(*s, generator=r, device="cuda")
+    K = torch.nn.functional.normalize(rand(B, H_k, n * C, 136), dim=-1).to(dtype)
+    V, beta = rand(B, H_v, n * C, 72).to(dtype), torch.sigmoid(rand(B, H_v, n * C))
+    g = -torch.nn.functional.softplus(rand(B, H_v, n * C))
+    if not flags & gdn.GDN_FLAG_G_RAW:
+        g = g.view(B, H_v, n, C).cumsum(-1).view(B, H_v, n * C)
+    many = gdn.chunk_prepare(K, V, beta, g, C, method=method, flags=flags)
+    for b in range(0, B, 12):
+        few = gdn.chunk_prepare(K[b:b + 12], V[b:b + 12], beta[b:b + 12], g[b:b + 12], C, method=method, flags=flags)
+        for x, y in zip(many, few):
+            assert torch.equal(x[b:b + 12], y)
+    assert gdn.gdn_device_status() == gdn.GDN_OK

@@ -171,3 +171,55 @@ def test_one_native_call_gives_what_the_two_calls_give(B, H_k, H_v, chunks, toke
         assert e.value.status == gdn.GDN_ERR_INVALID_ARG
     with pytest.raises(ValueError):
         gdn.gated_delta_layer(torch.stack((Q, Q), -1)[..., 0], K, V, beta, g, token_major=token_major)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,H_k,H_v,chunks,with_state", [(1, 16, 32, 1, True), (3, 2, 4, 5, False), (8, 16, 32, 3, True), (1, 1, 2, 40, True)])
+def test_layer_call_can_be_captured_and_replayed_on_new_inputs(B, H_k, H_v, chunks, with_state):
+    """The native call (its second launch is a programmatic edge of the graph) and the segmented form: what the replay writes are
+    the bits of a call outside of a graph, for the inputs captured and for others in their place."""
+    def inputs(seed):
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        r = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+        T = 64 * chunks
+        return [r(B, T, H_k, 128).bfloat16(), r(B, T, H_k, 128).bfloat16(), r(B, T, H_v, 128).bfloat16(), torch.sigmoid(r(B, T, H_v)),
+                -torch.nn.functional.softplus(r(B, T, H_v))] + ([0.3 * r(B, H_v, 128, 128)] if with_state else [])
+
+    x = inputs(1)
+    call = lambda t: gdn.gated_delta_layer(*t[:5], S_in=t[5] if with_state else None)
+    want = [[y.clone() for y in call(inputs(seed))] for seed in (1, 2, 3)]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        O, S = call(x)
+    for seed in (1, 2, 3):
+        for a, b in zip(x, inputs(seed)):
+            a.copy_(b)
+        graph.replay()
+        graph.replay()
+        assert torch.equal(O.view(torch.int16), want[seed - 1][0].view(torch.int16))
+        assert torch.equal(S.view(torch.int32), want[seed - 1][1].view(torch.int32))
+    assert gdn.gdn_device_status() == gdn.GDN_OK
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,H_k,H_v,T,cu", [(1, 16, 32, 4096, None), (8, 32, 32, 1024, None), (1, 16, 32, 64, None),
+                                            (1, 16, 32, 4111, [0, 5, 69, 700, 701, 1725, 2000, 3999, 4111])])
+def test_repeated_layer_calls_are_bit_identical(B, H_k, H_v, T, cu):
+    """No atomics on data and a fixed order of every sum, in the state passing too: repeated calls agree bit for bit, also while
+    another stream keeps the memory system busy."""
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    r = lambda *s: torch.randn(*(s if cu is None else s[1:]), generator=gen, device="cuda")
+    args = (r(B, T, H_k, 128).bfloat16(), r(B, T, H_k, 128).bfloat16(), r(B, T, H_v, 128).bfloat16(), torch.sigmoid(r(B, T, H_v)),
+            -torch.nn.functional.softplus(r(B, T, H_v)))
+    ref = gdn.gated_delta_layer(*args, cu_seqlens=cu)
+    assert gdn.gdn_device_status() == gdn.GDN_OK
+    side, junk = torch.cuda.Stream(), torch.empty(64 << 20, dtype=torch.uint8, device="cuda")
+    for rep in range(8):
+        if rep % 2 == 1:
+            with torch.cuda.stream(side):
+                for _ in range(8):
+                    junk.add_(1)
+        O, S = gdn.gated_delta_layer(*args, cu_seqlens=cu)
+        assert torch.equal(O.view(torch.int16), ref[0].view(torch.int16)) and torch.equal(S.view(torch.int32), ref[1].view(torch.int32))
+    torch.cuda.synchronize()
+    assert gdn.gdn_device_status() == gdn.GDN_OK

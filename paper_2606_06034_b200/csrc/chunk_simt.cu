@@ -22,6 +22,7 @@
 // of 4 (mod 8) words keeps the reads free of bank conflicts. C = 64, d = 128: 1024 chunks 111 us (one entry per thread and
 // step, two scalar reads per multiply-add: 1016 us), 8 chunks 21 us (216 us).
 #include "common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace gdn {
 namespace {
@@ -37,16 +38,12 @@ __device__ __forceinline__ void st4(__nv_bfloat16* p, float4 v) {
 __device__ __forceinline__ void st(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 
-typedef unsigned long long f2;  // two packed fp32
+using sm100::f2;
+using sm100::pair2;
 __device__ __forceinline__ void fma2(f2& acc, f2 a, f2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b)); }
-__device__ __forceinline__ f2 dup2(float x) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
-    return r;
-}
 __device__ __forceinline__ float2 split2(f2 v) {
     float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    sm100::unpair2(v, r.x, r.y);
     return r;
 }
 __device__ __forceinline__ float sum2(f2 v) {
@@ -161,7 +158,8 @@ __device__ __forceinline__ void prod_rows(f2 (&acc)[R][NC * 2], const float* X, 
                 for (int c = 0; c < NC; ++c) b[c] = *reinterpret_cast<const ulonglong2*>(B + (j + jj) * kLdk + col + c * 4 * G);
 #pragma unroll
                 for (int r = FULL ? 0 : q; r < R; ++r) {
-                    const f2 x = dup2(jj == 0 ? a[r].x : jj == 1 ? a[r].y : jj == 2 ? a[r].z : a[r].w);
+                    const float e = jj == 0 ? a[r].x : jj == 1 ? a[r].y : jj == 2 ? a[r].z : a[r].w;
+                    const f2 x = pair2(e, e);
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
                         fma2(acc[r][2 * c], x, b[c].x);

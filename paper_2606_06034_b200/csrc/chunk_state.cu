@@ -170,25 +170,9 @@ __device__ __forceinline__ void tmem_ld8_split8(uint32_t taddr, uint32_t (&r)[8]
                  : "r"(taddr)
                  : "memory");
 }
-typedef unsigned long long f2;  // two packed fp32
-__device__ __forceinline__ f2 pair2(float a, float b) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 __device__ __forceinline__ uint32_t pack_pair(f2 v) {
     float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    unpair2(v, a, b);
     return pack_bf16x2(a, b);
 }
 // half HI of a bf16 pair minus x, in fp32 (one instruction, no unpacking)

@@ -100,31 +100,6 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-// Two packed fp32: one instruction for two elements (the same roundings). In the A-build, the sums of the levels and the scaling of the W / U
-// operands: 4 x 16 heads x 4096 tokens 77.5 -> 76.8 us, chunks of 128 100.9 -> 99.9, layer call of 8 x 4096 tokens 636 -> 627.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 pair2(float a, float b) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpair2(f2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-    f2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 __device__ __forceinline__ void compute_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // bounded mbarrier wait: polls, and every 1024 polls compares the clock with a budget of about a second

@@ -116,10 +116,9 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity) {
 
 // The same for a whole warp, with one answer for all its lanes (the hardware barriers behind it count warps). It also gives
 // up when another warp has: the lanes still polling then vote on one last poll. Lanes that have left the loop have seen the
-// phase complete, so that poll sees it too. (A vote on every poll, or a look at `fail` before the first one, costs the chain of
-// the sequence 20 to 40 cycles a chunk: 32 heads x 32768 tokens 1217 and 1207 us instead of 1199.) What follows the first poll is
-// one function for the seven places that wait: in line it is code that a short call fetches for nothing (the same shape 1204
-// instead of 1192 us, one chunk 34.8 instead of 34.5).
+// phase complete, so that poll sees it too. (A vote on every poll gives the same times.) What follows the first poll is
+// one function for the places that wait. In line it is twice the code: layer calls of 8 x 4096 tokens 730 instead of 715 us, 32768
+// tokens 1026 instead of 1038, one chunk 22.6 instead of 22.9.
 __device__ __noinline__ bool wait_bar_slow(uint64_t* bar, uint32_t parity, const volatile int* fail) {
     const long long t0 = clock64();
     uint32_t i = 0;
@@ -270,8 +269,8 @@ chunk_state_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                    const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmU,
                    const __grid_constant__ CUtensorMap tmO, const ParamsS p) {
     extern __shared__ uint8_t smem_raw[];
-    // (an offset, so that the compiler goes on to know it as shared memory: 32768 tokens, 32 heads 992 -> 967 us for the layer call, 8 x 4096
-    // tokens 744 -> 691, 61 packed prompts 482 -> 469)
+    // (an offset, so that the compiler goes on to know it as shared memory: 32768 tokens, 32 heads 1052 -> 1038 us for the layer call, 8 x 4096
+    // tokens 740 -> 715, 61 packed prompts 482 -> 470)
     uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
     float* gtab = reinterpret_cast<float*>(smem + kOffG);  // (see kTab)
 

@@ -482,7 +482,12 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const int warp = tid >> 5;
     const int lane = tid & 31;
 
-    if constexpr (EX == 1 || EX == 3) launch_dependents();  // (the layer call's state passing follows: it waits for this kernel's end itself)
+    if constexpr (EX == 1 || EX == 3) {
+        // The layer call's state passing follows and waits for this kernel's end itself. It takes all of an SM's TMEM at its start: none of its
+        // CTAs (more than 200 KB of shared memory) may have room beside one of these that has not allocated its own columns yet.
+        static_assert(L::kTotal >= 64 * 1024, "the next kernel's CTAs must not fit beside these");
+        launch_dependents();
+    }
     if (tid == 0) {
         mbar_init(&bar_k, 1);
         mbar_init(&bar_v, 1);
@@ -515,8 +520,8 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_s;
 
-    // (S is known where the doubling form was chosen. As a constant it saves a register: chunks of 128 107 -> 101 us without a spill, layer call
-    // of 8 x 4096 tokens 662 -> 641; the default instantiation's code came out 1 % slower with it)
+    // (S is known where the doubling form was chosen; as a constant it saves a register: chunks of 128, 4 x 16 heads x 4096 tokens, 115.5 ->
+    // 108.1 us, layer call of 8 x 4096 tokens 724 -> 715, 61 packed prompts 482 -> 472)
     const int N = p.N, S = DBL != 0 && (MERGE || EX != 0) ? DBL : p.S;
     // width of the band kept in fp32 (lb[]): the order N, or all of NB for forward substitution
     const int n_band = (MODE == INV_NEUMANN) ? N : NB;
@@ -536,8 +541,8 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // rows, B operands) keeps using t; TMEM columns no longer depend on the chunk (the two chunks sit on different
     // lanes of the same columns); a warp holds two groups of 16 consecutive rows, which leave as two bulk stores.
     // M = 64 instructions take as long as M = 128 ones (and the doubling levels need twice as many of them), so at full
-    // clocks this form is ~10 % slower; it draws less power, and a launch long enough to run into the power cap is
-    // faster with it. The host picks it for large launches (launch_tc_bf16).
+    // clocks this form is 3 % slower; it draws less power, and on a GPU that runs at the power cap it is 3.5 % faster. The
+    // host picks it for large launches (launch_tc_bf16).
     static_assert(!PERM || (C == 64 && !MERGE && MODE == INV_NEUMANN && EX == 0 && DBL != 0), "built for the default 64-chunk path");
     constexpr bool kPerm = PERM;
     const int lrow = tid & 127;  // TMEM lane of this thread's row
@@ -709,9 +714,8 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         if (C == 64 && EX == 0 && !PERM && !MERGE && warp == 0 && has_next && elect_one()) {
             // The next tile's K can only land in shared memory once this tile's W products are done with the buffer,
             // which leaves its load little time before the next Gram product wants it: ask for it in L2 now. Only in the default
-            // form (4 x 16 heads x 4096 tokens 79.7 us with, 80.5 without): the M = 64 form for large launches loses by it (stress 4643 and
-            // 4520 us), chunks of 128 too (107 and 101), and with the optional layouts it costs 28 bytes of spill (8 x 4096 tokens of
-            // the layer call 698 and 680).
+            // form (4 x 16 heads x 4096 tokens 85.1 us with, 85.7 without): the others gain nothing by it (chunks of 128 109.0 and 108.1, layer
+            // call of 8 x 4096 tokens 721 and 715, the M = 64 form 2423 and 2417 for 65536 tiles).
             const TileCoord nc = tile_coord<EX>(pos_next, p);
             tma_prefetch_l2_3d(&tmK, nc.kx, nc.t0, nc.kz);
             tma_prefetch_l2_3d(&tmK, nc.kx + 64, nc.t0, nc.kz);
@@ -815,7 +819,9 @@ chunk_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     rj[0] = rq.x; rj[1] = rq.y; rj[2] = rq.z; rj[3] = rq.w;
                 }
                 if constexpr (C == 64) {
-                    // (see below: entries on and above the diagonal only have to be finite)
+                    // (see below: entries on and above the diagonal only have to be finite. Two elements an instruction here, in the sums of
+                    // the levels and in the scaling of the W / U operands: 4 x 16 heads x 4096 tokens 86.0 -> 85.1 us, layer call of 8 x 4096
+                    // tokens 721 -> 715.)
 #pragma unroll
                     for (int q = 0; q < 4; q += 2) {
                         const int jl = j4 * 4 + q;
@@ -1935,7 +1941,7 @@ int launch_c(const Maps& m, const Params& prm, cudaStream_t stream, bool perm = 
 
 
 namespace {
-constexpr long long kM64MinTiles = 32768;  // 65 536 chunks of 64 tokens: a launch of about 1.2 ms
+constexpr long long kM64MinTiles = 32768;  // 65 536 chunks of 64 tokens: a launch of 1.1 to 1.25 ms
 // waits on an mbarrier that never completes: wait_bar must give up after its budget and report it
 __global__ void wait_selftest_kernel(int* status) {
     __shared__ uint64_t bar;
@@ -1982,8 +1988,11 @@ int launch_tc_bf16(const Problem& p, InverseMode mode, cudaStream_t stream) {
     if (!make_map(&m.K, p.K, zk, t_in, ck, 64, in_rows, CU_TENSOR_MAP_SWIZZLE_128B)) return GDN_ERR_LAUNCH;
     if (!make_map(&m.V, p.V, zv, t_in, cv, 64, in_rows, CU_TENSOR_MAP_SWIZZLE_128B)) return GDN_ERR_LAUNCH;
     // Large launches of the default 64-chunk path (no flags, S = 8 or 15) run the form whose tensor-core products are
-    // M = 64 instructions per chunk (kPerm in the kernel): it draws less power, and a launch of a millisecond or more
-    // runs into the power cap, where that is worth more than the ~10 % it costs at full clocks. Its warps hold 16 rows
+    // M = 64 instructions per chunk (kPerm in the kernel): it draws less power. Which form is faster depends on the state of
+    // the GPU more than on the size. Default and M = 64, us, one launch after idle (full clocks) | launches back to back at
+    // the power cap (1627 to 1770 and 1770 to 1920 MHz): 2048 tiles 85, 87 | 85.5, 82.7; 8192 296, 307 | 320, 310; 32768 1092, 1126 | 1257,
+    // 1215; 131072 4182, 4314 | 4981, 4809; 1024 tiles do not reach the cap (45.5, 46.1). A launch of a millisecond or more
+    // is taken for work that keeps the GPU at the cap, a shorter one not. Its warps hold 16 rows
     // of each of a tile's two chunks, so its W, U and Tinv rows leave in boxes of 16 rows. (GDN_FORCE_M64 = 1 / 0 in the
     // environment forces the choice: the tests run both forms on small cases.)
     const long long n_tiles_all = (long long)p.B * p.H_v * ((p.T + kTile - 1) / kTile);

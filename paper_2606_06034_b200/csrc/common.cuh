@@ -98,8 +98,8 @@ enum InverseMode { INV_NEUMANN = 0, INV_FWDSUBST_ROWS = 1, INV_FWDSUBST_BLOCKED 
 
 // Launches a kernel that may be set up while the kernel before it in the stream still runs, if that one has allowed it
 // (launch_dependents); the kernel waits for that one's end and its writes (grid_dependency_wait) before it touches memory. Behind any
-// other kernel it is an ordinary launch. Layer calls, before and now: 32768 tokens, 32 heads 994 and 987 us, 8 x 4096 tokens 714 and 708, one
-// chunk of 32 heads (from a graph) 23.4 and 22.9. Between the four launches of the segmented call the same costs time (the pass
+// other kernel it is an ordinary launch. One chunk of 32 heads as a layer call 24.7 -> 22.9 us; long calls
+// gain less than their runs differ. Between the four launches of the segmented call the same costs time (the pass
 // that waits holds SMs that the one before could use: 993 and 1159).
 template <typename... P, typename... A>
 inline bool launch_behind(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, A... args) {
